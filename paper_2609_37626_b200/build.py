@@ -1,4 +1,5 @@
-"""Builds libsplash_mla.so in-tree with nvcc for sm_100a (cross-compiles without a GPU)."""
+"""Builds libsplash_mla.so in-tree with nvcc for sm_100a (cross-compiles without a GPU), and the extension module that
+takes torch tensors to it."""
 from __future__ import annotations
 
 import glob
@@ -9,6 +10,8 @@ import sys
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libsplash_mla.so")
+TORCH_SRC = os.path.join(CSRC, "splash_torch.cpp")
+TORCH_EXT = os.path.join(HERE, "_splash_torch.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -21,21 +24,40 @@ def sources():
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
 
 
-def needs_build() -> bool:
-    if not os.path.exists(LIB):
+def _older(target: str, deps) -> bool:
+    if not os.path.exists(target):
         return True
-    t = os.path.getmtime(LIB)
-    deps = sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(
-        os.path.join(HERE, "..", "include", "*.h"))
+    t = os.path.getmtime(target)
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def _headers():
+    return glob.glob(os.path.join(HERE, "..", "include", "*.h"))
+
+
+def _build_torch_ext() -> None:
+    """The extension is a host file against torch's C++ headers; it finds the library beside it and torch's libraries
+    in the process (the package imports torch first)."""
+    import sysconfig
+
+    from torch.utils import cpp_extension
+    flags = ["-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden", "-D_GLIBCXX_USE_CXX11_ABI=1"]
+    for path in cpp_extension.include_paths() + [sysconfig.get_paths()["include"], "/usr/local/cuda/include"]:
+        flags += ["-isystem", path]
+    libs = ["-L" + HERE, "-lsplash_mla"]
+    for path in cpp_extension.library_paths():
+        libs.append("-L" + path)
+    libs += ["-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_cuda", "-ltorch_python", "-Wl,-rpath,$ORIGIN"]
+    subprocess.check_call([os.environ.get("CXX", "g++")] + flags + ["-o", TORCH_EXT, TORCH_SRC] + libs)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    if not force and not needs_build():
-        return LIB
-    nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
-    cmd = [nvcc] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) + ["-o", LIB] + sources()
-    subprocess.check_call(cmd)
+    if force or _older(LIB, sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + _headers()):
+        nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
+        cmd = [nvcc] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) + ["-o", LIB] + sources()
+        subprocess.check_call(cmd)
+    if force or _older(TORCH_EXT, [TORCH_SRC] + _headers()):
+        _build_torch_ext()
     return LIB
 
 
