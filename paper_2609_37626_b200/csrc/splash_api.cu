@@ -255,27 +255,36 @@ int decode_dense(const splash_mla_shape *shape, const void *q, const void *kv_po
     const bool simt = (shape->flags & SPLASH_FLAG_SIMT) != 0;
     // R query rows per request: the kernels see R * num_heads virtual heads (head g, row r -> g * R + r: the rows
     // of a head are dense, so a virtual head is 576 / 512 elements from the next) and mask causally by
-    // (virtual head mod R); a slice wider than 128 virtual heads runs as several CTA pairs per KV worker in ONE launch
-    // chain (the loop below has a single pass).
+    // (virtual head mod R); a slice wider than 128 virtual heads runs as several CTA pairs per KV worker in one launch
     const int R = shape->q_rows > 1 ? (int)shape->q_rows : 1;
     const int vbegin = head_begin * R, vend = head_end * R;
-    const int vstep = vend - vbegin;
+    const int h = vend - vbegin;
+    cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     cudaError_t e = cudaSuccess;
     // a page-copy job: its table rewrite runs first; its page copy rides in the decode kernel if that is a CTA-pair
-    // kernel (one pass only), else runs as a kernel of its own after the decode
+    // kernel, else runs as a kernel of its own after the decode
     bool job_copy_pending = job != nullptr;
-    if (job != nullptr) e = run_migrate_job(job, true, false, static_cast<cudaStream_t>(stream_));
-    for (int vb = vbegin; vb < vend && e == cudaSuccess; vb += vstep) {
-    const int ve = vb + vstep < vend ? vb + vstep : vend;
-    const int h = ve - vb;
+    if (job != nullptr) e = run_migrate_job(job, true, false, stream);
     Tiling t = choose_tiling(shape, h, dev.sm_count, simt);
     const bool fused_sparse = sparse && sparse->fused && !simt;
     if (fused_sparse) { t.heads_per_group = 64; t.num_groups = 2; t.num_workers = dev.sm_count / 2 > 0 ? dev.sm_count / 2 : 1; t.pair_groups = 1; }
+    // where the work partition comes from (splash_common.cuh): a batch of up to 32 requests is planned by the decode kernel
+    // itself; if its contexts are short besides, no request is cut and the combine kernel is left out
+    int plan_mode = kPlanWorkspace;
+    if (!simt && !(shape->flags & SPLASH_FLAG_VALIDATE) && B <= kInlinePlanRequests) {
+        const int pages = sparse ? sparse->pages_per_request : shape->block_table_stride;
+        // (the e4m3 pair kernel's own plan saves 4 us and costs 2.6 % of its main loop: long contexts keep the plan kernel,
+        // unless the call takes a partition over, which may have been one that left nothing in the workspace)
+        const bool e4m3_pairs = shape->kv_dtype == SPLASH_KV_E4M3_TOKEN_SCALE && t.num_groups == 2 && t.heads_per_group == 64 &&
+                                !(shape->flags & (SPLASH_FLAG_NO_PAIR | SPLASH_FLAG_REUSE_PLAN));
+        if (!e4m3_pairs || (int64_t)B * pages * t.pair_groups <= kInlinePairPages)
+            plan_mode = pages <= kWholeRequestPages && B <= t.num_workers ? kPlanWhole : kPlanInline;
+        if (plan_mode == kPlanWhole) t.num_workers = B;
+    }
     PlanView v = make_plan_view(workspace, B, t.num_workers, h);
     if (workspace_bytes < v.bytes) {
         set_error("workspace has %zu bytes, %zu needed", workspace_bytes, v.bytes); return SPLASH_INVALID_ARG;
     }
-    cudaStream_t stream = static_cast<cudaStream_t>(stream_);
 
     DecodeParams p;
     memset(&p, 0, sizeof p);
@@ -284,13 +293,14 @@ int decode_dense(const splash_mla_shape *shape, const void *q, const void *kv_po
     p.q_stride_request = shape->q_stride_request; p.q_stride_head = R > 1 ? kDQK : shape->q_stride_head;
     p.out_stride_request = shape->out_stride_request; p.out_stride_head = R > 1 ? kDV : shape->out_stride_head;
     p.lse_stride_request = shape->lse_stride_request;
-    p.B = B; p.H = shape->num_heads * R; p.head_begin = vb; p.head_end = ve; p.q_rows = R;
+    p.B = B; p.H = shape->num_heads * R; p.head_begin = vbegin; p.head_end = vend; p.q_rows = R;
     p.table_stride = shape->block_table_stride; p.num_pool_pages = shape->num_pool_pages;
     p.heads_per_group = t.heads_per_group; p.num_groups = t.num_groups; p.num_workers = t.num_workers;
     p.pair_groups = t.pair_groups;
     p.softmax_scale = shape->softmax_scale;
     p.tile_start = v.tile_start; p.req_lo = v.req_lo; p.req_hi = v.req_hi; p.worker_begin = v.worker_begin;
-    p.worker_req = v.worker_req;
+    p.worker_req = v.worker_req; p.split_rec = v.split_rec;
+    p.plan_mode = plan_mode; p.kv_begin = kv_begin; p.kv_end = kv_end;
     p.status = v.status; p.partial_lse = v.partial_lse; p.partial_out = v.partial_out; p.partial_scale = v.partial_scale;
     p.trace = g_trace;
     p.len_cap = sparse ? sparse->max_selected : -1;
@@ -307,7 +317,7 @@ int decode_dense(const splash_mla_shape *shape, const void *q, const void *kv_po
         p.request_overhead_tiles = kRequestOverheadTilesPair;
     // the bf16 CTA-pair kernel writes its partial outputs as f16
     p.partial_f16 = (pair && shape->kv_dtype == SPLASH_KV_BF16 && !fused_sparse) ? 1 : 0;
-    if (job_copy_pending && pair && !fused_sparse && vend - vbegin <= vstep) {
+    if (job_copy_pending && pair && !fused_sparse) {
         p.mig_src = static_cast<const uint4 *>(job->src_pool); p.mig_dst = static_cast<uint4 *>(job->dst_pool);
         p.mig_src_scales = reinterpret_cast<const uint4 *>(job->src_scales); p.mig_dst_scales = reinterpret_cast<uint4 *>(job->dst_scales);
         p.mig_src_ids = job->src_page_ids; p.mig_dst_ids = job->dst_page_ids;
@@ -318,34 +328,31 @@ int decode_dense(const splash_mla_shape *shape, const void *q, const void *kv_po
     // the previous call's partition taken again (the same batch in the next layer): no plan kernel, only the error words
     // of the status block are cleared (word 8, the number of split requests, belongs to the plan)
     const bool reuse_plan = (shape->flags & SPLASH_FLAG_REUSE_PLAN) && !(shape->flags & SPLASH_FLAG_VALIDATE) && !sparse;
-    e = record_timing_event(0, stream);
-    if (e == cudaSuccess) {
-        if (reuse_plan) {
-            if (vb == vbegin) e = cudaMemsetAsync(v.status, 0, 8 * sizeof(int32_t), stream);
-        } else {
-            e = launch_plan(p, kv_begin, kv_end, v.tile_start, v.req_lo, v.req_hi, v.req_wfirst, v.req_wlast,
-                            v.cost_start, v.worker_begin, v.split_list, v.worker_req, v.split_rec, v.status, vb == vbegin, stream);
-        }
+    if (e == cudaSuccess) e = record_timing_event(0, stream);
+    if (e == cudaSuccess && plan_mode == kPlanWorkspace) {
+        if (!reuse_plan) e = launch_plan(p, v, stream);
+        else if (simt) e = cudaMemsetAsync(v.status, 0, 8 * sizeof(int32_t), stream);
+        else p.clear_status = 1;
     }
     if (e == cudaSuccess) e = record_timing_event(1, stream);
     // validation mode: the table entries the call will use, checked on the device before the decode kernel runs
-    if (e == cudaSuccess && (shape->flags & SPLASH_FLAG_VALIDATE) && !sparse && vb == vbegin)
+    if (e == cudaSuccess && (shape->flags & SPLASH_FLAG_VALIDATE) && !sparse)
         e = launch_validate_pages(p, v.req_lo, v.req_hi, stream);
     if (e == cudaSuccess && sparse && !fused_sparse)
         e = launch_sparse_gather(B, sparse->max_selected, sparse->pages_per_request, sparse->pool656, sparse->num_pool_pages,
                                  sparse->block_table, sparse->table_stride, sparse->ctx_lens, sparse->sel, sparse->sel_stride,
-                                 sparse->sel_count, const_cast<void *>(kv_pool), sparse->dense_table, dev.sm_count, stream);
+                                 sparse->sel_count, const_cast<void *>(kv_pool), sparse->dense_table, dev.sm_count,
+                                 plan_mode == kPlanWorkspace, stream);
     if (e == cudaSuccess) {
         if (simt) e = launch_decode_simt(p, shape->kv_dtype, stream);
         else if (fused_sparse) e = launch_decode_sparse_pair(p, stream);
         else e = launch_decode_umma(p, *shape, stream);
     }
     if (e == cudaSuccess) e = record_timing_event(2, stream);
-    if (e == cudaSuccess) e = launch_split_combine(p, v.split_rec, stream);
+    if (e == cudaSuccess && plan_mode != kPlanWhole) e = launch_split_combine(p, v.split_rec, stream);
     if (e == cudaSuccess) e = record_timing_event(3, stream);
     if (e == cudaSuccess && g_timing) g_events_recorded = true;
-    }
-    if (e == cudaSuccess && job_copy_pending) e = run_migrate_job(job, false, true, static_cast<cudaStream_t>(stream_));
+    if (e == cudaSuccess && job_copy_pending) e = run_migrate_job(job, false, true, stream);
     if (e != cudaSuccess) { set_error("CUDA error: %s", cudaGetErrorString(e)); return SPLASH_CUDA_ERROR; }
     return SPLASH_OK;
 }

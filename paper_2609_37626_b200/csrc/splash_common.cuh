@@ -139,6 +139,10 @@ struct DecodeParams {
     int64_t mig_page_vecs;
     int32_t mig_n;
     int32_t request_overhead_tiles;   // per-request cost the plan adds to the tile count
+    int32_t plan_mode;                // kPlanWorkspace, kPlanInline or kPlanWhole
+    int32_t clear_status;             // 1: no plan kernel ran (its partition is taken again): block 0 clears the error words
+    const int32_t *kv_begin, *kv_end; // the inline modes read the ranges themselves
+    int4 *split_rec;                  // kPlanInline: where block 0 leaves the combine kernel's records
     long long *trace;          // optional device buffer for pipeline timestamps (diagnostics), or NULL
 };
 
@@ -151,21 +155,176 @@ struct Segment {
     int32_t slot;                   // partial slot, or -1 when the piece is the whole request
 };
 
+// ---- programmatic dependent launch ---------------------------------------------
+// The three kernels of a decode call are chained with programmatic stream serialisation:
+// a dependent kernel may be scheduled while its predecessor is still running, does its
+// own set-up (barriers, tensor memory), and blocks in grid_dependency_wait() before it
+// touches anything the predecessor wrote.
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Where a decode kernel's partition comes from.  Workspace: the plan kernel wrote it.  Inline: a batch of at most 32
+// requests is one lane each, so a warp of every CTA works the partition out for itself in a shuffle scan while the plan
+// kernel of such a call would still be in its launch (a tiny decode: 16.4 us with the plan kernel in front, see
+// build_inline_plan); the numbers are the plan kernel's.  Whole: inline, and no request is cut -- worker i takes request
+// i -- so that there is nothing to combine either.
+enum { kPlanWorkspace = 0, kPlanInline = 1, kPlanWhole = 2 };
+constexpr int kInlinePlanRequests = 32;
+constexpr int kWholeRequestPages = 4;
+constexpr int kInlinePairPages = 8192;
+// shared-memory copy of an inline plan: tile_start[B + 1], lo[B], hi[B] (as in the workspace), then the worker's first
+// tile, its end, and the request that holds the first
+constexpr uint32_t kInlinePlanBytes = ((3 * kInlinePlanRequests + 4) * 4 + 15) / 16 * 16;
+
+// Effective range of request i (the rule of the plan kernel).
+__device__ __forceinline__ void effective_range(int s, const int32_t *kv_begin, const int32_t *kv_end, int i, int len_cap, int &lo, int &hi) {
+    if (len_cap >= 0 && (s < 0 || s > len_cap)) s = 1;     // a list count out of bounds: one (poisoned) row
+    lo = kv_begin ? kv_begin[i] : 0;
+    hi = kv_end ? kv_end[i] : s;
+    if (lo < 0) lo = 0;
+    if (hi > s) hi = s;
+    if (hi < lo) hi = lo;
+}
+
+// floor(total * w / W) without 64-bit division: total = a W + b, floor = a w + floor(b w / W)
+__device__ __forceinline__ int cost_target(int total, int w, int W) {
+    const int a = total / W, b = total - a * W;
+    return a * w + (b * w) / W;
+}
+
+// One warp of a CTA: the plan, as far as worker `worker` needs it.
+static __device__ __noinline__ void build_inline_plan(const DecodeParams &p, int worker, int32_t *sp, int lane) {
+    const int B = p.B, W = p.num_workers, overhead = p.request_overhead_tiles;
+    int lo = 0, hi = 0;
+    if (lane < B) effective_range(p.seq_lens[lane], p.kv_begin, p.kv_end, lane, p.len_cap, lo, hi);
+    const int n = hi > lo ? (hi + kPage - 1) / kPage - lo / kPage : 0;
+    const int c = n > 0 ? n + overhead : 0;
+    int sn = n, sc = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int a = __shfl_up_sync(0xffffffffu, sn, o), b = __shfl_up_sync(0xffffffffu, sc, o);
+        if (lane >= o) { sn += a; sc += b; }
+    }
+    if (lane == 0) sp[0] = 0;
+    if (lane < B) { sp[lane + 1] = sn; sp[B + 1 + lane] = lo; sp[2 * B + 1 + lane] = hi; }
+    if (p.plan_mode == kPlanWhole) {
+        if (lane == worker) { sp[3 * B + 1] = sn - n; sp[3 * B + 2] = sn; sp[3 * B + 3] = worker; }
+        return;
+    }
+    const int tiles = __shfl_sync(0xffffffffu, sn, 31), cost = __shfl_sync(0xffffffffu, sc, 31);
+    // first tile of worker w (the same w in all lanes) and the request that holds it: as many requests lie before it as
+    // end at or before its share of the cost
+    auto start = [&](int w, int &req) {
+        req = 0;
+        if (w >= W || cost == 0) return tiles;
+        const int target = cost_target(cost, w, W);
+        req = __popc(__ballot_sync(0xffffffffu, sc <= target));
+        const int off = target - __shfl_sync(0xffffffffu, sc - c, req) - overhead;
+        return __shfl_sync(0xffffffffu, sn - n, req) + max(off, 0);
+    };
+    int req, unused;
+    const int wb = start(worker, req), we = start(worker + 1, unused);
+    if (lane == 0) { sp[3 * B + 1] = wb; sp[3 * B + 2] = we; sp[3 * B + 3] = req; }
+}
+
+// The same warp of block 0, once its CTA is under way: clears the status block (this cannot wipe another CTA's report: the
+// first one a CTA can make is the end of a bounded wait, seconds after this) and leaves in the workspace what the combine
+// kernel reads, the workers' first tiles and the list of the requests that were cut.
+static __device__ __noinline__ void publish_inline_plan(const DecodeParams &p, const int32_t *ts, int lane) {
+    const int B = p.B, W = p.num_workers, overhead = p.request_overhead_tiles;
+    int split = 0;
+    if (p.plan_mode == kPlanInline) {
+        const int rs = lane < B ? ts[lane] : ts[B], re = lane < B ? ts[lane + 1] : rs;
+        const int c = re > rs ? re - rs + overhead : 0;
+        int sc = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int b = __shfl_up_sync(0xffffffffu, sc, o);
+            if (lane >= o) sc += b;
+        }
+        const int cost = __shfl_sync(0xffffffffu, sc, 31);
+        int32_t *const worker_begin = const_cast<int32_t *>(p.worker_begin);
+        int wf = -1, wl = -1;         // the last workers that start at or before the request's first / last tile
+        for (int w0 = 0; w0 <= W; w0 += 32) {
+            const int w = w0 + lane, target = w < W ? cost_target(cost, w, W) : 0;
+            int k = 0;
+            for (int j = 0; j < B; ++j) k += __shfl_sync(0xffffffffu, sc, j) <= target ? 1 : 0;
+            const int off = target - __shfl_sync(0xffffffffu, sc - c, k) - overhead;
+            int g = __shfl_sync(0xffffffffu, rs, k) + max(off, 0);
+            if (w >= W || cost == 0) g = ts[B];
+            if (w <= W) worker_begin[w] = g;
+            for (int j = 0; j < 32 && w0 + j < W; ++j) {
+                const int gj = __shfl_sync(0xffffffffu, g, j);
+                wf += gj <= rs ? 1 : 0;
+                wl += gj <= re - 1 ? 1 : 0;
+            }
+        }
+        const unsigned cut = __ballot_sync(0xffffffffu, re > rs && wf != wl);
+        split = __popc(cut);
+        if ((cut >> lane) & 1u) p.split_rec[__popc(cut & ((1u << lane) - 1u))] = make_int4(lane, wf, wl, rs);
+    }
+    if (lane < 16) p.status[lane] = lane == 8 ? split : 0;
+}
+
 // Iterates the segments of worker w in plan order.  Every thread of a CTA calls
-// it with the same arguments and gets the same answer.
+// it with the same arguments and gets the same answer.  kPlanOffset: where an inline plan lies in dynamic shared memory;
+// kPlanInWorkspace: the kernel is launched behind a plan kernel only.
+constexpr uint32_t kPlanInWorkspace = 0xffffffffu;
+template <uint32_t kPlanOffset>
 struct SegmentIter {
+    int32_t x, end, wb, i, w;
+    static __device__ __forceinline__ int32_t *inline_plan() {
+        extern __shared__ __align__(1024) uint8_t smem[];
+        return reinterpret_cast<int32_t *>(smem + kPlanOffset);
+    }
+    // tile_start[B + 1]; lo[B] and hi[B] follow it, in the workspace and in an inline plan alike
+    static __device__ __forceinline__ const int32_t *tile_start(const DecodeParams &p) {
+        return p.plan_mode != kPlanWorkspace ? inline_plan() : p.tile_start;
+    }
+    __device__ void init(const DecodeParams &p, int worker) {
+        w = worker;
+        // i: the request containing tile x (last i with ts[i] <= x and ts[i+1] > x): the plan has it, which saves every
+        // role of every CTA a bisection of a dozen dependent global loads before its first tile
+        if (p.plan_mode != kPlanWorkspace) {
+            const int32_t *own = inline_plan() + 3 * p.B + 1;
+            wb = own[0]; x = wb; end = own[1]; i = own[2];
+        } else {
+            wb = p.worker_begin[worker]; x = wb; end = p.worker_begin[worker + 1];
+            i = x < end ? p.worker_req[worker] : 0;
+        }
+    }
+    __device__ bool next(const DecodeParams &p, Segment &s) {
+        if (x >= end) return false;
+        const int32_t *ts = tile_start(p);
+        while (ts[i + 1] <= x) ++i;                    // skip finished / empty requests
+        int rs = ts[i], re = ts[i + 1];
+        int seg_end = re < end ? re : end;
+        s.request = i;
+        s.tile_begin = x - rs;
+        s.tile_end = seg_end - rs;
+        s.lo = ts[p.B + 1 + i];
+        s.hi = ts[2 * p.B + 1 + i];
+        bool full = (x == rs) && (seg_end == re);
+        s.slot = full ? -1 : 2 * w + (rs <= wb ? 0 : 1);
+        x = seg_end;
+        return true;
+    }
+};
+
+// The same on the workspace's arrays only.
+template <>
+struct SegmentIter<kPlanInWorkspace> {
     const int32_t *ts;
     int32_t B, x, end, wb, i, w;
+    static __device__ __forceinline__ const int32_t *tile_start(const DecodeParams &p) { return p.tile_start; }
     __device__ void init(const DecodeParams &p, int worker) {
         ts = p.tile_start; B = p.B; w = worker;
         wb = p.worker_begin[worker]; x = wb; end = p.worker_begin[worker + 1];
-        // the request containing tile x (last i with ts[i] <= x and ts[i+1] > x): the plan has it, which saves every
-        // role of every CTA a bisection of a dozen dependent global loads before its first tile
         i = x < end ? p.worker_req[worker] : 0;
     }
     __device__ bool next(const DecodeParams &p, Segment &s) {
         if (x >= end) return false;
-        while (ts[i + 1] <= x) ++i;                    // skip finished / empty requests
+        while (ts[i + 1] <= x) ++i;
         int rs = ts[i], re = ts[i + 1];
         int seg_end = re < end ? re : end;
         s.request = i;
@@ -180,10 +339,32 @@ struct SegmentIter {
     }
 };
 
+// The beginning of a decode kernel, all threads: the plan's origin by the call's mode.  `plan_warp`: a warp that is not
+// needed at once.
+template <uint32_t kPlanOffset>
+__device__ __forceinline__ void start_plan(const DecodeParams &p, int worker, int plan_warp, SegmentIter<kPlanOffset> &it) {
+    if constexpr (kPlanOffset != kPlanInWorkspace) {
+        if (p.plan_mode != kPlanWorkspace) {
+            const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+            int32_t *sp = it.inline_plan();
+            // no combine kernel follows and every CTA is running: the next call's first kernel may set up on the SMs left
+            if (p.plan_mode == kPlanWhole) grid_launch_dependents();
+            if (warp == plan_warp) build_inline_plan(p, worker, sp, lane);
+            __syncthreads();
+            if (blockIdx.x == 0 && warp == plan_warp) publish_inline_plan(p, sp, lane);
+            it.init(p, worker);
+            return;
+        }
+    }
+    if (p.clear_status && blockIdx.x == 0 && threadIdx.x < 8) p.status[threadIdx.x] = 0;      // (see publish_inline_plan)
+    it.init(p, worker);
+}
+
 // Requests whose effective KV range is empty belong to no segment: O = 0, LSE = -inf is
 // written by the decode CTA (worker, head group) with worker == request mod num_workers,
 // for its own heads.  Called by all threads of the CTA once its segments are done.
-__device__ __forceinline__ void fill_empty_requests(const DecodeParams &p, int worker, int head0, int heads_per_group,
+// `ts`: the plan's tile_start (SegmentIter::ts).
+__device__ __forceinline__ void fill_empty_requests(const DecodeParams &p, const int32_t *ts, int worker, int head0, int heads_per_group,
                                                     int tid, int nthreads) {
     // The plan's arrays are a launch old and have left the caches: a loop over this worker's requests that looks at one
     // request per iteration is a chain of round trips to DRAM at the very end of the CTA (seven on the rollout workload).
@@ -192,7 +373,7 @@ __device__ __forceinline__ void fill_empty_requests(const DecodeParams &p, int w
     const int lane = tid & 31, wid = tid >> 5, nwarps = nthreads >> 5;
     for (int64_t j0 = (int64_t)wid * 32; worker + j0 * p.num_workers < p.B; j0 += (int64_t)nwarps * 32) {
         const int64_t mine = worker + (j0 + lane) * p.num_workers;
-        const bool empty = mine < p.B && p.tile_start[mine + 1] == p.tile_start[mine];
+        const bool empty = mine < p.B && ts[mine + 1] == ts[mine];
         unsigned found = __ballot_sync(0xffffffffu, empty);
         while (found) {
             const int src = __ffs(found) - 1;
@@ -207,14 +388,6 @@ __device__ __forceinline__ void fill_empty_requests(const DecodeParams &p, int w
         }
     }
 }
-
-// ---- programmatic dependent launch ---------------------------------------------
-// The three kernels of a decode call are chained with programmatic stream serialisation:
-// a dependent kernel may be scheduled while its predecessor is still running, does its
-// own set-up (barriers, tensor memory), and blocks in grid_dependency_wait() before it
-// touches anything the predecessor wrote.
-__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
@@ -251,16 +424,13 @@ void set_error(const char *fmt, ...);
 void count_launch(int n = 1);
 
 // kernels' host launchers
-cudaError_t launch_plan(const DecodeParams &p, const int32_t *kv_begin, const int32_t *kv_end,
-                        int32_t *tile_start, int32_t *req_lo, int32_t *req_hi, int32_t *req_wfirst,
-                        int32_t *req_wlast, int32_t *cost_start, int32_t *worker_begin, int32_t *split_list, int32_t *worker_req, int4 *split_rec,
-                        int32_t *status, bool reset_status, cudaStream_t stream);
+cudaError_t launch_plan(const DecodeParams &p, const PlanView &v, cudaStream_t stream);
 cudaError_t launch_validate_pages(const DecodeParams &p, const int32_t *req_lo, const int32_t *req_hi, cudaStream_t stream);
 cudaError_t launch_decode_sparse_pair(const DecodeParams &p, cudaStream_t stream);
 cudaError_t launch_sparse_gather(int B, int max_sel, int pages_per_request, const void *kv_pool, int num_pool_pages,
                                  const int32_t *block_table, int64_t table_stride, const int32_t *seq_lens,
                                  const int32_t *sel, int64_t sel_stride, const int32_t *sel_count, void *dense_pool,
-                                 int32_t *dense_table, int sm_count, cudaStream_t stream);
+                                 int32_t *dense_table, int sm_count, bool after_plan, cudaStream_t stream);
 cudaError_t launch_dop_pack_rows(const void *a, const void *b, void *out, const int32_t *send_row, int64_t n, int h,
                                  int64_t a_bytes, int64_t b_bytes, int64_t a_row_pitch, int64_t a_head_pitch,
                                  int64_t b_row_pitch, int64_t b_head_pitch, int sm_count, cudaStream_t stream);

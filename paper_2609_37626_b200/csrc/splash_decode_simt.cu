@@ -35,7 +35,7 @@ __device__ __forceinline__ float elem_to_float(uint16_t v) {
 
 template <int KV_DTYPE>
 __global__ void __launch_bounds__(kSimtThreads)
-decode_simt_kernel(const DecodeParams p) {
+decode_simt_kernel(const __grid_constant__ DecodeParams p) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SimtSmem &sm = *reinterpret_cast<SimtSmem *>(smem_raw);
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -45,7 +45,7 @@ decode_simt_kernel(const DecodeParams p) {
     const int h = p.head_end - p.head_begin;
 
     grid_dependency_wait();       // the plan kernel's output is read from here on
-    SegmentIter it;
+    SegmentIter<kPlanInWorkspace> it;
     it.init(p, worker);
     Segment seg;
     while (it.next(p, seg)) {
@@ -189,7 +189,7 @@ decode_simt_kernel(const DecodeParams p) {
         }
         __syncthreads();
     }
-    fill_empty_requests(p, worker, head0, kSimtHeads, tid, kSimtThreads);
+    fill_empty_requests(p, it.tile_start(p), worker, head0, kSimtHeads, tid, kSimtThreads);
 }
 
 }  // namespace

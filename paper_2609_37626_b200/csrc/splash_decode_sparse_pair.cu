@@ -91,7 +91,8 @@ constexpr uint32_t kOffL = kOffAlpha + kN * 4;                  // float [64]
 constexpr uint32_t kOffXch = kOffL + kN * 4;                    // float [64][4]
 constexpr uint32_t kOffBar = kOffXch + kN * 16;
 constexpr uint32_t kOffMisc = (kOffBar + kNumBarriers * 8 + 15) / 16 * 16;
-constexpr uint32_t kSmemBytes = kOffMisc + 32;
+constexpr uint32_t kOffPlan = kOffMisc + 32;                    // inline plan
+constexpr uint32_t kSmemBytes = kOffPlan + kInlinePlanBytes;
 static_assert(kSmemBytes <= 232448, "shared memory overflow");
 static_assert(kOffQ % 1024 == 0 && kOffP1 % 1024 == 0 && kSlab % 1024 == 0, "swizzle atoms need 1024-byte alignment");
 static_assert(kOffRawK % 16 == 0 && kOffRawV % 16 == 0 && kOffRing % 8 == 0 && kOffBar % 8 == 0, "alignment");
@@ -133,7 +134,7 @@ __device__ __forceinline__ void umma_bf16_pair(uint32_t d_tmem, uint64_t a_desc,
 }
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
-decode_sparse_pair_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap tmap_q) {
+decode_sparse_pair_kernel(const __grid_constant__ DecodeParams p, const __grid_constant__ CUtensorMap tmap_q) {
     extern __shared__ __align__(1024) uint8_t smem[];
     const uint32_t sbase = smem_u32(smem);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -182,8 +183,8 @@ decode_sparse_pair_kernel(const DecodeParams p, const __grid_constant__ CUtensor
     const long long t_start = clock64();
     const unsigned long long ns_start = global_timer_ns();
 
-    SegmentIter it;
-    it.init(p, worker);
+    SegmentIter<kOffPlan> it;
+    start_plan(p, worker, kThreads / 32 - 1, it);
     Segment seg;
     seg.lo = seg.hi = seg.tile_begin = seg.tile_end = 0;
 
@@ -378,7 +379,7 @@ decode_sparse_pair_kernel(const DecodeParams p, const __grid_constant__ CUtensor
         const unsigned long long *ring = reinterpret_cast<const unsigned long long *>(smem + kOffRing);
         uint32_t total = 0;         // tiles of this worker: the building duties do not care about request boundaries
         {
-            SegmentIter it2 = it;
+            SegmentIter<kOffPlan> it2 = it;
             Segment seg2;
             while (it2.next(p, seg2)) total += (uint32_t)(seg2.tile_end - seg2.tile_begin);
         }
@@ -682,7 +683,7 @@ decode_sparse_pair_kernel(const DecodeParams p, const __grid_constant__ CUtensor
         }
     }
 
-    fill_empty_requests(p, worker, head0, kN, tid, kThreads);
+    fill_empty_requests(p, it.tile_start(p), worker, head0, kN, tid, kThreads);
     if (p.trace != nullptr && tid == 0) {   // per-CTA cycles and nanoseconds
         p.trace[512 + blockIdx.x] = clock64() - t_start;
         if (blockIdx.x < 256) p.trace[768 + blockIdx.x] = (long long)(global_timer_ns() - ns_start);

@@ -81,7 +81,8 @@ struct Layout {
     static constexpr uint32_t kOffL = kOffAlpha + N * 4;     // float [N]
     static constexpr uint32_t kOffBar = kOffL + N * 4;       // uint64 [kNumBarriers]
     static constexpr uint32_t kOffMisc = kOffBar + kNumBarriers * 8;   // u32: tmem base, abort, rescale flag
-    static constexpr uint32_t kBytes = kOffMisc + 16;
+    static constexpr uint32_t kOffPlan = kOffMisc + 16;
+    static constexpr uint32_t kBytes = kOffPlan + kInlinePlanBytes;
     // tensor memory columns
     static constexpr uint32_t kColO = 0;                     // 4 blocks x N columns
     // S^T is accumulated in kAcc independent partial sums (summed by the softmax warps): a
@@ -103,7 +104,7 @@ struct Layout {
 // ---------------------------------------------------------------- the kernel
 template <int N>
 __global__ void __launch_bounds__(kThreads, 1)
-decode_umma_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap tmap_kv,
+decode_umma_kernel(const __grid_constant__ DecodeParams p, const __grid_constant__ CUtensorMap tmap_kv,
                    const __grid_constant__ CUtensorMap tmap_q) {
     using L = Layout<N>;
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -142,8 +143,8 @@ decode_umma_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap tma
     grid_dependency_wait();       // the plan kernel's output is read from here on
     const long long t_start = clock64();
 
-    SegmentIter it;
-    it.init(p, worker);
+    SegmentIter<L::kOffPlan> it;
+    start_plan(p, worker, kThreads / 32 - 1, it);
     Segment seg;
     long long *const trace = blockIdx.x == 0 ? p.trace : nullptr;
     auto mark = [&](uint32_t tile, int ev) {
@@ -650,7 +651,7 @@ decode_umma_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap tma
         }
     }
 
-    fill_empty_requests(p, worker, head0, N, tid, kThreads);
+    fill_empty_requests(p, it.tile_start(p), worker, head0, N, tid, kThreads);
     if (p.trace != nullptr && tid == 0) p.trace[512 + blockIdx.x] = clock64() - t_start;   // per-CTA cycles
 
     // ---- teardown

@@ -72,14 +72,15 @@ constexpr uint32_t kOffTok = kOffL + kN * 4;                // float2 [64]: (log
 constexpr uint32_t kOffXch = kOffTok + 64 * 8;              // float [64][2]: per-head exchange between token halves
 constexpr uint32_t kOffBar = kOffXch + kN * 8;
 constexpr uint32_t kOffMisc = (kOffBar + kNumBarriers * 8 + 15) / 16 * 16;
-constexpr uint32_t kSmemBytes = kOffMisc + 32;
+constexpr uint32_t kOffPlan = kOffMisc + 32;                    // inline plan
+constexpr uint32_t kSmemBytes = kOffPlan + kInlinePlanBytes;
 static_assert(kSmemBytes <= 232448, "shared memory overflow");
 static_assert(kOffQHi % 512 == 0 && kOffQLo % 512 == 0 && kOffPHi % 512 == 0 && kOffPLo % 512 == 0, "alignment");
 // tensor memory: O^T 4 blocks x 64 columns, then 2 S buffers x 2 partial accumulators x 64 columns
 constexpr uint32_t kColO = 0, kColS = 256;
 
 __global__ void __launch_bounds__(kThreads, 1)
-decode_umma_fp8_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap tmap_kv) {
+decode_umma_fp8_kernel(const __grid_constant__ DecodeParams p, const __grid_constant__ CUtensorMap tmap_kv) {
     extern __shared__ __align__(1024) uint8_t smem[];
     const uint32_t sbase = smem_u32(smem);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -117,8 +118,8 @@ decode_umma_fp8_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap
     grid_dependency_wait();       // the plan kernel's output is read from here on
     const long long t_start = clock64();
 
-    SegmentIter it;
-    it.init(p, worker);
+    SegmentIter<kOffPlan> it;
+    start_plan(p, worker, kThreads / 32 - 1, it);
     Segment seg;
     long long *const trace = blockIdx.x == 0 ? p.trace : nullptr;
     auto mark = [&](uint32_t tile, int ev) {
@@ -535,7 +536,7 @@ decode_umma_fp8_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap
         }
     }
 
-    fill_empty_requests(p, worker, head0, kN, tid, kThreads);
+    fill_empty_requests(p, it.tile_start(p), worker, head0, kN, tid, kThreads);
 
     // ---- teardown
     if (p.trace != nullptr && tid == 0) p.trace[512 + blockIdx.x] = clock64() - t_start;   // per-CTA cycles

@@ -94,7 +94,8 @@ struct Layout {
     static constexpr uint32_t kOffL = kOffAlpha + N * 4;       // float [N]
     static constexpr uint32_t kOffBar = kOffL + N * 4;
     static constexpr uint32_t kOffMisc = (kOffBar + kNumBarriers * 8 + 15) / 16 * 16;   // u32: tmem base, abort
-    static constexpr uint32_t kBytes = kOffMisc + 16;
+    static constexpr uint32_t kOffPlan = kOffMisc + 16;        // inline plan
+    static constexpr uint32_t kBytes = kOffPlan + kInlinePlanBytes;
     static constexpr uint32_t kColO = 0;                       // 4 dv blocks x (N hi, N lo) columns
     static constexpr uint32_t kColS = 8 * N;                   // 2 buffers x kQkWarps partials x (N hi, N lo) columns
     static_assert(kColS + 2 * kQkWarps * 2 * N <= 512, "tensor memory overflow");
@@ -105,7 +106,7 @@ struct Layout {
 // ---------------------------------------------------------------- the kernel
 template <int N>
 __global__ void __launch_bounds__(Layout<N>::kThreads, 1)
-decode_umma_fp8_narrow_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap tmap_kv) {
+decode_umma_fp8_narrow_kernel(const __grid_constant__ DecodeParams p, const __grid_constant__ CUtensorMap tmap_kv) {
     using L = Layout<N>;
     constexpr int kStages = L::kStages, kThreads = L::kThreads, kNumSoftmaxWarps = L::kSoftmaxWarps, kWarpConvert = L::kWarpConvert;
     constexpr int kSoftmaxThreads = L::kSoftmaxThreads;
@@ -145,8 +146,8 @@ decode_umma_fp8_narrow_kernel(const DecodeParams p, const __grid_constant__ CUte
     grid_dependency_wait();       // the plan kernel's output is read from here on
     const long long t_start = clock64();
 
-    SegmentIter it;
-    it.init(p, worker);
+    SegmentIter<L::kOffPlan> it;
+    start_plan(p, worker, kThreads / 32 - 1, it);
     Segment seg;
     long long *const trace = blockIdx.x == 0 ? p.trace : nullptr;
     auto mark = [&](uint32_t tile, int ev) {
@@ -301,7 +302,7 @@ decode_umma_fp8_narrow_kernel(const DecodeParams p, const __grid_constant__ CUte
             const int part = ct & 3;
             {
                 // the rows of the request after this one: into L2 now, so that their loads, a request from now, are short
-                SegmentIter peek = it;
+                SegmentIter<L::kOffPlan> peek = it;
                 Segment nxt;
                 if (peek.next(p, nxt)) {
                     const char *row0 = reinterpret_cast<const char *>(static_cast<const __nv_bfloat16 *>(p.q) +
@@ -643,7 +644,7 @@ decode_umma_fp8_narrow_kernel(const DecodeParams p, const __grid_constant__ CUte
         }
     }
 
-    fill_empty_requests(p, worker, head0, N, tid, kThreads);
+    fill_empty_requests(p, it.tile_start(p), worker, head0, N, tid, kThreads);
     if (p.trace != nullptr && tid == 0) p.trace[512 + blockIdx.x] = clock64() - t_start;   // per-CTA cycles
 
     // ---- teardown

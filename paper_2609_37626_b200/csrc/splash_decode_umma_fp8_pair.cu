@@ -87,7 +87,8 @@ constexpr uint32_t kTokBytes = 32 * 8 + 32 * 4;                 // per warp: (sc
 constexpr uint32_t kOffTok = kOffXch + kN * 16;
 constexpr uint32_t kOffBar = kOffTok + kSoftmaxWarps * kTokBytes;
 constexpr uint32_t kOffMisc = (kOffBar + kNumBarriers * 8 + 15) / 16 * 16;
-constexpr uint32_t kSmemBytes = kOffMisc + 32;
+constexpr uint32_t kOffPlan = kOffMisc + 32;                    // inline plan
+constexpr uint32_t kSmemBytes = kOffPlan + kInlinePlanBytes;
 static_assert(kSmemBytes <= 232448, "shared memory overflow");
 static_assert(kOffQHi % 1024 == 0 && kOffP % 1024 == 0 && kOffTok % 16 == 0 && kTokBytes % 16 == 0, "alignment");
 // tensor memory: O two halves of dv x 128 columns, then 2 S buffers x 2 partials x 64 columns
@@ -100,8 +101,12 @@ __device__ __forceinline__ void umma_e4m3_pair(uint32_t d_tmem, uint64_t a_desc,
         "tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}"
         ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
 }
+
+// kInline: the variant that can plan for itself.  The kernel sits at its register cap, and a walk over the segments that
+// can read either plan costs the main loop 0.6 to 2.4 % of its cycles: calls behind a plan kernel have their own variant.
+template <bool kInline>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
-decode_umma_fp8_pair_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap tmap_page,
+decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid_constant__ CUtensorMap tmap_page,
                             const __grid_constant__ CUtensorMap tmap_pair, const __grid_constant__ CUtensorMap tmap_out,
                             const __grid_constant__ CUtensorMap tmap_part) {
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -153,8 +158,8 @@ decode_umma_fp8_pair_kernel(const DecodeParams p, const __grid_constant__ CUtens
     const long long t_start = clock64();
     const unsigned long long ns_start = global_timer_ns();
 
-    SegmentIter it;
-    it.init(p, worker);
+    SegmentIter<kInline ? kOffPlan : kPlanInWorkspace> it;
+    start_plan(p, worker, kThreads / 32 - 1, it);
     Segment seg;
     seg.lo = seg.hi = seg.tile_begin = seg.tile_end = 0;
     // geometry of supertile s of the current segment: page tiles 2s (page A, CTA 0) and 2s + 1 (page B, CTA 1)
@@ -633,7 +638,7 @@ decode_umma_fp8_pair_kernel(const DecodeParams p, const __grid_constant__ CUtens
         }
     }
 
-    fill_empty_requests(p, worker, head0, kN, tid, kThreads);
+    fill_empty_requests(p, it.tile_start(p), worker, head0, kN, tid, kThreads);
     if (p.trace != nullptr && tid == 0) {   // per-CTA cycles and nanoseconds
         p.trace[512 + blockIdx.x] = clock64() - t_start;
         if (blockIdx.x < 256) p.trace[768 + blockIdx.x] = (long long)(global_timer_ns() - ns_start);
@@ -675,7 +680,11 @@ cudaError_t launch_decode_umma_fp8_pair(const DecodeParams &p, cudaStream_t stre
     if (!make_store_map_3d(&mpart, p.partial_out, kDV, h, (uint64_t)2 * p.num_workers, (uint64_t)kDV * 4, h * kDV * 4, 32))
         return cudaErrorInvalidValue;
     static DeviceOnce once;
-    cudaError_t e = once.run([&] { return cudaFuncSetAttribute(decode_umma_fp8_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes); });
+    cudaError_t e = once.run([&] {
+        const cudaError_t e0 = cudaFuncSetAttribute(decode_umma_fp8_pair_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
+        if (e0 != cudaSuccess) return e0;
+        return cudaFuncSetAttribute(decode_umma_fp8_pair_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
+    });
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(p.num_workers * p.pair_groups * 2)); cfg.blockDim = dim3(kThreads);
@@ -684,7 +693,7 @@ cudaError_t launch_decode_umma_fp8_pair(const DecodeParams &p, cudaStream_t stre
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, decode_umma_fp8_pair_kernel, p, mpage, mpair, mout, mpart);
+    e = cudaLaunchKernelEx(&cfg, p.plan_mode == kPlanWorkspace ? decode_umma_fp8_pair_kernel<false> : decode_umma_fp8_pair_kernel<true>, p, mpage, mpair, mout, mpart);
     count_launch();
     return e;
 }

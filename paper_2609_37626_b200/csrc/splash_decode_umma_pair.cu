@@ -82,7 +82,8 @@ constexpr uint32_t kOffL = kOffAlpha + kN * 4;                  // float [64]
 constexpr uint32_t kOffXch = kOffL + kN * 4;                    // float [64][4]
 constexpr uint32_t kOffBar = kOffXch + kN * 16;
 constexpr uint32_t kOffMisc = (kOffBar + kNumBarriers * 8 + 15) / 16 * 16;
-constexpr uint32_t kSmemBytes = kOffMisc + 32;
+constexpr uint32_t kOffPlan = kOffMisc + 32;                    // inline plan
+constexpr uint32_t kSmemBytes = kOffPlan + kInlinePlanBytes;
 static_assert(kSmemBytes <= 232448, "shared memory overflow");
 static_assert(kOffQ % 1024 == 0 && kOffP1 % 1024 == 0 && kSlab % 1024 == 0, "swizzle atoms need 1024-byte alignment");
 // tensor memory: O two halves of dv x 128 columns, then 2 S buffers x 4 partials x 32 columns
@@ -97,7 +98,7 @@ __device__ __forceinline__ void umma_bf16_pair(uint32_t d_tmem, uint64_t a_desc,
 }
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
-decode_umma_pair_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap tmap_half,
+decode_umma_pair_kernel(const __grid_constant__ DecodeParams p, const __grid_constant__ CUtensorMap tmap_half,
                         const __grid_constant__ CUtensorMap tmap_peer, const __grid_constant__ CUtensorMap tmap_q) {
     extern __shared__ __align__(1024) uint8_t smem[];
     const uint32_t sbase = smem_u32(smem);
@@ -146,8 +147,8 @@ decode_umma_pair_kernel(const DecodeParams p, const __grid_constant__ CUtensorMa
     const long long t_start = clock64();
     const unsigned long long ns_start = global_timer_ns();
 
-    SegmentIter it;
-    it.init(p, worker);
+    SegmentIter<kOffPlan> it;
+    start_plan(p, worker, kThreads / 32 - 1, it);
     Segment seg;
     seg.lo = seg.hi = seg.tile_begin = seg.tile_end = 0;
 
@@ -548,7 +549,7 @@ decode_umma_pair_kernel(const DecodeParams p, const __grid_constant__ CUtensorMa
         }
     }
 
-    fill_empty_requests(p, worker, head0, kN, tid, kThreads);
+    fill_empty_requests(p, it.tile_start(p), worker, head0, kN, tid, kThreads);
     if (p.trace != nullptr && tid == 0) {   // per-CTA cycles and nanoseconds
         p.trace[512 + blockIdx.x] = clock64() - t_start;
         if (blockIdx.x < 256) p.trace[768 + blockIdx.x] = (long long)(global_timer_ns() - ns_start);

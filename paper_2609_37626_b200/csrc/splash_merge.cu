@@ -18,6 +18,8 @@ constexpr int kMergeThreads = 128;
 __global__ void __launch_bounds__(kMergeThreads)
 lse_merge_kernel(int num_parts, int64_t rows, int d_v, const float *__restrict__ part_out,
                  const float *__restrict__ part_lse, float *__restrict__ out, float *__restrict__ lse) {
+    grid_launch_dependents();
+    grid_dependency_wait();       // launched while the work before it on the stream still runs
     const int64_t r = blockIdx.x;
     float m = -INFINITY;
     for (int j = 0; j < num_parts; ++j) m = fmaxf(m, part_lse[(int64_t)j * rows + r]);
@@ -70,6 +72,7 @@ split_combine_kernel(const DecodeParams p, const int4 *__restrict__ split_rec) {
     const int h = p.head_end - p.head_begin;
     const int k = blockIdx.x % h, entry = blockIdx.x / h;
     const int g = p.head_begin + k;
+    grid_launch_dependents();     // a next call's first kernel may come in once every block of this grid has started
     grid_dependency_wait();       // the decode kernel's partial slots (and the plan) are read from here on
     // Three rounds of loads, each independent within itself (the plan's arrays have long left L2 by now, so every
     // dependent load is a trip to DRAM): the list length and this entry's record; then the worker boundaries and the
@@ -183,9 +186,10 @@ split_combine_kernel(const DecodeParams p, const int4 *__restrict__ split_rec) {
 
 cudaError_t launch_lse_merge(int num_parts, int64_t rows, int d_v, const float *part_out,
                              const float *part_lse, float *out, float *lse, cudaStream_t stream) {
-    lse_merge_kernel<<<(unsigned)rows, kMergeThreads, 0, stream>>>(num_parts, rows, d_v, part_out, part_lse, out, lse);
+    const cudaError_t e = launch_dependent(lse_merge_kernel, dim3((unsigned)rows), dim3(kMergeThreads), 0, stream, num_parts, rows, d_v,
+                                           part_out, part_lse, out, lse);
     count_launch();
-    return cudaGetLastError();
+    return e;
 }
 
 cudaError_t launch_split_combine(const DecodeParams &p, const int4 *split_rec, cudaStream_t stream) {

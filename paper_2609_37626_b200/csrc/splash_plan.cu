@@ -20,15 +20,17 @@ constexpr int kPlanThreads = 1024;
 constexpr int kPlanSmemRequests = 4096;
 constexpr int kPlanSmemWorkers = 512;
 
+// One CTA between the caller's work and the decode kernel: its time is latency (a load of the lengths, a scan, two
+// bisections, the stores) and comes on top of every call of more than 32 requests.  As many threads as there are requests
+// or workers, one barrier per 1,024 requests in the scan, 32-bit arithmetic.
 __global__ void __launch_bounds__(kPlanThreads)
-plan_kernel(int B, int W, int overhead, int len_cap, int reset_status, const int32_t *__restrict__ seq_lens, const int32_t *__restrict__ kv_begin,
+plan_kernel(int B, int W, int overhead, int len_cap, const int32_t *__restrict__ seq_lens, const int32_t *__restrict__ kv_begin,
             const int32_t *__restrict__ kv_end, int32_t *tile_start,
             int32_t *__restrict__ req_lo, int32_t *__restrict__ req_hi,
             int32_t *__restrict__ req_wfirst, int32_t *__restrict__ req_wlast,
             int32_t *cost_start, int32_t *worker_begin, int32_t *__restrict__ split_list, int32_t *__restrict__ worker_req,
             int4 *__restrict__ split_rec, int32_t *__restrict__ status) {
-    __shared__ long long warp_tot_tiles[32], warp_tot_cost[32];
-    __shared__ long long carry_tiles, carry_cost;
+    __shared__ int2 warp_tot[2][32];
     __shared__ int n_split;
     // The bisections below chase a dozen dependent loads each; for the usual sizes the
     // prefix arrays live in shared memory while the plan is built and are copied out at the end.
@@ -36,62 +38,61 @@ plan_kernel(int B, int W, int overhead, int len_cap, int reset_status, const int
     const bool staged = B <= kPlanSmemRequests && W <= kPlanSmemWorkers;
     int32_t *const g_tile_start = tile_start, *const g_cost_start = cost_start, *const g_worker_begin = worker_begin;
     if (staged) { tile_start = s_tile; cost_start = s_cost; worker_begin = s_wbeg; }
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    grid_launch_dependents();     // the decode kernel may start its set-up now; it waits for this grid before reading the plan
-    // the status block is cleared by the first pass of a call only: a later pass (more than 128 (head, row) pairs)
-    // must not wipe what an earlier one recorded
-    if (reset_status && tid < 16) status[tid] = 0;
-    if (tid == 0) { carry_tiles = 0; carry_cost = 0; tile_start[0] = 0; cost_start[0] = 0; n_split = 0; }
-    __syncthreads();
+    const int tid = threadIdx.x, nthreads = blockDim.x, lane = tid & 31, wid = tid >> 5;
+    grid_dependency_wait();       // launched while the work before it on the stream still runs
+    grid_launch_dependents();     // the next kernel may start its set-up now; it waits for this grid before reading the plan
+    if (tid < 16) status[tid] = 0;
+    if (tid == 0) { tile_start[0] = 0; cost_start[0] = 0; n_split = 0; }
 
     // pass 1: effective ranges, tile counts, exclusive prefixes of tiles and of cost
-    for (int base = 0; base < B; base += kPlanThreads) {
-        int i = base + tid;
-        long long n = 0;
+    int carry_tiles = 0, carry_cost = 0;
+    for (int base = 0, chunk = 0; base < B; base += nthreads, ++chunk) {
+        const int i = base + tid;
+        int n = 0;
         if (i < B) {
-            int s = seq_lens[i];
-            if (len_cap >= 0 && (s < 0 || s > len_cap)) s = 1;     // a list count out of bounds: one (poisoned) row
-            int lo = kv_begin ? kv_begin[i] : 0;
-            int hi = kv_end ? kv_end[i] : s;
-            if (lo < 0) lo = 0;
-            if (hi > s) hi = s;
-            if (hi < lo) hi = lo;
+            int lo, hi;
+            effective_range(seq_lens[i], kv_begin, kv_end, i, len_cap, lo, hi);
             req_lo[i] = lo; req_hi[i] = hi;
             if (hi > lo) n = (hi + kPage - 1) / kPage - lo / kPage;
         }
-        long long c = n > 0 ? n + overhead : 0;
-        long long sn = n, sc = c;
+        int sn = n, sc = n > 0 ? n + overhead : 0;
+#pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            long long a = __shfl_up_sync(0xffffffffu, sn, o);
-            long long b = __shfl_up_sync(0xffffffffu, sc, o);
+            const int a = __shfl_up_sync(0xffffffffu, sn, o), b = __shfl_up_sync(0xffffffffu, sc, o);
             if (lane >= o) { sn += a; sc += b; }
         }
-        if (lane == 31) { warp_tot_tiles[wid] = sn; warp_tot_cost[wid] = sc; }
+        if (lane == 31) warp_tot[chunk & 1][wid] = make_int2(sn, sc);
         __syncthreads();
-        long long offn = carry_tiles, offc = carry_cost;
-        for (int k = 0; k < wid; ++k) { offn += warp_tot_tiles[k]; offc += warp_tot_cost[k]; }
-        if (i < B) { tile_start[i + 1] = (int32_t)(offn + sn); cost_start[i + 1] = (int32_t)(offc + sc); }
-        __syncthreads();
-        if (tid == kPlanThreads - 1) { carry_tiles = offn + sn; carry_cost = offc + sc; }
-        __syncthreads();
+        // every warp scans the warps' totals for itself (two buffers: one barrier per chunk is enough)
+        int2 t = lane < (nthreads >> 5) ? warp_tot[chunk & 1][lane] : make_int2(0, 0);
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int a = __shfl_up_sync(0xffffffffu, t.x, o), b = __shfl_up_sync(0xffffffffu, t.y, o);
+            if (lane >= o) { t.x += a; t.y += b; }
+        }
+        const int before_n = wid > 0 ? __shfl_sync(0xffffffffu, t.x, (wid + 31) & 31) : 0;
+        const int before_c = wid > 0 ? __shfl_sync(0xffffffffu, t.y, (wid + 31) & 31) : 0;
+        if (i < B) { tile_start[i + 1] = carry_tiles + before_n + sn; cost_start[i + 1] = carry_cost + before_c + sc; }
+        carry_tiles += __shfl_sync(0xffffffffu, t.x, 31);
+        carry_cost += __shfl_sync(0xffffffffu, t.y, 31);
     }
-    const long long total_cost = carry_cost;
-    const int total_tiles = (int)carry_tiles;
+    const int total_cost = carry_cost, total_tiles = carry_tiles;
+    __threadfence_block();
+    __syncthreads();
 
     // pass 2: worker w starts at cost floor(w * total_cost / W); the request whose
     // cost interval [cost_start[i], cost_start[i+1]) holds that value is found by
     // bisection, and a start that falls into the request's fixed overhead snaps to
     // its first tile.
-    for (int w = tid; w <= W; w += kPlanThreads) {
+    for (int w = tid; w <= W; w += nthreads) {
         int g = total_tiles, first_req = 0;
         if (w < W && total_cost > 0) {
-            long long target = (total_cost * w) / W;
+            const int target = cost_target(total_cost, w, W);
             int lo = 0, hi = B;   // invariant cost_start[lo] <= target < cost_start[hi]
             while (hi - lo > 1) { int mid = (lo + hi) >> 1; if (cost_start[mid] <= target) lo = mid; else hi = mid; }
             while (cost_start[lo + 1] <= target) ++lo;   // (defensive; bisection already lands on a non-empty request)
-            long long off = target - cost_start[lo] - overhead;
-            if (off < 0) off = 0;
-            g = tile_start[lo] + (int)off;
+            const int off = target - cost_start[lo] - overhead;
+            g = tile_start[lo] + max(off, 0);
             first_req = lo;
         }
         worker_begin[w] = g;
@@ -101,18 +102,19 @@ plan_kernel(int B, int W, int overhead, int len_cap, int reset_status, const int
     __syncthreads();
 
     // pass 3: first / last worker of every request
-    for (int i = tid; i < B; i += kPlanThreads) {
-        int rs = tile_start[i], re = tile_start[i + 1];
+    for (int i = tid; i < B; i += nthreads) {
+        const int rs = tile_start[i], re = tile_start[i + 1];
         int wf = -1, wl = -1;
         if (re > rs) {
-            // worker containing tile x: the w with worker_begin[w] <= x < worker_begin[w+1]
-            int lo = 0, hi = W;   // invariant worker_begin[lo] <= rs < worker_begin[hi]
-            while (hi - lo > 1) { int mid = (lo + hi) >> 1; if (worker_begin[mid] <= rs) lo = mid; else hi = mid; }
-            wf = lo;
-            int x = re - 1;
-            lo = 0; hi = W;
-            while (hi - lo > 1) { int mid = (lo + hi) >> 1; if (worker_begin[mid] <= x) lo = mid; else hi = mid; }
-            wl = lo;
+            // worker containing tile x: the w with worker_begin[w] <= x < worker_begin[w+1]; both bisections side by side
+            int hi0 = W, hi1 = W;
+            wf = wl = 0;          // invariant worker_begin[w] <= x < worker_begin[hi]
+            while (hi0 - wf > 1 || hi1 - wl > 1) {
+                const int m0 = (wf + hi0) >> 1, m1 = (wl + hi1) >> 1;
+                const int b0 = worker_begin[m0], b1 = worker_begin[m1];
+                if (hi0 - wf > 1) { if (b0 <= rs) wf = m0; else hi0 = m0; }
+                if (hi1 - wl > 1) { if (b1 <= re - 1) wl = m1; else hi1 = m1; }
+            }
         }
         req_wfirst[i] = wf; req_wlast[i] = wl;
         // requests cut into several pieces are listed for the combine kernel (at most W - 1 of them;
@@ -123,12 +125,12 @@ plan_kernel(int B, int W, int overhead, int len_cap, int reset_status, const int
             split_rec[e] = make_int4(i, wf, wl, rs);      // all the combine kernel needs to know about the request, in one load
         }
     }
+    if (staged) {
+        for (int i = tid; i <= B; i += nthreads) { g_tile_start[i] = s_tile[i]; g_cost_start[i] = s_cost[i]; }
+        for (int w = tid; w <= W; w += nthreads) g_worker_begin[w] = s_wbeg[w];
+    }
     __syncthreads();
     if (tid == 0) status[8] = n_split;
-    if (staged) {
-        for (int i = tid; i <= B; i += kPlanThreads) { g_tile_start[i] = s_tile[i]; g_cost_start[i] = s_cost[i]; }
-        for (int w = tid; w <= W; w += kPlanThreads) g_worker_begin[w] = s_wbeg[w];
-    }
 }
 
 // Validation mode: every block-table entry of a page that intersects a request's effective range must name a page of
@@ -157,20 +159,20 @@ cudaError_t launch_validate_pages(const DecodeParams &p, const int32_t *req_lo, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_plan(const DecodeParams &p, const int32_t *kv_begin, const int32_t *kv_end,
-                        int32_t *tile_start, int32_t *req_lo, int32_t *req_hi, int32_t *req_wfirst,
-                        int32_t *req_wlast, int32_t *cost_start, int32_t *worker_begin, int32_t *split_list,
-                        int32_t *worker_req, int4 *split_rec, int32_t *status, bool reset_status, cudaStream_t stream) {
+cudaError_t launch_plan(const DecodeParams &p, const PlanView &v, cudaStream_t stream) {
     // same shared-memory carve-out as the decode kernel that follows: no reconfiguration between them
     static DeviceOnce once;
     once.run([&] {
         cudaFuncSetAttribute(plan_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
         return cudaSuccess;     // a preference: a failure is not an error
     });
-    plan_kernel<<<1, kPlanThreads, 0, stream>>>(p.B, p.num_workers, p.request_overhead_tiles, p.len_cap, reset_status ? 1 : 0, p.seq_lens, kv_begin, kv_end, tile_start,
-                                                req_lo, req_hi, req_wfirst, req_wlast, cost_start, worker_begin, split_list, worker_req, split_rec, status);
+    const int items = p.B > p.num_workers + 1 ? p.B : p.num_workers + 1;
+    const int threads = items >= kPlanThreads ? kPlanThreads : (items + 31) / 32 * 32;
+    const cudaError_t e = launch_dependent(plan_kernel, dim3(1), dim3(threads), 0, stream, p.B, p.num_workers, p.request_overhead_tiles,
+                                           p.len_cap, p.seq_lens, p.kv_begin, p.kv_end, v.tile_start, v.req_lo, v.req_hi, v.req_wfirst,
+                                           v.req_wlast, v.cost_start, v.worker_begin, v.split_list, v.worker_req, v.split_rec, v.status);
     count_launch();
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace splash

@@ -40,10 +40,13 @@ __global__ void __launch_bounds__(kGatherThreads, 4)
 sparse_gather_kernel(int B, int max_sel, int pages_per_request, const uint8_t *__restrict__ kv_pool, int num_pool_pages,
                      const int32_t *__restrict__ block_table, int64_t table_stride, const int32_t *__restrict__ seq_lens,
                      const int32_t *__restrict__ sel, int64_t sel_stride, const int32_t *__restrict__ sel_count,
-                     uint8_t *__restrict__ dense_pool, int32_t *__restrict__ dense_table) {
-    // Launched as a programmatic dependent of the plan kernel, whose output it does not read: it runs beside it,
-    // lets the decode kernel behind it set up early, and waits for the plan only before it exits, so that the
-    // decode kernel, which waits for this grid, finds both the plan and the dense cache complete.
+                     uint8_t *__restrict__ dense_pool, int32_t *__restrict__ dense_table, int after_plan) {
+    // Launched as a programmatic dependent of the plan kernel, whose output it does not read and which lets it start once
+    // the work before it on the stream is done: it runs beside it, lets the decode kernel behind it set up early, and
+    // waits for the plan only before it exits, so that the decode kernel, which waits for this grid, finds both the
+    // plan and the dense cache complete.  Without a plan kernel (a batch that the decode kernel plans itself) what comes
+    // before it is the caller's own work, which its inputs may depend on.
+    if (!after_plan) grid_dependency_wait();
     grid_launch_dependents();
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * kGatherThreads + threadIdx.x) >> 5;
@@ -145,7 +148,7 @@ sparse_gather_kernel(int B, int max_sel, int pages_per_request, const uint8_t *_
             }
         }
     }
-    grid_dependency_wait();
+    if (after_plan) grid_dependency_wait();
 }
 
 }  // namespace
@@ -153,7 +156,7 @@ sparse_gather_kernel(int B, int max_sel, int pages_per_request, const uint8_t *_
 cudaError_t launch_sparse_gather(int B, int max_sel, int pages_per_request, const void *kv_pool, int num_pool_pages,
                                  const int32_t *block_table, int64_t table_stride, const int32_t *seq_lens,
                                  const int32_t *sel, int64_t sel_stride, const int32_t *sel_count, void *dense_pool,
-                                 int32_t *dense_table, int sm_count, cudaStream_t stream) {
+                                 int32_t *dense_table, int sm_count, bool after_plan, cudaStream_t stream) {
     const int64_t groups = ((int64_t)B * pages_per_request * kPage + 31) / 32;
     const int warps_per_block = kGatherThreads / 32;
     int64_t blocks = (groups + warps_per_block - 1) / warps_per_block;
@@ -163,7 +166,7 @@ cudaError_t launch_sparse_gather(int B, int max_sel, int pages_per_request, cons
     cudaError_t e = launch_dependent(sparse_gather_kernel, dim3((unsigned)blocks), dim3(kGatherThreads), 0, stream, B, max_sel,
                                      pages_per_request, static_cast<const uint8_t *>(kv_pool), num_pool_pages, block_table,
                                      table_stride, seq_lens, sel, sel_stride, sel_count, static_cast<uint8_t *>(dense_pool),
-                                     dense_table);
+                                     dense_table, after_plan ? 1 : 0);
     count_launch();
     return e;
 }
