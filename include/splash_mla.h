@@ -287,7 +287,7 @@ SPLASH_API size_t splash_kv_page_migrate_workspace_bytes(int32_t max_page_id);
  * How: slices of 65..128 (head, row) pairs run on CTA pairs in which the MMA-issuing warps of
  * each pair's second CTA have nothing to do; those warps copy the job's pages (16-byte
  * streaming loads and stores, byte-exact) while the rest of the kernel decodes, on SMs and
- * HBM bandwidth the decode leaves unused.  The job's table rewrite (three small kernels) runs
+ * HBM bandwidth the decode leaves unused.  The job's table rewrite (two small kernels) runs
  * on `stream` before the decode.  Calls that do not run on the CTA-pair kernels (narrower
  * slices, SPLASH_FLAG_SIMT / NO_PAIR, more than 128 (head, row) pairs) run the plain page-copy
  * kernel after the decode instead: same results, no overlap.
@@ -341,7 +341,7 @@ SPLASH_API int splash_mla_decode_migrating(const splash_mla_shape *shape,
  *   - The first call on each device looks up the array's device address (a host-side
  *     query, no allocation); make that first call outside any stream capture.
  *   - All calls on a device share the one table, and it keeps the previous call's
- *     contents: each call first resets the entries [0, max_page_id) on `stream`.  Two
+ *     contents: each call writes its own entries on `stream` and believes no others.  Two
  *     calls that can overlap on the GPU (different streams, no ordering between them)
  *     race on it -- order them, or give one of them its own workspace through
  *     splash_kv_page_migrate.

@@ -1,66 +1,85 @@
 // KV page migration between two page pools in HBM, with block-table rewrite: the
 // single-GPU part of a layout switch (kept blocks are repacked into the destination
 // view; the table is the page metadata that must follow them).  Byte-exact.
-#include "splash_common.cuh"
+#include "splash_copy.cuh"
 
 namespace splash {
 
 namespace {
 
-constexpr int kCopyThreads = 256;
-constexpr int kCopyCtasPerPage = 4;
+constexpr int kScaleVecs = kPage * 4 / 16;  // 16-byte vectors of a scale page
 
-__global__ void remap_fill_kernel(int32_t *remap, int32_t n) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) remap[i] = -1;
-}
-
-__global__ void remap_scatter_kernel(int32_t *remap, const int32_t *__restrict__ src_ids,
-                                     const int32_t *__restrict__ dst_ids, int64_t n, int32_t src_base,
-                                     int32_t dst_base, int32_t max_page_id) {
-    int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j < n) {
-        int32_t s = src_base + src_ids[j];
-        if (s >= 0 && s < max_page_id) remap[s] = dst_base + dst_ids[j];
-    }
-}
-
-__global__ void table_rewrite_kernel(int32_t *table, int64_t num_entries, const int32_t *__restrict__ remap,
-                                     int32_t max_page_id) {
-    int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e < num_entries) {
-        int32_t id = table[e];
-        if (id >= 0 && id < max_page_id) {
-            int32_t r = remap[id];
-            if (r >= 0) table[e] = r;
-        }
-    }
-}
-
-// grid (n, kCopyCtasPerPage): 16-byte vector copy of one quarter of page j; CTA 0 of
-// a page also moves its scale page.
+// Entry s of the remap table: which listed page has the table id s.  The table is not cleared first (that was a kernel of
+// its own): an entry nobody wrote in this call holds anything, and the rewrite believes an entry only if the page that it
+// names does have that id.
 __global__ void __launch_bounds__(kCopyThreads)
-page_copy_kernel(const uint4 *__restrict__ src_pool, uint4 *__restrict__ dst_pool,
-                 const uint4 *__restrict__ src_scales, uint4 *__restrict__ dst_scales,
-                 int64_t page_vecs, const int32_t *__restrict__ src_ids, const int32_t *__restrict__ dst_ids) {
-    const int64_t j = blockIdx.x;
-    const int part = blockIdx.y;
-    const int64_t s = src_ids[j], d = dst_ids[j];
-    const uint4 *src = src_pool + s * page_vecs;
-    uint4 *dst = dst_pool + d * page_vecs;
-    const int64_t per = (page_vecs + kCopyCtasPerPage - 1) / kCopyCtasPerPage;
-    const int64_t begin = per * part;
-    const int64_t end = begin + per < page_vecs ? begin + per : page_vecs;
-    int64_t c = begin + threadIdx.x;
-    // four independent 16-byte loads in flight per thread
-    for (; c + 3 * kCopyThreads < end; c += 4 * kCopyThreads) {
-        uint4 v0 = __ldg(src + c), v1 = __ldg(src + c + kCopyThreads);
-        uint4 v2 = __ldg(src + c + 2 * kCopyThreads), v3 = __ldg(src + c + 3 * kCopyThreads);
-        dst[c] = v0; dst[c + kCopyThreads] = v1; dst[c + 2 * kCopyThreads] = v2; dst[c + 3 * kCopyThreads] = v3;
+remap_scatter_kernel(int32_t *remap, const int32_t *__restrict__ src_ids, int64_t n, int32_t src_base, int32_t max_page_id) {
+    grid_dependency_wait();         // launched while the work before it on the stream still runs
+    grid_launch_dependents();       // the pages may be copied meanwhile; the table's blocks wait for this grid
+    const int64_t j = (int64_t)blockIdx.x * kCopyThreads + threadIdx.x;
+    if (j < n) {
+        const int32_t s = src_base + src_ids[j];
+        if (s >= 0 && s < max_page_id) remap[s] = (int32_t)j;
     }
-    for (; c < end; c += kCopyThreads) dst[c] = __ldg(src + c);
-    if (src_scales != nullptr && part == 0 && threadIdx.x < kPage * 4 / 16)
-        dst_scales[d * (kPage * 4 / 16) + threadIdx.x] = __ldg(src_scales + s * (kPage * 4 / 16) + threadIdx.x);
+}
+
+struct MigrateParams {
+    const void *src_pool;
+    void *dst_pool;
+    const uint4 *src_scales;
+    uint4 *dst_scales;
+    int64_t page_bytes;
+    const int32_t *src_ids, *dst_ids;
+    int32_t n, src_base, dst_base, max_page_id;
+    int32_t *table;
+    const int32_t *remap;
+    int64_t num_entries;
+    int32_t table_blocks, spacing;   // block r * spacing, r < table_blocks, rewrites a piece of the table, the others copy a page
+    int32_t after_scatter;           // 1: a remap_scatter_kernel, which has waited for the work before it, comes before this grid
+};
+
+constexpr int kEntriesPerBlock = kCopyThreads * 4;
+
+__device__ __forceinline__ void rewrite_entries(const MigrateParams &p, int64_t piece) {
+    int64_t e[4];
+    int32_t id[4], j[4];
+    // four chains of table entry -> page -> its ids per thread, a round trip for each link of all four
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        e[k] = piece * kEntriesPerBlock + k * kCopyThreads + threadIdx.x;
+        id[k] = e[k] < p.num_entries ? p.table[e[k]] : -1;
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) j[k] = id[k] >= 0 && id[k] < p.max_page_id ? p.remap[id[k]] : -1;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        if (j[k] < 0 || j[k] >= p.n) continue;
+        const int32_t s = p.src_base + p.src_ids[j[k]], d = p.dst_base + p.dst_ids[j[k]];
+        if (s == id[k] && d >= 0) p.table[e[k]] = d;
+    }
+}
+
+// One block per page, with its scale page, and the table's rewrite in blocks spread evenly between them.  Bound by HBM.
+template <typename Vec>
+__global__ void __launch_bounds__(kCopyThreads, 4)
+page_migrate_kernel(const __grid_constant__ MigrateParams p) {
+    if (!p.after_scatter) grid_dependency_wait();
+    grid_launch_dependents();
+    const int b = blockIdx.x;
+    const int before = min(p.table_blocks, b / p.spacing + 1);     // table blocks up to and including this place
+    if (b % p.spacing == 0 && b / p.spacing < p.table_blocks) {
+        if (p.after_scatter) grid_dependency_wait();
+        rewrite_entries(p, b / p.spacing);
+        return;
+    }
+    const int j = b - before;
+    const int64_t s = p.src_ids[j], d = p.dst_ids[j];
+    const int vecs = (int)(p.page_bytes / (int64_t)sizeof(Vec));
+    const Vec *src = reinterpret_cast<const Vec *>(static_cast<const char *>(p.src_pool) + s * p.page_bytes);
+    Vec *dst = reinterpret_cast<Vec *>(static_cast<char *>(p.dst_pool) + d * p.page_bytes);
+    copy_row(dst, vecs, [&](int c) { return src + c; });
+    if (p.src_scales != nullptr && threadIdx.x < kScaleVecs)
+        p.dst_scales[d * kScaleVecs + threadIdx.x] = __ldg(p.src_scales + s * kScaleVecs + threadIdx.x);
 }
 
 // Remap table of the allocation-free entry point: lives in the library's device image,
@@ -97,28 +116,31 @@ cudaError_t launch_page_migrate(const void *src_pool, const float *src_scales, v
                                 const int32_t *dst_ids, int64_t n, int32_t src_base, int32_t dst_base,
                                 int32_t max_page_id, int32_t *block_table, int64_t num_entries,
                                 int32_t *remap, bool do_table, bool do_copy, cudaStream_t stream) {
-    cudaError_t e;
-    if (do_table && num_entries > 0 && max_page_id > 0) {
-        remap_fill_kernel<<<(max_page_id + 255) / 256, 256, 0, stream>>>(remap, max_page_id);
+    MigrateParams p;
+    p.src_pool = src_pool; p.dst_pool = dst_pool;
+    p.src_scales = reinterpret_cast<const uint4 *>(src_scales); p.dst_scales = reinterpret_cast<uint4 *>(dst_scales);
+    p.page_bytes = page_bytes; p.src_ids = src_ids; p.dst_ids = dst_ids; p.n = (int32_t)n;
+    p.src_base = src_base; p.dst_base = dst_base; p.max_page_id = max_page_id;
+    p.table = block_table; p.remap = remap; p.num_entries = num_entries;
+    const bool table = do_table && num_entries > 0 && max_page_id > 0;
+    const int64_t pages = do_copy ? n : 0;
+    p.table_blocks = table ? (int32_t)((num_entries + kEntriesPerBlock - 1) / kEntriesPerBlock) : 0;
+    p.after_scatter = table ? 1 : 0;
+    const int64_t blocks = pages + p.table_blocks;
+    if (blocks == 0) return cudaSuccess;
+    p.spacing = p.table_blocks > 0 ? (int32_t)(blocks / p.table_blocks) : 1;
+    cudaError_t e = cudaSuccess;
+    if (table) {
+        e = launch_dependent(remap_scatter_kernel, dim3((unsigned)((n + kCopyThreads - 1) / kCopyThreads)), dim3(kCopyThreads), 0, stream,
+                             remap, src_ids, n, src_base, max_page_id);
         count_launch();
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        remap_scatter_kernel<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(remap, src_ids, dst_ids, n, src_base,
-                                                                               dst_base, max_page_id);
-        count_launch();
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        table_rewrite_kernel<<<(unsigned)((num_entries + 255) / 256), 256, 0, stream>>>(block_table, num_entries,
-                                                                                        remap, max_page_id);
-        count_launch();
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if (e != cudaSuccess) return e;
     }
-    if (!do_copy) return cudaSuccess;
-    dim3 grid((unsigned)n, kCopyCtasPerPage);
-    page_copy_kernel<<<grid, kCopyThreads, 0, stream>>>(
-        static_cast<const uint4 *>(src_pool), static_cast<uint4 *>(dst_pool),
-        reinterpret_cast<const uint4 *>(src_scales), reinterpret_cast<uint4 *>(dst_scales),
-        page_bytes / 16, src_ids, dst_ids);
+    // 32-byte accesses where the pages lie on 32-byte boundaries (they do in every pool of whole pages whose base does)
+    const bool wide = copy_width(address_bits(src_pool) | address_bits(dst_pool) | (uint64_t)page_bytes) == 32;
+    e = launch_dependent(wide ? page_migrate_kernel<Vec32> : page_migrate_kernel<uint4>, dim3((unsigned)blocks), dim3(kCopyThreads), 0, stream, p);
     count_launch();
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace splash
