@@ -567,10 +567,8 @@ int splash_dop_pack_rows(const void *a, int64_t a_part_bytes, int64_t a_row_pitc
     }
     if (a_head_pitch < a_part_bytes || (b && b_head_pitch < b_part_bytes)) { set_error("head pitch smaller than the part"); return SPLASH_INVALID_ARG; }
     if (n > 0x7fffffffLL) { set_error("too many rows"); return SPLASH_INVALID_ARG; }
-    DeviceInfo dev;
-    if (!current_device_info(dev)) return SPLASH_CUDA_ERROR;
     cudaError_t e = launch_dop_pack_rows(a, b, send, send_row, n, h, a_part_bytes, b_part_bytes, a_row_pitch, a_head_pitch,
-                                         b_row_pitch, b_head_pitch, dev.sm_count, static_cast<cudaStream_t>(stream_));
+                                         b_row_pitch, b_head_pitch, static_cast<cudaStream_t>(stream_));
     if (e != cudaSuccess) { set_error("CUDA error: %s", cudaGetErrorString(e)); return SPLASH_CUDA_ERROR; }
     return SPLASH_OK;
 }
@@ -585,9 +583,7 @@ int splash_dop_swap_outer(const void *in, int64_t A, int64_t B, int64_t inner_by
         const int64_t bytes = A * B * inner_bytes;
         if (po < pi + bytes && pi < po + bytes) { set_error("out overlaps in"); return SPLASH_INVALID_ARG; }
     }
-    DeviceInfo dev;
-    if (!current_device_info(dev)) return SPLASH_CUDA_ERROR;
-    cudaError_t e = launch_dop_swap_outer(in, out, A, B, inner_bytes, dev.sm_count, static_cast<cudaStream_t>(stream_));
+    cudaError_t e = launch_dop_swap_outer(in, out, A, B, inner_bytes, static_cast<cudaStream_t>(stream_));
     if (e != cudaSuccess) { set_error("CUDA error: %s", cudaGetErrorString(e)); return SPLASH_CUDA_ERROR; }
     return SPLASH_OK;
 }
@@ -601,9 +597,7 @@ int splash_dop_unpack_rows(const void *recv, const int32_t *send_row, int64_t n,
         set_error("a required pointer is NULL or misaligned"); return SPLASH_INVALID_ARG;
     }
     if (out_row_pitch < row_bytes) { set_error("out_row_pitch smaller than a row"); return SPLASH_INVALID_ARG; }
-    DeviceInfo dev;
-    if (!current_device_info(dev)) return SPLASH_CUDA_ERROR;
-    cudaError_t e = launch_dop_unpack_rows(recv, out, send_row, n, row_bytes, out_row_pitch, dev.sm_count,
+    cudaError_t e = launch_dop_unpack_rows(recv, out, send_row, n, row_bytes, out_row_pitch,
                                            static_cast<cudaStream_t>(stream_));
     if (e != cudaSuccess) { set_error("CUDA error: %s", cudaGetErrorString(e)); return SPLASH_CUDA_ERROR; }
     return SPLASH_OK;
