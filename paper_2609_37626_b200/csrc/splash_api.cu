@@ -104,7 +104,7 @@ Tiling choose_tiling(const splash_mla_shape *s, int h, int sm_count, bool simt) 
     t.pair_groups = 1;
     if (!simt && s->q_rows > 1) {      // several query rows per request: always CTA pairs, whatever the width
         // more than 128 (head, row) pairs: several pairs per KV worker, side by side on the same pages
-        t.heads_per_group = 64; t.num_groups = 2;
+        t.heads_per_group = s->kv_dtype != SPLASH_KV_BF16 && h <= 64 ? 32 : 64; t.num_groups = 2;
         t.pair_groups = (h + kMaxHeads - 1) / kMaxHeads;
         const int w = (sm_count / 2) / t.pair_groups;
         t.num_workers = w > 0 ? w : 1;
@@ -118,7 +118,7 @@ Tiling choose_tiling(const splash_mla_shape *s, int h, int sm_count, bool simt) 
         t.num_workers = w > 0 ? w : 1;
         return t;
     }
-    umma_tiling(s->kv_dtype, h, sm_count, &t.heads_per_group, &t.num_groups, &t.num_workers);
+    umma_tiling(s->kv_dtype, h, sm_count, (s->flags & SPLASH_FLAG_NO_PAIR) == 0, &t.heads_per_group, &t.num_groups, &t.num_workers);
     return t;
 }
 
@@ -149,10 +149,12 @@ size_t splash_mla_decode_workspace_bytes(const splash_mla_shape *shape, int32_t 
     const int R = shape->q_rows > 1 ? (int)shape->q_rows : 1;
     const int h = (head_end - head_begin) * R;
     if (h == 0 || shape->num_requests == 0) return 256;
-    // the larger of the two kernels' needs, so one workspace serves both paths
+    // the largest of the kernels' needs, so one workspace serves every path (SPLASH_FLAG_SIMT, SPLASH_FLAG_NO_PAIR)
     size_t need = 0;
-    for (int simt = 0; simt < 2; ++simt) {
-        Tiling t = choose_tiling(shape, h, dev.sm_count, simt != 0);
+    for (int path = 0; path < 3; ++path) {
+        splash_mla_shape s = *shape;
+        s.flags = path == 2 ? s.flags | SPLASH_FLAG_NO_PAIR : s.flags & ~SPLASH_FLAG_NO_PAIR;
+        Tiling t = choose_tiling(&s, h, dev.sm_count, path == 1);
         PlanView v = make_plan_view(nullptr, shape->num_requests, t.num_workers, h);
         if (v.bytes > need) need = v.bytes;
     }
@@ -275,7 +277,7 @@ int decode_dense(const splash_mla_shape *shape, const void *q, const void *kv_po
         const int pages = sparse ? sparse->pages_per_request : shape->block_table_stride;
         // (the e4m3 pair kernel's own plan saves 4 us and costs 2.6 % of its main loop: long contexts keep the plan kernel,
         // unless the call takes a partition over, which may have been one that left nothing in the workspace)
-        const bool e4m3_pairs = shape->kv_dtype == SPLASH_KV_E4M3_TOKEN_SCALE && t.num_groups == 2 && t.heads_per_group == 64 &&
+        const bool e4m3_pairs = shape->kv_dtype == SPLASH_KV_E4M3_TOKEN_SCALE && t.num_groups == 2 &&
                                 !(shape->flags & (SPLASH_FLAG_NO_PAIR | SPLASH_FLAG_REUSE_PLAN));
         if (!e4m3_pairs || (int64_t)B * pages * t.pair_groups <= kInlinePairPages)
             plan_mode = pages <= kWholeRequestPages && B <= t.num_workers ? kPlanWhole : kPlanInline;
@@ -310,9 +312,9 @@ int decode_dense(const splash_mla_shape *shape, const void *q, const void *kv_po
         p.ctx_lens = sparse->ctx_lens;
     }
     p.request_overhead_tiles = kRequestOverheadTilesDefault;
-    const bool pair = !simt && t.num_groups == 2 && t.heads_per_group == 64 && !(shape->flags & SPLASH_FLAG_NO_PAIR);
+    const bool pair = !simt && t.num_groups == 2 && !(shape->flags & SPLASH_FLAG_NO_PAIR);
     if (!simt && shape->kv_dtype == SPLASH_KV_E4M3_TOKEN_SCALE)
-        p.request_overhead_tiles = pair ? kRequestOverheadTilesFp8Pair : kRequestOverheadTilesFp8;
+        p.request_overhead_tiles = !pair ? kRequestOverheadTilesFp8 : t.heads_per_group == 32 ? kRequestOverheadTilesFp8Pair32 : kRequestOverheadTilesFp8Pair;
     else if (pair)
         p.request_overhead_tiles = kRequestOverheadTilesPair;
     // the bf16 CTA-pair kernel writes its partial outputs as f16

@@ -29,6 +29,7 @@ constexpr int kRequestOverheadTilesDefault = 4;
 constexpr int kRequestOverheadTilesFp8 = 6;        // also right for the 16- / 32-head e4m3 kernel: a TP-8 share of the rollout
                                                    // workload takes 237 / 232 / 228 / 224 / 227 / 232 / 239 us with 2 / 3 / 4 / 6 / 8 / 10 / 14
 constexpr int kRequestOverheadTilesPair = 5;       // bf16 CTA-pair kernel (a segment costs 7,500 cycles, a tile 1,650)
+constexpr int kRequestOverheadTilesFp8Pair32 = 8;  // the same kernel with 32 heads per CTA
 constexpr int kRequestOverheadTilesFp8Pair = 13;   // CTA-pair kernel: tiles are cheaper, the per-request work is not
 
 // ---- workspace layout ------------------------------------------------------
@@ -440,7 +441,7 @@ cudaError_t launch_dop_swap_outer(const void *in, void *out, int64_t A, int64_t 
 cudaError_t launch_decode_simt(const DecodeParams &p, int kv_dtype, cudaStream_t stream);
 int simt_heads_per_group();
 // tcgen05 kernel: how it cuts a head slice of width h into CTAs, and its launcher
-void umma_tiling(int kv_dtype, int h, int sm_count, int *heads_per_group, int *num_groups, int *num_workers);
+void umma_tiling(int kv_dtype, int h, int sm_count, bool pairs, int *heads_per_group, int *num_groups, int *num_workers);
 cudaError_t launch_decode_umma(const DecodeParams &p, const splash_mla_shape &shape, cudaStream_t stream);
 cudaError_t launch_decode_umma_fp8(const DecodeParams &p, cudaStream_t stream);
 cudaError_t launch_decode_umma_fp8_narrow(const DecodeParams &p, cudaStream_t stream);   // 16 / 32 heads per CTA

@@ -683,9 +683,10 @@ cudaError_t launch_n(const DecodeParams &p, const CUtensorMap &mkv, const CUtens
 
 }  // namespace
 
-void umma_tiling(int kv_dtype, int h, int sm_count, int *heads_per_group, int *num_groups, int *num_workers) {
-    (void)kv_dtype;       // both cache formats have 16-, 32- and 64-head kernels
-    const int n = h <= 16 ? 16 : (h <= 32 ? 32 : 64);
+void umma_tiling(int kv_dtype, int h, int sm_count, bool pairs, int *heads_per_group, int *num_groups, int *num_workers) {
+    // both cache formats have 16-, 32- and 64-head kernels; 33..64 heads over an e4m3 cache run as a CTA pair of 32 each
+    // (100 requests of 500 to 20,000 tokens, 64 heads: 147 us with one CTA per worker, 130 us with pairs, the SMs at the power limit)
+    const int n = h <= 16 ? 16 : (h <= 32 || (h <= 64 && pairs && kv_dtype != SPLASH_KV_BF16) ? 32 : 64);
     *heads_per_group = n;
     *num_groups = (h + n - 1) / n;
     const int w = sm_count / *num_groups;
@@ -694,7 +695,7 @@ void umma_tiling(int kv_dtype, int h, int sm_count, int *heads_per_group, int *n
 
 cudaError_t launch_decode_umma(const DecodeParams &p, const splash_mla_shape &shape, cudaStream_t stream) {
     if (shape.kv_dtype != SPLASH_KV_BF16) {
-        // slices of more than 64 heads run on CTA pairs (cta_group::2) unless the caller opts out
+        // slices of more than 32 heads run on CTA pairs (cta_group::2) unless the caller opts out
         if (p.num_groups == 2 && !(shape.flags & SPLASH_FLAG_NO_PAIR)) {
             const cudaError_t e = launch_decode_umma_fp8_pair(p, stream);
             if (e != cudaErrorNotSupported) return e;      // output rows not 16-byte aligned: no TMA stores

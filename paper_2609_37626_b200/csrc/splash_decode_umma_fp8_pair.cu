@@ -1,17 +1,23 @@
-// e4m3 decode kernel for slices of 65..128 heads: a CLUSTER OF TWO CTAs per KV worker that
-// issues its MMAs with tcgen05 cta_group::2.
+// e4m3 decode kernel for slices of 33..128 heads: a CLUSTER OF TWO CTAs per KV worker that
+// issues its MMAs with tcgen05 cta_group::2.  H = 64 or 32 heads per CTA.
 //
-// Why: with both operands in shared memory a small MMA costs what its operands cost to
-// stream ((A + B bytes) / 128 B per cycle).  Two independent 64-head CTAs each stream every
-// K row and every V row themselves.  A CTA pair shares them:
+// Why pairs: with both operands in shared memory a small MMA costs what its operands cost to
+// stream ((A + B bytes) / 128 B per cycle).  Two independent CTAs each stream every
+// K row and every V row themselves.  A CTA pair shares them.  A "supertile" is two consecutive
+// page tiles of a segment; each CTA supplies ONE page (64 tokens) as its half of the B operand.
+// bf16 x e4m3 is not an MMA type pair, so q (one scale per head) and P are each split into two
+// 8-bit terms, hi + lo:
 //
-//   S [128 heads x 128 tokens] = Q K^T      M = 128 (64 heads per CTA), N = 128: each CTA supplies
-//                                            ONE page (64 tokens) as its half of the B operand
-//   O [128 heads x 256 dv]    += P V        M = 128, N = 256 (x 2 halves of dv): each CTA supplies
-//                                            its 64 heads of P and 128 of the 256 dv columns
+//   H = 64:  S [128 heads x 128 tokens]  = q hi K^T + q lo K^T    M = 128 (64 heads per CTA), N = 128, 36 MMAs of K = 32
+//            O [128 heads x 256 dv]     += P hi V + P lo V        M = 128, N = 256 (x 2 halves of dv): each CTA supplies
+//                                                                  its 64 heads of P and 128 of the 256 dv columns
+//   H = 32:  the same shapes, but the two terms are ROWS of one A operand (16 hi rows and the 16 lo rows of the same
+//            heads in turn: a TMEM lane quadrant holds both terms of its heads), half as many MMAs:
+//            S [(hi, lo) x 64 heads x 128 tokens] = [q hi; q lo] K^T,  O [(hi, lo) x 64 heads x 256 dv] += [P hi; 16 P lo] V
+//            the softmax adds the two halves of a logit, the epilogue hi + lo / 16
 //
-// so per 128 tokens and per CTA the tensor cores read 72 KB (QK^T) + 96 KB (P.V) instead of
-// 288 + 192 KB.  A "supertile" is two consecutive page tiles of a segment: CTA r loads page r
+// so per 128 tokens and per CTA the tensor cores read 72 + 96 KB (H = 64) or 36 + 48 KB (H = 32).
+// CTA r loads page r
 // (all 9 chunks of 64 columns) into a stage for QK^T.  For P.V CTA r supplies dv columns
 // [256 n + 128 r, + 128) of BOTH pages, at the same shared-memory offsets in both CTAs (the
 // two CTAs of an MMA share one descriptor).  Its own page already has them in chunk slots
@@ -19,11 +25,14 @@
 // columns only the peer needs, so once QK^T of the stage has retired they are overwritten
 // with the peer page's chunks 4 n + 2 r, 4 n + 2 r + 1.  The MMAs over page g then start at
 // slot 4 n + 2 g in both CTAs.  That second load hides behind the softmax of the supertile.
-// Accumulators: CTA r holds its 64 heads; a head's row is TMEM lane h (tokens / dv of the
-// first half of N) and lane 64 + h (second half).
+// Accumulators: CTA r holds its 64 rows; row i is TMEM lane i (tokens / dv of the
+// first half of N) and lane 64 + i (second half).
 //
-// Roles per CTA (576 threads): K-page + scale producer, 2 QK^T issuers and 2 P.V issuers
+// Roles per CTA (512 threads): K-page + scale producer, QK^T issuer and P.V issuer
 // (leader CTA only), 8 softmax warps, 4 query converters, 1 producer of the peer chunks.
+// An issuer warp stays converged and one elected lane issues: what the MMAs take is the same in all lanes then and lives
+// in uniform registers.  Issued from a branch that lane 0 alone takes, an MMA costs 65 to 90 cycles, because every
+// descriptor has to be moved there first; converged, 35 to 48, and one warp does what took two.
 // Barriers that the issuers wait on live in the leader; the peer's warps arrive on them across
 // the cluster (relaxed arrivals: what they announce is already in place on the peer's SM), and
 // TMA loads of the peer complete on them too.
@@ -36,92 +45,101 @@ namespace {
 
 using namespace umma;
 
-constexpr int kQkWarps = 2, kPvWarps = 2, kSoftmaxWarps = 8, kConvertWarps = 4;
+constexpr int kIssuerWarps = 2, kSoftmaxWarps = 8, kConvertWarps = 4;
 constexpr int kWarpProducer = 0;
 constexpr int kWarpQk = 1;
-constexpr int kWarpPv = kWarpQk + kQkWarps;
-constexpr int kWarpSoftmax = kWarpPv + kPvWarps;
+constexpr int kWarpPv = 2;
+constexpr int kWarpSoftmax = kWarpQk + kIssuerWarps;
 constexpr int kWarpConvert = kWarpSoftmax + kSoftmaxWarps;
 constexpr int kWarpVProducer = kWarpConvert + kConvertWarps;
-constexpr int kThreads = (kWarpVProducer + 1) * 32;    // 18 warps = 576 threads
-constexpr int kN = 64;                              // heads per CTA
+constexpr int kThreads = (kWarpVProducer + 1) * 32;    // 16 warps = 512 threads
 constexpr uint32_t kSlab = 64 * 64;                 // 64 rows x 64 B
 constexpr uint32_t kPageBytes = 9 * kSlab;          // 36,864
 constexpr uint32_t kPeerBytes = 4 * kSlab;          // the peer page's chunks this CTA multiplies: 16,384
 constexpr uint32_t kScaleBytes = 256;
-constexpr int kStages = 3;
 constexpr int kPrefetchAhead = 1;                    // supertiles between the L2 prefetch of a page and its use (4: 1.5 % slower; none: 5 %)
 constexpr int kPrefetchAheadBusy = 4;                // the same while the call carries a page-copy job
 constexpr float kTau = 7.0f;                          // (6 / 2.75: 0.3 % slower on the rollout workload, 4 / 4.75 more)
 constexpr float kLift = 1.75f;
 
-enum BarrierId {
-    kBarKFull = 0,                        // [3] leader: both CTAs' pages landed (tx bytes of both)
-    kBarQkDone = kBarKFull + kStages,     // [3] QK^T of the stage retired (multicast commit): peer chunks may land
-    kBarVFull = kBarQkDone + kStages,     // [3] leader: both CTAs' peer chunks landed
-    kBarStageEmpty = kBarVFull + kStages, // [3] P.V of the stage retired (multicast commit): stage, its scales and
-                                          //     the P buffer are free, O is up to date
-    kBarScFull = kBarStageEmpty + kStages,// [3] local: scale pages of the stage landed
-    kBarQFull = kBarScFull + kStages,     // leader: query operands of both CTAs written
-    kBarQLocal,                           // local: this CTA's query scales written
-    kBarQEmpty,                           // last QK^T of the request retired (multicast commit)
-    kBarQsRead,                           // local: the softmax warps have picked up the request's query scales
-    kBarSFull,                            // [2] S buffer written (multicast commit)
-    kBarSEmpty = kBarSFull + 2,           // [2] S buffer read (leader: by both CTAs)
-    kBarPFull = kBarSEmpty + 2,           // [2] P buffer written (leader: by both CTAs)
-    kBarOFull = kBarPFull + 2,            // last P.V of the request retired (multicast commit)
-    kBarOEmpty,                           // O drained (leader: by both CTAs)
-    kNumBarriers
+// H = 64: three stages are what shared memory holds beside 73,728 B of query operands; H = 32: four.
+template <int H>
+struct Layout {
+    static constexpr int kStages = H == 64 ? 3 : 4;
+    enum BarrierId {
+        kBarKFull = 0,                        // [stages] leader: both CTAs' pages landed (tx bytes of both)
+        kBarQkDone = kBarKFull + kStages,     // [stages] QK^T of the stage retired (multicast commit): peer chunks may land
+        kBarVFull = kBarQkDone + kStages,     // [stages] leader: both CTAs' peer chunks landed
+        kBarStageEmpty = kBarVFull + kStages, // [stages] P.V of the stage retired (multicast commit): stage, its scales and
+                                              //     the P buffer are free, O is up to date
+        kBarScFull = kBarStageEmpty + kStages,// [stages] local: scale pages of the stage landed
+        kBarQFull = kBarScFull + kStages,     // leader: query operands of both CTAs written
+        kBarQLocal,                           // local: this CTA's query scales written
+        kBarQEmpty,                           // last QK^T of the request retired (multicast commit)
+        kBarQsRead,                           // local: the softmax warps have picked up the request's query scales
+        kBarSFull,                            // [2] S buffer written (multicast commit)
+        kBarSEmpty = kBarSFull + 2,           // [2] S buffer read (leader: by both CTAs)
+        kBarPFull = kBarSEmpty + 2,           // [2] P buffer written (leader: by both CTAs)
+        kBarOFull = kBarPFull + 2,            // last P.V of the request retired (multicast commit)
+        kBarOEmpty,                           // O drained (leader: by both CTAs)
+        kNumBarriers
+    };
+    // query operand: 9 chunk slabs of 64 rows x 64 B for q hi and as many for q lo (H = 64), or both as rows of one (H = 32)
+    static constexpr uint32_t kQTerm = H == 64 ? 9 * kSlab : 16 * 64;        // from a head's hi row to its lo row
+    static constexpr uint32_t kPTerm = H == 64 ? 2 * kSlab : 16 * 64;        // the same in P
+    static constexpr uint32_t kPBuf = H == 64 ? 4 * kSlab : 2 * kSlab;
+    static constexpr uint32_t kOffK = 0;                            // [stages] 9 chunk slots
+    static constexpr uint32_t kOffQ = kOffK + kStages * kPageBytes;
+    static constexpr uint32_t kOffP = kOffQ + 2 * H * kDQK;         // [2 buffers] ([hi, lo]) [2 page slabs] x 4096
+    static constexpr uint32_t kOffScale = kOffP + 2 * kPBuf;        // float [stages][2 pages][64]
+    static constexpr uint32_t kOffQs = kOffScale + kStages * 2 * kScaleBytes;    // float [4][H]
+    static constexpr uint32_t kOffAlpha = kOffQs + 4 * H * 4;       // float [H]
+    static constexpr uint32_t kOffL = kOffAlpha + H * 4;            // float [H]
+    static constexpr uint32_t kOffXch = kOffL + H * 4;              // float [H][4]
+    static constexpr uint32_t kTokBytes = 32 * 8 + 32 * 4;          // per warp: (scale, log2 scale) x 32, 1 / scale x 32
+    static constexpr uint32_t kOffTok = kOffXch + H * 16;
+    static constexpr uint32_t kOffBar = kOffTok + kSoftmaxWarps * kTokBytes;
+    static constexpr uint32_t kOffMisc = (kOffBar + kNumBarriers * 8 + 15) / 16 * 16;
+    static constexpr uint32_t kOffPlan = kOffMisc + 32;             // inline plan
+    static constexpr uint32_t kSmemBytes = kOffPlan + kInlinePlanBytes;
+    static_assert(kSmemBytes <= 232448, "shared memory overflow");
+    static_assert(kOffQ % 1024 == 0 && kOffP % 1024 == 0 && kOffTok % 16 == 0 && kTokBytes % 16 == 0, "alignment");
+    // tensor memory: O two halves of dv x 128 columns, then 2 S buffers x 64 columns
+    static constexpr uint32_t kColO = 0, kColS = 256;
 };
 
-constexpr uint32_t kOffK = 0;                                   // [3 stages] 9 chunk slots
-constexpr uint32_t kOffQHi = kOffK + kStages * kPageBytes;
-constexpr uint32_t kOffQLo = kOffQHi + kN * kDQK;
-constexpr uint32_t kOffP = kOffQLo + kN * kDQK;                 // [2 buffers][hi, lo][2 page slabs] x 4096
-constexpr uint32_t kOffScale = kOffP + 2 * 2 * 2 * kSlab;       // float [3 stages][2 pages][64]
-constexpr uint32_t kOffQs = kOffScale + kStages * 2 * kScaleBytes;    // float [4][64]
-constexpr uint32_t kOffAlpha = kOffQs + 4 * kN * 4;             // float [64]
-constexpr uint32_t kOffL = kOffAlpha + kN * 4;                  // float [64]
-constexpr uint32_t kOffXch = kOffL + kN * 4;                    // float [64][4]
-constexpr uint32_t kTokBytes = 32 * 8 + 32 * 4;                 // per warp: (scale, log2 scale) x 32, 1 / scale x 32
-constexpr uint32_t kOffTok = kOffXch + kN * 16;
-constexpr uint32_t kOffBar = kOffTok + kSoftmaxWarps * kTokBytes;
-constexpr uint32_t kOffMisc = (kOffBar + kNumBarriers * 8 + 15) / 16 * 16;
-constexpr uint32_t kOffPlan = kOffMisc + 32;                    // inline plan
-constexpr uint32_t kSmemBytes = kOffPlan + kInlinePlanBytes;
-static_assert(kSmemBytes <= 232448, "shared memory overflow");
-static_assert(kOffQHi % 1024 == 0 && kOffP % 1024 == 0 && kOffTok % 16 == 0 && kTokBytes % 16 == 0, "alignment");
-// tensor memory: O two halves of dv x 128 columns, then 2 S buffers x 2 partials x 64 columns
-constexpr uint32_t kColO = 0, kColS = 256;
-
-__device__ __forceinline__ void umma_e4m3_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+// Issued by the elected lane of a converged warp; the operands are uniform.
+__device__ __forceinline__ void umma_e4m3_pair(uint32_t elected, uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
+        "{\n\t.reg .pred p, q;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
+        "setp.ne.b32 q, %5, 0;\n\t"
+        "@q tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(elected) : "memory");
 }
 
 // kInline: the variant that can plan for itself.  The kernel sits at its register cap, and a walk over the segments that
 // can read either plan costs the main loop 0.6 to 2.4 % of its cycles: calls behind a plan kernel have their own variant.
-template <bool kInline>
+template <int H, bool kInline>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid_constant__ CUtensorMap tmap_page,
                             const __grid_constant__ CUtensorMap tmap_pair, const __grid_constant__ CUtensorMap tmap_out,
                             const __grid_constant__ CUtensorMap tmap_part) {
+    using L = Layout<H>;
+    constexpr int kStages = L::kStages;
     extern __shared__ __align__(1024) uint8_t smem[];
     const uint32_t sbase = smem_u32(smem);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t rank = cluster_ctarank();             // 0 = leader: issues the MMAs
-    const int pair_id = blockIdx.x >> 1;                // CTA pair: (KV worker, group of 128 heads)
+    const int pair_id = blockIdx.x >> 1;                // CTA pair: (KV worker, group of 2 H heads)
     const int worker = pair_id / p.pair_groups;
-    const int head0 = p.head_begin + (pair_id % p.pair_groups) * (2 * kN) + (int)rank * kN;
+    const int head0 = p.head_begin + (pair_id % p.pair_groups) * (2 * H) + (int)rank * H;
     const int h = p.head_end - p.head_begin;
 
-    volatile uint32_t *misc = reinterpret_cast<volatile uint32_t *>(smem + kOffMisc);
+    volatile uint32_t *misc = reinterpret_cast<volatile uint32_t *>(smem + L::kOffMisc);
     Ctx ctx{misc + 1, p.status};
-    auto bar = [&](int id) -> uint32_t { return sbase + kOffBar + 8u * (uint32_t)id; };
-    auto leader_bar = [&](int id) -> uint32_t { return map_to_cta(sbase + kOffBar + 8u * (uint32_t)id, 0); };
+    auto bar = [&](int id) -> uint32_t { return sbase + L::kOffBar + 8u * (uint32_t)id; };
+    auto leader_bar = [&](int id) -> uint32_t { return map_to_cta(sbase + L::kOffBar + 8u * (uint32_t)id, 0); };
     // one arrival of a warp of either CTA on a barrier that lives in the leader
     auto arrive_on_leader = [&](int id) {
         if (rank == 0) mbar_arrive(bar(id));
@@ -131,22 +149,22 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
     if (tid == 0) {
         // barriers the leader's issuers wait on count the warps of both CTAs (the peer's copies are unused)
         for (int s = 0; s < kStages; ++s) {
-            mbar_init(bar(kBarKFull + s), 1); mbar_init(bar(kBarQkDone + s), kQkWarps);
-            mbar_init(bar(kBarVFull + s), 1); mbar_init(bar(kBarStageEmpty + s), kPvWarps);
-            mbar_init(bar(kBarScFull + s), 1);
+            mbar_init(bar(L::kBarKFull + s), 1); mbar_init(bar(L::kBarQkDone + s), 1);
+            mbar_init(bar(L::kBarVFull + s), 1); mbar_init(bar(L::kBarStageEmpty + s), 1);
+            mbar_init(bar(L::kBarScFull + s), 1);
         }
-        mbar_init(bar(kBarQFull), 2 * kConvertWarps); mbar_init(bar(kBarQLocal), kConvertWarps); mbar_init(bar(kBarQEmpty), kQkWarps);
-        mbar_init(bar(kBarQsRead), kSoftmaxWarps);
+        mbar_init(bar(L::kBarQFull), 2 * kConvertWarps); mbar_init(bar(L::kBarQLocal), kConvertWarps); mbar_init(bar(L::kBarQEmpty), 1);
+        mbar_init(bar(L::kBarQsRead), kSoftmaxWarps);
         for (int b = 0; b < 2; ++b) {
-            mbar_init(bar(kBarSFull + b), kQkWarps); mbar_init(bar(kBarSEmpty + b), 2 * kSoftmaxWarps);
-            mbar_init(bar(kBarPFull + b), 2 * kSoftmaxWarps);
+            mbar_init(bar(L::kBarSFull + b), 1); mbar_init(bar(L::kBarSEmpty + b), 2 * kSoftmaxWarps);
+            mbar_init(bar(L::kBarPFull + b), 2 * kSoftmaxWarps);
         }
-        mbar_init(bar(kBarOFull), kPvWarps); mbar_init(bar(kBarOEmpty), 2 * kSoftmaxWarps);
+        mbar_init(bar(L::kBarOFull), 1); mbar_init(bar(L::kBarOEmpty), 2 * kSoftmaxWarps);
         misc[1] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(sbase + kOffMisc), "r"(512u) : "memory");
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(sbase + L::kOffMisc), "r"(512u) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
     tcgen05_fence_before();
@@ -158,7 +176,7 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
     const long long t_start = clock64();
     const unsigned long long ns_start = global_timer_ns();
 
-    SegmentIter<kInline ? kOffPlan : kPlanInWorkspace> it;
+    SegmentIter<kInline ? L::kOffPlan : kPlanInWorkspace> it;
     start_plan(p, worker, kThreads / 32 - 1, it);
     Segment seg;
     seg.lo = seg.hi = seg.tile_begin = seg.tile_end = 0;
@@ -189,7 +207,7 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
                 const PairGeom g = pair_geom(s);
                 const int ta = seg.tile_begin + 2 * s;
                 const uint32_t stage = st_it % kStages, ph = (st_it / kStages) & 1;
-                const uint32_t k0 = sbase + kOffK + stage * kPageBytes;
+                const uint32_t k0 = sbase + L::kOffK + stage * kPageBytes;
                 // the page this warp fetches: its CTA's own for QK^T, the other CTA's for the P.V chunks.  A tile cut at
                 // both ends inside its page is written by hand instead (zeros outside the range); only a request whose
                 // whole range lies inside one page has such a tile, and it is page A.
@@ -199,26 +217,26 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
                     page_a = table[first_page + ta];
                     page_b = g.has_b ? table[first_page + ta + 1] : p.num_pool_pages;   // a page past the pool reads as zeros
                     if (!is_v) {
-                        ok = mbar_wait(ctx, bar(kBarStageEmpty + stage), ph ^ 1, kBarStageEmpty + stage);
+                        ok = mbar_wait(ctx, bar(L::kBarStageEmpty + stage), ph ^ 1, L::kBarStageEmpty + stage);
                         if (ok) {
                             // the leader's barrier expects the pages of both CTAs
-                            if (rank == 0) mbar_expect_tx(bar(kBarKFull + stage), 2 * kPageBytes);
+                            if (rank == 0) mbar_expect_tx(bar(L::kBarKFull + stage), 2 * kPageBytes);
                             if (!tg.both)
-                                tma_load_4d_pair(k0, &tmap_page, leader_bar(kBarKFull + stage), 0, tg.tok0, 0, rank == 0 ? page_a : page_b);
+                                tma_load_4d_pair(k0, &tmap_page, leader_bar(L::kBarKFull + stage), 0, tg.tok0, 0, rank == 0 ? page_a : page_b);
                             // scale pages of both pages, for this CTA's softmax warps
                             const bool in_a = page_a >= 0 && page_a < p.num_pool_pages;
                             const bool in_b = g.has_b && page_b >= 0 && page_b < p.num_pool_pages;
                             if (!in_a || (g.has_b && !in_b)) {     // a page outside the pool reads as zeros; give its tokens the scale 1
-                                float *sc1 = reinterpret_cast<float *>(smem + kOffScale + stage * 2 * kScaleBytes);
+                                float *sc1 = reinterpret_cast<float *>(smem + L::kOffScale + stage * 2 * kScaleBytes);
                                 for (int t = 0; t < kPage; ++t) {
                                     if (!in_a) sc1[t] = 1.0f;
                                     if (g.has_b && !in_b) sc1[kPage + t] = 1.0f;
                                 }
                             }
-                            mbar_expect_tx(bar(kBarScFull + stage), (in_a ? kScaleBytes : 0u) + (in_b ? kScaleBytes : 0u));
-                            const uint32_t sdst = sbase + kOffScale + stage * 2 * kScaleBytes;
-                            if (in_a) bulk_load(sdst, p.kv_scales + (int64_t)page_a * kPage, kScaleBytes, bar(kBarScFull + stage));
-                            if (in_b) bulk_load(sdst + kScaleBytes, p.kv_scales + (int64_t)page_b * kPage, kScaleBytes, bar(kBarScFull + stage));
+                            mbar_expect_tx(bar(L::kBarScFull + stage), (in_a ? kScaleBytes : 0u) + (in_b ? kScaleBytes : 0u));
+                            const uint32_t sdst = sbase + L::kOffScale + stage * 2 * kScaleBytes;
+                            if (in_a) bulk_load(sdst, p.kv_scales + (int64_t)page_a * kPage, kScaleBytes, bar(L::kBarScFull + stage));
+                            if (in_b) bulk_load(sdst + kScaleBytes, p.kv_scales + (int64_t)page_b * kPage, kScaleBytes, bar(L::kBarScFull + stage));
                             // A stage is held from its load until P.V has read it, about three supertiles, so the
                             // load of supertile s + 3 starts only when the issuers are about to need it: have its
                             // page in L2 by then.
@@ -230,14 +248,14 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
                             }
                         }
                     } else {
-                        ok = mbar_wait(ctx, bar(kBarQkDone + stage), ph, kBarQkDone + stage);
+                        ok = mbar_wait(ctx, bar(L::kBarQkDone + stage), ph, L::kBarQkDone + stage);
                         if (ok) {
-                            if (rank == 0) mbar_expect_tx(bar(kBarVFull + stage), 2 * kPeerBytes);
+                            if (rank == 0) mbar_expect_tx(bar(L::kBarVFull + stage), 2 * kPeerBytes);
                             // peer page chunks 4n + 2 rank, + 1 -> slots 4n + 2 (1 - rank), + 1
                             if (!tg.both) {
 #pragma unroll
                                 for (int n = 0; n < 2; ++n)
-                                    tma_load_4d_pair(k0 + (4 * n + 2 * (1 - (int)rank)) * kSlab, &tmap_pair, leader_bar(kBarVFull + stage), 0,
+                                    tma_load_4d_pair(k0 + (4 * n + 2 * (1 - (int)rank)) * kSlab, &tmap_pair, leader_bar(L::kBarVFull + stage), 0,
                                                      tg.tok0, 4 * n + 2 * (int)rank, rank == 0 ? page_b : page_a);
                             }
                         }
@@ -248,7 +266,7 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
                     const int page = __shfl_sync(0xffffffffu, (rank == 0) != is_v ? page_a : page_b, 0);
                     const uint8_t *src = page >= 0 && page < p.num_pool_pages
                         ? static_cast<const uint8_t *>(p.kv_pool) + (size_t)page * (kPage * kDQK) : nullptr;
-                    uint8_t *slabs = smem + kOffK + stage * kPageBytes;
+                    uint8_t *slabs = smem + L::kOffK + stage * kPageBytes;
                     if (!is_v) {
                         fill_rows_by_hand<64>(slabs, kSlab, kPage, src, tg.tok0, tg.a, tg.b, 0, 0, 9, lane);
                     } else {
@@ -258,111 +276,115 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
                     }
                     fence_proxy_async();
                     __syncwarp();
-                    if (lane == 0) mbar_complete_tx_cluster(leader_bar(is_v ? kBarVFull + stage : kBarKFull + stage), is_v ? kPeerBytes : kPageBytes);
+                    if (lane == 0) mbar_complete_tx_cluster(leader_bar(is_v ? L::kBarVFull + stage : L::kBarKFull + stage), is_v ? kPeerBytes : kPageBytes);
                 }
             }
         }
-    } else if (warp >= kWarpQk && warp < kWarpQk + kQkWarps && rank == 0) {
-        // ===================================================== QK^T issuers (leader CTA)
-        if (lane == 0) {
-            const int a = warp - kWarpQk;                 // partial accumulator a
-            constexpr uint32_t kIdescQK = make_idesc_e4m3(128, 128, 0);
-            uint32_t st_it = 0, seg_it = 0;
-            bool ok = true;
-            while (ok && it.next(p, seg)) {
-                const int nsuper = (seg.tile_end - seg.tile_begin + 1) >> 1;
-                ok = mbar_wait_cluster(ctx, bar(kBarQFull), seg_it & 1, kBarQFull);
-                for (int s = 0; ok && s < nsuper; ++s, ++st_it) {
-                    const uint32_t stage = st_it % kStages, b = st_it & 1;
-                    ok = mbar_wait_cluster(ctx, bar(kBarKFull + stage), (st_it / kStages) & 1, kBarKFull + stage) &&
-                         mbar_wait_cluster(ctx, bar(kBarSEmpty + b), ((st_it >> 1) & 1) ^ 1, kBarSEmpty + b);
-                    if (!ok) break;
-                    tcgen05_fence_after();
-                    const uint32_t k0 = sbase + kOffK + stage * kPageBytes;
-                    const uint32_t d = tmem_base + kColS + (b * kQkWarps + a) * kN;
-                    // 18 K = 32 steps x (q hi, q lo) = 36 MMAs per supertile; this issuer takes every second
+    } else if (warp == kWarpQk && rank == 0) {
+        // ===================================================== QK^T issuer (leader CTA)
+        constexpr uint32_t kIdescQK = make_idesc_e4m3(128, 128, 0);
+        const uint32_t elected = elect_one(), tmem_u = uniform(tmem_base);
+        uint32_t st_it = 0, seg_it = 0;
+        bool ok = true;
+        while (ok && it.next(p, seg)) {
+            const int nsuper = (int)uniform((uint32_t)((seg.tile_end - seg.tile_begin + 1) >> 1));
+            ok = mbar_wait_cluster(ctx, bar(L::kBarQFull), seg_it & 1, L::kBarQFull);
+            for (int s = 0; ok && s < nsuper; ++s, ++st_it) {
+                const uint32_t stage = st_it % kStages, b = st_it & 1;
+                ok = mbar_wait_cluster(ctx, bar(L::kBarKFull + stage), (st_it / kStages) & 1, L::kBarKFull + stage) &&
+                     mbar_wait_cluster(ctx, bar(L::kBarSEmpty + b), ((st_it >> 1) & 1) ^ 1, L::kBarSEmpty + b);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                tcgen05_fence_after();
+                const uint32_t d = tmem_u + L::kColS + b * 64;
+                const uint64_t dq = make_desc_sw64(sbase + L::kOffQ, 16, 512);                            // A: 2 x 64 rows x 32
+                const uint64_t dk = make_desc_sw64(sbase + L::kOffK + stage * kPageBytes, 16, 512);       // B: 2 x 64 tokens x 32
+                // 18 K = 32 steps, for H = 64 with q hi and then with q lo
 #pragma unroll
-                    for (int t = 0; t < 36 / kQkWarps; ++t) {
-                        const int idx = t * kQkWarps + a, hl = idx / 18, ks = idx % 18, c = ks >> 1, k = ks & 1;
-                        const uint32_t q0 = sbase + (hl ? kOffQLo : kOffQHi);
-                        uint64_t dq = make_desc_sw64(q0 + c * kSlab + k * 32, 16, 512);     // A: 2 x 64 heads x 32
-                        uint64_t dk = make_desc_sw64(k0 + c * kSlab + k * 32, 16, 512);     // B: 2 x 64 tokens x 32
-                        umma_e4m3_pair(d, dq, dk, kIdescQK, t != 0);
-                    }
-                    umma_commit_pair(bar(kBarSFull + b));
-                    umma_commit_pair(bar(kBarQkDone + stage));
+                for (int t = 0; t < (H == 64 ? 36 : 18); ++t) {
+                    const uint32_t ks = t % 18, at = (ks >> 1) * kSlab + (ks & 1) * 32;
+                    umma_e4m3_pair(elected, d, dq + (((t / 18) * L::kQTerm + at) >> 4), dk + (at >> 4), kIdescQK, t != 0);
                 }
-                if (ok) umma_commit_pair(bar(kBarQEmpty));
-                ++seg_it;
+                if (elected) { umma_commit_pair(bar(L::kBarSFull + b)); umma_commit_pair(bar(L::kBarQkDone + stage)); }
+                __syncwarp();
             }
+            if (ok && elected) umma_commit_pair(bar(L::kBarQEmpty));
+            __syncwarp();
+            ++seg_it;
         }
-    } else if (warp >= kWarpPv && warp < kWarpPv + kPvWarps && rank == 0) {
-        // ===================================================== P.V issuers (leader CTA)
-        if (lane == 0) {
-            const int n = warp - kWarpPv;                 // dv half: columns [256 n, 256 n + 256)
-            constexpr uint32_t kIdescPV = make_idesc_e4m3(128, 256, 0, 0, 1, 0);
-            constexpr uint32_t kIdescPVLo = make_idesc_e4m3(128, 256, 0, 0, 1, 1);   // P lo is e5m2 (A operand)
-            uint32_t st_it = 0, seg_it = 0;
-            bool ok = true;
-            while (ok && it.next(p, seg)) {
-                const int ntiles = seg.tile_end - seg.tile_begin;
-                const int nsuper = (ntiles + 1) >> 1;
-                for (int s = 0; ok && s < nsuper; ++s, ++st_it) {
-                    const uint32_t stage = st_it % kStages, pb = st_it & 1;
-                    ok = mbar_wait_cluster(ctx, bar(kBarVFull + stage), (st_it / kStages) & 1, kBarVFull + stage) &&
-                         mbar_wait_cluster(ctx, bar(kBarPFull + pb), (st_it >> 1) & 1, kBarPFull + pb);
-                    if (ok && s == 0) ok = mbar_wait_cluster(ctx, bar(kBarOEmpty), (seg_it & 1) ^ 1, kBarOEmpty);
-                    if (!ok) break;
-                    tcgen05_fence_after();
-                    const uint32_t k0 = sbase + kOffK + stage * kPageBytes;
-                    const bool has_b = 2 * s + 1 < ntiles;
-                    const int ksteps = has_b ? 4 : 2;     // 32 tokens each; page B's are skipped when it does not exist
+    } else if (warp == kWarpPv && rank == 0) {
+        // ===================================================== P.V issuer (leader CTA)
+        constexpr uint32_t kIdescPV = make_idesc_e4m3(128, 256, 0, 0, 1, 0);
+        constexpr uint32_t kIdescPVLo = make_idesc_e4m3(128, 256, 0, 0, 1, 1);   // P lo is e5m2 (A operand; H = 64)
+        const uint32_t elected = elect_one(), tmem_u = uniform(tmem_base);
+        uint32_t st_it = 0, seg_it = 0;
+        bool ok = true;
+        while (ok && it.next(p, seg)) {
+            const int ntiles = (int)uniform((uint32_t)(seg.tile_end - seg.tile_begin));
+            const int nsuper = (ntiles + 1) >> 1;
+            for (int s = 0; ok && s < nsuper; ++s, ++st_it) {
+                const uint32_t stage = st_it % kStages, pb = st_it & 1;
+                ok = mbar_wait_cluster(ctx, bar(L::kBarVFull + stage), (st_it / kStages) & 1, L::kBarVFull + stage) &&
+                     mbar_wait_cluster(ctx, bar(L::kBarPFull + pb), (st_it >> 1) & 1, L::kBarPFull + pb);
+                if (ok && s == 0) ok = mbar_wait_cluster(ctx, bar(L::kBarOEmpty), (seg_it & 1) ^ 1, L::kBarOEmpty);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                tcgen05_fence_after();
+                const int pages = 2 * s + 1 < ntiles ? 2 : 1;     // page B's MMAs are skipped when it does not exist
+                // A: P rows, slab = page, 32 tokens; B: slots 4n + 2 page, + 1 (two 64-wide dv chunks, LBO), 32 tokens
+                const uint64_t da = make_desc_sw64(sbase + L::kOffP + pb * L::kPBuf, 16, 512);
+                const uint64_t db = make_desc_sw64(sbase + L::kOffK + stage * kPageBytes, kSlab, 512);
 #pragma unroll
-                    for (int hl = 0; hl < 2; ++hl) {
-                        const uint32_t p0 = sbase + kOffP + (pb * 2 + hl) * 2 * kSlab;
-                        for (int ks = 0; ks < ksteps; ++ks) {
-                            // A: P rows, slab = page, 32 tokens; B: slots 4n + 2 page, + 1 (two 64-wide dv chunks, LBO), 32 tokens
-                            const int pg = ks >> 1;
-                            uint64_t da = make_desc_sw64(p0 + pg * kSlab + (ks & 1) * 32, 16, 512);
-                            uint64_t db = make_desc_sw64(k0 + (4 * n + 2 * pg) * kSlab + (ks & 1) * 2048, kSlab, 512);
-                            umma_e4m3_pair(tmem_base + kColO + n * 128, da, db, hl ? kIdescPVLo : kIdescPV, (s != 0) || (hl | ks) != 0);
+                for (int hl = 0; hl < (H == 64 ? 2 : 1); ++hl) {
+                    for (int pg = 0; pg < pages; ++pg) {
+#pragma unroll
+                        for (int k = 0; k < 2; ++k) {
+#pragma unroll
+                            for (int n = 0; n < 2; ++n)           // dv half: columns [256 n, 256 n + 256)
+                                umma_e4m3_pair(elected, tmem_u + L::kColO + n * 128, da + ((hl * L::kPTerm + pg * kSlab + k * 32) >> 4),
+                                               db + (((4 * n + 2 * pg) * kSlab + k * 2048) >> 4), hl ? kIdescPVLo : kIdescPV,
+                                               (uint32_t)s | (uint32_t)(hl | pg | k));
                         }
                     }
-                    umma_commit_pair(bar(kBarStageEmpty + stage));
-                    if (s + 1 == nsuper) umma_commit_pair(bar(kBarOFull));
                 }
-                ++seg_it;
+                if (elected) {
+                    umma_commit_pair(bar(L::kBarStageEmpty + stage));
+                    if (s + 1 == nsuper) umma_commit_pair(bar(L::kBarOFull));
+                }
+                __syncwarp();
             }
+            ++seg_it;
         }
     } else if (warp >= kWarpQk && warp < kWarpSoftmax) {
         // the issuer warps of the peer CTA have nothing to do for the attention itself: they carry the call's page-copy
         // job, if it has one (a layer's pages on the move while this layer decodes)
         if (p.mig_n > 0)
-            copy_pages_in_idle_warp(p, pair_id * (kQkWarps + kPvWarps) + (warp - kWarpQk), p.num_workers * p.pair_groups * (kQkWarps + kPvWarps), lane);
+            copy_pages_in_idle_warp(p, pair_id * kIssuerWarps + (warp - kWarpQk), p.num_workers * p.pair_groups * kIssuerWarps, lane);
     } else if (warp >= kWarpConvert && warp < kWarpConvert + kConvertWarps) {
-        // ===================================================== query converters (this CTA's 64 heads)
+        // ===================================================== query converters (this CTA's heads)
         const int ct = (warp - kWarpConvert) * 32 + lane;   // 0..127
-        float *qs_s = reinterpret_cast<float *>(smem + kOffQs);
+        float *qs_s = reinterpret_cast<float *>(smem + L::kOffQs);
         uint32_t seg_it = 0;
         bool ok = true;
         while (ok && it.next(p, seg)) {
             {
-                const int hd = ct >> 1, part = ct & 1;
+                constexpr int kParts = 128 / H, kVecs = 72 / kParts;      // threads per head, 16-byte loads per thread
+                const int hd = ct / kParts, part = ct % kParts;
                 const int gh = head0 + hd;
                 const bool live = gh < p.head_end;
                 const uint4 *src = reinterpret_cast<const uint4 *>(
                     static_cast<const __nv_bfloat16 *>(p.q) + (int64_t)seg.request * p.q_stride_request +
-                    (int64_t)(live ? gh : p.head_begin) * p.q_stride_head + part * 288);
+                    (int64_t)(live ? gh : p.head_begin) * p.q_stride_head + part * (kVecs * 8));
                 // first pass (row maximum) while the previous request is still being multiplied
                 float amax = 0.f;
                 if (live) {
 #pragma unroll 1
-                    for (int v0 = 0; v0 < 36; v0 += 12) {
-                        uint4 x[12];
+                    for (int v0 = 0; v0 < kVecs; v0 += kVecs / 3) {
+                        uint4 x[kVecs / 3];
 #pragma unroll
-                        for (int i = 0; i < 12; ++i) x[i] = __ldg(src + v0 + i);
+                        for (int i = 0; i < kVecs / 3; ++i) x[i] = __ldg(src + v0 + i);
 #pragma unroll
-                        for (int i = 0; i < 12; ++i) {
+                        for (int i = 0; i < kVecs / 3; ++i) {
                             const uint32_t w[4] = {x[i].x, x[i].y, x[i].z, x[i].w};
 #pragma unroll
                             for (int k = 0; k < 4; ++k) {
@@ -372,11 +394,12 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
                         }
                     }
                 }
-                amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 1));
+#pragma unroll
+                for (int o = 1; o < kParts; o <<= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
                 const float qs = amax > 0.f ? amax * (1.0f / 448.0f) : 1.0f;
                 const float inv = amax > 0.f ? 448.0f / amax : 1.0f;
-                if (part == 0) qs_s[(seg_it & 3) * kN + hd] = qs;
-                // second pass in four batches of nine 16-byte loads, a batch ahead: the first batch is in
+                if (part == 0) qs_s[(seg_it & 3) * H + hd] = qs;
+                // second pass in batches of nine 16-byte loads, a batch ahead: the first batch is in
                 // flight while this warp waits for the operand buffers, which are free once the last
                 // QK^T of the previous request has retired
                 uint4 xa[9], xb[9];
@@ -394,36 +417,41 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
                             const float e0 = __uint_as_float(w[k] << 16) * inv, e1 = __uint_as_float(w[k] & 0xffff0000u) * inv;
                             split_e4m3_e4m3_x2(e0, e1, hi[k], lo[k]);      // packed f16 arithmetic: half the instructions
                         }
-                        const uint32_t d = (uint32_t)(part * 288 + (v0 + i) * 8);
-                        const uint32_t off = (d >> 6) * kSlab + sw64((uint32_t)hd, d & 63);
-                        *reinterpret_cast<uint2 *>(smem + kOffQHi + off) =
+                        const uint32_t d = (uint32_t)(part * (kVecs * 8) + (v0 + i) * 8);
+                        const uint32_t row = H == 64 ? hd : 2 * hd - (hd & 15);      // H = 32: 32 (hd / 16) + hd mod 16
+                        const uint32_t off = (d >> 6) * kSlab + sw64(row, d & 63);
+                        *reinterpret_cast<uint2 *>(smem + L::kOffQ + off) =
                             make_uint2((uint32_t)hi[0] | ((uint32_t)hi[1] << 16), (uint32_t)hi[2] | ((uint32_t)hi[3] << 16));
-                        *reinterpret_cast<uint2 *>(smem + kOffQLo + off) =
+                        *reinterpret_cast<uint2 *>(smem + L::kOffQ + L::kQTerm + off) =
                             make_uint2((uint32_t)lo[0] | ((uint32_t)lo[1] << 16), (uint32_t)lo[2] | ((uint32_t)lo[3] << 16));
                     }
                 };
                 load_batch(xa, 0);
-                ok = mbar_wait(ctx, bar(kBarQEmpty), (seg_it & 1) ^ 1, kBarQEmpty);
+                ok = mbar_wait(ctx, bar(L::kBarQEmpty), (seg_it & 1) ^ 1, L::kBarQEmpty);
                 if (!ok) break;
                 load_batch(xb, 9);  convert_batch(xa, 0);
-                load_batch(xa, 18); convert_batch(xb, 9);
-                load_batch(xb, 27); convert_batch(xa, 18);
-                convert_batch(xb, 27);
+                if constexpr (H == 64) {
+                    load_batch(xa, 18); convert_batch(xb, 9);
+                    load_batch(xb, 27); convert_batch(xa, 18);
+                    convert_batch(xb, 27);
+                } else {
+                    convert_batch(xb, 9);
+                }
                 fence_proxy_async();
                 __syncwarp();
                 // The softmax warps wait on QLocal by phase parity, so it must never complete two phases
                 // ahead of them: hold this request's arrival until they have entered the previous one.
                 if (lane == 0) {
-                    if (seg_it > 0) ok = mbar_wait(ctx, bar(kBarQsRead), (seg_it - 1) & 1, kBarQsRead);
-                    mbar_arrive(bar(kBarQLocal)); arrive_on_leader(kBarQFull);
+                    if (seg_it > 0) ok = mbar_wait(ctx, bar(L::kBarQsRead), (seg_it - 1) & 1, L::kBarQsRead);
+                    mbar_arrive(bar(L::kBarQLocal)); arrive_on_leader(L::kBarQFull);
                 }
                 ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
             }
             ++seg_it;
         }
-    } else {
+    } else if constexpr (H == 64) {
         // ===================================================== softmax + epilogue warps
-        // S partial layout per CTA: TMEM lane L < 64 = head L, tokens of page A in 64 columns;
+        // S layout per CTA: TMEM lane L < 64 = head L, tokens of page A in 64 columns;
         // lane 64 + L = head L, tokens of page B.  Two warps per quadrant take 32 columns each,
         // so a thread owns ONE head and 32 tokens of one page.
         const int sw = warp - kWarpSoftmax;             // 0..7
@@ -433,15 +461,15 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
         const int hd = 32 * (q4 & 1) + lane;            // this thread's head (0..63 within the CTA)
         const int half_id = q4 & 1;                     // heads 0-31 or 32-63: the four warps that share them sync on bar 2 + half_id
         const uint32_t lane_addr = (uint32_t)(32 * q4) << 16;
-        float *qs_s = reinterpret_cast<float *>(smem + kOffQs);
-        float *alpha_s = reinterpret_cast<float *>(smem + kOffAlpha);
-        float *l_s = reinterpret_cast<float *>(smem + kOffL);
-        float *xch = reinterpret_cast<float *>(smem + kOffXch);
+        float *qs_s = reinterpret_cast<float *>(smem + L::kOffQs);
+        float *alpha_s = reinterpret_cast<float *>(smem + L::kOffAlpha);
+        float *l_s = reinterpret_cast<float *>(smem + L::kOffL);
+        float *xch = reinterpret_cast<float *>(smem + L::kOffXch);
         // per-warp table of its 32 tokens, read back as 16-byte broadcasts:
         // tok_a[j / 2] = (scale_j, log2 scale_j, scale_j+1, log2 scale_j+1), tok_r[j / 4] = 1 / scale of four tokens
-        float4 *tok_a = reinterpret_cast<float4 *>(smem + kOffTok + sw * kTokBytes);
+        float4 *tok_a = reinterpret_cast<float4 *>(smem + L::kOffTok + sw * L::kTokBytes);
         float4 *tok_r = tok_a + 16;
-        const float *scale_s = reinterpret_cast<const float *>(smem + kOffScale);
+        const float *scale_s = reinterpret_cast<const float *>(smem + L::kOffScale);
         const float scale_log2 = p.softmax_scale * kLog2e;
         const int slot4 = pg * 2 + cf;                  // this thread's slot among the 4 threads of its head
         uint32_t st_it = 0, seg_it = 0;
@@ -449,10 +477,10 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
         // thread still meets the named barriers -- once the CTA aborts, waits return at once.
         bool ok = true;
         while (it.next(p, seg)) {
-            ok &= mbar_wait(ctx, bar(kBarQLocal), seg_it & 1, kBarQLocal);
-            const float cq = scale_log2 * qs_s[(seg_it & 3) * kN + hd];
+            ok &= mbar_wait(ctx, bar(L::kBarQLocal), seg_it & 1, L::kBarQLocal);
+            const float cq = scale_log2 * qs_s[(seg_it & 3) * H + hd];
             __syncwarp();
-            if (lane == 0) mbar_arrive(bar(kBarQsRead));
+            if (lane == 0) mbar_arrive(bar(L::kBarQsRead));
             float m = -INFINITY, l = 0.f;
             const int nsuper = (seg.tile_end - seg.tile_begin + 1) >> 1;
             // several query rows per request: this thread's (virtual) head is row (head mod R) and sees the
@@ -462,15 +490,12 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
                 const PairGeom g = pair_geom(s);
                 const TileGeom geo = pg ? g.b : g.a;
                 const uint32_t stage = st_it % kStages, b = st_it & 1;
-                ok &= mbar_wait(ctx, bar(kBarSFull + b), (st_it >> 1) & 1, kBarSFull + b);
-                ok &= mbar_wait(ctx, bar(kBarScFull + stage), (st_it / kStages) & 1, kBarScFull + stage);
+                ok &= mbar_wait(ctx, bar(L::kBarSFull + b), (st_it >> 1) & 1, L::kBarSFull + b);
+                ok &= mbar_wait(ctx, bar(L::kBarScFull + stage), (st_it / kStages) & 1, L::kBarScFull + stage);
                 tcgen05_fence_after();
                 float sv[32];
                 {
-                    float part[32];
-                    const uint32_t sb = tmem_base + lane_addr + kColS + (b * kQkWarps) * kN + 32 * cf;
-                    tmem_ld32(sb, sv);
-                    tmem_ld32(sb + kN, part);
+                    tmem_ld32(tmem_base + lane_addr + L::kColS + b * 64 + 32 * cf, sv);
                     // meanwhile: lane j prepares token 32 cf + j.  A token outside the range gets scale 0 and
                     // log2 scale -inf; its row of K may hold anything, so its logit is also forced below.
                     const int r = 32 * cf + lane;
@@ -479,12 +504,10 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
                     reinterpret_cast<float2 *>(tok_a)[lane] = make_float2(ts, v ? fast_log2(ts) : -INFINITY);
                     reinterpret_cast<float *>(tok_r)[lane] = v ? fast_rcp(ts) : 0.f;
                     tmem_wait_ld();
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) sv[j] += part[j];
                 }
                 tcgen05_fence_before();
                 __syncwarp();
-                if (lane == 0) arrive_on_leader(kBarSEmpty + b);
+                if (lane == 0) arrive_on_leader(L::kBarSEmpty + b);
                 uint32_t valid = __ballot_sync(0xffffffffu, 32 * cf + lane >= geo.r_lo && 32 * cf + lane < geo.r_hi);
                 {
                     // how many of this thread's 32 tokens lie below its head's causal end: token j of the thread is
@@ -542,16 +565,16 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
                 const bool rescale = named_bar_or<1, kSoftmaxWarps * 32>(grew);
                 // P.V of the supertile that last used this P buffer (two back) must be done; a rescale
                 // of O also needs the previous supertile's P.V
-                if (st_it > 1) ok &= mbar_wait(ctx, bar(kBarStageEmpty + (st_it - 2) % kStages), ((st_it - 2) / kStages) & 1, kBarStageEmpty);
+                if (st_it > 1) ok &= mbar_wait(ctx, bar(L::kBarStageEmpty + (st_it - 2) % kStages), ((st_it - 2) / kStages) & 1, L::kBarStageEmpty);
                 if (rescale && s > 0) {
-                    ok &= mbar_wait(ctx, bar(kBarStageEmpty + (st_it - 1) % kStages), ((st_it - 1) / kStages) & 1, kBarStageEmpty);
+                    ok &= mbar_wait(ctx, bar(L::kBarStageEmpty + (st_it - 1) % kStages), ((st_it - 1) / kStages) & 1, L::kBarStageEmpty);
                     tcgen05_fence_after();
                     // O rows are TMEM lanes: this thread scales its lane's columns [128 cf, 128 cf + 128)
                     const float a_row = alpha_s[hd];
 #pragma unroll 1
                     for (int c = 0; c < 4; ++c) {
                         float o[32];
-                        const uint32_t addr = tmem_base + lane_addr + kColO + 128 * cf + c * 32;
+                        const uint32_t addr = tmem_base + lane_addr + L::kColO + 128 * cf + c * 32;
                         tmem_ld32(addr, o);
                         tmem_wait_ld();
 #pragma unroll
@@ -563,8 +586,8 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
                 }
                 {
                     // P hi / lo: K-major, 64-byte swizzle; slab = page, row = head, bytes [32 cf, 32 cf + 32)
-                    uint8_t *ph = smem + kOffP + ((b * 2 + 0) * 2 + pg) * kSlab;
-                    uint8_t *pl = smem + kOffP + ((b * 2 + 1) * 2 + pg) * kSlab;
+                    uint8_t *ph = smem + L::kOffP + ((b * 2 + 0) * 2 + pg) * kSlab;
+                    uint8_t *pl = smem + L::kOffP + ((b * 2 + 1) * 2 + pg) * kSlab;
 #pragma unroll
                     for (int u16 = 0; u16 < 2; ++u16) {
                         const uint32_t o = sw64((uint32_t)hd, (uint32_t)(32 * cf + 16 * u16));
@@ -575,7 +598,7 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
                 fence_proxy_async();
                 tcgen05_fence_before();
                 __syncwarp();
-                if (lane == 0) arrive_on_leader(kBarPFull + b);
+                if (lane == 0) arrive_on_leader(L::kBarPFull + b);
             }
             // ---- row sums of the 4 threads of a head
             xch[hd * 4 + slot4] = l;
@@ -595,7 +618,7 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
             // ---- epilogue: lane L < 64 holds head L, dv [256 n, 256 n + 128) in columns n * 128 + j;
             // lane 64 + L holds head L, dv [256 n + 128, 256 n + 256).  The two warps of a quadrant
             // take one n each.
-            ok &= mbar_wait(ctx, bar(kBarOFull), seg_it & 1, kBarOFull);
+            ok &= mbar_wait(ctx, bar(L::kBarOFull), seg_it & 1, L::kBarOFull);
             tcgen05_fence_after();
             // Every warp drains its [32 heads x 128 dv] block in four rounds of 32 columns through a
             // 4 KB tile of the P buffers (idle now: the last P.V has retired): a thread writes its row
@@ -605,7 +628,7 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
                 const int n = cf;
                 const int dv0 = 256 * n + 128 * pg;
                 const int row0 = 32 * (q4 & 1);
-                uint8_t *stg = smem + kOffP + sw * 4096;
+                uint8_t *stg = smem + L::kOffP + sw * 4096;
                 const float inv_l = l_s[hd];
                 const bool final_out = seg.slot < 0;
                 const CUtensorMap *omap = final_out ? &tmap_out : &tmap_part;
@@ -614,7 +637,7 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
 #pragma unroll 1
                 for (int c = 0; c < 4; ++c) {
                     float o[32];
-                    tmem_ld32(tmem_base + lane_addr + kColO + n * 128 + c * 32, o);
+                    tmem_ld32(tmem_base + lane_addr + L::kColO + n * 128 + c * 32, o);
                     tmem_wait_ld();
                     if (c > 0) {                          // the previous round's store has read the tile
                         if (lane == 0) bulk_wait_group_read();
@@ -633,12 +656,261 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
             }
             tcgen05_fence_before();
             __syncwarp();
-            if (lane == 0) arrive_on_leader(kBarOEmpty);
+            if (lane == 0) arrive_on_leader(L::kBarOEmpty);
+            ++seg_it;
+        }
+    } else {
+        // ===================================================== softmax + epilogue warps, 32 heads
+        // Two heads per thread, in the accumulator fragment layout: hA and hA + 8 of a quadrant's sixteen, hi terms in
+        // lanes 0..15 of the quadrant and lo terms in lanes 16..31, so both terms of a logit arrive in the same register of two
+        // loads.  Quadrants 0, 1 hold page A and 2, 3 page B of 16 heads each; the two warps of a quadrant take 32 tokens
+        // each, a thread tokens 8 k + 2 tq + {0, 1} of them.
+        const int sw = warp - kWarpSoftmax;             // 0..7
+        const int q4 = warp & 3;                        // TMEM lane quadrant
+        const int cf = sw >> 2;                         // tokens [32 cf, 32 cf + 32) of the page
+        const int pg = q4 >> 1;                         // 0: page A, 1: page B
+        const int head16 = q4 & 1;                      // heads 0-15 or 16-31: the four warps that share them sync on bar 2 + head16
+        const int hA = 16 * head16 + (lane >> 2), tq = lane & 3;
+        const int slot4 = pg * 2 + cf;                  // this warp's slot among the four
+        const uint32_t lane_addr = (uint32_t)(32 * q4) << 16;
+        float *qs_s = reinterpret_cast<float *>(smem + L::kOffQs);
+        float *alpha_s = reinterpret_cast<float *>(smem + L::kOffAlpha);
+        float *l_s = reinterpret_cast<float *>(smem + L::kOffL);
+        float *xch = reinterpret_cast<float *>(smem + L::kOffXch);
+        // what the four warps that share a head have found
+        auto exchange = [&](float (&v)[2], auto op) {
+            if (tq == 0) { xch[hA * 4 + slot4] = v[0]; xch[(hA + 8) * 4 + slot4] = v[1]; }
+            named_bar_sync_dyn<128>(2 + head16);
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const float4 x = *reinterpret_cast<const float4 *>(&xch[(hA + 8 * e) * 4]);
+                v[e] = op(op(x.x, x.y), op(x.z, x.w));
+            }
+        };
+        // per-warp table of its 32 tokens: tok_a[j / 2] = (scale_j, log2 scale_j, scale_j+1, log2 scale_j+1), tok_r[j] = 1 / scale_j
+        float4 *tok_a = reinterpret_cast<float4 *>(smem + L::kOffTok + sw * L::kTokBytes);
+        float *tok_r = reinterpret_cast<float *>(tok_a + 16);
+        const float *scale_s = reinterpret_cast<const float *>(smem + L::kOffScale);
+        const float scale_log2 = p.softmax_scale * kLog2e;
+        uint32_t st_it = 0, seg_it = 0;
+        bool ok = true;                                 // (a failed wait only clears it, as above)
+        while (it.next(p, seg)) {
+            ok &= mbar_wait(ctx, bar(L::kBarQLocal), seg_it & 1, L::kBarQLocal);
+            const float cqA = scale_log2 * qs_s[(seg_it & 3) * H + hA], cqB = scale_log2 * qs_s[(seg_it & 3) * H + hA + 8];
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(L::kBarQsRead));
+            float mA = -INFINITY, mB = -INFINITY, lA = 0.f, lB = 0.f;
+            const int nsuper = (seg.tile_end - seg.tile_begin + 1) >> 1;
+            // causal ends of the two (virtual) heads' rows
+            int endA = 0x3fffffff, endB = 0x3fffffff;
+            if (p.q_rows > 1) {
+                const int len = p.seq_lens[seg.request] - (p.q_rows - 1);
+                endA = len + (head0 + hA) % p.q_rows; endB = len + (head0 + hA + 8) % p.q_rows;
+            }
+            for (int s = 0; s < nsuper; ++s, ++st_it) {
+                const PairGeom g = pair_geom(s);
+                const TileGeom geo = pg ? g.b : g.a;
+                const uint32_t stage = st_it % kStages, b = st_it & 1;
+                ok &= mbar_wait(ctx, bar(L::kBarSFull + b), (st_it >> 1) & 1, L::kBarSFull + b);
+                ok &= mbar_wait(ctx, bar(L::kBarScFull + stage), (st_it / kStages) & 1, L::kBarScFull + stage);
+                tcgen05_fence_after();
+                float sv[16];                     // [4 k + e]: head hA, token 8 k + 2 tq + e; [4 k + 2 + e]: head hA + 8
+                {
+                    float part[16];
+                    const uint32_t sb = tmem_base + lane_addr + L::kColS + b * 64 + 32 * cf;
+                    tmem_ld_frag<32>(sb, sv);
+                    tmem_ld_frag<32>(sb + (16u << 16), part);
+                    // meanwhile: lane j prepares token 32 cf + j.  A token outside the range gets scale 0 and
+                    // log2 scale -inf; its row of K may hold anything, so its logit is also forced below.
+                    const int r = 32 * cf + lane;
+                    const bool v = r >= geo.r_lo && r < geo.r_hi;
+                    const float ts = v ? scale_s[(stage * 2 + pg) * 64 + geo.tok0 + r] : 0.f;
+                    reinterpret_cast<float2 *>(tok_a)[lane] = make_float2(ts, v ? fast_log2(ts) : -INFINITY);
+                    tok_r[lane] = v ? fast_rcp(ts) : 0.f;
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) sv[j] += part[j];
+                }
+                tcgen05_fence_before();
+                __syncwarp();
+                if (lane == 0) arrive_on_leader(L::kBarSEmpty + b);
+                // the warp's tokens [first, limA) / [first, limB) count for its two heads
+                float mt[2] = {-INFINITY, -INFINITY};
+                const int t_first = (seg.lo / kPage + seg.tile_begin + 2 * s + pg) * kPage + geo.tok0;    // token of row 0
+                const int limA = min(geo.r_hi, endA - t_first) - 32 * cf, limB = min(geo.r_hi, endB - t_first) - 32 * cf;
+                const int first = geo.r_lo - 32 * cf;
+                if (__all_sync(0xffffffffu, first <= 0 && limA >= 32 && limB >= 32)) {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const float4 t = tok_a[4 * k + tq];
+                        sv[4 * k] = fmaf(sv[4 * k], cqA * t.x, t.y);
+                        sv[4 * k + 1] = fmaf(sv[4 * k + 1], cqA * t.z, t.w);
+                        sv[4 * k + 2] = fmaf(sv[4 * k + 2], cqB * t.x, t.y);
+                        sv[4 * k + 3] = fmaf(sv[4 * k + 3], cqB * t.z, t.w);
+                    }
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const float4 t = tok_a[4 * k + tq];
+                        const int j0 = 8 * k + 2 * tq, j1 = j0 + 1;
+                        sv[4 * k] = j0 >= first && j0 < limA ? fmaf(sv[4 * k], cqA * t.x, t.y) : -INFINITY;
+                        sv[4 * k + 1] = j1 >= first && j1 < limA ? fmaf(sv[4 * k + 1], cqA * t.z, t.w) : -INFINITY;
+                        sv[4 * k + 2] = j0 >= first && j0 < limB ? fmaf(sv[4 * k + 2], cqB * t.x, t.y) : -INFINITY;
+                        sv[4 * k + 3] = j1 >= first && j1 < limB ? fmaf(sv[4 * k + 3], cqB * t.z, t.w) : -INFINITY;
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    mt[0] = fmaxf(mt[0], fmaxf(sv[4 * k], sv[4 * k + 1]));
+                    mt[1] = fmaxf(mt[1], fmaxf(sv[4 * k + 2], sv[4 * k + 3]));
+                }
+                // row maximum: the four threads of a head in this warp, then the four warps
+#pragma unroll
+                for (int o = 1; o < 4; o <<= 1) {
+                    mt[0] = fmaxf(mt[0], __shfl_xor_sync(0xffffffffu, mt[0], o));
+                    mt[1] = fmaxf(mt[1], __shfl_xor_sync(0xffffffffu, mt[1], o));
+                }
+                exchange(mt, [](float x, float y) { return fmaxf(x, y); });
+                bool grew = false;
+                float alA = 1.f, alB = 1.f;
+                if (mt[0] > mA + kTau) { alA = (mA == -INFINITY) ? 0.f : fast_exp2(mA - mt[0]); mA = mt[0]; lA *= alA; grew = true; }
+                if (mt[1] > mB + kTau) { alB = (mB == -INFINITY) ? 0.f : fast_exp2(mB - mt[1]); mB = mt[1]; lB *= alB; grew = true; }
+                if (tq == 0 && slot4 == 0) { alpha_s[hA] = alA; alpha_s[hA + 8] = alB; }
+                // a head that has seen no token yet: all weights 0, not NaN
+                const float offA = kLift - (mA == -INFINITY ? 0.f : mA), offB = kLift - (mB == -INFINITY ? 0.f : mB);
+                uint32_t wA[4], wB[4];            // two tokens each: hi bytes below, lo bytes above
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const float2 rt = *reinterpret_cast<const float2 *>(&tok_r[8 * k + 2 * tq]);
+                    const float a0 = fast_exp2(sv[4 * k] + offA), a1 = fast_exp2(sv[4 * k + 1] + offA);
+                    const float b0 = fast_exp2(sv[4 * k + 2] + offB), b1 = fast_exp2(sv[4 * k + 3] + offB);
+                    lA = fmaf(a1, rt.y, fmaf(a0, rt.x, lA));
+                    lB = fmaf(b1, rt.y, fmaf(b0, rt.x, lB));
+                    uint16_t main, rest;
+                    split_e4m3_e4m3x16_x2(a0, a1, main, rest);
+                    wA[k] = (uint32_t)main | ((uint32_t)rest << 16);
+                    split_e4m3_e4m3x16_x2(b0, b1, main, rest);
+                    wB[k] = (uint32_t)main | ((uint32_t)rest << 16);
+                }
+                const bool rescale = named_bar_or<1, kSoftmaxWarps * 32>(grew);
+                // P.V of the supertile that last used this P buffer (two back) must be done; a rescale
+                // of O also needs the previous supertile's P.V
+                if (st_it > 1) ok &= mbar_wait(ctx, bar(L::kBarStageEmpty + (st_it - 2) % kStages), ((st_it - 2) / kStages) & 1, L::kBarStageEmpty);
+                if (rescale && s > 0) {
+                    ok &= mbar_wait(ctx, bar(L::kBarStageEmpty + (st_it - 1) % kStages), ((st_it - 1) / kStages) & 1, L::kBarStageEmpty);
+                    tcgen05_fence_after();
+                    // O rows are TMEM lanes (hi and lo rows of the same sixteen heads): this thread scales its lane's columns
+                    // [128 cf, 128 cf + 128)
+                    const float a_row = alpha_s[16 * head16 + (lane & 15)];
+#pragma unroll 1
+                    for (int c = 0; c < 4; ++c) {
+                        float o[32];
+                        const uint32_t addr = tmem_base + lane_addr + L::kColO + 128 * cf + c * 32;
+                        tmem_ld32(addr, o);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int k = 0; k < 32; ++k) o[k] *= a_row;
+                        tmem_st16(addr, *reinterpret_cast<float(*)[16]>(&o[0]));
+                        tmem_st16(addr + 16, *reinterpret_cast<float(*)[16]>(&o[16]));
+                    }
+                    tmem_wait_st();
+                }
+                {
+                    // P: K-major, 64-byte swizzle; slab = page, byte = token, rows like the query operand's.  Neighbouring lanes swap
+                    // so that a thread holds four consecutive tokens, of group k (even lanes) or k + 1 (odd lanes): 4-byte
+                    // stores without conflicts.
+                    const bool odd = tq & 1;
+                    uint8_t *const ph = smem + L::kOffP + b * L::kPBuf + pg * kSlab + (odd ? 8 : 0) + 4 * (tq >> 1);
+#pragma unroll
+                    for (int k = 0; k < 4; k += 2) {
+                        const uint32_t o = sw64((uint32_t)(2 * hA - (hA & 15)), (uint32_t)(32 * cf + 8 * k));
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) {
+                            const uint32_t w0 = e ? wB[k] : wA[k], w1 = e ? wB[k + 1] : wA[k + 1];
+                            const uint32_t got = __shfl_xor_sync(0xffffffffu, odd ? w0 : w1, 1);
+                            const uint32_t lower = odd ? got : w0, upper = odd ? w1 : got;
+                            uint8_t *const dst = ph + o + e * (8 * 64);          // head hA + 8: same swizzle phase
+                            *reinterpret_cast<uint32_t *>(dst) = __byte_perm(lower, upper, 0x5410);
+                            *reinterpret_cast<uint32_t *>(dst + L::kPTerm) = __byte_perm(lower, upper, 0x7632);
+                        }
+                    }
+                }
+                fence_proxy_async();
+                tcgen05_fence_before();
+                __syncwarp();
+                if (lane == 0) arrive_on_leader(L::kBarPFull + b);
+            }
+            // ---- row sums of a head: its four threads here, then the four warps
+            float lt[2] = {lA, lB};
+#pragma unroll
+            for (int o = 1; o < 4; o <<= 1) {
+                lt[0] += __shfl_xor_sync(0xffffffffu, lt[0], o);
+                lt[1] += __shfl_xor_sync(0xffffffffu, lt[1], o);
+            }
+            exchange(lt, [](float x, float y) { return x + y; });
+            if (tq == 0 && slot4 == 0) {
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const int hh = hA + 8 * e, gh = head0 + hh;
+                    l_s[hh] = lt[e] > 0.f ? 1.f / lt[e] : 0.f;       // no token at all (an empty causal range): O = 0, LSE = -inf
+                    if (gh < p.head_end) {
+                        const float lse = lt[e] > 0.f ? ((e ? mB : mA) - kLift + log2f(lt[e])) * kLn2 : -INFINITY;
+                        if (seg.slot < 0) p.lse[(int64_t)seg.request * p.lse_stride_request + gh] = lse;
+                        else p.partial_lse[(int64_t)seg.slot * h + (gh - p.head_begin)] = lse;
+                    }
+                }
+            }
+            named_bar_sync<1, kSoftmaxWarps * 32>();
+            // ---- epilogue: quadrants 0, 1 hold dv [256 n, 256 n + 128) in columns n * 128 + j, quadrants 2, 3
+            // dv [256 n + 128, 256 n + 256).  The two warps of a quadrant take one n each: [16 heads x 128 dv] as hi and lo
+            // rows, in four rounds of 32 columns through a 2 KB tile of the P buffers (idle now) and a TMA store per round.
+            ok &= mbar_wait(ctx, bar(L::kBarOFull), seg_it & 1, L::kBarOFull);
+            tcgen05_fence_after();
+            {
+                const int n = cf;
+                const int dv0 = 256 * n + 128 * pg;
+                const int row0 = 16 * head16;
+                uint8_t *stg = smem + L::kOffP + sw * 2048;
+                const bool final_out = seg.slot < 0;
+                const CUtensorMap *omap = final_out ? &tmap_out : &tmap_part;
+                const int rowc = final_out ? head0 + row0 : head0 - p.head_begin + row0;
+                const int outer = final_out ? seg.request : seg.slot;
+                const int r = lane >> 2;                      // rows r and r + 8: same swizzle phase
+                const float inv_a = l_s[row0 + r], inv_b = l_s[row0 + r + 8];
+#pragma unroll 1
+                for (int c = 0; c < 4; ++c) {
+                    const uint32_t addr = tmem_base + lane_addr + L::kColO + n * 128 + c * 32;
+                    float o[16], lo[16];
+                    tmem_ld_frag<32>(addr, o);
+                    tmem_ld_frag<32>(addr + (16u << 16), lo);
+                    tmem_wait_ld();
+                    if (c > 0) {                              // the previous round's store has read the tile
+                        if (lane == 0) bulk_wait_group_read();
+                        __syncwarp();
+                    }
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        uint8_t *const dst = stg + r * 128 + (((2 * k + (tq >> 1)) ^ r) << 4) + (tq & 1) * 8;
+                        *reinterpret_cast<float2 *>(dst) =
+                            make_float2(fmaf(lo[4 * k], 0.0625f, o[4 * k]) * inv_a, fmaf(lo[4 * k + 1], 0.0625f, o[4 * k + 1]) * inv_a);
+                        *reinterpret_cast<float2 *>(dst + 8 * 128) =
+                            make_float2(fmaf(lo[4 * k + 2], 0.0625f, o[4 * k + 2]) * inv_b, fmaf(lo[4 * k + 3], 0.0625f, o[4 * k + 3]) * inv_b);
+                    }
+                    fence_proxy_async();
+                    __syncwarp();
+                    if (lane == 0) { tma_store_3d(omap, smem_u32(stg), dv0 + 32 * c, rowc, outer); bulk_commit_group(); }
+                }
+                if (lane == 0) bulk_wait_group_read();        // the tile goes back to being a P buffer
+                __syncwarp();
+            }
+            tcgen05_fence_before();
+            __syncwarp();
+            if (lane == 0) arrive_on_leader(L::kBarOEmpty);
             ++seg_it;
         }
     }
 
-    fill_empty_requests(p, it.tile_start(p), worker, head0, kN, tid, kThreads);
+    fill_empty_requests(p, it.tile_start(p), worker, head0, H, tid, kThreads);
     if (p.trace != nullptr && tid == 0) {   // per-CTA cycles and nanoseconds
         p.trace[512 + blockIdx.x] = clock64() - t_start;
         if (blockIdx.x < 256) p.trace[768 + blockIdx.x] = (long long)(global_timer_ns() - ns_start);
@@ -658,9 +930,8 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
     }
 }
 
-}  // namespace
-
-cudaError_t launch_decode_umma_fp8_pair(const DecodeParams &p, cudaStream_t stream) {
+template <int H>
+cudaError_t launch_pair(const DecodeParams &p, cudaStream_t stream) {
     alignas(64) CUtensorMap mpage, mpair;
     const uint64_t pages = (uint64_t)(p.num_pool_pages > 0 ? p.num_pool_pages : 1);
     if (!make_map_4d(&mpage, CU_TENSOR_MAP_DATA_TYPE_UINT8, CU_TENSOR_MAP_SWIZZLE_64B, p.kv_pool, kPage, pages,
@@ -674,28 +945,30 @@ cudaError_t launch_decode_umma_fp8_pair(const DecodeParams &p, cudaStream_t stre
     if (p.out_stride_head % 4 || p.out_stride_request % 4) return cudaErrorNotSupported;   // rows must start on 16-byte boundaries
     const uint64_t hbytes = (uint64_t)p.out_stride_head * 4;
     if (!make_store_map_3d(&mout, p.out, kDV, (uint64_t)p.head_end, (uint64_t)p.B, hbytes,
-                           p.B > 1 ? (uint64_t)p.out_stride_request * 4 : hbytes * (uint64_t)p.head_end, 32))
+                           p.B > 1 ? (uint64_t)p.out_stride_request * 4 : hbytes * (uint64_t)p.head_end, H / 2))
         return cudaErrorNotSupported;
     const uint64_t h = (uint64_t)(p.head_end - p.head_begin);
-    if (!make_store_map_3d(&mpart, p.partial_out, kDV, h, (uint64_t)2 * p.num_workers, (uint64_t)kDV * 4, h * kDV * 4, 32))
+    if (!make_store_map_3d(&mpart, p.partial_out, kDV, h, (uint64_t)2 * p.num_workers, (uint64_t)kDV * 4, h * kDV * 4, H / 2))
         return cudaErrorInvalidValue;
+    const int smem = (int)Layout<H>::kSmemBytes;
     static DeviceOnce once;
     cudaError_t e = once.run([&] {
-        const cudaError_t e0 = cudaFuncSetAttribute(decode_umma_fp8_pair_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
+        const cudaError_t e0 = cudaFuncSetAttribute(decode_umma_fp8_pair_kernel<H, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e0 != cudaSuccess) return e0;
-        return cudaFuncSetAttribute(decode_umma_fp8_pair_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
+        return cudaFuncSetAttribute(decode_umma_fp8_pair_kernel<H, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     });
     if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(p.num_workers * p.pair_groups * 2)); cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = kSmemBytes; cfg.stream = stream;
-    cudaLaunchAttribute attr[1];      // (the cluster shape is part of the kernel's declaration)
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, p.plan_mode == kPlanWorkspace ? decode_umma_fp8_pair_kernel<false> : decode_umma_fp8_pair_kernel<true>, p, mpage, mpair, mout, mpart);
+    // (the cluster shape is part of the kernel's declaration)
+    e = launch_dependent(p.plan_mode == kPlanWorkspace ? decode_umma_fp8_pair_kernel<H, false> : decode_umma_fp8_pair_kernel<H, true>,
+                         dim3((unsigned)(p.num_workers * p.pair_groups * 2)), dim3(kThreads), (size_t)smem, stream, p, mpage, mpair, mout, mpart);
     count_launch();
     return e;
+}
+
+}  // namespace
+
+cudaError_t launch_decode_umma_fp8_pair(const DecodeParams &p, cudaStream_t stream) {
+    return p.heads_per_group == 32 ? launch_pair<32>(p, stream) : launch_pair<64>(p, stream);
 }
 
 }  // namespace splash
