@@ -23,8 +23,10 @@
 // Accumulators: CTA r holds its 64 heads; a head's row is TMEM lane h (first half of N) and
 // lane 64 + h (second half).
 //
-// Roles per CTA (512 threads): page + query producer, 4 QK^T issuers and 2 P.V issuers
-// (leader CTA only), 8 softmax warps, 1 producer of the peer chunks.  Barriers that the
+// Roles per CTA (384 threads): page + query producer, QK^T issuer and P.V issuer
+// (leader CTA only), 8 softmax warps, 1 producer of the peer chunks.  An issuer warp stays converged and an elected lane
+// issues, with all that the MMAs take in uniform registers (issued from a branch of lane 0 alone an MMA costs 65 to 90
+// cycles, and it took four QK^T issuers with a partial accumulator each, which the softmax had to add up).  Barriers that the
 // issuers wait on live in the leader; the peer's warps arrive on them across the cluster
 // (relaxed arrivals: what they announce is already in place on the peer's SM), and TMA loads
 // of the peer complete on them too.
@@ -38,13 +40,13 @@ namespace {
 
 using namespace umma;
 
-constexpr int kQkWarps = 4, kPvWarps = 2, kSoftmaxWarps = 8;
+constexpr int kIssuerWarps = 2, kSoftmaxWarps = 8;
 constexpr int kWarpProducer = 0;
 constexpr int kWarpQk = 1;
-constexpr int kWarpPv = kWarpQk + kQkWarps;
-constexpr int kWarpSoftmax = kWarpPv + kPvWarps;       // 7: TMEM quadrant = warp & 3
+constexpr int kWarpPv = 2;
+constexpr int kWarpSoftmax = kWarpQk + kIssuerWarps;   // TMEM quadrant = warp & 3
 constexpr int kWarpVProducer = kWarpSoftmax + kSoftmaxWarps;
-constexpr int kThreads = (kWarpVProducer + 1) * 32;    // 16 warps = 512 threads
+constexpr int kThreads = (kWarpVProducer + 1) * 32;    // 12 warps = 384 threads
 constexpr int kN = 64;                              // heads per CTA
 constexpr int kHalf = 32;                           // tokens per CTA and tile
 constexpr uint32_t kSlab = kHalf * 128;             // one chunk of a half-page: 32 tokens x 128 B
@@ -86,15 +88,17 @@ constexpr uint32_t kOffPlan = kOffMisc + 32;                    // inline plan
 constexpr uint32_t kSmemBytes = kOffPlan + kInlinePlanBytes;
 static_assert(kSmemBytes <= 232448, "shared memory overflow");
 static_assert(kOffQ % 1024 == 0 && kOffP1 % 1024 == 0 && kSlab % 1024 == 0, "swizzle atoms need 1024-byte alignment");
-// tensor memory: O two halves of dv x 128 columns, then 2 S buffers x 4 partials x 32 columns
+// tensor memory: O two halves of dv x 128 columns, then 2 S buffers x 32 columns
 constexpr uint32_t kColO = 0, kColS = 256;
 
-__device__ __forceinline__ void umma_bf16_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+// Issued by the elected lane of a converged warp; the operands are uniform.
+__device__ __forceinline__ void umma_bf16_pair(uint32_t elected, uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
+        "{\n\t.reg .pred p, q;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
+        "setp.ne.b32 q, %5, 0;\n\t"
+        "@q tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(elected) : "memory");
 }
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
@@ -122,15 +126,15 @@ decode_umma_pair_kernel(const __grid_constant__ DecodeParams p, const __grid_con
     if (tid == 0) {
         // barriers the leader's issuers wait on count the warps of both CTAs (the peer's copies are unused)
         for (int s = 0; s < kStages; ++s) {
-            mbar_init(bar(kBarKFull + s), 1); mbar_init(bar(kBarQkDone + s), kQkWarps);
-            mbar_init(bar(kBarVFull + s), 1); mbar_init(bar(kBarStageEmpty + s), kPvWarps);
+            mbar_init(bar(kBarKFull + s), 1); mbar_init(bar(kBarQkDone + s), 1);
+            mbar_init(bar(kBarVFull + s), 1); mbar_init(bar(kBarStageEmpty + s), 1);
         }
-        mbar_init(bar(kBarQFull), 1); mbar_init(bar(kBarQEmpty), kQkWarps);
+        mbar_init(bar(kBarQFull), 1); mbar_init(bar(kBarQEmpty), 1);
         for (int b = 0; b < 2; ++b) {
-            mbar_init(bar(kBarSFull + b), kQkWarps); mbar_init(bar(kBarSEmpty + b), 2 * kSoftmaxWarps);
+            mbar_init(bar(kBarSFull + b), 1); mbar_init(bar(kBarSEmpty + b), 2 * kSoftmaxWarps);
             mbar_init(bar(kBarPFull + b), 2 * kSoftmaxWarps);
         }
-        mbar_init(bar(kBarOFull), kPvWarps); mbar_init(bar(kBarOEmpty), 2 * kSoftmaxWarps);
+        mbar_init(bar(kBarOFull), 1); mbar_init(bar(kBarOEmpty), 2 * kSoftmaxWarps);
         misc[1] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -233,81 +237,80 @@ decode_umma_pair_kernel(const __grid_constant__ DecodeParams p, const __grid_con
             }
             ++seg_it;
         }
-    } else if (warp >= kWarpQk && warp < kWarpQk + kQkWarps && rank == 0) {
-        // ===================================================== QK^T issuers (leader CTA)
-        // One thread sustains one tcgen05.mma per ~65 cycles and a chain of MMAs into one accumulator
-        // runs at the MMA latency, so the 36 K = 16 steps of a tile go to four issuers with a partial
-        // accumulator each.
-        if (lane == 0) {
-            const int a = warp - kWarpQk;
-            constexpr uint32_t kIdescQK = make_idesc(128, 64, 0, 0);
-            uint32_t kv_it = 0, seg_it = 0;
-            bool ok = true;
-            while (ok && it.next(p, seg)) {
-                ok = mbar_wait_cluster(ctx, bar(kBarQFull), seg_it & 1, kBarQFull);
-                for (int tile = seg.tile_begin; ok && tile < seg.tile_end; ++tile, ++kv_it) {
-                    const uint32_t stage = kv_it % kStages, b = kv_it & 1;
-                    ok = mbar_wait_cluster(ctx, bar(kBarKFull + stage), (kv_it / kStages) & 1, kBarKFull + stage) &&
-                         mbar_wait_cluster(ctx, bar(kBarSEmpty + b), ((kv_it >> 1) & 1) ^ 1, kBarSEmpty + b);
-                    if (!ok) break;
-                    tcgen05_fence_after();
-                    const uint32_t k0 = sbase + kOffK + stage * kStageBytes;
-                    const uint32_t d = tmem_base + kColS + (b * kQkWarps + a) * kHalf;
+    } else if (warp == kWarpQk && rank == 0) {
+        // ===================================================== QK^T issuer (leader CTA)
+        constexpr uint32_t kIdescQK = make_idesc(128, 64, 0, 0);
+        const uint32_t elected = elect_one(), tmem_u = uniform(tmem_base);
+        uint32_t kv_it = 0, seg_it = 0;
+        bool ok = true;
+        while (ok && it.next(p, seg)) {
+            const int ntiles = (int)uniform((uint32_t)(seg.tile_end - seg.tile_begin));
+            ok = mbar_wait_cluster(ctx, bar(kBarQFull), seg_it & 1, kBarQFull);
+            for (int i = 0; ok && i < ntiles; ++i, ++kv_it) {
+                const uint32_t stage = kv_it % kStages, b = kv_it & 1;
+                ok = mbar_wait_cluster(ctx, bar(kBarKFull + stage), (kv_it / kStages) & 1, kBarKFull + stage) &&
+                     mbar_wait_cluster(ctx, bar(kBarSEmpty + b), ((kv_it >> 1) & 1) ^ 1, kBarSEmpty + b);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                tcgen05_fence_after();
+                const uint32_t d = tmem_u + kColS + b * kHalf;
+                const uint64_t dq = make_desc(sbase + kOffQ, 16, 1024);                          // A: 2 x 64 heads x 16
+                const uint64_t dk = make_desc(sbase + kOffK + stage * kStageBytes, 16, 1024);    // B: 2 x 32 tokens x 16
 #pragma unroll
-                    for (int t = 0; t < 36 / kQkWarps; ++t) {
-                        const int idx = t * kQkWarps + a, c = idx >> 2, k = idx & 3;
-                        uint64_t dq = make_desc(sbase + kOffQ + c * kQSlab + k * 32, 16, 1024);   // A: 2 x 64 heads x 16
-                        uint64_t dk = make_desc(k0 + c * kSlab + k * 32, 16, 1024);             // B: 2 x 32 tokens x 16
-                        umma_bf16_pair(d, dq, dk, kIdescQK, t != 0);
-                    }
-                    umma_commit_pair(bar(kBarSFull + b));
-                    umma_commit_pair(bar(kBarQkDone + stage));
-                }
-                if (ok) umma_commit_pair(bar(kBarQEmpty));
-                ++seg_it;
+                for (int t = 0; t < 36; ++t)
+                    umma_bf16_pair(elected, d, dq + (((t >> 2) * kQSlab + (t & 3) * 32) >> 4), dk + (((t >> 2) * kSlab + (t & 3) * 32) >> 4), kIdescQK, t != 0);
+                if (elected) { umma_commit_pair(bar(kBarSFull + b)); umma_commit_pair(bar(kBarQkDone + stage)); }
+                __syncwarp();
             }
+            if (ok && elected) umma_commit_pair(bar(kBarQEmpty));
+            __syncwarp();
+            ++seg_it;
         }
-    } else if (warp >= kWarpPv && warp < kWarpPv + kPvWarps && rank == 0) {
-        // ===================================================== P.V issuers (leader CTA)
-        if (lane == 0) {
-            const int n = warp - kWarpPv;                 // dv half: columns [256 n, 256 n + 256)
-            constexpr uint32_t kIdescPV = make_idesc(128, 256, 0, 1);
-            uint32_t kv_it = 0, seg_it = 0;
-            bool ok = true;
-            while (ok && it.next(p, seg)) {
-                for (int tile = seg.tile_begin; ok && tile < seg.tile_end; ++tile, ++kv_it) {
-                    const uint32_t stage = kv_it % kStages, pb = kv_it & 1;
-                    ok = mbar_wait_cluster(ctx, bar(kBarVFull + stage), (kv_it / kStages) & 1, kBarVFull + stage) &&
-                         mbar_wait_cluster(ctx, bar(kBarPFull + pb), (kv_it >> 1) & 1, kBarPFull + pb);
-                    if (ok && tile == seg.tile_begin) ok = mbar_wait_cluster(ctx, bar(kBarOEmpty), (seg_it & 1) ^ 1, kBarOEmpty);
-                    if (!ok) break;
-                    tcgen05_fence_after();
-                    const uint32_t k0 = sbase + kOffK + stage * kStageBytes;
+    } else if (warp == kWarpPv && rank == 0) {
+        // ===================================================== P.V issuer (leader CTA)
+        constexpr uint32_t kIdescPV = make_idesc(128, 256, 0, 1);
+        const uint32_t elected = elect_one(), tmem_u = uniform(tmem_base);
+        uint32_t kv_it = 0, seg_it = 0;
+        bool ok = true;
+        while (ok && it.next(p, seg)) {
+            const int ntiles = (int)uniform((uint32_t)(seg.tile_end - seg.tile_begin));
+            for (int i = 0; ok && i < ntiles; ++i, ++kv_it) {
+                const uint32_t stage = kv_it % kStages, pb = kv_it & 1;
+                ok = mbar_wait_cluster(ctx, bar(kBarVFull + stage), (kv_it / kStages) & 1, kBarVFull + stage) &&
+                     mbar_wait_cluster(ctx, bar(kBarPFull + pb), (kv_it >> 1) & 1, kBarPFull + pb);
+                if (ok && i == 0) ok = mbar_wait_cluster(ctx, bar(kBarOEmpty), (seg_it & 1) ^ 1, kBarOEmpty);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                tcgen05_fence_after();
+                const uint32_t k0 = sbase + kOffK + stage * kStageBytes;
+                // 16 tokens of half-page j / 2.  A: P rows (heads), 32 bytes of the 64-byte row (half-page 0: in the
+                // stage's rope slot, 1: in its own buffer);
+                // B: slots 4n + 2g, + 1 (two 64-wide dv chunks, LBO apart), 16 token rows, MN-major
+                const uint64_t da0 = make_desc_sw64(k0 + 8 * kSlab, 16, 512), da1 = make_desc_sw64(sbase + kOffP1 + pb * kPHalfBytes, 16, 512);
+                const uint64_t db = make_desc(k0, kSlab, 1024);
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        // 16 tokens of half-page g.  A: P rows (heads), 32 bytes of the 64-byte row (g = 0: in the
-                        // stage's rope slot, g = 1: in its own buffer);
-                        // B: slots 4n + 2g, + 1 (two 64-wide dv chunks, LBO apart), 16 token rows, MN-major
-                        const int g = j >> 1;
-                        const uint32_t p0 = g == 0 ? k0 + 8 * kSlab : sbase + kOffP1 + pb * kPHalfBytes;
-                        uint64_t da = make_desc_sw64(p0 + (j & 1) * 32, 16, 512);
-                        uint64_t db = make_desc(k0 + (4 * n + 2 * g) * kSlab + (j & 1) * 2048, kSlab, 1024);
-                        umma_bf16_pair(tmem_base + kColO + n * 128, da, db, kIdescPV, (tile != seg.tile_begin) || j != 0);
-                    }
-                    umma_commit_pair(bar(kBarStageEmpty + stage));
-                    if (tile + 1 == seg.tile_end) umma_commit_pair(bar(kBarOFull));
+                for (int j = 0; j < 4; ++j) {
+#pragma unroll
+                    for (int n = 0; n < 2; ++n)                  // dv half: columns [256 n, 256 n + 256)
+                        umma_bf16_pair(elected, tmem_u + kColO + n * 128, (j < 2 ? da0 : da1) + (((j & 1) * 32) >> 4),
+                                       db + (((4 * n + 2 * (j >> 1)) * kSlab + (j & 1) * 2048) >> 4), kIdescPV, (uint32_t)i | (uint32_t)j);
                 }
-                ++seg_it;
+                if (elected) {
+                    umma_commit_pair(bar(kBarStageEmpty + stage));
+                    if (i + 1 == ntiles) umma_commit_pair(bar(kBarOFull));
+                }
+                __syncwarp();
             }
+            ++seg_it;
         }
     } else if (warp >= kWarpQk && warp < kWarpSoftmax) {
         // the issuer warps of the peer CTA have nothing to do for the attention itself: they carry the call's page-copy
         // job, if it has one (a layer's pages on the move while this layer decodes)
         if (p.mig_n > 0)
-            copy_pages_in_idle_warp(p, pair_id * (kQkWarps + kPvWarps) + (warp - kWarpQk), p.num_workers * p.pair_groups * (kQkWarps + kPvWarps), lane);
+            copy_pages_in_idle_warp(p, pair_id * kIssuerWarps + (warp - kWarpQk), p.num_workers * p.pair_groups * kIssuerWarps, lane);
     } else {
         // ===================================================== softmax + epilogue warps
-        // S partial layout per CTA: TMEM lane L < 64 = head L, tokens of half-page 0 in 32 columns;
+        // S layout per CTA: TMEM lane L < 64 = head L, tokens of half-page 0 in 32 columns;
         // lane 64 + L = head L, tokens of half-page 1.  Two warps per quadrant take 16 columns each,
         // so a thread owns ONE head and 16 tokens of one half-page.
         const int sw = warp - kWarpSoftmax;             // 0..7
@@ -340,15 +343,10 @@ decode_umma_pair_kernel(const __grid_constant__ DecodeParams p, const __grid_con
                 tcgen05_fence_after();
                 float sv[16];
                 {
-                    float pa[16], pb[16], pc[16];
-                    const uint32_t sb = tmem_base + lane_addr + kColS + (b * kQkWarps) * kHalf + 16 * cf;
-                    tmem_ld16(sb, sv);
-                    tmem_ld16(sb + kHalf, pa);
-                    tmem_ld16(sb + 2 * kHalf, pb);
-                    tmem_ld16(sb + 3 * kHalf, pc);
+                    tmem_ld16(tmem_base + lane_addr + kColS + b * kHalf + 16 * cf, sv);
                     tmem_wait_ld();
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) sv[j] = ((sv[j] + pa[j]) + (pb[j] + pc[j])) * scale_log2;
+                    for (int j = 0; j < 16; ++j) sv[j] *= scale_log2;
                 }
                 tcgen05_fence_before();
                 __syncwarp();
