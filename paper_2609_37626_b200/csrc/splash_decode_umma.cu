@@ -12,20 +12,17 @@
 // of the K rows (the latent), taken as an MN-major operand, so every KV byte crosses
 // HBM once per head group.
 //
-// Warp roles (288 threads):
+// Warp roles (224 threads):
 //   warp 0     TMA producer: block-table driven page gathers into a ring of stages
 //              (nine 64x64-element boxes per page, 128-byte swizzle), and the query
 //              rows of each segment.  Page tails and unaligned KV ranges are handled
 //              by shifting the box in the token dimension so that out-of-range tokens
 //              fall outside the page and are zero-filled by the TMA unit.
-//   warps 1-4  MMA issuers (one thread each).  One thread sustains only one tcgen05.mma
-//              per ~65 cycles whatever the shape, far below the pipe's rate for these
-//              small-N MMAs, so the work is spread: every issuer owns one of the
-//              independent S^T partial accumulators and one of the four dv blocks of
-//              O^T, runs its own ready-driven loop over the barriers and commits its
-//              own MMAs (the consumer barriers count one arrival per issuer).  QK^T of
-//              tile i+1 is issued while the softmax warps handle tile i.
-//   warps 5-8  online softmax over tokens (= TMEM lanes): per-head maxima by a
+//   warp 1     QK^T issuer: S^T of tile i + 1 while the softmax warps handle tile i (two S^T buffers)
+//   warp 2     P.V issuer.  An issuer warp stays converged and an elected lane issues, with all that the MMAs take in
+//              uniform registers.  (Issued from a branch of lane 0 alone, an MMA costs about 65 cycles whatever its shape,
+//              far above the pipe's time for these small-N ones: that took four issuers with a partial sum of S^T each.)
+//   warps 3-6  online softmax over tokens (= TMEM lanes): per-head maxima by a
 //              warp-shuffle reduce-scatter plus a small shared-memory exchange, lazy
 //              rescaling of O^T (only when a maximum grows by more than 2^8), P written
 //              to shared memory as the K-major B operand, epilogue.
@@ -41,8 +38,8 @@ namespace {
 
 using namespace umma;
 
-constexpr int kThreads = 288;                      // 9 warps: producer, 4 MMA issuers, 4 softmax
-constexpr int kMmaWarps = 4;
+constexpr int kThreads = 224;                      // 7 warps: producer, 2 MMA issuers, 4 softmax
+constexpr int kWarpQk = 1, kWarpPv = 2, kWarpSoftmax = 3;
 constexpr int kNumSoftmaxWarps = 4;                // barriers fed by the softmax role count one arrival per warp
 constexpr int kChunks = 9;                         // 576 / 64-element (128 B) chunks
 constexpr uint32_t kSlabBytes = 64 * 128;          // one chunk of one page: 64 tokens x 128 B
@@ -85,18 +82,12 @@ struct Layout {
     static constexpr uint32_t kBytes = kOffPlan + kInlinePlanBytes;
     // tensor memory columns
     static constexpr uint32_t kColO = 0;                     // 4 blocks x N columns
-    // S^T is accumulated in kAcc independent partial sums (summed by the softmax warps): a
-    // chain of 36 small MMAs into ONE accumulator runs at the MMA latency, not its rate.
     // 64-head groups compute S = Q K^T with the heads on the MMA's M (a softmax row lives in
     // one thread: no shuffles, no exchange); narrower groups compute S^T with the tokens on M
     // so that a 16- or 32-head slice is not padded to 64 rows.
     static constexpr bool kHeadsOnM = N == 64;
-    static constexpr int kAcc = 4;                           // = number of issuers that take part in QK^T
-    // two S buffers let QK^T run a tile ahead of the softmax; the 64-head kernel has tensor
-    // memory for one only (O^T 256 columns + 4 partials x 64)
-    static constexpr int kSBufs = N >= 64 ? 1 : 2;
-    static constexpr uint32_t kColS = 4 * N;                 // kSBufs buffers x kAcc x N columns
-    static_assert(kColS + kSBufs * kAcc * N <= 512, "tensor memory overflow");
+    static constexpr uint32_t kColS = 4 * N;                 // two buffers (QK^T runs a tile ahead of the softmax) x N columns
+    static_assert(kColS + 2 * N <= 512, "tensor memory overflow");
     static_assert(kBytes <= 232448, "shared memory overflow");
     static_assert(kOffQ % 1024 == 0 && kOffP % 1024 == 0 && (N * 128) % 1024 == 0, "swizzle atoms need 1024-byte alignment");
 };
@@ -124,11 +115,11 @@ decode_umma_kernel(const __grid_constant__ DecodeParams p, const __grid_constant
         return;
     }
     if (tid == 0) {
-        for (int s = 0; s < kStages; ++s) { mbar_init(bar(kBarKvFull + s), 1); mbar_init(bar(kBarKvEmpty + s), kMmaWarps); }
-        mbar_init(bar(kBarQFull), 1); mbar_init(bar(kBarQEmpty), L::kAcc);
-        for (int b = 0; b < L::kSBufs; ++b) { mbar_init(bar(kBarSFull + b), L::kAcc); mbar_init(bar(kBarSEmpty + b), kNumSoftmaxWarps); }
+        for (int s = 0; s < kStages; ++s) { mbar_init(bar(kBarKvFull + s), 1); mbar_init(bar(kBarKvEmpty + s), 1); }
+        mbar_init(bar(kBarQFull), 1); mbar_init(bar(kBarQEmpty), 1);
+        for (int b = 0; b < 2; ++b) { mbar_init(bar(kBarSFull + b), 1); mbar_init(bar(kBarSEmpty + b), kNumSoftmaxWarps); }
         mbar_init(bar(kBarPFull), kNumSoftmaxWarps);
-        mbar_init(bar(kBarOFull), kMmaWarps); mbar_init(bar(kBarOEmpty), kNumSoftmaxWarps);
+        mbar_init(bar(kBarOFull), 1); mbar_init(bar(kBarOEmpty), kNumSoftmaxWarps);
         misc[1] = 0; misc[2] = 0; misc[3] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -207,107 +198,82 @@ decode_umma_kernel(const __grid_constant__ DecodeParams p, const __grid_constant
             }
             ++seg_it;
         }
-    } else if (warp <= kMmaWarps) {
-        // ===================================================== MMA issuers
-        if (lane == 0) {
-            const int mw = warp - 1;                 // issuer index: S^T accumulator mw, dv block mw
-            const bool does_qk = mw < L::kAcc;
-            constexpr uint32_t kIdescQK = L::kHeadsOnM ? make_idesc(64, 64, 0, 0) : make_idesc(64, N, 0, 0);
-            // P^T is K-major (swizzled) when the softmax has the heads on M, MN-major (plain) when it has the tokens on M
-            constexpr uint32_t kIdescPV = make_idesc(128, N, 1, L::kHeadsOnM ? 0 : 1);
-            uint32_t kv_it = 0, s_it = 0, p_it = 0, seg_it = 0;
-            bool ok = true;
-            // This issuer's share of S^T for the tile with global index kv: the K = 16 steps
-            // idx = mw, mw + kAcc, ... of the 36, into partial accumulator mw.
-            auto issue_qk = [&](uint32_t kv, uint32_t sidx) {
-                const uint32_t stage = kv % kStages, b = sidx % L::kSBufs;
-                if (mw == 0) mark(kv, 2);
+    } else if (warp == kWarpQk) {
+        // ===================================================== QK^T issuer
+        constexpr uint32_t kIdescQK = L::kHeadsOnM ? make_idesc(64, 64, 0, 0) : make_idesc(64, N, 0, 0);
+        const uint32_t elected = elect_one(), tmem_u = uniform(tmem_base);
+        uint32_t kv = 0, seg_it = 0;
+        bool ok = true;
+        while (ok && it.next(p, seg)) {
+            const int ntiles = (int)uniform((uint32_t)(seg.tile_end - seg.tile_begin));
+            ok = mbar_wait(ctx, bar(kBarQFull), seg_it & 1, kBarQFull);
+            for (int i = 0; ok && i < ntiles; ++i, ++kv) {
+                const uint32_t stage = kv % kStages, b = kv & 1;
+                ok = mbar_wait(ctx, bar(kBarKvFull + stage), (kv / kStages) & 1, kBarKvFull + stage) &&
+                     mbar_wait(ctx, bar(kBarSEmpty + b), ((kv >> 1) & 1) ^ 1, kBarSEmpty + b);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                if (elected) mark(kv, 2);
                 tcgen05_fence_after();
-                const uint32_t a0 = sbase + L::kOffKv + stage * kStageBytes;
-                const uint32_t b0 = sbase + L::kOffQ;
-                const uint32_t d = tmem_base + L::kColS + (b * L::kAcc + mw) * N;
+                const uint64_t dk = make_desc(sbase + L::kOffKv + stage * kStageBytes, 16, 1024);     // K tile rows = tokens
+                const uint64_t dq = make_desc(sbase + L::kOffQ, 16, 1024);                            // Q rows = heads
+                const uint32_t d = tmem_u + L::kColS + b * N;
 #pragma unroll
-                for (int t = 0; t < 36 / L::kAcc; ++t) {
-                    const int idx = t * L::kAcc + mw, c = idx >> 2, k = idx & 3;
-                    uint64_t dk = make_desc(a0 + c * kSlabBytes + k * 32, 16, 1024);      // K tile rows = tokens
-                    uint64_t dq = make_desc(b0 + c * (N * 128) + k * 32, 16, 1024);       // Q rows = heads
-                    if constexpr (L::kHeadsOnM) umma_bf16(d, dq, dk, kIdescQK, t != 0);   // S  [heads x tokens]
-                    else umma_bf16(d, dk, dq, kIdescQK, t != 0);                          // S^T [tokens x heads]
+                for (int t = 0; t < 36; ++t) {       // K = 16 steps
+                    const uint64_t k_t = dk + (((t >> 2) * kSlabBytes + (t & 3) * 32) >> 4), q_t = dq + (((t >> 2) * (N * 128) + (t & 3) * 32) >> 4);
+                    if constexpr (L::kHeadsOnM) umma_bf16(elected, d, q_t, k_t, kIdescQK, t != 0);    // S  [heads x tokens]
+                    else umma_bf16(elected, d, k_t, q_t, kIdescQK, t != 0);                           // S^T [tokens x heads]
                 }
-                umma_commit(bar(kBarSFull + b));
-                if (mw == 0) mark(kv, 3);
-            };
-            // O^T block mw += V^T block mw (128 dv x 64 tokens) * P^T, four K = 16 steps.
-            auto issue_pv = [&](uint32_t stage, bool first_tile) {
+                if (elected) { umma_commit(bar(kBarSFull + b)); mark(kv, 3); }
+                __syncwarp();
+            }
+            if (ok && elected) umma_commit(bar(kBarQEmpty));
+            __syncwarp();
+            ++seg_it;
+        }
+    } else if (warp == kWarpPv) {
+        // ===================================================== P.V issuer
+        // P^T is K-major (swizzled) when the softmax has the heads on M, MN-major (plain) when it has the tokens on M
+        constexpr uint32_t kIdescPV = make_idesc(128, N, 1, L::kHeadsOnM ? 0 : 1);
+        const uint32_t elected = elect_one(), tmem_u = uniform(tmem_base);
+        uint32_t kv = 0, seg_it = 0;
+        bool ok = true;
+        while (ok && it.next(p, seg)) {
+            const int ntiles = (int)uniform((uint32_t)(seg.tile_end - seg.tile_begin));
+            for (int i = 0; ok && i < ntiles; ++i, ++kv) {
+                const uint32_t stage = kv % kStages;
+                // (one P buffer: the softmax warps cannot fill it again before this tile's P.V has retired)
+                ok = mbar_wait(ctx, bar(kBarPFull), kv & 1, kBarPFull);
+                if (ok && i == 0) ok = mbar_wait(ctx, bar(kBarOEmpty), (seg_it & 1) ^ 1, kBarOEmpty);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                if (elected) mark(kv, 6);
                 tcgen05_fence_after();
-                const uint32_t v0 = sbase + L::kOffKv + stage * kStageBytes + (2 * mw) * kSlabBytes;
-                const uint32_t p0 = sbase + L::kOffP;
+                // A: dv block j = two 64-element chunks (LBO apart) x 16 tokens (SBO per 8 tokens), MN-major
+                const uint64_t da = make_desc(sbase + L::kOffKv + stage * kStageBytes, kSlabBytes, 1024);
+                // B: 16 tokens x N heads.  K-major: 32 B into the swizzled rows; MN-major: two groups of eight tokens
+                // (128 B apart) x groups of eight heads (1,024 B apart)
+                const uint64_t db = L::kHeadsOnM ? make_desc(sbase + L::kOffP, 16, 1024) : make_desc_mn_plain(sbase + L::kOffP, 128, 1024);
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    // A: two 64-element chunks (LBO apart) x 16 tokens (SBO per 8 tokens), MN-major
-                    uint64_t da = make_desc(v0 + k * 2048, kSlabBytes, 1024);
-                    // B: 16 tokens x N heads.  K-major: 32 B into the swizzled rows; MN-major: two groups of eight tokens
-                    // (128 B apart) x groups of eight heads (1,024 B apart)
-                    uint64_t db = L::kHeadsOnM ? make_desc(p0 + k * 32, 16, 1024) : make_desc_mn_plain(p0 + k * 256, 128, 1024);
-                    umma_bf16(tmem_base + L::kColO + mw * N, da, db, kIdescPV, (!first_tile) || k != 0);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        umma_bf16(elected, tmem_u + L::kColO + j * N, da + ((2 * j * kSlabBytes + k * 2048) >> 4),
+                                  db + ((k * (L::kHeadsOnM ? 32 : 256)) >> 4), kIdescPV, (uint32_t)i | (uint32_t)k);
                 }
-            };
-            while (ok && it.next(p, seg)) {
-                const int ntiles = seg.tile_end - seg.tile_begin;
-                if (does_qk) {
-                    ok = mbar_wait(ctx, bar(kBarQFull), seg_it & 1, kBarQFull);
-                    if (!ok) break;
+                if (elected) {
+                    umma_commit(bar(kBarKvEmpty + stage));   // P.V done: stage free, P buffer free, O^T updated
+                    if (i + 1 == ntiles) umma_commit(bar(kBarOFull));
+                    mark(kv, 7);
                 }
-                // Issue whatever is ready: P.V of tile pv_i (frees a stage) or QK^T of tile qk_i
-                // (at most one tile ahead of the softmax: two S buffers).
-                int qk_i = does_qk ? 0 : ntiles, pv_i = 0;
-                unsigned long long idle_since = 0;
-                uint32_t idle_polls = 0;          // the wall clock is read once per 256 idle polls: reading it costs hundreds of cycles
-                while (pv_i < ntiles) {
-                    bool progressed = false;
-                    if ((qk_i > pv_i) && mbar_test_wait(bar(kBarPFull), (p_it + pv_i) & 1)) {
-                        if (pv_i == 0 && !mbar_wait(ctx, bar(kBarOEmpty), (seg_it & 1) ^ 1, kBarOEmpty)) { ok = false; break; }
-                        if (mw == 0) mark(kv_it + pv_i, 6);
-                        const uint32_t stage = (kv_it + pv_i) % kStages;
-                        issue_pv(stage, pv_i == 0);
-                        umma_commit(bar(kBarKvEmpty + stage));   // P.V done: stage free, P buffer free, O^T updated
-                        if (pv_i + 1 == ntiles) umma_commit(bar(kBarOFull));
-                        if (mw == 0) mark(kv_it + pv_i, 7);
-                        ++pv_i;
-                        progressed = true;
-                    }
-                    if (does_qk && qk_i < ntiles && qk_i < pv_i + 2) {
-                        const uint32_t kv = kv_it + qk_i, sidx = s_it + qk_i;
-                        if (mbar_test_wait(bar(kBarKvFull + kv % kStages), (kv / kStages) & 1) &&
-                            mbar_test_wait(bar(kBarSEmpty + sidx % L::kSBufs), ((sidx / L::kSBufs) & 1) ^ 1)) {
-                            issue_qk(kv, sidx);
-                            ++qk_i;
-                            if (qk_i == ntiles) umma_commit(bar(kBarQEmpty));
-                            progressed = true;
-                        }
-                    }
-                    if (progressed) { idle_since = 0; idle_polls = 0; continue; }
-                    if ((++idle_polls & 255u) != 0u) continue;
-                    if (*ctx.abort_flag) { ok = false; break; }
-                    const unsigned long long now = global_timer_ns();
-                    if (idle_since == 0) idle_since = now;
-                    else if (now - idle_since > kWaitLimitNs) {
-                        *ctx.abort_flag = 1;
-                        if (atomicCAS(ctx.status, 0, (int)SPLASH_DEVICE_TIMEOUT) == 0) {
-                            ctx.status[1] = (int)blockIdx.x; ctx.status[2] = 100 + (qk_i > pv_i ? kBarPFull : kBarKvFull);
-                            ctx.status[3] = pv_i;
-                        }
-                        ok = false; break;
-                    }
-                }
-                kv_it += ntiles; s_it += ntiles; p_it += ntiles;
-                ++seg_it;
+                __syncwarp();
             }
+            ++seg_it;
         }
     } else {
         // ===================================================== softmax + epilogue warps
         const int q4 = warp & 3;                       // TMEM lane quadrant of this warp
-        const int sw = warp - 1 - kMmaWarps;           // softmax warp 0..3
+        const int sw = warp - kWarpSoftmax;            // softmax warp 0..3
         const int st = sw * 32 + lane;                 // 0..127
         const uint32_t lane_addr = (uint32_t)(32 * q4) << 16;
         float *red = reinterpret_cast<float *>(smem + L::kOffRed);
@@ -334,8 +300,8 @@ decode_umma_kernel(const __grid_constant__ DecodeParams p, const __grid_constant
             const int ntiles = seg.tile_end - seg.tile_begin;
             for (int i = 0; i < ntiles; ++i) {
                 const TileGeom g = tile_geom(seg.lo, seg.hi, (first_page + seg.tile_begin + i) * kPage);
-                const uint32_t b = s_it % L::kSBufs;
-                ok &= mbar_wait(ctx, bar(kBarSFull + b), (s_it / L::kSBufs) & 1, kBarSFull + b);
+                const uint32_t b = s_it & 1;
+                ok &= mbar_wait(ctx, bar(kBarSFull + b), (s_it >> 1) & 1, kBarSFull + b);
                 if (st == 0) mark(s_it, 4);
                 tcgen05_fence_after();
                 if constexpr (L::kHeadsOnM) {
@@ -343,18 +309,7 @@ decode_umma_kernel(const __grid_constant__ DecodeParams p, const __grid_constant
                 // fragment load spreads those over all 32 threads: this thread holds heads
                 // hA = 16 q4 + lane/4 and hB = hA + 8, tokens 8k + 2(lane%4) + {0,1}, k = 0..7.
                 float s[32];
-                {
-                    const uint32_t sb = tmem_base + lane_addr + L::kColS + b * (L::kAcc * N);
-                    tmem_ld_16x256b_x8(sb, s);
-#pragma unroll
-                    for (int a = 1; a < L::kAcc; ++a) {
-                        float part[32];
-                        tmem_ld_16x256b_x8(sb + a * N, part);
-                        tmem_wait_ld();
-#pragma unroll
-                        for (int n = 0; n < 32; ++n) s[n] += part[n];
-                    }
-                }
+                tmem_ld_16x256b_x8(tmem_base + lane_addr + L::kColS + b * N, s);
                 tmem_wait_ld();
                 tcgen05_fence_before();
                 __syncwarp();
@@ -427,18 +382,8 @@ decode_umma_kernel(const __grid_constant__ DecodeParams p, const __grid_constant
                 const int rA = 16 * q4 + (lane >> 2), rB = rA + 8, tq = lane & 3;
                 const bool vA = rA >= g.r_lo && rA < g.r_hi, vB = rB >= g.r_lo && rB < g.r_hi;
                 float s[4 * kR];
-                {
-                    float t0[4 * kR], t1[4 * kR], t2[4 * kR];
-                    const uint32_t sb = tmem_base + lane_addr + L::kColS + b * (L::kAcc * N);
-                    tmem_ld_frag<N>(sb, s);
-                    tmem_ld_frag<N>(sb + N, t0);
-                    tmem_ld_frag<N>(sb + 2 * N, t1);
-                    tmem_ld_frag<N>(sb + 3 * N, t2);
-                    tmem_wait_ld();
-#pragma unroll
-                    for (int n = 0; n < 4 * kR; ++n) s[n] = (s[n] + t0[n]) + (t1[n] + t2[n]);
-                    static_assert(L::kAcc == 4, "four partial accumulators are summed here");
-                }
+                tmem_ld_frag<N>(tmem_base + lane_addr + L::kColS + b * N, s);
+                tmem_wait_ld();
                 tcgen05_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bar(kBarSEmpty + b));

@@ -215,7 +215,7 @@ decode_umma_fp8_kernel(const __grid_constant__ DecodeParams p, const __grid_cons
                         const uint32_t q0 = sbase + (hl ? kOffQLo : kOffQHi);
                         uint64_t dq = make_desc_sw64(q0 + c * kSlab + k * 32, 16, 512);     // A: 64 heads x 32
                         uint64_t dk = make_desc_sw64(k0 + c * kSlab + k * 32, 16, 512);     // B: 64 tokens x 32
-                        umma_e4m3(d, dq, dk, kIdescQK, t != 0);
+                        umma_e4m3(1u, d, dq, dk, kIdescQK, t != 0);
                     }
                     umma_commit(bar(kBarSFull + b));
                     if (a == 0) mark(kv, 3);
@@ -253,7 +253,7 @@ decode_umma_fp8_kernel(const __grid_constant__ DecodeParams p, const __grid_cons
                                 // A: two 64-element chunks (LBO apart) x 32 tokens (SBO per 8 tokens), MN-major
                                 uint64_t da = make_desc_sw64(v0 + (2 * j) * kSlab + k * 2048, kSlab, 512);
                                 uint64_t db = make_desc_sw64(sbase + (hl ? kOffPLo : kOffPHi) + (kv & 1) * (kN * 64) + k * 32, 16, 512);
-                                umma_e4m3(tmem_base + kColO + j * kN, da, db, hl ? kIdescPVLo : kIdescPV, (i != 0) || (hl | k) != 0);
+                                umma_e4m3(1u, tmem_base + kColO + j * kN, da, db, hl ? kIdescPVLo : kIdescPV, (i != 0) || (hl | k) != 0);
                             }
                         }
                     }

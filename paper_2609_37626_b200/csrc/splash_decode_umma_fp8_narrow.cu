@@ -28,9 +28,9 @@
 // barrier-wide OR per tile, and only then do they reduce the maxima across tokens, move the
 // references and rescale O^T.  Row sums stay per thread until the request ends.
 //
-// Warp roles (352 threads, 480 with 32 heads): TMA producer (pages + scale pages, next page pulled into L2), 2 QK^T
-// issuers (one partial accumulator of S^T each), 2 P.V issuers (two dv blocks each), N / 4 softmax /
-// epilogue warps (one per TMEM lane quadrant and group of 16 heads), 2 query converter warps (a request ahead: the query operands are double buffered).  Every wait is bounded; on expiry the CTA records
+// Warp roles (352 threads, 480 with 32 heads): TMA producer (pages + scale pages, next page pulled into L2), QK^T
+// issuer, P.V issuer (converged warps whose elected lane issues with uniform operands), N / 4 softmax /
+// epilogue warps (one per TMEM lane quadrant and group of 16 heads), 4 query converter warps (a request ahead: the query operands are double buffered).  Every wait is bounded; on expiry the CTA records
 // SPLASH_DEVICE_TIMEOUT and leaves in order.
 #include "splash_fp8.cuh"
 #include "splash_pair.cuh"
@@ -41,11 +41,9 @@ namespace {
 
 using namespace umma;
 
-constexpr int kQkWarps = 2;                        // = partial accumulators of S^T
-constexpr int kPvWarps = 2;                        // each owns two of the four dv blocks of O^T
 constexpr int kWarpQk = 1;
-constexpr int kWarpPv = kWarpQk + kQkWarps;
-constexpr int kWarpSoftmax = kWarpPv + kPvWarps;            // 5: TMEM lane quadrant = warp & 3
+constexpr int kWarpPv = 2;
+constexpr int kWarpSoftmax = 3;                    // TMEM lane quadrant = warp & 3
 constexpr int kChunks = 9;                         // 576 / 64-element (64 B) chunks
 constexpr uint32_t kSlab = 64 * 64;                // one chunk of one page: 64 tokens x 64 B
 constexpr uint32_t kStageBytes = kChunks * kSlab;  // 36,864
@@ -61,7 +59,7 @@ enum BarrierId {
     kBarKvFull = 0,                    // [stages]
     kBarKvEmpty = kBarKvFull + kMaxStages,
     kBarQFull = kBarKvEmpty + kMaxStages,   // [2]: one per query operand buffer
-    kBarQEmpty = kBarQFull + 2,        // [2]: the QK^T issuers are done with the buffer AND the softmax warps with the request
+    kBarQEmpty = kBarQFull + 2,        // [2]: the QK^T issuer is done with the buffer AND the softmax warps with the request
                                        // (they stage its output tile there)
     kBarSFull = kBarQEmpty + 2,        // [2]
     kBarSEmpty = kBarSFull + 2,        // [2]
@@ -78,7 +76,7 @@ struct Layout {
     static constexpr int kSoftmaxWarps = N / 4;                // one per TMEM lane quadrant and group of 16 heads
     static constexpr int kSoftmaxThreads = 32 * kSoftmaxWarps;
     static constexpr int kWarpConvert = kWarpSoftmax + kSoftmaxWarps;
-    static constexpr int kNumConvertWarps = 2;                 // four threads per head, 16 heads per pass
+    static constexpr int kNumConvertWarps = 4;                 // eight threads per head, 16 heads per pass
     static constexpr int kThreads = (kWarpConvert + kNumConvertWarps) * 32;   // 352 (N = 16) or 480 (N = 32)
     static constexpr uint32_t kQSlab = 2 * N * 64;             // one chunk of the query operand: (N hi rows, N lo rows) x 64 B
     static constexpr uint32_t kQBytes = kChunks * kQSlab;      // one buffer; there are two (request parity)
@@ -97,8 +95,8 @@ struct Layout {
     static constexpr uint32_t kOffPlan = kOffMisc + 16;        // inline plan
     static constexpr uint32_t kBytes = kOffPlan + kInlinePlanBytes;
     static constexpr uint32_t kColO = 0;                       // 4 dv blocks x (N hi, N lo) columns
-    static constexpr uint32_t kColS = 8 * N;                   // 2 buffers x kQkWarps partials x (N hi, N lo) columns
-    static_assert(kColS + 2 * kQkWarps * 2 * N <= 512, "tensor memory overflow");
+    static constexpr uint32_t kColS = 8 * N;                   // 2 buffers x (N hi, N lo) columns
+    static_assert(kColS + 2 * 2 * N <= 512, "tensor memory overflow");
     static_assert(kBytes <= 232448, "shared memory overflow");
     static_assert(kOffQ % 1024 == 0 && kQSlab % 512 == 0 && kOffP % 128 == 0, "operands need aligned windows");
 };
@@ -127,11 +125,11 @@ decode_umma_fp8_narrow_kernel(const __grid_constant__ DecodeParams p, const __gr
         return;
     }
     if (tid == 0) {
-        for (int s = 0; s < kStages; ++s) { mbar_init(bar(kBarKvFull + s), 1); mbar_init(bar(kBarKvEmpty + s), kPvWarps); }
-        for (int b = 0; b < 2; ++b) { mbar_init(bar(kBarQFull + b), L::kNumConvertWarps); mbar_init(bar(kBarQEmpty + b), kQkWarps + kNumSoftmaxWarps); }
-        for (int b = 0; b < 2; ++b) { mbar_init(bar(kBarSFull + b), kQkWarps); mbar_init(bar(kBarSEmpty + b), kNumSoftmaxWarps); }
+        for (int s = 0; s < kStages; ++s) { mbar_init(bar(kBarKvFull + s), 1); mbar_init(bar(kBarKvEmpty + s), 1); }
+        for (int b = 0; b < 2; ++b) { mbar_init(bar(kBarQFull + b), L::kNumConvertWarps); mbar_init(bar(kBarQEmpty + b), 1 + kNumSoftmaxWarps); }
+        for (int b = 0; b < 2; ++b) { mbar_init(bar(kBarSFull + b), 1); mbar_init(bar(kBarSEmpty + b), kNumSoftmaxWarps); }
         for (int b = 0; b < 2; ++b) mbar_init(bar(kBarPFull + b), kNumSoftmaxWarps);
-        mbar_init(bar(kBarOFull), kPvWarps); mbar_init(bar(kBarOEmpty), kNumSoftmaxWarps);
+        mbar_init(bar(kBarOFull), 1); mbar_init(bar(kBarOEmpty), kNumSoftmaxWarps);
         misc[1] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -214,92 +212,88 @@ decode_umma_fp8_narrow_kernel(const __grid_constant__ DecodeParams p, const __gr
                 ++kv_it;
             }
         }
-    } else if (warp < kWarpPv) {
-        // ===================================================== QK^T issuers: S^T = K [q hi | q lo]^T
-        if (lane == 0) {
-            const int a = warp - kWarpQk;            // partial accumulator a
-            constexpr uint32_t kIdescQK = make_idesc_e4m3(64, 2 * N, 0);
-            uint32_t kv = 0, seg_it = 0;
-            bool ok = true;
-            while (ok && it.next(p, seg)) {
-                const int ntiles = seg.tile_end - seg.tile_begin;
-                const uint32_t qb = seg_it & 1;
-                ok = mbar_wait(ctx, bar(kBarQFull + qb), (seg_it >> 1) & 1, kBarQFull + qb);
-                for (int i = 0; ok && i < ntiles; ++i, ++kv) {
-                    const uint32_t stage = kv % kStages, b = kv & 1;
-                    ok = mbar_wait(ctx, bar(kBarKvFull + stage), (kv / kStages) & 1, kBarKvFull + stage) &&
-                         mbar_wait(ctx, bar(kBarSEmpty + b), ((kv >> 1) & 1) ^ 1, kBarSEmpty + b);
-                    if (!ok) break;
-                    if (a == 0) mark(kv, 2);
-                    tcgen05_fence_after();
-                    const uint32_t k0 = sbase + L::kOffKv + stage * kStageBytes;
-                    const uint32_t d = tmem_base + L::kColS + (b * kQkWarps + a) * (2 * N);
-                    // 18 K = 32 steps per tile; this issuer takes every second
+    } else if (warp == kWarpQk) {
+        // ===================================================== QK^T issuer: S^T = K [q hi | q lo]^T
+        constexpr uint32_t kIdescQK = make_idesc_e4m3(64, 2 * N, 0);
+        const uint32_t elected = elect_one(), tmem_u = uniform(tmem_base);
+        uint32_t kv = 0, seg_it = 0;
+        bool ok = true;
+        while (ok && it.next(p, seg)) {
+            const int ntiles = (int)uniform((uint32_t)(seg.tile_end - seg.tile_begin));
+            const uint32_t qb = seg_it & 1;
+            ok = mbar_wait(ctx, bar(kBarQFull + qb), (seg_it >> 1) & 1, kBarQFull + qb);
+            for (int i = 0; ok && i < ntiles; ++i, ++kv) {
+                const uint32_t stage = kv % kStages, b = kv & 1;
+                ok = mbar_wait(ctx, bar(kBarKvFull + stage), (kv / kStages) & 1, kBarKvFull + stage) &&
+                     mbar_wait(ctx, bar(kBarSEmpty + b), ((kv >> 1) & 1) ^ 1, kBarSEmpty + b);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                if (elected) mark(kv, 2);
+                tcgen05_fence_after();
+                const uint64_t dk = make_desc_sw64(sbase + L::kOffKv + stage * kStageBytes, 16, 512);    // A: 64 tokens x 32
+                const uint64_t dq = make_desc_sw64(sbase + L::kOffQ + qb * L::kQBytes, 16, 512);         // B: 2N rows x 32
+                const uint32_t d = tmem_u + L::kColS + b * (2 * N);
 #pragma unroll
-                    for (int t = 0; t < 18 / kQkWarps; ++t) {
-                        const int ks = t * kQkWarps + a, c = ks >> 1, k = ks & 1;
-                        uint64_t dk = make_desc_sw64(k0 + c * kSlab + k * 32, 16, 512);                      // A: 64 tokens x 32
-                        uint64_t dq = make_desc_sw64(sbase + L::kOffQ + qb * L::kQBytes + c * L::kQSlab + k * 32, 16, 512);    // B: 2N rows x 32
-                        umma_e4m3(d, dk, dq, kIdescQK, t != 0);
-                    }
-                    umma_commit(bar(kBarSFull + b));
-                    if (a == 0) mark(kv, 3);
-                }
-                if (ok) umma_commit(bar(kBarQEmpty + qb));
-                ++seg_it;
+                for (int ks = 0; ks < 18; ++ks)      // K = 32 steps
+                    umma_e4m3(elected, d, dk + (((ks >> 1) * kSlab + (ks & 1) * 32) >> 4), dq + (((ks >> 1) * L::kQSlab + (ks & 1) * 32) >> 4), kIdescQK, ks != 0);
+                if (elected) { umma_commit(bar(kBarSFull + b)); mark(kv, 3); }
+                __syncwarp();
             }
+            if (ok && elected) umma_commit(bar(kBarQEmpty + qb));
+            __syncwarp();
+            ++seg_it;
         }
-    } else if (warp < kWarpSoftmax) {
-        // ===================================================== P.V issuers: [O^T hi | O^T lo] += V^T [P hi | 16 P lo]^T
-        if (lane == 0) {
-            const int pj = warp - kWarpPv;           // dv blocks 2 pj and 2 pj + 1
-            constexpr uint32_t kIdescPV = make_idesc_e4m3(128, 2 * N, 1, 0, 1);
-            uint32_t kv = 0, seg_it = 0;
-            bool ok = true;
-            while (ok && it.next(p, seg)) {
-                const int ntiles = seg.tile_end - seg.tile_begin;
-                for (int i = 0; ok && i < ntiles; ++i, ++kv) {
-                    const uint32_t stage = kv % kStages;
-                    ok = mbar_wait(ctx, bar(kBarPFull + (kv & 1)), (kv >> 1) & 1, kBarPFull + (kv & 1));
-                    if (ok && i == 0) ok = mbar_wait(ctx, bar(kBarOEmpty), (seg_it & 1) ^ 1, kBarOEmpty);
-                    if (!ok) break;
-                    if (pj == 0) mark(kv, 6);
-                    tcgen05_fence_after();
-                    const uint32_t v0 = sbase + L::kOffKv + stage * kStageBytes;
+    } else if (warp == kWarpPv) {
+        // ===================================================== P.V issuer: [O^T hi | O^T lo] += V^T [P hi | 16 P lo]^T
+        constexpr uint32_t kIdescPV = make_idesc_e4m3(128, 2 * N, 1, 0, 1);
+        const uint32_t elected = elect_one(), tmem_u = uniform(tmem_base);
+        uint32_t kv = 0, seg_it = 0;
+        bool ok = true;
+        while (ok && it.next(p, seg)) {
+            const int ntiles = (int)uniform((uint32_t)(seg.tile_end - seg.tile_begin));
+            for (int i = 0; ok && i < ntiles; ++i, ++kv) {
+                const uint32_t stage = kv % kStages;
+                ok = mbar_wait(ctx, bar(kBarPFull + (kv & 1)), (kv >> 1) & 1, kBarPFull + (kv & 1));
+                if (ok && i == 0) ok = mbar_wait(ctx, bar(kBarOEmpty), (seg_it & 1) ^ 1, kBarOEmpty);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                if (elected) mark(kv, 6);
+                tcgen05_fence_after();
+                // A: dv block j = two 64-element chunks (LBO apart) x 32 tokens (SBO per 8 tokens), MN-major
+                const uint64_t da = make_desc_sw64(sbase + L::kOffKv + stage * kStageBytes, kSlab, 512);
+                // B: 32 tokens (four groups of eight, 128 B apart) x 2N columns (groups of 16, 1024 B apart)
+                const uint64_t db = make_desc_mn_plain(sbase + L::kOffP + (kv & 1) * L::kPBytes, 128, 1024);
 #pragma unroll
-                    for (int k = 0; k < 2; ++k) {
+                for (int k = 0; k < 2; ++k) {
 #pragma unroll
-                        for (int jj = 0; jj < 2; ++jj) {
-                            const int j = 2 * pj + jj;
-                            // A: two 64-element chunks (LBO apart) x 32 tokens (SBO per 8 tokens), MN-major
-                            uint64_t da = make_desc_sw64(v0 + (2 * j) * kSlab + k * 2048, kSlab, 512);
-                            // B: 32 tokens (four groups of eight, 128 B apart) x 2N columns (groups of 16, 1024 B apart)
-                            uint64_t db = make_desc_mn_plain(sbase + L::kOffP + (kv & 1) * L::kPBytes + k * 512, 128, 1024);
-                            umma_e4m3(tmem_base + L::kColO + j * (2 * N), da, db, kIdescPV, (i != 0) || k != 0);
-                        }
-                    }
+                    for (int j = 0; j < 4; ++j)
+                        umma_e4m3(elected, tmem_u + L::kColO + j * (2 * N), da + ((2 * j * kSlab + k * 2048) >> 4), db + ((k * 512) >> 4), kIdescPV,
+                                  (uint32_t)i | (uint32_t)k);
+                }
+                if (elected) {
                     umma_commit(bar(kBarKvEmpty + stage));   // P.V done: stage free, P buffers free, O^T updated
                     if (i + 1 == ntiles) umma_commit(bar(kBarOFull));
-                    if (pj == 0) mark(kv, 7);
+                    mark(kv, 7);
                 }
-                ++seg_it;
+                __syncwarp();
             }
+            ++seg_it;
         }
     } else if (warp >= kWarpConvert) {
         // ===================================================== query converters
-        // bf16 query rows -> e4m3 hi + lo operands with one scale per head, four threads per head.  The operands are
+        // bf16 query rows -> e4m3 hi + lo operands with one scale per head, eight threads per head.  The operands are
         // double buffered, so the converters work a whole request ahead: the row is read once, into registers, and
         // the latency of those loads (several microseconds while the cache streams at full rate) stays off the
         // path from one request's last tile to the next one's first.
-        constexpr int kVecs = 18;                      // 8-element vectors per thread: a quarter of a row
-        const int ct = (warp - kWarpConvert) * 32 + lane;   // 0..63: head ct / 4 of a pass, quarter ct % 4
+        constexpr int kVecs = 9;                       // 8-element vectors per thread: an eighth of a row
+        const int ct = (warp - kWarpConvert) * 32 + lane;   // 0..127: head ct / 8 of a pass, eighth ct % 8
         float *qs_s = reinterpret_cast<float *>(smem + L::kOffQs);
         uint32_t seg_it = 0;
         bool ok = true;
         while (ok && it.next(p, seg)) {
             const uint32_t qb = seg_it & 1;
             uint8_t *qdst = smem + L::kOffQ + qb * L::kQBytes;
-            const int part = ct & 3;
+            const int part = ct & 7;
             {
                 // the rows of the request after this one: into L2 now, so that their loads, a request from now, are short
                 SegmentIter<L::kOffPlan> peek = it;
@@ -308,39 +302,35 @@ decode_umma_fp8_narrow_kernel(const __grid_constant__ DecodeParams p, const __gr
                     const char *row0 = reinterpret_cast<const char *>(static_cast<const __nv_bfloat16 *>(p.q) +
                                        (int64_t)nxt.request * p.q_stride_request + (int64_t)head0 * p.q_stride_head);
                     const int64_t bytes = (int64_t)min(N, p.head_end - head0) * p.q_stride_head * 2;
-                    for (int64_t o = (int64_t)ct * 128; o < bytes; o += 64 * 128)
+                    for (int64_t o = (int64_t)ct * 128; o < bytes; o += L::kNumConvertWarps * 32 * 128)
                         asm volatile("prefetch.global.L2 [%0];" ::"l"(row0 + o));
                 }
             }
 #pragma unroll 1
             for (int pass = 0; pass < N / 16; ++pass) {
-                const int hd = pass * 16 + (ct >> 2);
+                const int hd = pass * 16 + (ct >> 3);
                 const int gh = head0 + hd;
                 const bool live = gh < p.head_end;
                 const uint4 *src = reinterpret_cast<const uint4 *>(
                     static_cast<const __nv_bfloat16 *>(p.q) + (int64_t)seg.request * p.q_stride_request +
                     (int64_t)(live ? gh : p.head_begin) * p.q_stride_head + part * (kVecs * 8));
-                // 16 heads keep the quarter row in registers between the two passes; with 32 heads (480 threads, 128
-                // registers each) it is read again, nine vectors at a time, from the cache it has just come into
-                constexpr int kBatch = N == 16 ? kVecs : kVecs / 2;
-                uint4 x[kBatch];
+                // (kept in registers between the maximum and the conversion)
+                uint4 x[kVecs];
                 float amax = 0.f;
-#pragma unroll 1
-                for (int v0 = 0; v0 < kVecs; v0 += kBatch) {
 #pragma unroll
-                    for (int v = 0; v < kBatch; ++v) x[v] = live ? __ldg(src + v0 + v) : make_uint4(0u, 0u, 0u, 0u);
+                for (int v = 0; v < kVecs; ++v) x[v] = live ? __ldg(src + v) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
-                    for (int v = 0; v < kBatch; ++v) {
-                        const uint32_t w[4] = {x[v].x, x[v].y, x[v].z, x[v].w};
+                for (int v = 0; v < kVecs; ++v) {
+                    const uint32_t w[4] = {x[v].x, x[v].y, x[v].z, x[v].w};
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            amax = fmaxf(amax, fabsf(__uint_as_float(w[k] << 16)));
-                            amax = fmaxf(amax, fabsf(__uint_as_float(w[k] & 0xffff0000u)));
-                        }
+                    for (int k = 0; k < 4; ++k) {
+                        amax = fmaxf(amax, fabsf(__uint_as_float(w[k] << 16)));
+                        amax = fmaxf(amax, fabsf(__uint_as_float(w[k] & 0xffff0000u)));
                     }
                 }
                 amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 1));
                 amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 2));
+                amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 4));
                 const float qs = amax > 0.f ? amax * (1.0f / 448.0f) : 1.0f;
                 const float inv = amax > 0.f ? 448.0f / amax : 1.0f;
                 if (pass == 0) {
@@ -349,29 +339,22 @@ decode_umma_fp8_narrow_kernel(const __grid_constant__ DecodeParams p, const __gr
                     if (!ok) break;
                 }
                 if (part == 0) qs_s[(seg_it & 3) * N + hd] = qs;
-#pragma unroll 1
-                for (int v0 = 0; v0 < kVecs; v0 += kBatch) {
-                    if (kBatch < kVecs) {
 #pragma unroll
-                        for (int v = 0; v < kBatch; ++v) x[v] = live ? __ldg(src + v0 + v) : make_uint4(0u, 0u, 0u, 0u);
+                for (int v = 0; v < kVecs; ++v) {
+                    const uint32_t w[4] = {x[v].x, x[v].y, x[v].z, x[v].w};
+                    uint16_t hi[4], lo[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const float e0 = __uint_as_float(w[k] << 16) * inv, e1 = __uint_as_float(w[k] & 0xffff0000u) * inv;
+                        split_e4m3_e4m3_x2(e0, e1, hi[k], lo[k]);
                     }
-#pragma unroll
-                    for (int v = 0; v < kBatch; ++v) {
-                        const uint32_t w[4] = {x[v].x, x[v].y, x[v].z, x[v].w};
-                        uint16_t hi[4], lo[4];
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            const float e0 = __uint_as_float(w[k] << 16) * inv, e1 = __uint_as_float(w[k] & 0xffff0000u) * inv;
-                            split_e4m3_e4m3_x2(e0, e1, hi[k], lo[k]);
-                        }
-                        const uint32_t d = (uint32_t)(part * (kVecs * 8) + (v0 + v) * 8);
-                        // the lo rows follow the N hi rows of the chunk (N is a multiple of 8: same swizzle phase)
-                        const uint32_t off = (d >> 6) * L::kQSlab + sw64((uint32_t)hd, d & 63);
-                        *reinterpret_cast<uint2 *>(qdst + off) =
-                            make_uint2((uint32_t)hi[0] | ((uint32_t)hi[1] << 16), (uint32_t)hi[2] | ((uint32_t)hi[3] << 16));
-                        *reinterpret_cast<uint2 *>(qdst + N * 64 + off) =
-                            make_uint2((uint32_t)lo[0] | ((uint32_t)lo[1] << 16), (uint32_t)lo[2] | ((uint32_t)lo[3] << 16));
-                    }
+                    const uint32_t d = (uint32_t)(part * (kVecs * 8) + v * 8);
+                    // the lo rows follow the N hi rows of the chunk (N is a multiple of 8: same swizzle phase)
+                    const uint32_t off = (d >> 6) * L::kQSlab + sw64((uint32_t)hd, d & 63);
+                    *reinterpret_cast<uint2 *>(qdst + off) =
+                        make_uint2((uint32_t)hi[0] | ((uint32_t)hi[1] << 16), (uint32_t)hi[2] | ((uint32_t)hi[3] << 16));
+                    *reinterpret_cast<uint2 *>(qdst + N * 64 + off) =
+                        make_uint2((uint32_t)lo[0] | ((uint32_t)lo[1] << 16), (uint32_t)lo[2] | ((uint32_t)lo[3] << 16));
                 }
             }
             if (!ok) break;
@@ -427,16 +410,14 @@ decode_umma_fp8_narrow_kernel(const __grid_constant__ DecodeParams p, const __gr
                 tcgen05_fence_after();
                 float s[4 * kR];
                 {
-                    // S^T = the sum of four N-column pieces: (partial 0, partial 1) x (q hi, q lo)
-                    float t0[4 * kR], t1[4 * kR], t2[4 * kR];
-                    const uint32_t sb = tmem_base + lane_addr + L::kColS + b * (2 * kQkWarps * N) + h0;
+                    // S^T = the sum of two N-column pieces: q hi, q lo
+                    float t0[4 * kR];
+                    const uint32_t sb = tmem_base + lane_addr + L::kColS + b * (2 * N) + h0;
                     tmem_ld_16x256b_x2(sb, s);
                     tmem_ld_16x256b_x2(sb + N, t0);
-                    tmem_ld_16x256b_x2(sb + 2 * N, t1);
-                    tmem_ld_16x256b_x2(sb + 3 * N, t2);
                     tmem_wait_ld();
 #pragma unroll
-                    for (int n = 0; n < 4 * kR; ++n) s[n] = (s[n] + t0[n]) + (t1[n] + t2[n]);
+                    for (int n = 0; n < 4 * kR; ++n) s[n] += t0[n];
                 }
                 tcgen05_fence_before();
                 __syncwarp();
