@@ -79,9 +79,8 @@ enum {
     /* slices of 65..128 heads: use two independent 64-head CTAs per KV worker instead of a CTA
      * pair issuing cta_group::2 MMAs.  A diagnostic path. */
     SPLASH_FLAG_NO_PAIR = 2u,
-    /* splash_mla_decode_sparse only: one kernel that gathers, dequantises and multiplies (CTA pairs) instead of
-     * the gather kernel followed by the dense kernels.  Every listed row crosses HBM once; tile, query rows and
-     * P are f16 in that kernel (values must lie within f16's range).  Correct, not yet the faster of the two. */
+    /* splash_mla_decode_sparse only: accepted, without effect.  (It asked for one kernel that gathers, dequantises and
+     * multiplies instead of a gather kernel followed by the dense ones; every sparse call runs that way now.) */
     SPLASH_FLAG_SPARSE_FUSED = 4u,
     /* splash_mla_decode only: validation mode.  One more (small) kernel between the plan and the decode kernel checks
      * every block-table entry of a page that intersects a request's range against [0, num_pool_pages) and records

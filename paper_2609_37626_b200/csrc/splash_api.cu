@@ -165,7 +165,7 @@ size_t splash_mla_decode_workspace_bytes(const splash_mla_shape *shape, int32_t 
 
 namespace {
 
-// The first stage of a sparse call: gathers the listed rows into the dense cache that the decode then reads.
+// A sparse call: where the listed rows come from, and the dense cache that the fp32 kernel has them gathered into.
 struct SparseStage {
     const void *pool656;
     int num_pool_pages;
@@ -175,7 +175,6 @@ struct SparseStage {
     int64_t sel_stride;
     int max_selected, pages_per_request;
     int32_t *dense_table;
-    bool fused;        // one kernel gathers, dequantises and multiplies (CTA pairs); else gather kernel + dense kernels
 };
 
 // Argument checks shared by the page-migration entry points (the workspace variant, the job of a decode call).
@@ -217,8 +216,9 @@ cudaError_t run_migrate_job(const splash_migrate_job *job, bool do_table, bool d
                                job->num_table_entries, static_cast<int32_t *>(job->workspace), do_table, do_copy, stream);
 }
 
-// One dense decode call: plan, decode kernel, combine.  With a sparse stage, seq_lens are the list counts, kv_pool
-// and block_table the dense cache and its table, and the gather kernel runs between the plan and the decode kernel.
+// One decode call: plan, decode kernel, combine.  With a sparse stage, seq_lens are the list counts; the decode kernel gathers
+// the listed rows itself, except the fp32 kernel, which runs over the dense cache behind kv_pool and block_table that the gather
+// kernel has filled.
 int decode_dense(const splash_mla_shape *shape, const void *q, const void *kv_pool, const float *kv_scales,
                  const int32_t *block_table, const int32_t *seq_lens, int32_t head_begin, int32_t head_end,
                  const int32_t *kv_begin, const int32_t *kv_end, float *out, float *lse,
@@ -268,8 +268,6 @@ int decode_dense(const splash_mla_shape *shape, const void *q, const void *kv_po
     bool job_copy_pending = job != nullptr;
     if (job != nullptr) e = run_migrate_job(job, true, false, stream);
     Tiling t = choose_tiling(shape, h, dev.sm_count, simt);
-    const bool fused_sparse = sparse && sparse->fused && !simt;
-    if (fused_sparse) { t.heads_per_group = 64; t.num_groups = 2; t.num_workers = dev.sm_count / 2 > 0 ? dev.sm_count / 2 : 1; t.pair_groups = 1; }
     // where the work partition comes from (splash_common.cuh): a batch of up to 32 requests is planned by the decode kernel
     // itself; if its contexts are short besides, no request is cut and the combine kernel is left out
     int plan_mode = kPlanWorkspace;
@@ -306,7 +304,8 @@ int decode_dense(const splash_mla_shape *shape, const void *q, const void *kv_po
     p.status = v.status; p.partial_lse = v.partial_lse; p.partial_out = v.partial_out; p.partial_scale = v.partial_scale;
     p.trace = g_trace;
     p.len_cap = sparse ? sparse->max_selected : -1;
-    if (fused_sparse) {
+    if (sparse && !simt) {
+        p.sparse = 1;
         p.kv_pool = sparse->pool656; p.block_table = sparse->block_table; p.table_stride = sparse->table_stride;
         p.num_pool_pages = sparse->num_pool_pages; p.sel = sparse->sel; p.sel_stride = sparse->sel_stride;
         p.ctx_lens = sparse->ctx_lens;
@@ -318,8 +317,8 @@ int decode_dense(const splash_mla_shape *shape, const void *q, const void *kv_po
     else if (pair)
         p.request_overhead_tiles = kRequestOverheadTilesPair;
     // the bf16 CTA-pair kernel writes its partial outputs as f16
-    p.partial_f16 = (pair && shape->kv_dtype == SPLASH_KV_BF16 && !fused_sparse) ? 1 : 0;
-    if (job_copy_pending && pair && !fused_sparse) {
+    p.partial_f16 = (pair && shape->kv_dtype == SPLASH_KV_BF16) ? 1 : 0;
+    if (job_copy_pending && pair) {
         p.mig_src = static_cast<const uint4 *>(job->src_pool); p.mig_dst = static_cast<uint4 *>(job->dst_pool);
         p.mig_src_scales = reinterpret_cast<const uint4 *>(job->src_scales); p.mig_dst_scales = reinterpret_cast<uint4 *>(job->dst_scales);
         p.mig_src_ids = job->src_page_ids; p.mig_dst_ids = job->dst_page_ids;
@@ -340,14 +339,13 @@ int decode_dense(const splash_mla_shape *shape, const void *q, const void *kv_po
     // validation mode: the table entries the call will use, checked on the device before the decode kernel runs
     if (e == cudaSuccess && (shape->flags & SPLASH_FLAG_VALIDATE) && !sparse)
         e = launch_validate_pages(p, v.req_lo, v.req_hi, stream);
-    if (e == cudaSuccess && sparse && !fused_sparse)
+    if (e == cudaSuccess && sparse && simt)
         e = launch_sparse_gather(B, sparse->max_selected, sparse->pages_per_request, sparse->pool656, sparse->num_pool_pages,
                                  sparse->block_table, sparse->table_stride, sparse->ctx_lens, sparse->sel, sparse->sel_stride,
                                  sparse->sel_count, const_cast<void *>(kv_pool), sparse->dense_table, dev.sm_count,
-                                 plan_mode == kPlanWorkspace, stream);
+                                 stream);
     if (e == cudaSuccess) {
         if (simt) e = launch_decode_simt(p, shape->kv_dtype, stream);
-        else if (fused_sparse) e = launch_decode_sparse_pair(p, stream);
         else e = launch_decode_umma(p, *shape, stream);
     }
     if (e == cudaSuccess) e = record_timing_event(2, stream);
@@ -445,8 +443,7 @@ int splash_mla_decode_sparse(const splash_mla_shape *shape, const void *q, const
     st.table_stride = shape->block_table_stride; st.ctx_lens = seq_lens; st.sel = sel_tokens; st.sel_count = sel_count;
     st.sel_stride = sel_stride; st.max_selected = max_selected; st.pages_per_request = v.pages_per_request;
     st.dense_table = reinterpret_cast<int32_t *>(ws + v.off_table);
-    st.fused = (shape->flags & SPLASH_FLAG_SPARSE_FUSED) != 0 && (shape->flags & (SPLASH_FLAG_NO_PAIR | SPLASH_FLAG_SIMT)) == 0;
-    // plan (over the list counts) -> gather into the dense cache -> decode kernel over the dense cache -> combine
+    // plan (over the list counts) -> decode kernel, whose CTAs gather the rows of their own tiles -> combine
     return decode_dense(&v.dense, q, ws + v.off_pool, nullptr, st.dense_table, sel_count, head_begin, head_end, nullptr, nullptr,
                         out, lse, workspace, v.inner_bytes, stream_, &st);
 }

@@ -126,10 +126,11 @@ struct DecodeParams {
                                // each row scaled by a power of two so that its largest entry sits just below f16's maximum
                                // (exact, and no limit on the magnitude of the cache values)
     int32_t len_cap;           // >= 0: seq_lens holds list counts; one outside [0, len_cap] counts as 1 (sparse decode)
-    // fused sparse decode: kv_pool holds 656-byte rows, block_table / num_pool_pages describe it, and request i
+    // sparse decode: kv_pool holds 656-byte rows, block_table / num_pool_pages describe it, and request i
     // attends over the tokens sel[i * sel_stride + j], j < seq_lens[i], each below ctx_lens[i]
     const int32_t *sel, *ctx_lens;
     int64_t sel_stride;
+    int32_t sparse;
     int32_t num_workers;
     // optional page-copy job carried along by the CTA-pair kernels in warps that have nothing else to do (the issuer
     // warps of each pair's second CTA): page mig_src_ids[j] of mig_src -> page mig_dst_ids[j] of mig_dst, j < mig_n,
@@ -427,11 +428,10 @@ void count_launch(int n = 1);
 // kernels' host launchers
 cudaError_t launch_plan(const DecodeParams &p, const PlanView &v, cudaStream_t stream);
 cudaError_t launch_validate_pages(const DecodeParams &p, const int32_t *req_lo, const int32_t *req_hi, cudaStream_t stream);
-cudaError_t launch_decode_sparse_pair(const DecodeParams &p, cudaStream_t stream);
 cudaError_t launch_sparse_gather(int B, int max_sel, int pages_per_request, const void *kv_pool, int num_pool_pages,
                                  const int32_t *block_table, int64_t table_stride, const int32_t *seq_lens,
                                  const int32_t *sel, int64_t sel_stride, const int32_t *sel_count, void *dense_pool,
-                                 int32_t *dense_table, int sm_count, bool after_plan, cudaStream_t stream);
+                                 int32_t *dense_table, int sm_count, cudaStream_t stream);
 cudaError_t launch_dop_pack_rows(const void *a, const void *b, void *out, const int32_t *send_row, int64_t n, int h,
                                  int64_t a_bytes, int64_t b_bytes, int64_t a_row_pitch, int64_t a_head_pitch,
                                  int64_t b_row_pitch, int64_t b_head_pitch, cudaStream_t stream);

@@ -30,6 +30,7 @@
 // Every mbarrier wait is bounded by a wall-clock limit; on expiry the CTA records
 // SPLASH_DEVICE_TIMEOUT in the workspace status block, raises a CTA-wide abort flag,
 // lets copies in flight land, frees its tensor memory and returns.
+#include "splash_gather.cuh"
 #include "splash_pair.cuh"
 
 namespace splash {
@@ -39,7 +40,7 @@ namespace {
 using namespace umma;
 
 constexpr int kThreads = 224;                      // 7 warps: producer, 2 MMA issuers, 4 softmax
-constexpr int kWarpQk = 1, kWarpPv = 2, kWarpSoftmax = 3;
+constexpr int kWarpQk = 1, kWarpPv = 2, kWarpSoftmax = 3, kWarpGather = 7;    // (sparse decode: eight more warps, which write the stages)
 constexpr int kNumSoftmaxWarps = 4;                // barriers fed by the softmax role count one arrival per warp
 constexpr int kChunks = 9;                         // 576 / 64-element (128 B) chunks
 constexpr uint32_t kSlabBytes = 64 * 128;          // one chunk of one page: 64 tokens x 128 B
@@ -93,11 +94,12 @@ struct Layout {
 };
 
 // ---------------------------------------------------------------- the kernel
-template <int N>
-__global__ void __launch_bounds__(kThreads, 1)
+template <int N, bool kSparse>
+__global__ void __launch_bounds__(kThreads + (kSparse ? 32 * kGatherWarps : 0), 1)
 decode_umma_kernel(const __grid_constant__ DecodeParams p, const __grid_constant__ CUtensorMap tmap_kv,
                    const __grid_constant__ CUtensorMap tmap_q) {
     using L = Layout<N>;
+    constexpr int kNumThreads = kThreads + (kSparse ? 32 * kGatherWarps : 0);
     extern __shared__ __align__(1024) uint8_t smem[];
     const uint32_t sbase = smem_u32(smem);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -115,7 +117,7 @@ decode_umma_kernel(const __grid_constant__ DecodeParams p, const __grid_constant
         return;
     }
     if (tid == 0) {
-        for (int s = 0; s < kStages; ++s) { mbar_init(bar(kBarKvFull + s), 1); mbar_init(bar(kBarKvEmpty + s), 1); }
+        for (int s = 0; s < kStages; ++s) { mbar_init(bar(kBarKvFull + s), kSparse ? kGatherWarps : 1); mbar_init(bar(kBarKvEmpty + s), 1); }
         mbar_init(bar(kBarQFull), 1); mbar_init(bar(kBarQEmpty), 1);
         for (int b = 0; b < 2; ++b) { mbar_init(bar(kBarSFull + b), 1); mbar_init(bar(kBarSEmpty + b), kNumSoftmaxWarps); }
         mbar_init(bar(kBarPFull), kNumSoftmaxWarps);
@@ -135,7 +137,7 @@ decode_umma_kernel(const __grid_constant__ DecodeParams p, const __grid_constant
     const long long t_start = clock64();
 
     SegmentIter<L::kOffPlan> it;
-    start_plan(p, worker, kThreads / 32 - 1, it);
+    start_plan(p, worker, kWarpGather - 1, it);
     Segment seg;
     long long *const trace = blockIdx.x == 0 ? p.trace : nullptr;
     auto mark = [&](uint32_t tile, int ev) {
@@ -158,7 +160,7 @@ decode_umma_kernel(const __grid_constant__ DecodeParams p, const __grid_constant
             const int first_page = seg.lo / kPage;
             const int32_t *table = p.block_table + (int64_t)seg.request * p.table_stride;
             int entry = 0;
-            for (int tile = seg.tile_begin; ok && tile < seg.tile_end; ++tile) {
+            for (int tile = seg.tile_begin; !kSparse && ok && tile < seg.tile_end; ++tile) {
                 const int rel = tile - seg.tile_begin;
                 if ((rel & 31) == 0) {
                     int idx = tile + lane;
@@ -270,6 +272,18 @@ decode_umma_kernel(const __grid_constant__ DecodeParams p, const __grid_constant
             }
             ++seg_it;
         }
+    } else if (kSparse && warp >= kWarpGather) {
+        // ===================================================== sparse decode: rows into the stages, in place of the TMA producer
+        if constexpr (kSparse)
+            gather_tiles<kPage>(
+                p, it, warp - kWarpGather, lane, 0, [&](uint32_t t) { return smem + L::kOffKv + (t % kStages) * kStageBytes; },
+                [&](uint32_t t) { return mbar_wait(ctx, bar(kBarKvEmpty + t % kStages), ((t / kStages) & 1) ^ 1, kBarKvEmpty); },
+                [&](uint32_t t) {
+                    fence_proxy_async();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar(kBarKvFull + t % kStages));
+                },
+                [](uint32_t) { return true; }, [](uint32_t) {});
     } else {
         // ===================================================== softmax + epilogue warps
         const int q4 = warp & 3;                       // TMEM lane quadrant of this warp
@@ -596,7 +610,7 @@ decode_umma_kernel(const __grid_constant__ DecodeParams p, const __grid_constant
         }
     }
 
-    fill_empty_requests(p, it.tile_start(p), worker, head0, N, tid, kThreads);
+    fill_empty_requests(p, it.tile_start(p), worker, head0, N, tid, kNumThreads);
     if (p.trace != nullptr && tid == 0) p.trace[512 + blockIdx.x] = clock64() - t_start;   // per-CTA cycles
 
     // ---- teardown
@@ -614,14 +628,14 @@ decode_umma_kernel(const __grid_constant__ DecodeParams p, const __grid_constant
 }
 
 // ---------------------------------------------------------------- host side
-template <int N>
+template <int N, bool kSparse>
 cudaError_t launch_n(const DecodeParams &p, const CUtensorMap &mkv, const CUtensorMap &mq, cudaStream_t stream) {
     const int smem = (int)Layout<N>::kBytes;
     static DeviceOnce once;
-    cudaError_t e = once.run([&] { return cudaFuncSetAttribute(decode_umma_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); });
+    cudaError_t e = once.run([&] { return cudaFuncSetAttribute(decode_umma_kernel<N, kSparse>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); });
     if (e != cudaSuccess) return e;
-    e = launch_dependent(decode_umma_kernel<N>, dim3((unsigned)(p.num_workers * p.num_groups)), dim3(kThreads), (size_t)smem,
-                         stream, p, mkv, mq);
+    e = launch_dependent(decode_umma_kernel<N, kSparse>, dim3((unsigned)(p.num_workers * p.num_groups)),
+                         dim3(kThreads + (kSparse ? 32 * kGatherWarps : 0)), (size_t)smem, stream, p, mkv, mq);
     count_launch();
     return e;
 }
@@ -650,7 +664,8 @@ cudaError_t launch_decode_umma(const DecodeParams &p, const splash_mla_shape &sh
     if (p.num_groups == 2 && p.heads_per_group == 64 && !(shape.flags & SPLASH_FLAG_NO_PAIR)) return launch_decode_umma_pair(p, stream);
     alignas(64) CUtensorMap mkv, mq;
     const int n = p.heads_per_group;
-    if (!make_map_4d(&mkv, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, CU_TENSOR_MAP_SWIZZLE_128B, p.kv_pool, kPage,
+    // (the rows of a sparse call do not come by TMA)
+    if (!p.sparse && !make_map_4d(&mkv, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, CU_TENSOR_MAP_SWIZZLE_128B, p.kv_pool, kPage,
                      (uint64_t)(p.num_pool_pages > 0 ? p.num_pool_pages : 1), (uint64_t)kDQK * 2, 128,
                      (uint64_t)kPage * kDQK * 2, 64))
         return cudaErrorInvalidValue;
@@ -658,10 +673,11 @@ cudaError_t launch_decode_umma(const DecodeParams &p, const splash_mla_shape &sh
                      (uint64_t)p.B, (uint64_t)p.q_stride_head * 2, 128,
                      (uint64_t)(p.B > 1 ? p.q_stride_request : p.q_stride_head * p.H) * 2, (uint32_t)n))
         return cudaErrorInvalidValue;
+    if (p.sparse) mkv = mq;
     switch (n) {
-        case 16: return launch_n<16>(p, mkv, mq, stream);
-        case 32: return launch_n<32>(p, mkv, mq, stream);
-        case 64: return launch_n<64>(p, mkv, mq, stream);
+        case 16: return p.sparse ? launch_n<16, true>(p, mkv, mq, stream) : launch_n<16, false>(p, mkv, mq, stream);
+        case 32: return p.sparse ? launch_n<32, true>(p, mkv, mq, stream) : launch_n<32, false>(p, mkv, mq, stream);
+        case 64: return p.sparse ? launch_n<64, true>(p, mkv, mq, stream) : launch_n<64, false>(p, mkv, mq, stream);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -32,6 +32,7 @@
 // of the peer complete on them too.
 #include <cuda_fp16.h>
 
+#include "splash_gather.cuh"
 #include "splash_pair.cuh"
 
 namespace splash {
@@ -46,7 +47,7 @@ constexpr int kWarpQk = 1;
 constexpr int kWarpPv = 2;
 constexpr int kWarpSoftmax = kWarpQk + kIssuerWarps;   // TMEM quadrant = warp & 3
 constexpr int kWarpVProducer = kWarpSoftmax + kSoftmaxWarps;
-constexpr int kThreads = (kWarpVProducer + 1) * 32;    // 12 warps = 384 threads
+constexpr int kThreads = (kWarpVProducer + 1) * 32;    // 12 warps = 384 threads; sparse decode: 8 more, which write the stages
 constexpr int kN = 64;                              // heads per CTA
 constexpr int kHalf = 32;                           // tokens per CTA and tile
 constexpr uint32_t kSlab = kHalf * 128;             // one chunk of a half-page: 32 tokens x 128 B
@@ -101,9 +102,11 @@ __device__ __forceinline__ void umma_bf16_pair(uint32_t elected, uint32_t d_tmem
         ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(elected) : "memory");
 }
 
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
+template <bool kSparse>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads + (kSparse ? 32 * kGatherWarps : 0), 1)
 decode_umma_pair_kernel(const __grid_constant__ DecodeParams p, const __grid_constant__ CUtensorMap tmap_half,
                         const __grid_constant__ CUtensorMap tmap_peer, const __grid_constant__ CUtensorMap tmap_q) {
+    constexpr int kNumThreads = kThreads + (kSparse ? 32 * kGatherWarps : 0);
     extern __shared__ __align__(1024) uint8_t smem[];
     const uint32_t sbase = smem_u32(smem);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -126,8 +129,9 @@ decode_umma_pair_kernel(const __grid_constant__ DecodeParams p, const __grid_con
     if (tid == 0) {
         // barriers the leader's issuers wait on count the warps of both CTAs (the peer's copies are unused)
         for (int s = 0; s < kStages; ++s) {
-            mbar_init(bar(kBarKFull + s), 1); mbar_init(bar(kBarQkDone + s), 1);
-            mbar_init(bar(kBarVFull + s), 1); mbar_init(bar(kBarStageEmpty + s), 1);
+            constexpr int kFilled = kSparse ? 2 * kGatherWarps : 1;       // by the gathering warps of both CTAs, or by bytes
+            mbar_init(bar(kBarKFull + s), kFilled); mbar_init(bar(kBarQkDone + s), 1);
+            mbar_init(bar(kBarVFull + s), kFilled); mbar_init(bar(kBarStageEmpty + s), 1);
         }
         mbar_init(bar(kBarQFull), 1); mbar_init(bar(kBarQEmpty), 1);
         for (int b = 0; b < 2; ++b) {
@@ -152,7 +156,7 @@ decode_umma_pair_kernel(const __grid_constant__ DecodeParams p, const __grid_con
     const unsigned long long ns_start = global_timer_ns();
 
     SegmentIter<kOffPlan> it;
-    start_plan(p, worker, kThreads / 32 - 1, it);
+    start_plan(p, worker, kWarpVProducer, it);
     Segment seg;
     seg.lo = seg.hi = seg.tile_begin = seg.tile_end = 0;
 
@@ -175,7 +179,7 @@ decode_umma_pair_kernel(const __grid_constant__ DecodeParams p, const __grid_con
             ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
             const int first_page = seg.lo / kPage;
             const int32_t *table = p.block_table + (int64_t)seg.request * p.table_stride;
-            for (int tile = seg.tile_begin; ok && tile < seg.tile_end; ++tile, ++kv_it) {
+            for (int tile = seg.tile_begin; !kSparse && ok && tile < seg.tile_end; ++tile, ++kv_it) {
                 const TileGeom g = tile_geom(seg.lo, seg.hi, (first_page + tile) * kPage);
                 const uint32_t stage = kv_it % kStages, ph = (kv_it / kStages) & 1;
                 const uint32_t k0 = sbase + kOffK + stage * kStageBytes;
@@ -308,6 +312,23 @@ decode_umma_pair_kernel(const __grid_constant__ DecodeParams p, const __grid_con
         // job, if it has one (a layer's pages on the move while this layer decodes)
         if (p.mig_n > 0)
             copy_pages_in_idle_warp(p, pair_id * kIssuerWarps + (warp - kWarpQk), p.num_workers * p.pair_groups * kIssuerWarps, lane);
+    } else if (kSparse && warp > kWarpVProducer) {
+        // ===================================================== sparse decode: rows into the stages, in place of the TMA producers
+        if constexpr (kSparse)
+            gather_tiles<kHalf>(
+                p, it, warp - kWarpVProducer - 1, lane, (int)rank, [&](uint32_t t) { return smem + kOffK + (t % kStages) * kStageBytes; },
+                [&](uint32_t t) { return mbar_wait(ctx, bar(kBarStageEmpty + t % kStages), ((t / kStages) & 1) ^ 1, kBarStageEmpty); },
+                [&](uint32_t t) {
+                    fence_proxy_async();
+                    __syncwarp();
+                    if (lane == 0) arrive_on_leader(kBarKFull + t % kStages);
+                },
+                [&](uint32_t t) { return mbar_wait(ctx, bar(kBarQkDone + t % kStages), (t / kStages) & 1, kBarQkDone); },
+                [&](uint32_t t) {
+                    fence_proxy_async();
+                    __syncwarp();
+                    if (lane == 0) arrive_on_leader(kBarVFull + t % kStages);
+                });
     } else {
         // ===================================================== softmax + epilogue warps
         // S layout per CTA: TMEM lane L < 64 = head L, tokens of half-page 0 in 32 columns;
@@ -547,7 +568,7 @@ decode_umma_pair_kernel(const __grid_constant__ DecodeParams p, const __grid_con
         }
     }
 
-    fill_empty_requests(p, it.tile_start(p), worker, head0, kN, tid, kThreads);
+    fill_empty_requests(p, it.tile_start(p), worker, head0, kN, tid, kNumThreads);
     if (p.trace != nullptr && tid == 0) {   // per-CTA cycles and nanoseconds
         p.trace[512 + blockIdx.x] = clock64() - t_start;
         if (blockIdx.x < 256) p.trace[768 + blockIdx.x] = (long long)(global_timer_ns() - ns_start);
@@ -572,27 +593,28 @@ decode_umma_pair_kernel(const __grid_constant__ DecodeParams p, const __grid_con
 cudaError_t launch_decode_umma_pair(const DecodeParams &p, cudaStream_t stream) {
     alignas(64) CUtensorMap mhalf, mpeer, mq;
     const uint64_t pages = (uint64_t)(p.num_pool_pages > 0 ? p.num_pool_pages : 1);
-    if (!make_map_4d(&mhalf, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, CU_TENSOR_MAP_SWIZZLE_128B, p.kv_pool, kPage, pages,
-                     (uint64_t)kDQK * 2, 128, (uint64_t)kPage * kDQK * 2, kHalf, 9))
+    // (the rows of a sparse call do not come by TMA)
+    if (!p.sparse && !make_map_4d(&mhalf, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, CU_TENSOR_MAP_SWIZZLE_128B, p.kv_pool, kPage, pages,
+                                  (uint64_t)kDQK * 2, 128, (uint64_t)kPage * kDQK * 2, kHalf, 9))
         return cudaErrorInvalidValue;
-    if (!make_map_4d(&mpeer, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, CU_TENSOR_MAP_SWIZZLE_128B, p.kv_pool, kPage, pages,
-                     (uint64_t)kDQK * 2, 128, (uint64_t)kPage * kDQK * 2, kHalf, 2))
+    if (!p.sparse && !make_map_4d(&mpeer, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, CU_TENSOR_MAP_SWIZZLE_128B, p.kv_pool, kPage, pages,
+                                  (uint64_t)kDQK * 2, 128, (uint64_t)kPage * kDQK * 2, kHalf, 2))
         return cudaErrorInvalidValue;
     if (!make_map_4d(&mq, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, CU_TENSOR_MAP_SWIZZLE_128B, p.q, (uint64_t)p.H,
                      (uint64_t)p.B, (uint64_t)p.q_stride_head * 2, 128,
                      (uint64_t)(p.B > 1 ? p.q_stride_request : p.q_stride_head * p.H) * 2, (uint32_t)kN, 9))
         return cudaErrorInvalidValue;
+    if (p.sparse) mhalf = mpeer = mq;
     static DeviceOnce once;
-    cudaError_t e = once.run([&] { return cudaFuncSetAttribute(decode_umma_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes); });
+    cudaError_t e = once.run([&] {
+        const cudaError_t e0 = cudaFuncSetAttribute(decode_umma_pair_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
+        if (e0 != cudaSuccess) return e0;
+        return cudaFuncSetAttribute(decode_umma_pair_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
+    });
     if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(p.num_workers * p.pair_groups * 2)); cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = kSmemBytes; cfg.stream = stream;
-    cudaLaunchAttribute attr[1];      // (the cluster shape is part of the kernel's declaration)
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, decode_umma_pair_kernel, p, mhalf, mpeer, mq);
+    // (the cluster shape is part of the kernel's declaration)
+    e = launch_dependent(p.sparse ? decode_umma_pair_kernel<true> : decode_umma_pair_kernel<false>, dim3((unsigned)(p.num_workers * p.pair_groups * 2)),
+                         dim3(kThreads + (p.sparse ? 32 * kGatherWarps : 0)), (size_t)kSmemBytes, stream, p, mhalf, mpeer, mq);
     count_launch();
     return e;
 }
