@@ -349,7 +349,7 @@ int decode_dense(const splash_mla_shape *shape, const void *q, const void *kv_po
         else e = launch_decode_umma(p, *shape, stream);
     }
     if (e == cudaSuccess) e = record_timing_event(2, stream);
-    if (e == cudaSuccess && plan_mode != kPlanWhole) e = launch_split_combine(p, v.split_rec, stream);
+    if (e == cudaSuccess && plan_mode != kPlanWhole) e = launch_split_combine(p, v.split_rec, dev.sm_count, stream);
     if (e == cudaSuccess) e = record_timing_event(3, stream);
     if (e == cudaSuccess && g_timing) g_events_recorded = true;
     if (e == cudaSuccess && job_copy_pending) e = run_migrate_job(job, false, true, stream);

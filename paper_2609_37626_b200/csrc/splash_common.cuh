@@ -181,8 +181,8 @@ constexpr uint32_t kInlinePlanBytes = ((3 * kInlinePlanRequests + 4) * 4 + 15) /
 // Effective range of request i (the rule of the plan kernel).
 __device__ __forceinline__ void effective_range(int s, const int32_t *kv_begin, const int32_t *kv_end, int i, int len_cap, int &lo, int &hi) {
     if (len_cap >= 0 && (s < 0 || s > len_cap)) s = 1;     // a list count out of bounds: one (poisoned) row
-    lo = kv_begin ? kv_begin[i] : 0;
-    hi = kv_end ? kv_end[i] : s;
+    lo = kv_begin ? __ldcg(kv_begin + i) : 0;
+    hi = kv_end ? __ldcg(kv_end + i) : s;
     if (lo < 0) lo = 0;
     if (hi > s) hi = s;
     if (hi < lo) hi = lo;
@@ -194,11 +194,15 @@ __device__ __forceinline__ int cost_target(int total, int w, int W) {
     return a * w + (b * w) / W;
 }
 
-// One warp of a CTA: the plan, as far as worker `worker` needs it.
-static __device__ __noinline__ void build_inline_plan(const DecodeParams &p, int worker, int32_t *sp, int lane) {
+// The lengths of a batch of at most 32 requests, a request per lane: its effective range.
+__device__ __forceinline__ void lane_range(const DecodeParams &p, int lane, int &lo, int &hi) {
+    lo = hi = 0;
+    if (lane < p.B) effective_range(__ldcg(p.seq_lens + lane), p.kv_begin, p.kv_end, lane, p.len_cap, lo, hi);
+}
+
+// One warp of a CTA: the plan, as far as worker `worker` needs it, from the lanes' ranges.
+static __device__ __noinline__ void build_inline_plan(const DecodeParams &p, int worker, int32_t *sp, int lane, int lo, int hi) {
     const int B = p.B, W = p.num_workers, overhead = p.request_overhead_tiles;
-    int lo = 0, hi = 0;
-    if (lane < B) effective_range(p.seq_lens[lane], p.kv_begin, p.kv_end, lane, p.len_cap, lo, hi);
     const int n = hi > lo ? (hi + kPage - 1) / kPage - lo / kPage : 0;
     const int c = n > 0 ? n + overhead : 0;
     int sn = n, sc = c;
@@ -227,6 +231,42 @@ static __device__ __noinline__ void build_inline_plan(const DecodeParams &p, int
     int req, unused;
     const int wb = start(worker, req), we = start(worker + 1, unused);
     if (lane == 0) { sp[3 * B + 1] = wb; sp[3 * B + 2] = we; sp[3 * B + 3] = req; }
+}
+
+// What of the cache a CTA loads first: `bytes` at `offset` of the pages of the worker's first `count` tiles; and its heads.
+struct FirstLoads { uint32_t page_bytes, offset, bytes; int count, head0, heads; };
+
+// Before grid_dependency_wait, the same warp: the plan from the lengths as they lie there now, and from it the worker's first
+// pages, their scales and its first request's query rows into L2, while the work before this call on the stream still
+// runs (in a loop over layers the combine kernel of the one before: microseconds in which DRAM is idle).  Nothing of this is
+// relied on: the lengths are read again after the wait, and the plan made again if they differ; what is prefetched is
+// only that.  All reads go to L2 (a line in L1 would be stale after the wait).
+static __device__ __noinline__ void plan_ahead(const DecodeParams &p, int worker, int32_t *sp, int lane, const FirstLoads &f, int &lo, int &hi) {
+    lane_range(p, lane, lo, hi);
+    build_inline_plan(p, worker, sp, lane, lo, hi);
+    __syncwarp();
+    const int B = p.B, wb = sp[3 * B + 1], we = sp[3 * B + 2], req = sp[3 * B + 3];
+    if (wb < 0 || wb >= we || req < 0 || req >= B) return;
+    const int x = wb + lane;
+    if (!p.sparse && lane < f.count && x < we) {
+        int r = req;
+        while (r + 1 < B && sp[r + 1] <= x) ++r;
+        const int64_t idx = (int64_t)sp[B + 1 + r] / kPage + (x - sp[r]);
+        if (idx >= 0 && idx < p.table_stride) {
+            const int page = __ldcg(p.block_table + (int64_t)r * p.table_stride + idx);
+            if (page >= 0 && page < p.num_pool_pages) {
+                asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;"
+                             ::"l"(static_cast<const uint8_t *>(p.kv_pool) + (size_t)page * f.page_bytes + f.offset), "r"(f.bytes) : "memory");
+                if (p.kv_scales != nullptr) {
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(p.kv_scales + (size_t)page * kPage));
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(p.kv_scales + (size_t)page * kPage + 32));
+                }
+            }
+        }
+    }
+    const char *q = static_cast<const char *>(p.q) + ((int64_t)req * p.q_stride_request + (int64_t)f.head0 * p.q_stride_head) * 2;
+    const int rows = min(f.heads, p.head_end - f.head0);
+    for (int i = lane; i < rows * 9; i += 32) asm volatile("prefetch.global.L2 [%0];" ::"l"(q + (int64_t)(i / 9) * p.q_stride_head * 2 + (i % 9) * 128));
 }
 
 // The same warp of block 0, once its CTA is under way: clears the status block (this cannot wipe another CTA's report: the
@@ -341,23 +381,34 @@ struct SegmentIter<kPlanInWorkspace> {
     }
 };
 
-// The beginning of a decode kernel, all threads: the plan's origin by the call's mode.  `plan_warp`: a warp that is not
-// needed at once.
-template <uint32_t kPlanOffset>
-__device__ __forceinline__ void start_plan(const DecodeParams &p, int worker, int plan_warp, SegmentIter<kPlanOffset> &it) {
+// The beginning of a decode kernel, all threads, around its grid_dependency_wait: the plan's origin by the call's mode.
+// `plan_warp`: a warp that is not needed at once.  kAhead: the kernel leaves a combine block room beside its CTA, so its CTAs are
+// there well before the wait ends and may plan ahead; where they come in only as the blocks before them leave, planning twice
+// is time lost (1 us of a call).  A call that cuts no request has no combine kernel in front of the next one: always ahead.
+template <bool kAhead, uint32_t kPlanOffset>
+__device__ __forceinline__ void start_plan(const DecodeParams &p, int worker, int plan_warp, SegmentIter<kPlanOffset> &it, const FirstLoads &f) {
     if constexpr (kPlanOffset != kPlanInWorkspace) {
         if (p.plan_mode != kPlanWorkspace) {
             const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
             int32_t *sp = it.inline_plan();
+            int lo = 0, hi = 0;
+            const bool ahead = kAhead || p.plan_mode == kPlanWhole;
+            if (ahead && warp == plan_warp) plan_ahead(p, worker, sp, lane, f, lo, hi);
+            grid_dependency_wait();
             // no combine kernel follows and every CTA is running: the next call's first kernel may set up on the SMs left
             if (p.plan_mode == kPlanWhole) grid_launch_dependents();
-            if (warp == plan_warp) build_inline_plan(p, worker, sp, lane);
+            if (warp == plan_warp) {
+                int lo2, hi2;
+                lane_range(p, lane, lo2, hi2);
+                if (!ahead || __any_sync(0xffffffffu, lo2 != lo || hi2 != hi)) build_inline_plan(p, worker, sp, lane, lo2, hi2);
+            }
             __syncthreads();
             if (blockIdx.x == 0 && warp == plan_warp) publish_inline_plan(p, sp, lane);
             it.init(p, worker);
             return;
         }
     }
+    grid_dependency_wait();       // the plan kernel's output is read from here on
     if (p.clear_status && blockIdx.x == 0 && threadIdx.x < 8) p.status[threadIdx.x] = 0;      // (see publish_inline_plan)
     it.init(p, worker);
 }
@@ -447,7 +498,7 @@ cudaError_t launch_decode_umma_fp8(const DecodeParams &p, cudaStream_t stream);
 cudaError_t launch_decode_umma_fp8_narrow(const DecodeParams &p, cudaStream_t stream);   // 16 / 32 heads per CTA
 cudaError_t launch_decode_umma_fp8_pair(const DecodeParams &p, cudaStream_t stream);
 cudaError_t launch_decode_umma_pair(const DecodeParams &p, cudaStream_t stream);
-cudaError_t launch_split_combine(const DecodeParams &p, const int4 *split_rec, cudaStream_t stream);
+cudaError_t launch_split_combine(const DecodeParams &p, const int4 *split_rec, int sm_count, cudaStream_t stream);
 cudaError_t launch_lse_merge(int num_parts, int64_t rows, int d_v, const float *part_out,
                              const float *part_lse, float *out, float *lse, cudaStream_t stream);
 cudaError_t launch_page_migrate(const void *src_pool, const float *src_scales, void *dst_pool,

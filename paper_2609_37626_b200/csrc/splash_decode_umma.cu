@@ -69,9 +69,9 @@ struct Layout {
     static constexpr uint32_t kOffKv = 0;
     static constexpr uint32_t kOffQ = kOffKv + kStages * kStageBytes;
     static constexpr uint32_t kOffP = kOffQ + kQBytes;
-    // output staging for the narrow groups, [N heads][256 dv] floats: the finished tile leaves through the bulk-copy engine
+    // output staging for the narrow groups, [16 heads][512 dv] floats: the finished tile leaves through the bulk-copy engine
     // (64-head groups have no shared memory left for it and store from registers)
-    static constexpr uint32_t kOutBytes = N < 64 ? N * 1024 : 0;
+    static constexpr uint32_t kOutBytes = N < 64 ? 16 * kDV * 4 : 0;
     static constexpr uint32_t kOffOut = kOffP + kPBytes;
     static constexpr uint32_t kOffRed = kOffOut + kOutBytes; // float [N][4]
     static constexpr uint32_t kOffM = kOffRed + N * 16;      // float [N] running max, log2 domain
@@ -133,11 +133,10 @@ decode_umma_kernel(const __grid_constant__ DecodeParams p, const __grid_constant
     __syncthreads();
     tcgen05_fence_after();
     const uint32_t tmem_base = misc[0];
-    grid_dependency_wait();       // the plan kernel's output is read from here on
+    SegmentIter<L::kOffPlan> it;
+    start_plan<N < 64>(p, worker, kWarpGather - 1, it, FirstLoads{kStageBytes, 0u, kStageBytes, kStages + 1, head0, N});
     const long long t_start = clock64();
 
-    SegmentIter<L::kOffPlan> it;
-    start_plan(p, worker, kWarpGather - 1, it);
     Segment seg;
     long long *const trace = blockIdx.x == 0 ? p.trace : nullptr;
     auto mark = [&](uint32_t tile, int ev) {
@@ -537,6 +536,7 @@ decode_umma_kernel(const __grid_constant__ DecodeParams p, const __grid_constant
                     }
                 }
             }
+            if constexpr (N < 64) bulk_wait_group_read();      // the staging buffer's last rows have left
             softmax_bar_sync();
             // ---- epilogue: O^T block j holds dv = 128 j + TMEM lane, one column per head
             ok &= mbar_wait(ctx, bar(kBarOFull), seg_it & 1, kBarOFull);
@@ -551,42 +551,33 @@ decode_umma_kernel(const __grid_constant__ DecodeParams p, const __grid_constant
                 ostride = kDV;
             }
             const int nvalid = min(N, p.head_end - head0);
-            bool staged = false;
             if constexpr (N < 64) {
-                if (((reinterpret_cast<uintptr_t>(obase) | (uintptr_t)(ostride * 4)) & 15) == 0) {
-                    // Through shared memory and the bulk-copy engine: plain stores of this tile (one 128-byte line per
-                    // warp instruction, 64 of them per thread) take ~6,000 cycles while the cache streams, 2.5 times this.
-                    staged = true;
-                    float *stg = reinterpret_cast<float *>(smem + L::kOffOut);
+                // Through shared memory and the bulk-copy engine, sixteen heads at a time, four rows of 2 KB from each warp: plain
+                // stores of this tile (one 128-byte line per warp instruction, 64 of them per thread) take ~6,000 cycles while
+                // the cache streams.  The staging buffer is this epilogue's own: the copies are waited for before the next one.
+                float *stg = reinterpret_cast<float *>(smem + L::kOffOut);
 #pragma unroll 1
-                    for (int half = 0; half < 2; ++half) {
-#pragma unroll
-                        for (int jj = 0; jj < 2; ++jj) {
-                            const int j = 2 * half + jj;
-#pragma unroll
-                            for (int c = 0; c < N / 16; ++c) {
-                                float o[16];
-                                tmem_ld16(tmem_base + lane_addr + L::kColO + j * N + c * 16, o);
-                                tmem_wait_ld();
-#pragma unroll
-                                for (int k = 0; k < 16; ++k) {
-                                    const int n = c * 16 + k;
-                                    stg[n * 256 + jj * 128 + 32 * q4 + lane] = o[k] * l_s[n];
-                                }
-                            }
-                        }
-                        fence_proxy_async();
-                        softmax_bar_sync();
-                        if (st < nvalid) {
-                            bulk_store(obase + (int64_t)st * ostride + half * 256, smem_u32(stg + st * 256), 1024);
-                            bulk_commit_group();
-                            bulk_wait_group_read();          // the row has left shared memory
-                        }
+                for (int n0 = 0; n0 < N; n0 += 16) {
+                    if (n0 > 0) {
+                        bulk_wait_group_read();
                         softmax_bar_sync();
                     }
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        float o[16];
+                        tmem_ld16(tmem_base + lane_addr + L::kColO + j * N + n0, o);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int k = 0; k < 16; ++k) stg[k * kDV + 128 * j + 32 * q4 + lane] = o[k] * l_s[n0 + k];
+                    }
+                    fence_proxy_async();
+                    softmax_bar_sync();
+                    if (lane < 4 && n0 + 4 * sw + lane < nvalid) {
+                        bulk_store(obase + (int64_t)(n0 + 4 * sw + lane) * ostride, smem_u32(stg + (4 * sw + lane) * kDV), kDV * 4);
+                        bulk_commit_group();
+                    }
                 }
-            }
-            if (!staged) {
+            } else {
 #pragma unroll 1
                 for (int j = 0; j < 4; ++j) {
                     const int dv = 128 * j + 32 * q4 + lane;
@@ -608,6 +599,7 @@ decode_umma_kernel(const __grid_constant__ DecodeParams p, const __grid_constant
             if (lane == 0) mbar_arrive(bar(kBarOEmpty));
             ++seg_it;
         }
+        if constexpr (N < 64) bulk_wait_group_read();          // (nor may the CTA leave before)
     }
 
     fill_empty_requests(p, it.tile_start(p), worker, head0, N, tid, kNumThreads);

@@ -115,11 +115,10 @@ decode_umma_fp8_kernel(const __grid_constant__ DecodeParams p, const __grid_cons
     __syncthreads();
     tcgen05_fence_after();
     const uint32_t tmem_base = misc[0];
-    grid_dependency_wait();       // the plan kernel's output is read from here on
+    SegmentIter<kOffPlan> it;
+    start_plan<false>(p, worker, kThreads / 32 - 1, it, FirstLoads{kStageBytes, 0u, kStageBytes, kStages, head0, kN});
     const long long t_start = clock64();
 
-    SegmentIter<kOffPlan> it;
-    start_plan(p, worker, kThreads / 32 - 1, it);
     Segment seg;
     long long *const trace = blockIdx.x == 0 ? p.trace : nullptr;
     auto mark = [&](uint32_t tile, int ev) {

@@ -103,7 +103,7 @@ struct Layout {
 
 // ---------------------------------------------------------------- the kernel
 template <int N>
-__global__ void __launch_bounds__(Layout<N>::kThreads, 1)
+__global__ void __launch_bounds__(512, 1)      // (at most 128 registers: a combine block fits beside a CTA of 16 heads)
 decode_umma_fp8_narrow_kernel(const __grid_constant__ DecodeParams p, const __grid_constant__ CUtensorMap tmap_kv) {
     using L = Layout<N>;
     constexpr int kStages = L::kStages, kThreads = L::kThreads, kNumSoftmaxWarps = L::kSoftmaxWarps, kWarpConvert = L::kWarpConvert;
@@ -141,11 +141,10 @@ decode_umma_fp8_narrow_kernel(const __grid_constant__ DecodeParams p, const __gr
     __syncthreads();
     tcgen05_fence_after();
     const uint32_t tmem_base = misc[0];
-    grid_dependency_wait();       // the plan kernel's output is read from here on
+    SegmentIter<L::kOffPlan> it;
+    start_plan<N == 16>(p, worker, kThreads / 32 - 1, it, FirstLoads{kStageBytes, 0u, kStageBytes, kStages, head0, N});
     const long long t_start = clock64();
 
-    SegmentIter<L::kOffPlan> it;
-    start_plan(p, worker, kThreads / 32 - 1, it);
     Segment seg;
     long long *const trace = blockIdx.x == 0 ? p.trace : nullptr;
     auto mark = [&](uint32_t tile, int ev) {
@@ -169,7 +168,7 @@ decode_umma_fp8_narrow_kernel(const __grid_constant__ DecodeParams p, const __gr
                 const int page = __shfl_sync(0xffffffffu, entry, rel & 31);
                 // the next page (when its table entry is among the 32 this warp holds): pulled into L2 now
                 const int page_ahead = __shfl_sync(0xffffffffu, entry, (rel + 1) & 31);
-                const bool ahead_ok = (rel & 31) + 1 < 32 && tile + 1 < seg.tile_end;
+                const bool ahead_ok = (kv_it + 1 >= kStages || p.plan_mode == kPlanWorkspace) && (rel & 31) + 1 < 32 && tile + 1 < seg.tile_end;     // (else its load goes out at once, and plan_ahead has asked for it)
                 const TileGeom g = tile_geom(seg.lo, seg.hi, (first_page + tile) * kPage);
                 const uint32_t stage = kv_it % kStages, ph = (kv_it / kStages) & 1;
                 // a page id outside the pool reads as zeros through the tensor map; its tokens get the scale 1
@@ -563,56 +562,44 @@ decode_umma_fp8_narrow_kernel(const __grid_constant__ DecodeParams p, const __gr
                 ostride = kDV;
             }
             const int nvalid = min(N, p.head_end - head0);
-            if (((reinterpret_cast<uintptr_t>(obase) | (uintptr_t)(ostride * 4)) & 15) == 0) {
+            {
                 // Through shared memory and the bulk-copy engine: plain stores of this tile (one 128-byte line per warp
-                // instruction, 64 of them per thread) take ~6,000 cycles while the cache streams, 2.5 times this.  The
-                // finished request's query operands are dead by now and serve as the staging buffer, [N heads][256 dv]
-                // floats, filled and drained twice.
+                // instruction, 64 of them per thread) take ~6,000 cycles while the cache streams.  The finished request's query
+                // operands are dead by now and serve as the staging buffer, [N / 2 heads][512 dv] floats, filled and
+                // drained twice; a warp sends two rows of 2 KB (a bulk copy costs its warp about 90 cycles: sixteen of 1 KB per
+                // half, all from one warp, made this epilogue 800 cycles longer: 4,800).
                 float *stg = reinterpret_cast<float *>(smem + L::kOffQ + (seg_it & 1) * L::kQBytes);
-                static_assert(N * 256 * 4 <= (int)L::kQBytes, "the staging tile must fit a query operand buffer");
+                static_assert(N / 2 * kDV * 4 <= (int)L::kQBytes, "the staging tile must fit a query operand buffer");
+                static_assert(N / 2 == 2 * L::kSoftmaxWarps, "two rows per warp and half");
 #pragma unroll 1
                 for (int half = 0; half < 2; ++half) {
+                    const int row = 8 * (sw >> 2), n0 = half * (N / 2) + row;       // this warp's eight heads
 #pragma unroll
-                    for (int jj = 0; jj < 2; ++jj) {
-                        const int j = 2 * half + jj;
-                        {
-                            const int c = sw >> 2;        // this warp's 16 heads of the block
-                            float o[16], o_lo[16];
-                            tmem_ld16(tmem_base + lane_addr + L::kColO + j * (2 * N) + c * 16, o);
-                            tmem_ld16(tmem_base + lane_addr + L::kColO + j * (2 * N) + N + c * 16, o_lo);
-                            tmem_wait_ld();
+                    for (int j = 0; j < 4; j += 2) {
+                        float o[2][8], o_lo[2][8];
 #pragma unroll
-                            for (int k = 0; k < 16; ++k) {
-                                const int n = c * 16 + k;
-                                stg[n * 256 + jj * 128 + 32 * q4 + lane] = fmaf(o_lo[k], 0.0625f, o[k]) * l_s[n];
-                            }
+                        for (int jj = 0; jj < 2; ++jj) {
+                            tmem_ld8(tmem_base + lane_addr + L::kColO + (j + jj) * (2 * N) + n0, o[jj]);
+                            tmem_ld8(tmem_base + lane_addr + L::kColO + (j + jj) * (2 * N) + N + n0, o_lo[jj]);
                         }
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int jj = 0; jj < 2; ++jj)
+#pragma unroll
+                            for (int k = 0; k < 8; ++k)
+                                stg[(row + k) * kDV + 128 * (j + jj) + 32 * q4 + lane] = fmaf(o_lo[jj][k], 0.0625f, o[jj][k]) * l_s[n0 + k];
                     }
                     fence_proxy_async();
                     named_bar_sync<1, kSoftmaxThreads>();
-                    if (st < nvalid) {
-                        bulk_store(obase + (int64_t)st * ostride + half * 256, smem_u32(stg + st * 256), 1024);
-                        bulk_commit_group();
-                        bulk_wait_group_read();          // the row has left shared memory
-                    }
-                    named_bar_sync<1, kSoftmaxThreads>();
-                }
-            } else {
-#pragma unroll 1
-                for (int j = 0; j < 4; ++j) {
-                    const int dv = 128 * j + 32 * q4 + lane;
-                    {
-                        const int c = sw >> 2;
-                        float o[16], o_lo[16];
-                        tmem_ld16(tmem_base + lane_addr + L::kColO + j * (2 * N) + c * 16, o);
-                        tmem_ld16(tmem_base + lane_addr + L::kColO + j * (2 * N) + N + c * 16, o_lo);
-                        tmem_wait_ld();
-#pragma unroll
-                        for (int k = 0; k < 16; ++k) {
-                            const int n = c * 16 + k;
-                            if (n < nvalid) obase[(int64_t)n * ostride + dv] = fmaf(o_lo[k], 0.0625f, o[k]) * l_s[n];
+                    if (lane < 2) {
+                        const int r = 2 * sw + lane, n = half * (N / 2) + r;
+                        if (n < nvalid) {
+                            bulk_store(obase + (int64_t)n * ostride, smem_u32(stg + r * kDV), kDV * 4);
+                            bulk_commit_group();
+                            bulk_wait_group_read();          // the row has left shared memory
                         }
                     }
+                    named_bar_sync<1, kSoftmaxThreads>();
                 }
             }
             tcgen05_fence_before();

@@ -172,12 +172,11 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
     cluster_sync_all();                                   // barriers of both CTAs exist before anyone signals them
     tcgen05_fence_after();
     const uint32_t tmem_base = misc[0];
-    grid_dependency_wait();                               // the plan kernel's output is read from here on
+    SegmentIter<kInline ? L::kOffPlan : kPlanInWorkspace> it;
+    start_plan<false>(p, worker, kThreads / 32 - 1, it, FirstLoads{kPageBytes, 0u, kPageBytes, kStages, head0, H});
     const long long t_start = clock64();
     const unsigned long long ns_start = global_timer_ns();
 
-    SegmentIter<kInline ? L::kOffPlan : kPlanInWorkspace> it;
-    start_plan(p, worker, kThreads / 32 - 1, it);
     Segment seg;
     seg.lo = seg.hi = seg.tile_begin = seg.tile_end = 0;
     // geometry of supertile s of the current segment: page tiles 2s (page A, CTA 0) and 2s + 1 (page B, CTA 1)

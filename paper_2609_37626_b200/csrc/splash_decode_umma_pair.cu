@@ -151,12 +151,11 @@ decode_umma_pair_kernel(const __grid_constant__ DecodeParams p, const __grid_con
     cluster_sync_all();                                   // barriers of both CTAs exist before anyone signals them
     tcgen05_fence_after();
     const uint32_t tmem_base = misc[0];
-    grid_dependency_wait();                               // the plan kernel's output is read from here on
+    SegmentIter<kOffPlan> it;
+    start_plan<false>(p, worker, kWarpVProducer, it, FirstLoads{2 * kStageBytes, rank * kStageBytes, kStageBytes, kStages, head0, kN});
     const long long t_start = clock64();
     const unsigned long long ns_start = global_timer_ns();
 
-    SegmentIter<kOffPlan> it;
-    start_plan(p, worker, kWarpVProducer, it);
     Segment seg;
     seg.lo = seg.hi = seg.tile_begin = seg.tile_end = 0;
 

@@ -182,6 +182,116 @@ split_combine_kernel(const DecodeParams p, const int4 *__restrict__ split_rec) {
     if (c == 0) *lse = L;
 }
 
+// The same for launches of no more rows than SMs (a small batch): four groups of 128 threads take every fourth piece and add
+// their sums in shared memory.  2 KB of that and 32 registers, so that a block fits beside a decode CTA of 16 heads:
+// the next call's CTAs come in, plan and prefetch while this kernel runs (eight layers of 8 requests: with the kernel above, 6 KB
+// a block, they came in 1.6 to 4.4 us later, one by one as its blocks left).
+constexpr int kGroupedParts = 160, kCombineGroups = 4;
+template <bool kF16>
+__global__ void __launch_bounds__(kCombineGroups * kMergeThreads, 4)
+grouped_combine_kernel(const DecodeParams p, const int4 *__restrict__ split_rec) {
+    constexpr int kThreads = kCombineGroups * kMergeThreads, kDepth = 4;
+    // weights, slots and (f16 pieces) the power of two each row was divided by; then the groups' sums
+    constexpr int kFloats = (kF16 ? 3 : 2) * kGroupedParts;
+    __shared__ __align__(16) float smem_f[kFloats > 4 * kMergeThreads ? kFloats : 4 * kMergeThreads];
+    __shared__ float max_s[kThreads / 32], sum_s[kThreads / 32];
+    float *const w_s = smem_f, *const sc_s = smem_f + 2 * kGroupedParts;
+    int *const slot_s = reinterpret_cast<int *>(smem_f + kGroupedParts);
+    const int h = p.head_end - p.head_begin;
+    const int k = blockIdx.x % h, entry = blockIdx.x / h;
+    const int g = p.head_begin + k;
+    grid_launch_dependents();
+    grid_dependency_wait();
+    const int n_entries = p.status[8];
+    const int4 rec = split_rec[entry];
+    if (entry >= n_entries) return;
+    const int i = rec.x, wf = rec.y, nparts = rec.z - rec.y + 1, rs = rec.w;
+    float4 *o4 = reinterpret_cast<float4 *>(p.out + (int64_t)i * p.out_stride_request + (int64_t)g * p.out_stride_head);
+    float *lse = p.lse + (int64_t)i * p.lse_stride_request + g;
+    const int tid = threadIdx.x, c = tid % kMergeThreads, group = tid / kMergeThreads;
+    float L = -INFINITY;
+    if (tid < nparts) {                    // (kThreads >= kGroupedParts: a piece per thread)
+        const int w = wf + tid;
+        const int wb0 = p.worker_begin[w], wb1 = p.worker_begin[w + 1];
+        const float L0 = p.partial_lse[(int64_t)(2 * w) * h + k];
+        const float L1 = tid == 0 ? p.partial_lse[(int64_t)(2 * w + 1) * h + k] : 0.f;
+        float S0 = 1.f, S1 = 1.f;
+        if constexpr (kF16) {
+            S0 = p.partial_scale[(int64_t)(2 * w) * h + k];
+            if (tid == 0) S1 = p.partial_scale[(int64_t)(2 * w + 1) * h + k];
+        }
+        const int slot = 2 * w + (rs <= wb0 ? 0 : 1);
+        if (wb1 > wb0) L = (slot & 1) ? L1 : L0;
+        if constexpr (kF16) sc_s[tid] = (slot & 1) ? S1 : S0;
+        slot_s[tid] = slot;
+    }
+    float m = L;
+    for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((tid & 31) == 0) max_s[tid >> 5] = m;
+    __syncthreads();
+    m = max_s[0];
+#pragma unroll
+    for (int x = 1; x < kThreads / 32; ++x) m = fmaxf(m, max_s[x]);
+    if (m == -INFINITY) {                  // no piece saw a token
+        if (group == 0) o4[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (tid == 0) *lse = -INFINITY;
+        return;
+    }
+    float Z = tid < nparts ? expf(L - m) : 0.f;
+    if (tid < nparts) w_s[tid] = Z;
+    for (int o = 16; o; o >>= 1) Z += __shfl_xor_sync(0xffffffffu, Z, o);
+    if ((tid & 31) == 0) sum_s[tid >> 5] = Z;
+    __syncthreads();
+    Z = sum_s[0];
+#pragma unroll
+    for (int x = 1; x < kThreads / 32; ++x) Z += sum_s[x];       // same order in every thread: one value of Z
+    const float inv_z = 1.f / Z;
+    using Raw = typename std::conditional<kF16, uint2, float4>::type;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int j0 = group; j0 < nparts; j0 += kCombineGroups * kDepth) {
+        Raw raw[kDepth];
+#pragma unroll
+        for (int u = 0; u < kDepth; ++u)
+            if (j0 + u * kCombineGroups < nparts) {
+                const int64_t row = (int64_t)slot_s[j0 + u * kCombineGroups] * h + k;
+                if constexpr (kF16) raw[u] = reinterpret_cast<const uint2 *>(reinterpret_cast<const __half *>(p.partial_out) + row * kDV)[c];
+                else raw[u] = reinterpret_cast<const float4 *>(p.partial_out + row * kDV)[c];
+            }
+#pragma unroll
+        for (int u = 0; u < kDepth; ++u) {
+            const int j = j0 + u * kCombineGroups;
+            float wgt = j < nparts ? w_s[j] * inv_z : 0.f;
+            if (wgt != 0.f) {              // a dead worker's slot holds stale bytes
+                float4 v;
+                if constexpr (kF16) {
+                    wgt *= sc_s[j];
+                    const float2 a = __half22float2(*reinterpret_cast<const __half2 *>(&raw[u].x)), b = __half22float2(*reinterpret_cast<const __half2 *>(&raw[u].y));
+                    v = make_float4(a.x, a.y, b.x, b.y);
+                } else {
+                    v = raw[u];
+                }
+                acc.x = fmaf(wgt, v.x, acc.x); acc.y = fmaf(wgt, v.y, acc.y);
+                acc.z = fmaf(wgt, v.z, acc.z); acc.w = fmaf(wgt, v.w, acc.w);
+            }
+        }
+    }
+    float4 *const total = reinterpret_cast<float4 *>(smem_f);
+    __syncthreads();                       // the weights have been read
+#pragma unroll 1
+    for (int x = kCombineGroups - 1; x >= 0; --x) {
+        if (group == x) {
+            if (x < kCombineGroups - 1) {
+                const float4 v = total[c];
+                acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
+            }
+            if (x > 0) total[c] = acc;
+            else o4[c] = acc;
+        }
+        if (x > 0) __syncthreads();
+    }
+    if (tid == 0) *lse = m + logf(Z);
+}
+
 }  // namespace
 
 cudaError_t launch_lse_merge(int num_parts, int64_t rows, int d_v, const float *part_out,
@@ -192,7 +302,7 @@ cudaError_t launch_lse_merge(int num_parts, int64_t rows, int d_v, const float *
     return e;
 }
 
-cudaError_t launch_split_combine(const DecodeParams &p, const int4 *split_rec, cudaStream_t stream) {
+cudaError_t launch_split_combine(const DecodeParams &p, const int4 *split_rec, int sm_count, cudaStream_t stream) {
     // at most one request straddles each boundary between consecutive workers
     const int max_split = p.num_workers < p.B ? p.num_workers : p.B;
     dim3 grid((unsigned)((int64_t)(p.head_end - p.head_begin) * max_split));
@@ -202,13 +312,16 @@ cudaError_t launch_split_combine(const DecodeParams &p, const int4 *split_rec, c
         cudaFuncSetAttribute(split_combine_kernel<true, false>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
         cudaFuncSetAttribute(split_combine_kernel<false, true>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
         cudaFuncSetAttribute(split_combine_kernel<true, true>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+        cudaFuncSetAttribute(grouped_combine_kernel<false>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+        cudaFuncSetAttribute(grouped_combine_kernel<true>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
         return cudaSuccess;
     });
     // many requests per worker: every request is cut into a few pieces at most
     const bool lean = (int64_t)p.B * 4 >= p.num_workers;
-    auto kernel = p.partial_f16 ? (lean ? split_combine_kernel<true, true> : split_combine_kernel<true, false>)
+    const bool grouped = !lean && grid.x <= (unsigned)sm_count && p.num_workers <= kGroupedParts;
+    auto kernel = grouped ? (p.partial_f16 ? grouped_combine_kernel<true> : grouped_combine_kernel<false>) : p.partial_f16 ? (lean ? split_combine_kernel<true, true> : split_combine_kernel<true, false>)
                                 : (lean ? split_combine_kernel<false, true> : split_combine_kernel<false, false>);
-    cudaError_t e = launch_dependent(kernel, grid, dim3(kMergeThreads), 0, stream, p, split_rec);
+    cudaError_t e = launch_dependent(kernel, grid, dim3(grouped ? kCombineGroups * kMergeThreads : kMergeThreads), 0, stream, p, split_rec);
     count_launch();
     return e;
 }
