@@ -605,10 +605,11 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
             if (slot4 == 0) {
                 const float4 x4 = *reinterpret_cast<const float4 *>(&xch[hd * 4]);
                 const float lt = (x4.x + x4.y) + (x4.z + x4.w);
-                l_s[hd] = lt > 0.f ? 1.f / lt : 0.f;       // no token at all (an empty causal range): O = 0, LSE = -inf
+                // no token at all (an empty causal range): O = 0, LSE = -inf.  Exactly 0: a NaN in the request's data stays one.
+                l_s[hd] = lt == 0.f ? 0.f : 1.f / lt;
                 const int gh = head0 + hd;
                 if (gh < p.head_end) {
-                    float lse = lt > 0.f ? (m - kLift + log2f(lt)) * kLn2 : -INFINITY;
+                    float lse = lt == 0.f ? -INFINITY : (m - kLift + log2f(lt)) * kLn2;
                     if (seg.slot < 0) p.lse[(int64_t)seg.request * p.lse_stride_request + gh] = lse;
                     else p.partial_lse[(int64_t)seg.slot * h + (gh - p.head_begin)] = lse;
                 }
@@ -851,9 +852,9 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
                     const int hh = hA + 8 * e, gh = head0 + hh;
-                    l_s[hh] = lt[e] > 0.f ? 1.f / lt[e] : 0.f;       // no token at all (an empty causal range): O = 0, LSE = -inf
+                    l_s[hh] = lt[e] == 0.f ? 0.f : 1.f / lt[e];      // no token at all: O = 0, LSE = -inf, as above
                     if (gh < p.head_end) {
-                        const float lse = lt[e] > 0.f ? ((e ? mB : mA) - kLift + log2f(lt[e])) * kLn2 : -INFINITY;
+                        const float lse = lt[e] == 0.f ? -INFINITY : ((e ? mB : mA) - kLift + log2f(lt[e])) * kLn2;
                         if (seg.slot < 0) p.lse[(int64_t)seg.request * p.lse_stride_request + gh] = lse;
                         else p.partial_lse[(int64_t)seg.slot * h + (gh - p.head_begin)] = lse;
                     }

@@ -440,10 +440,11 @@ decode_umma_pair_kernel(const __grid_constant__ DecodeParams p, const __grid_con
             if (slot4 == 0) {
                 const float4 x4 = *reinterpret_cast<const float4 *>(&xch[hd * 4]);
                 const float lt = (x4.x + x4.y) + (x4.z + x4.w);
-                l_s[hd] = lt > 0.f ? 1.f / lt : 0.f;       // no token at all (an empty causal range): O = 0, LSE = -inf
+                // no token at all (an empty causal range): O = 0, LSE = -inf.  Exactly 0: a NaN in the request's data stays one.
+                l_s[hd] = lt == 0.f ? 0.f : 1.f / lt;
                 const int gh = head0 + hd;
                 if (gh < p.head_end) {
-                    float lse = lt > 0.f ? (m + log2f(lt)) * kLn2 : -INFINITY;
+                    float lse = lt == 0.f ? -INFINITY : (m + log2f(lt)) * kLn2;
                     if (seg.slot < 0) p.lse[(int64_t)seg.request * p.lse_stride_request + gh] = lse;
                     else p.partial_lse[(int64_t)seg.slot * h + (gh - p.head_begin)] = lse;
                 }

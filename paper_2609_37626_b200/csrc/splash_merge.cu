@@ -14,6 +14,10 @@ namespace {
 
 constexpr int kMergeThreads = 128;
 
+// What the LSEs of a row are measured against: their largest, or 0 where that is -inf.  Either no part saw a token then, and the
+// weights add up to exactly 0, or an LSE is NaN (which fmaxf passes over), and so is the sum: the row becomes NaN, not empty.
+__device__ __forceinline__ float reference_max(float m) { return m == -INFINITY ? 0.f : m; }
+
 // One CTA per row; each thread owns float4 columns tid, tid + 128, ...  The parts' LSEs come in one load each, a part per
 // thread, and the parts' rows kDepth loads at a time: taken one after the other in every thread they were a chain of round trips
 // (the decode of a CP shard with the merge of eight parts of 128 rows behind it: 28.2 us, now 27.1).  Where the rows are more
@@ -35,18 +39,18 @@ lse_merge_kernel(int num_parts, int64_t rows, int d_v, const float *__restrict__
     for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
     if ((tid & 31) == 0) red_s[0][tid >> 5] = m;
     __syncthreads();
-    m = fmaxf(fmaxf(red_s[0][0], red_s[0][1]), fmaxf(red_s[0][2], red_s[0][3]));
-    if (m == -INFINITY) {
-        for (int c = tid; c < nvec; c += kMergeThreads) o4[c] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (tid == 0) lse[r] = -INFINITY;
-        return;
-    }
+    m = reference_max(fmaxf(fmaxf(red_s[0][0], red_s[0][1]), fmaxf(red_s[0][2], red_s[0][3])));
     float Z = expf(first - m);        // (0 for a part without tokens)
     for (int j = tid + kMergeThreads; j < num_parts; j += kMergeThreads) Z += expf(part_lse[(int64_t)j * rows + r] - m);
     for (int o = 16; o; o >>= 1) Z += __shfl_xor_sync(0xffffffffu, Z, o);
     if ((tid & 31) == 0) red_s[1][tid >> 5] = Z;
     __syncthreads();
     Z = (red_s[1][0] + red_s[1][1]) + (red_s[1][2] + red_s[1][3]);       // the same in every thread
+    if (Z == 0.f) {                   // no part saw a token
+        for (int c = tid; c < nvec; c += kMergeThreads) o4[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (tid == 0) lse[r] = -INFINITY;
+        return;
+    }
     const float L = m + logf(Z);
     for (int j0 = 0; j0 < num_parts; j0 += kMergeThreads) {              // as many parts at a time as there are weights in shared memory
         const int n = min(kMergeThreads, num_parts - j0);
@@ -136,16 +140,16 @@ split_combine_kernel(const DecodeParams p, const int4 *__restrict__ split_rec) {
     for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
     if ((c & 31) == 0) red_s[c >> 5] = m;
     __syncthreads();
-    m = fmaxf(fmaxf(red_s[0], red_s[1]), fmaxf(red_s[2], red_s[3]));
-    if (m == -INFINITY) {                  // no piece saw a token (a query row whose causal range is empty)
-        o4[c] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (c == 0) *lse = -INFINITY;
-        return;
-    }
+    m = reference_max(fmaxf(fmaxf(red_s[0], red_s[1]), fmaxf(red_s[2], red_s[3])));
     for (int j = c; j < nparts; j += kMergeThreads) w_s[j] = expf(w_s[j] - m);     // 0 for dead workers
     __syncthreads();
     float Z = 0.f;
     for (int j = 0; j < nparts; ++j) Z += w_s[j];          // same order in every thread: one value of Z
+    if (Z == 0.f) {                        // no piece saw a token (a query row whose causal range is empty)
+        o4[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (c == 0) *lse = -INFINITY;
+        return;
+    }
     const float L = m + logf(Z);
     const float inv_z = 1.f / Z;
     // this thread's four columns of a slot's row as they lie in memory (loads first, conversions with the arithmetic:
@@ -256,11 +260,7 @@ grouped_combine_kernel(const DecodeParams p, const int4 *__restrict__ split_rec)
     m = max_s[0];
 #pragma unroll
     for (int x = 1; x < kThreads / 32; ++x) m = fmaxf(m, max_s[x]);
-    if (m == -INFINITY) {                  // no piece saw a token
-        if (group == 0) o4[c] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (tid == 0) *lse = -INFINITY;
-        return;
-    }
+    m = reference_max(m);
     float Z = tid < nparts ? expf(L - m) : 0.f;
     if (tid < nparts) w_s[tid] = Z;
     for (int o = 16; o; o >>= 1) Z += __shfl_xor_sync(0xffffffffu, Z, o);
@@ -269,6 +269,11 @@ grouped_combine_kernel(const DecodeParams p, const int4 *__restrict__ split_rec)
     Z = sum_s[0];
 #pragma unroll
     for (int x = 1; x < kThreads / 32; ++x) Z += sum_s[x];       // same order in every thread: one value of Z
+    if (Z == 0.f) {                        // no piece saw a token
+        if (group == 0) o4[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (tid == 0) *lse = -INFINITY;
+        return;
+    }
     const float inv_z = 1.f / Z;
     using Raw = typename std::conditional<kF16, uint2, float4>::type;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
