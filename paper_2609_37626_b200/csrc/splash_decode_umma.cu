@@ -207,7 +207,7 @@ decode_umma_kernel(const __grid_constant__ DecodeParams p, const __grid_constant
         bool ok = true;
         while (ok && it.next(p, seg)) {
             const int ntiles = (int)uniform((uint32_t)(seg.tile_end - seg.tile_begin));
-            ok = mbar_wait(ctx, bar(kBarQFull), seg_it & 1, kBarQFull);
+            mbar_wait(ctx, bar(kBarQFull), seg_it & 1, kBarQFull);       // (its answer goes unused: past a wait that gave up nothing counts, and a wait below ends the walk)
             for (int i = 0; ok && i < ntiles; ++i, ++kv) {
                 const uint32_t stage = kv % kStages, b = kv & 1;
                 ok = mbar_wait(ctx, bar(kBarKvFull + stage), (kv / kStages) & 1, kBarKvFull + stage) &&
@@ -276,13 +276,13 @@ decode_umma_kernel(const __grid_constant__ DecodeParams p, const __grid_constant
         if constexpr (kSparse)
             gather_tiles<kPage>(
                 p, it, warp - kWarpGather, lane, 0, [&](uint32_t t) { return smem + L::kOffKv + (t % kStages) * kStageBytes; },
-                [&](uint32_t t) { return mbar_wait(ctx, bar(kBarKvEmpty + t % kStages), ((t / kStages) & 1) ^ 1, kBarKvEmpty); },
+                [&](uint32_t t) { mbar_wait(ctx, bar(kBarKvEmpty + t % kStages), ((t / kStages) & 1) ^ 1, kBarKvEmpty); },
                 [&](uint32_t t) {
                     fence_proxy_async();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(bar(kBarKvFull + t % kStages));
                 },
-                [](uint32_t) { return true; }, [](uint32_t) {});
+                [](uint32_t) {}, [](uint32_t) {});
     } else {
         // ===================================================== softmax + epilogue warps
         const int q4 = warp & 3;                       // TMEM lane quadrant of this warp

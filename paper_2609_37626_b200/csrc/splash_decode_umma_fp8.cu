@@ -273,7 +273,7 @@ decode_umma_fp8_kernel(const __grid_constant__ DecodeParams p, const __grid_cons
         uint32_t seg_it = 0;
         bool ok = true;
         while (ok && it.next(p, seg)) {
-            ok = mbar_wait(ctx, bar(kBarQEmpty), (seg_it & 1) ^ 1, kBarQEmpty);
+            ok = warp_wait(ctx, bar(kBarQEmpty), (seg_it & 1) ^ 1, kBarQEmpty);
             if (!ok) break;
             {
                 const int hd = ct >> 1, part = ct & 1;

@@ -220,7 +220,7 @@ decode_umma_fp8_narrow_kernel(const __grid_constant__ DecodeParams p, const __gr
         while (ok && it.next(p, seg)) {
             const int ntiles = (int)uniform((uint32_t)(seg.tile_end - seg.tile_begin));
             const uint32_t qb = seg_it & 1;
-            ok = mbar_wait(ctx, bar(kBarQFull + qb), (seg_it >> 1) & 1, kBarQFull + qb);
+            mbar_wait(ctx, bar(kBarQFull + qb), (seg_it >> 1) & 1, kBarQFull + qb);       // (its answer goes unused: past a wait that gave up nothing counts, and a wait below ends the walk)
             for (int i = 0; ok && i < ntiles; ++i, ++kv) {
                 const uint32_t stage = kv % kStages, b = kv & 1;
                 ok = mbar_wait(ctx, bar(kBarKvFull + stage), (kv / kStages) & 1, kBarKvFull + stage) &&
@@ -334,7 +334,7 @@ decode_umma_fp8_narrow_kernel(const __grid_constant__ DecodeParams p, const __gr
                 const float inv = amax > 0.f ? 448.0f / amax : 1.0f;
                 if (pass == 0) {
                     // this buffer's previous request (two back): its QK^T retired, its output tile staged and gone
-                    ok = mbar_wait(ctx, bar(kBarQEmpty + qb), ((seg_it >> 1) & 1) ^ 1, kBarQEmpty + qb);
+                    ok = warp_wait(ctx, bar(kBarQEmpty + qb), ((seg_it >> 1) & 1) ^ 1, kBarQEmpty + qb);
                     if (!ok) break;
                 }
                 if (part == 0) qs_s[(seg_it & 3) * N + hd] = qs;

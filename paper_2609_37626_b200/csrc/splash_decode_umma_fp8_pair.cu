@@ -287,7 +287,7 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
         bool ok = true;
         while (ok && it.next(p, seg)) {
             const int nsuper = (int)uniform((uint32_t)((seg.tile_end - seg.tile_begin + 1) >> 1));
-            ok = mbar_wait_cluster(ctx, bar(L::kBarQFull), seg_it & 1, L::kBarQFull);
+            mbar_wait_cluster(ctx, bar(L::kBarQFull), seg_it & 1, L::kBarQFull);       // (its answer goes unused: past a wait that gave up nothing counts, and a wait below ends the walk)
             for (int s = 0; ok && s < nsuper; ++s, ++st_it) {
                 const uint32_t stage = st_it % kStages, b = st_it & 1;
                 ok = mbar_wait_cluster(ctx, bar(L::kBarKFull + stage), (st_it / kStages) & 1, L::kBarKFull + stage) &&
@@ -426,7 +426,7 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
                     }
                 };
                 load_batch(xa, 0);
-                ok = mbar_wait(ctx, bar(L::kBarQEmpty), (seg_it & 1) ^ 1, L::kBarQEmpty);
+                ok = warp_wait(ctx, bar(L::kBarQEmpty), (seg_it & 1) ^ 1, L::kBarQEmpty);
                 if (!ok) break;
                 load_batch(xb, 9);  convert_batch(xa, 0);
                 if constexpr (H == 64) {

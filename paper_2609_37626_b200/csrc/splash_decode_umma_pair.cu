@@ -248,7 +248,7 @@ decode_umma_pair_kernel(const __grid_constant__ DecodeParams p, const __grid_con
         bool ok = true;
         while (ok && it.next(p, seg)) {
             const int ntiles = (int)uniform((uint32_t)(seg.tile_end - seg.tile_begin));
-            ok = mbar_wait_cluster(ctx, bar(kBarQFull), seg_it & 1, kBarQFull);
+            mbar_wait_cluster(ctx, bar(kBarQFull), seg_it & 1, kBarQFull);       // (its answer goes unused: past a wait that gave up nothing counts, and a wait below ends the walk)
             for (int i = 0; ok && i < ntiles; ++i, ++kv_it) {
                 const uint32_t stage = kv_it % kStages, b = kv_it & 1;
                 ok = mbar_wait_cluster(ctx, bar(kBarKFull + stage), (kv_it / kStages) & 1, kBarKFull + stage) &&
@@ -316,13 +316,13 @@ decode_umma_pair_kernel(const __grid_constant__ DecodeParams p, const __grid_con
         if constexpr (kSparse)
             gather_tiles<kHalf>(
                 p, it, warp - kWarpVProducer - 1, lane, (int)rank, [&](uint32_t t) { return smem + kOffK + (t % kStages) * kStageBytes; },
-                [&](uint32_t t) { return mbar_wait(ctx, bar(kBarStageEmpty + t % kStages), ((t / kStages) & 1) ^ 1, kBarStageEmpty); },
+                [&](uint32_t t) { mbar_wait(ctx, bar(kBarStageEmpty + t % kStages), ((t / kStages) & 1) ^ 1, kBarStageEmpty); },
                 [&](uint32_t t) {
                     fence_proxy_async();
                     __syncwarp();
                     if (lane == 0) arrive_on_leader(kBarKFull + t % kStages);
                 },
-                [&](uint32_t t) { return mbar_wait(ctx, bar(kBarQkDone + t % kStages), (t / kStages) & 1, kBarQkDone); },
+                [&](uint32_t t) { mbar_wait(ctx, bar(kBarQkDone + t % kStages), (t / kStages) & 1, kBarQkDone); },
                 [&](uint32_t t) {
                     fence_proxy_async();
                     __syncwarp();

@@ -118,8 +118,8 @@ struct Resolver {
 // Warp gw of kGatherWarps: its rows of every tile of the worker.  kRows rows of a tile are this CTA's own (all 576 columns, for
 // QK^T and P.V); of a pair, whose CTAs own 32 rows each, the two 128-column blocks of the OTHER 32 rows that this CTA multiplies
 // follow two tiles later, into the chunk slots that QK^T has left (splash_decode_umma_pair.cu).
-// stage(t): the first slab of tile t's stage.  wait_stage(t), wait_qk(t): it may be written, its other half's slots may
-// (false: give up).  done_own(t), done_peer(t): all lanes, after their stores.
+// stage(t): the first slab of tile t's stage.  wait_stage(t), wait_qk(t): it may be written, its other half's slots may.  Nothing here
+// depends on whether a wait gave up: the warp walks its tiles to the end (no wait blocks once the CTA aborts), in step.  done_own(t), done_peer(t): all lanes, after their stores.
 template <int kRows, typename Iter, typename Stage, typename WaitStage, typename DoneOwn, typename WaitQk, typename DonePeer>
 __device__ __forceinline__ void gather_tiles(const DecodeParams &p, const Iter &it, int gw, int lane, int rank, Stage &&stage, WaitStage &&wait_stage,
                                              DoneOwn &&done_own, WaitQk &&wait_qk, DonePeer &&done_peer) {
@@ -178,7 +178,7 @@ __device__ __forceinline__ void gather_tiles(const DecodeParams &p, const Iter &
             const uint32_t t = (uint32_t)i / kBatches;
             const int r = gw * kShare + (i % kBatches) * 4 + (lane >> 3);
             const unsigned long long next = __shfl_sync(0xffffffffu, k == 7 ? res.row[0] : own, ((k + 1) & 7) * 4 + (lane >> 3));
-            if (i % kBatches == 0 && !wait_stage(t)) return;
+            if (i % kBatches == 0) wait_stage(t);
             uint8_t *const slab_row = stage(t) + r * 128;
             const float s[4] = {scale.x, scale.y, scale.z, scale.w};
 #pragma unroll
@@ -195,7 +195,7 @@ __device__ __forceinline__ void gather_tiles(const DecodeParams &p, const Iter &
             // the other half's rows of tile i - kLag, then the loads for the next one's (L2 hits, mostly: the peer reads them too)
             const int j = i - kLag;
             if (j >= 0) {
-                if (!wait_qk((uint32_t)j)) return;
+                wait_qk((uint32_t)j);
                 const int r = gw * kShare + (lane >> 3);
                 uint8_t *const slab_row = stage((uint32_t)j) + r * 128;
 #pragma unroll

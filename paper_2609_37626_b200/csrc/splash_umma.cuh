@@ -79,6 +79,11 @@ __device__ __forceinline__ bool mbar_wait(const Ctx &ctx, uint32_t bar, uint32_t
     if (mbar_try_wait(bar, parity)) return true;
     return mbar_wait_slow(ctx, bar, parity, bar_id);
 }
+// The same by all lanes of a converged warp, for a wait that decides where the warp goes: when a wait gives up, its lanes need not all
+// have seen the same, and some in the loop's next collective while the others wait behind the loop would never meet.
+__device__ __forceinline__ bool warp_wait(const Ctx &ctx, uint32_t bar, uint32_t parity, int bar_id) {
+    return __all_sync(0xffffffffu, mbar_wait(ctx, bar, parity, bar_id));
+}
 
 // TMA store of a shared-memory tile (bulk async-group completion); coordinates outside the
 // tensor are clipped
