@@ -110,6 +110,18 @@ PyObject *raise_status(int rc) {
 
 void *ptr(const at::Tensor *t) { return t ? t->data_ptr() : nullptr; }
 
+// A call into the library without the GIL: with the stream's launch queue full a launch blocks until the GPU has caught up, which may
+// itself wait for this process's other threads.  (Given back on every way out; addresses are read from the tensors before, where an
+// exception finds the GIL held.)
+template <typename F>
+int without_gil(F &&call) {
+    struct Released {
+        PyThreadState *state = PyEval_SaveThread();
+        ~Released() { PyEval_RestoreThread(state); }
+    } released;
+    return call();
+}
+
 at::Tensor new_tensor(at::IntArrayRef size, at::ScalarType dtype, const at::Tensor &like) {
     return at::Tensor(at::detail::empty_cuda(size, dtype, like.device(), std::nullopt));
 }
@@ -210,26 +222,27 @@ PyObject *mla_decode(PyObject *, PyObject *const *args, Py_ssize_t nargs, PyObje
     if (!ws) ws = &cached_workspace(*q, splash_mla_decode_workspace_bytes(&shape, (int32_t)first, (int32_t)last), "decode");
     const at::Tensor keep = *ws;                    // another thread may replace the cached one while the GIL is released
     const size_t ws_bytes = (size_t)keep.numel() * keep.element_size();
+    const void *q_at = q->data_ptr(), *kv_at = kv->data_ptr(), *scales_at = ptr(scales), *table_at = table->data_ptr(), *lens_at = lens->data_ptr();
+    const void *begin_at = ptr(begin), *end_at = ptr(end);
+    void *out_at = out.data_ptr(), *lse_at = lse.data_ptr(), *ws_at = keep.data_ptr();
+    auto decode = [&](const splash_migrate_job *job) {
+        return without_gil([&] {
+            return splash_mla_decode_migrating(&shape, q_at, kv_at, (const float *)scales_at, (const int32_t *)table_at, (const int32_t *)lens_at,
+                                               (int32_t)first, (int32_t)last, (const int32_t *)begin_at, (const int32_t *)end_at, (float *)out_at,
+                                               (float *)lse_at, ws_at, ws_bytes, stream, job);
+        });
+    };
     int rc;
     if (given(v[15])) {                             // (splash_migrate_job as a ctypes structure, what keeps it alive)
         PyObject *job = PySequence_GetItem(v[15], 0);
         Py_buffer view;
         if (!job) return nullptr;
         if (PyObject_GetBuffer(job, &view, PyBUF_SIMPLE) != 0) { Py_DECREF(job); return nullptr; }
-        rc = (size_t)view.len == sizeof(splash_migrate_job)
-                 ? splash_mla_decode_migrating(&shape, q->data_ptr(), kv->data_ptr(), (const float *)ptr(scales), (const int32_t *)table->data_ptr(),
-                                               (const int32_t *)lens->data_ptr(), (int32_t)first, (int32_t)last, (const int32_t *)ptr(begin),
-                                               (const int32_t *)ptr(end), (float *)out.data_ptr(), (float *)lse.data_ptr(), keep.data_ptr(), ws_bytes,
-                                               stream, (const splash_migrate_job *)view.buf)
-                 : SPLASH_INVALID_ARG;
+        rc = (size_t)view.len == sizeof(splash_migrate_job) ? decode((const splash_migrate_job *)view.buf) : SPLASH_INVALID_ARG;
         PyBuffer_Release(&view);
         Py_DECREF(job);
     } else {
-        Py_BEGIN_ALLOW_THREADS
-        rc = splash_mla_decode(&shape, q->data_ptr(), kv->data_ptr(), (const float *)ptr(scales), (const int32_t *)table->data_ptr(),
-                               (const int32_t *)lens->data_ptr(), (int32_t)first, (int32_t)last, (const int32_t *)ptr(begin),
-                               (const int32_t *)ptr(end), (float *)out.data_ptr(), (float *)lse.data_ptr(), keep.data_ptr(), ws_bytes, stream);
-        Py_END_ALLOW_THREADS
+        rc = decode(nullptr);
     }
     if (rc != SPLASH_OK) return raise_status(rc);
     return pair_of(v[10], out, v[11], lse);
@@ -272,13 +285,16 @@ PyObject *mla_decode_sparse(PyObject *, PyObject *const *args, Py_ssize_t nargs,
         ws = &cached_workspace(*q, need, "decode");
     }
     const at::Tensor keep = *ws;
-    int rc;
-    Py_BEGIN_ALLOW_THREADS
-    rc = splash_mla_decode_sparse(&shape, q->data_ptr(), kv->data_ptr(), (const int32_t *)table->data_ptr(), (const int32_t *)lens->data_ptr(),
-                                  (const int32_t *)sel->data_ptr(), q->size(0) > 0 ? sel->stride(0) : 0, (const int32_t *)count->data_ptr(),
-                                  (int32_t)most, (int32_t)first, (int32_t)last, (float *)out.data_ptr(), (float *)lse.data_ptr(), keep.data_ptr(),
-                                  (size_t)keep.numel() * keep.element_size(), stream);
-    Py_END_ALLOW_THREADS
+    const void *q_at = q->data_ptr(), *kv_at = kv->data_ptr(), *table_at = table->data_ptr(), *lens_at = lens->data_ptr(), *sel_at = sel->data_ptr();
+    const void *count_at = count->data_ptr();
+    void *out_at = out.data_ptr(), *lse_at = lse.data_ptr(), *ws_at = keep.data_ptr();
+    const int64_t sel_stride = q->size(0) > 0 ? sel->stride(0) : 0;
+    const size_t ws_bytes = (size_t)keep.numel() * keep.element_size();
+    const int rc = without_gil([&] {
+        return splash_mla_decode_sparse(&shape, q_at, kv_at, (const int32_t *)table_at, (const int32_t *)lens_at, (const int32_t *)sel_at, sel_stride,
+                                        (const int32_t *)count_at, (int32_t)most, (int32_t)first, (int32_t)last, (float *)out_at, (float *)lse_at,
+                                        ws_at, ws_bytes, stream);
+    });
     if (rc != SPLASH_OK) return raise_status(rc);
     return pair_of(v[10], out, v[11], lse);
     END_HANDLE_TH_ERRORS
@@ -303,8 +319,11 @@ PyObject *lse_merge(PyObject *, PyObject *const *args, Py_ssize_t nargs, PyObjec
     else lse = new_tensor({rows}, at::kFloat, *po);
     void *stream;
     if (!stream_of(v[4], stream)) return nullptr;
-    const int rc = splash_lse_merge((int32_t)parts, rows, (int32_t)dv, (const float *)po->data_ptr(), (const float *)pl->data_ptr(),
-                                    (float *)out.data_ptr(), (float *)lse.data_ptr(), stream);
+    const void *po_at = po->data_ptr(), *pl_at = pl->data_ptr();
+    void *out_at = out.data_ptr(), *lse_at = lse.data_ptr();
+    const int rc = without_gil([&] {
+        return splash_lse_merge((int32_t)parts, rows, (int32_t)dv, (const float *)po_at, (const float *)pl_at, (float *)out_at, (float *)lse_at, stream);
+    });
     if (rc != SPLASH_OK) return raise_status(rc);
     return pair_of(v[2], out, v[3], lse);
     END_HANDLE_TH_ERRORS
@@ -335,19 +354,21 @@ PyObject *migrate(PyObject *const *args, Py_ssize_t nargs, PyObject *kwnames, bo
     void *stream;
     if (!stream_of(v[with_workspace ? 11 : 10], stream)) return nullptr;
     const int64_t page_bytes = src->size(1) * src->size(2) * src->element_size();
-    int rc;
-    if (with_workspace) {
-        if (!ws) ws = &cached_workspace(*src, splash_kv_page_migrate_workspace_bytes((int32_t)most), "migrate");
-        const at::Tensor keep = *ws;
-        rc = splash_kv_page_migrate(src->data_ptr(), (const float *)ptr(ss), dst->data_ptr(), (float *)ptr(ds), page_bytes,
-                                    (const int32_t *)sid->data_ptr(), (const int32_t *)did->data_ptr(), sid->numel(), (int32_t)src_base,
-                                    (int32_t)dst_base, (int32_t)most, (int32_t *)table->data_ptr(), table->numel(), keep.data_ptr(),
-                                    (size_t)keep.numel(), stream);
-    } else {
-        rc = splash_kv_page_migrate_static(src->data_ptr(), (const float *)ptr(ss), dst->data_ptr(), (float *)ptr(ds), page_bytes,
-                                           (const int32_t *)sid->data_ptr(), (const int32_t *)did->data_ptr(), sid->numel(), (int32_t)src_base,
-                                           (int32_t)dst_base, (int32_t)most, (int32_t *)table->data_ptr(), table->numel(), stream);
-    }
+    if (with_workspace && !ws) ws = &cached_workspace(*src, splash_kv_page_migrate_workspace_bytes((int32_t)most), "migrate");
+    const at::Tensor keep = with_workspace ? *ws : at::Tensor();
+    const void *src_at = src->data_ptr(), *ss_at = ptr(ss), *sid_at = sid->data_ptr(), *did_at = did->data_ptr();
+    void *dst_at = dst->data_ptr(), *ds_at = ptr(ds), *table_at = table->data_ptr(), *ws_at = with_workspace ? keep.data_ptr() : nullptr;
+    const int64_t n = sid->numel(), entries = table->numel();
+    const size_t ws_bytes = with_workspace ? (size_t)keep.numel() : 0;
+    const int rc = without_gil([&] {
+        return with_workspace
+                   ? splash_kv_page_migrate(src_at, (const float *)ss_at, dst_at, (float *)ds_at, page_bytes, (const int32_t *)sid_at,
+                                            (const int32_t *)did_at, n, (int32_t)src_base, (int32_t)dst_base, (int32_t)most, (int32_t *)table_at,
+                                            entries, ws_at, ws_bytes, stream)
+                   : splash_kv_page_migrate_static(src_at, (const float *)ss_at, dst_at, (float *)ds_at, page_bytes, (const int32_t *)sid_at,
+                                                   (const int32_t *)did_at, n, (int32_t)src_base, (int32_t)dst_base, (int32_t)most,
+                                                   (int32_t *)table_at, entries, stream);
+    });
     if (rc != SPLASH_OK) return raise_status(rc);
     Py_RETURN_NONE;
 }
@@ -390,8 +411,12 @@ PyObject *dop_pack_rows(PyObject *, PyObject *const *args, Py_ssize_t nargs, PyO
     SPLASH_ASSERT(out.is_contiguous() && out.sizes() == at::IntArrayRef({n, h, da + db}));
     void *stream;
     if (!stream_of(v[4], stream)) return nullptr;
-    const int rc = splash_dop_pack_rows(a->data_ptr(), da * es, a->stride(0) * es, a->stride(1) * es, ptr(b), db * es, b ? b->stride(0) * es : 0,
-                                        b ? b->stride(1) * es : 0, (const int32_t *)row->data_ptr(), n, (int32_t)h, out.data_ptr(), stream);
+    const void *a_at = a->data_ptr(), *b_at = ptr(b), *row_at = row->data_ptr();
+    void *out_at = out.data_ptr();
+    const int64_t a_row = a->stride(0) * es, a_head = a->stride(1) * es, b_row = b ? b->stride(0) * es : 0, b_head = b ? b->stride(1) * es : 0;
+    const int rc = without_gil([&] {
+        return splash_dop_pack_rows(a_at, da * es, a_row, a_head, b_at, db * es, b_row, b_head, (const int32_t *)row_at, n, (int32_t)h, out_at, stream);
+    });
     if (rc != SPLASH_OK) return raise_status(rc);
     return given(v[3]) ? Py_NewRef(v[3]) : THPVariable_Wrap(out);
     END_HANDLE_TH_ERRORS
@@ -422,7 +447,10 @@ PyObject *dop_swap_outer(PyObject *, PyObject *const *args, Py_ssize_t nargs, Py
     SPLASH_ASSERT(out.is_contiguous());
     void *stream;
     if (!stream_of(v[2], stream)) return nullptr;
-    const int rc = splash_dop_swap_outer(x->data_ptr(), x->size(0), x->size(1), inner, out.data_ptr(), stream);
+    const void *x_at = x->data_ptr();
+    void *out_at = out.data_ptr();
+    const int64_t A = x->size(0), Bn = x->size(1);
+    const int rc = without_gil([&] { return splash_dop_swap_outer(x_at, A, Bn, inner, out_at, stream); });
     if (rc != SPLASH_OK) return raise_status(rc);
     return given(v[1]) ? Py_NewRef(v[1]) : THPVariable_Wrap(out);
     END_HANDLE_TH_ERRORS
@@ -450,8 +478,10 @@ PyObject *dop_unpack_rows(PyObject *, PyObject *const *args, Py_ssize_t nargs, P
     for (int64_t k = 1; k < recv->dim(); ++k) row_bytes *= recv->size(k);
     void *stream;
     if (!stream_of(v[3], stream)) return nullptr;
-    const int rc = splash_dop_unpack_rows(recv->data_ptr(), (const int32_t *)row->data_ptr(), row->numel(), row_bytes, out->data_ptr(),
-                                          out->stride(0) * out->element_size(), stream);
+    const void *recv_at = recv->data_ptr(), *row_at = row->data_ptr();
+    void *out_at = out->data_ptr();
+    const int64_t n = row->numel(), pitch = out->stride(0) * out->element_size();
+    const int rc = without_gil([&] { return splash_dop_unpack_rows(recv_at, (const int32_t *)row_at, n, row_bytes, out_at, pitch, stream); });
     if (rc != SPLASH_OK) return raise_status(rc);
     return Py_NewRef(v[2]);
     END_HANDLE_TH_ERRORS
