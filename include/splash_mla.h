@@ -283,13 +283,8 @@ SPLASH_API size_t splash_kv_page_migrate_workspace_bytes(int32_t max_page_id);
  * none of the job's destination pages and not the job's block table (the usual case: the job
  * moves the pages of ANOTHER layer's cache; source pages may be shared, they are only read).
  *
- * How: slices of 65..128 (head, row) pairs run on CTA pairs in which the MMA-issuing warps of
- * each pair's second CTA have nothing to do; those warps copy the job's pages (16-byte
- * streaming loads and stores, byte-exact) while the rest of the kernel decodes, on SMs and
- * HBM bandwidth the decode leaves unused.  The job's table rewrite (two small kernels) runs
- * on `stream` before the decode.  Calls that do not run on the CTA-pair kernels (narrower
- * slices, SPLASH_FLAG_SIMT / NO_PAIR, more than 128 (head, row) pairs) run the plain page-copy
- * kernel after the decode instead: same results, no overlap.
+ * How: the job's kernels (splash_kv_page_migrate's) run on `stream` in front of the decode's, each started under the
+ * tail of the one before it, so that the call takes about the time of both parts.
  *
  * job == NULL or job->n == 0: exactly splash_mla_decode.  The job's fields are the arguments of
  * splash_kv_page_migrate, validated the same way; on an error nothing has been launched.

@@ -210,10 +210,10 @@ int check_migrate_job(const splash_migrate_job *job) {
                               job->workspace, job->workspace_bytes);
 }
 
-cudaError_t run_migrate_job(const splash_migrate_job *job, bool do_table, bool do_copy, cudaStream_t stream) {
+cudaError_t run_migrate_job(const splash_migrate_job *job, cudaStream_t stream) {
     return launch_page_migrate(job->src_pool, job->src_scales, job->dst_pool, job->dst_scales, job->page_bytes, job->src_page_ids,
                                job->dst_page_ids, job->n, job->src_id_base, job->dst_id_base, job->max_page_id, job->block_table,
-                               job->num_table_entries, static_cast<int32_t *>(job->workspace), do_table, do_copy, stream);
+                               job->num_table_entries, static_cast<int32_t *>(job->workspace), stream);
 }
 
 // One decode call: plan, decode kernel, combine.  With a sparse stage, seq_lens are the list counts; the decode kernel gathers
@@ -235,7 +235,7 @@ int decode_dense(const splash_mla_shape *shape, const void *q, const void *kv_po
     const int B = shape->num_requests;
     if (B == 0 || head_end == head_begin) {     // idle rank: no attention to compute; its pages still move
         if (job != nullptr) {
-            cudaError_t e = run_migrate_job(job, true, true, static_cast<cudaStream_t>(stream_));
+            cudaError_t e = run_migrate_job(job, static_cast<cudaStream_t>(stream_));
             if (e != cudaSuccess) { set_error("CUDA error: %s", cudaGetErrorString(e)); return SPLASH_CUDA_ERROR; }
         }
         return SPLASH_OK;
@@ -263,10 +263,11 @@ int decode_dense(const splash_mla_shape *shape, const void *q, const void *kv_po
     const int h = vend - vbegin;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     cudaError_t e = cudaSuccess;
-    // a page-copy job: its table rewrite runs first; its page copy rides in the decode kernel if that is a CTA-pair
-    // kernel, else runs as a kernel of its own after the decode
-    bool job_copy_pending = job != nullptr;
-    if (job != nullptr) e = run_migrate_job(job, true, false, stream);
+    // A migration job: its two kernels, at the copy rate, then the decode's, which come in as its last pages move.  (A copy carried by
+    // the idle issuer warps of the CTA pairs, under the decode, is not the faster one: the pages and the cache share the DRAM, and two
+    // warps a pair stay far below its rate.  10,000 pages beside 16 contexts of 32,768 tokens on 128 heads over e4m3: 463 us, 246 this
+    // way; 2,000 beside one of 262,144 over bf16: 188 and 122; with four and six such warps a pair they had been 367 and 140.)
+    if (job != nullptr) e = run_migrate_job(job, stream);
     Tiling t = choose_tiling(shape, h, dev.sm_count, simt);
     // where the work partition comes from (splash_common.cuh): a batch of up to 32 requests is planned by the decode kernel
     // itself; if its contexts are short besides, no request is cut and the combine kernel is left out
@@ -318,13 +319,6 @@ int decode_dense(const splash_mla_shape *shape, const void *q, const void *kv_po
         p.request_overhead_tiles = kRequestOverheadTilesPair;
     // the bf16 CTA-pair kernel writes its partial outputs as f16
     p.partial_f16 = (pair && shape->kv_dtype == SPLASH_KV_BF16) ? 1 : 0;
-    if (job_copy_pending && pair) {
-        p.mig_src = static_cast<const uint4 *>(job->src_pool); p.mig_dst = static_cast<uint4 *>(job->dst_pool);
-        p.mig_src_scales = reinterpret_cast<const uint4 *>(job->src_scales); p.mig_dst_scales = reinterpret_cast<uint4 *>(job->dst_scales);
-        p.mig_src_ids = job->src_page_ids; p.mig_dst_ids = job->dst_page_ids;
-        p.mig_page_vecs = job->page_bytes / 16; p.mig_n = (int32_t)job->n;
-        job_copy_pending = false;
-    }
 
     // the previous call's partition taken again (the same batch in the next layer): no plan kernel, only the error words
     // of the status block are cleared (word 8, the number of split requests, belongs to the plan)
@@ -352,7 +346,6 @@ int decode_dense(const splash_mla_shape *shape, const void *q, const void *kv_po
     if (e == cudaSuccess && plan_mode != kPlanWhole) e = launch_split_combine(p, v.split_rec, dev.sm_count, stream);
     if (e == cudaSuccess) e = record_timing_event(3, stream);
     if (e == cudaSuccess && g_timing) g_events_recorded = true;
-    if (e == cudaSuccess && job_copy_pending) e = run_migrate_job(job, false, true, stream);
     if (e != cudaSuccess) { set_error("CUDA error: %s", cudaGetErrorString(e)); return SPLASH_CUDA_ERROR; }
     return SPLASH_OK;
 }
@@ -485,7 +478,7 @@ int splash_kv_page_migrate(const void *src_pool, const float *src_scales, void *
     if (rc != SPLASH_OK || n == 0) return rc;
     cudaError_t e = launch_page_migrate(src_pool, src_scales, dst_pool, dst_scales, page_bytes, src_page_ids,
                                         dst_page_ids, n, src_id_base, dst_id_base, max_page_id, block_table,
-                                        num_table_entries, static_cast<int32_t *>(workspace), true, true,
+                                        num_table_entries, static_cast<int32_t *>(workspace),
                                         static_cast<cudaStream_t>(stream_));
     if (e != cudaSuccess) { set_error("CUDA error: %s", cudaGetErrorString(e)); return SPLASH_CUDA_ERROR; }
     return SPLASH_OK;
@@ -516,7 +509,7 @@ int splash_kv_page_migrate_static(const void *src_pool, const float *src_scales,
     cudaError_t e = static_remap_address(&remap);      // first call on a device looks the symbol up
     if (e != cudaSuccess) { set_error("cudaGetSymbolAddress failed: %s", cudaGetErrorString(e)); return SPLASH_CUDA_ERROR; }
     e = launch_page_migrate(src_pool, src_scales, dst_pool, dst_scales, page_bytes, src_page_ids, dst_page_ids, n,
-                            src_id_base, dst_id_base, max_page_id, block_table, num_table_entries, remap, true, true,
+                            src_id_base, dst_id_base, max_page_id, block_table, num_table_entries, remap,
                             static_cast<cudaStream_t>(stream_));
     if (e != cudaSuccess) { set_error("CUDA error: %s", cudaGetErrorString(e)); return SPLASH_CUDA_ERROR; }
     return SPLASH_OK;

@@ -58,7 +58,6 @@ constexpr uint32_t kPageBytes = 9 * kSlab;          // 36,864
 constexpr uint32_t kPeerBytes = 4 * kSlab;          // the peer page's chunks this CTA multiplies: 16,384
 constexpr uint32_t kScaleBytes = 256;
 constexpr int kPrefetchAhead = 1;                    // supertiles between the L2 prefetch of a page and its use (4: 1.5 % slower; none: 5 %)
-constexpr int kPrefetchAheadBusy = 4;                // the same while the call carries a page-copy job
 constexpr float kTau = 7.0f;                          // (6 / 2.75: 0.3 % slower on the rollout workload, 4 / 4.75 more)
 constexpr float kLift = 1.75f;
 
@@ -239,8 +238,7 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
                             // A stage is held from its load until P.V has read it, about three supertiles, so the
                             // load of supertile s + 3 starts only when the issuers are about to need it: have its
                             // page in L2 by then.
-                            // (further ahead while a page-copy job shares the memory system: the loads then take longer)
-                            const int tf = ta + 2 * (p.mig_n > 0 ? kPrefetchAheadBusy : kPrefetchAhead) + (int)rank;
+                            const int tf = ta + 2 * kPrefetchAhead + (int)rank;
                             if (tf < seg.tile_end) {
                                 const int page_f = table[first_page + tf];
                                 if (page_f >= 0 && page_f < p.num_pool_pages) tma_prefetch_4d(&tmap_page, 0, 0, 0, page_f);
@@ -355,10 +353,7 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
             ++seg_it;
         }
     } else if (warp >= kWarpQk && warp < kWarpSoftmax) {
-        // the issuer warps of the peer CTA have nothing to do for the attention itself: they carry the call's page-copy
-        // job, if it has one (a layer's pages on the move while this layer decodes)
-        if (p.mig_n > 0)
-            copy_pages_in_idle_warp(p, pair_id * kIssuerWarps + (warp - kWarpQk), p.num_workers * p.pair_groups * kIssuerWarps, lane);
+        // (the issuer warps of the peer CTA have nothing to do)
     } else if (warp >= kWarpConvert && warp < kWarpConvert + kConvertWarps) {
         // ===================================================== query converters (this CTA's heads)
         const int ct = (warp - kWarpConvert) * 32 + lane;   // 0..127

@@ -58,7 +58,6 @@ constexpr uint32_t kQBytes = 9 * kQSlab;            // 73,728
 constexpr uint32_t kPHalfBytes = kN * 64;           // P of one half-page: 64 heads x 32 tokens bf16
 constexpr int kStages = 4;
 constexpr int kPrefetchAhead = 1;                   // tiles between the L2 prefetch of a page and its use (4: 3 % slower; none: 4 %)
-constexpr int kPrefetchAheadBusy = 4;               // the same while the call carries a page-copy job
 constexpr float kTau = 8.0f;                        // O is rescaled only when a row maximum grows by more than 2^8
 
 enum BarrierId {
@@ -194,8 +193,7 @@ decode_umma_pair_kernel(const __grid_constant__ DecodeParams p, const __grid_con
                             // A stage is held from its load until P.V has read it, about three tiles, so the
                             // load of tile t + 3 starts only when the issuers are about to need it: have its
                             // half of the page in L2 by then.
-                            // (further ahead while a page-copy job shares the memory system: the loads then take longer)
-                            const int tf = tile + (p.mig_n > 0 ? kPrefetchAheadBusy : kPrefetchAhead);
+                            const int tf = tile + kPrefetchAhead;
                             if (tf < seg.tile_end) {
                                 const int page_f = table[first_page + tf];
                                 // this CTA's half of the page is 32 consecutive rows: one contiguous range
@@ -307,10 +305,7 @@ decode_umma_pair_kernel(const __grid_constant__ DecodeParams p, const __grid_con
             ++seg_it;
         }
     } else if (warp >= kWarpQk && warp < kWarpSoftmax) {
-        // the issuer warps of the peer CTA have nothing to do for the attention itself: they carry the call's page-copy
-        // job, if it has one (a layer's pages on the move while this layer decodes)
-        if (p.mig_n > 0)
-            copy_pages_in_idle_warp(p, pair_id * kIssuerWarps + (warp - kWarpQk), p.num_workers * p.pair_groups * kIssuerWarps, lane);
+        // (the issuer warps of the peer CTA have nothing to do)
     } else if (kSparse && warp > kWarpVProducer) {
         // ===================================================== sparse decode: rows into the stages, in place of the TMA producers
         if constexpr (kSparse)

@@ -115,19 +115,17 @@ cudaError_t launch_page_migrate(const void *src_pool, const float *src_scales, v
                                 float *dst_scales, int64_t page_bytes, const int32_t *src_ids,
                                 const int32_t *dst_ids, int64_t n, int32_t src_base, int32_t dst_base,
                                 int32_t max_page_id, int32_t *block_table, int64_t num_entries,
-                                int32_t *remap, bool do_table, bool do_copy, cudaStream_t stream) {
+                                int32_t *remap, cudaStream_t stream) {
     MigrateParams p;
     p.src_pool = src_pool; p.dst_pool = dst_pool;
     p.src_scales = reinterpret_cast<const uint4 *>(src_scales); p.dst_scales = reinterpret_cast<uint4 *>(dst_scales);
     p.page_bytes = page_bytes; p.src_ids = src_ids; p.dst_ids = dst_ids; p.n = (int32_t)n;
     p.src_base = src_base; p.dst_base = dst_base; p.max_page_id = max_page_id;
     p.table = block_table; p.remap = remap; p.num_entries = num_entries;
-    const bool table = do_table && num_entries > 0 && max_page_id > 0;
-    const int64_t pages = do_copy ? n : 0;
+    const bool table = num_entries > 0 && max_page_id > 0;
     p.table_blocks = table ? (int32_t)((num_entries + kEntriesPerBlock - 1) / kEntriesPerBlock) : 0;
     p.after_scatter = table ? 1 : 0;
-    const int64_t blocks = pages + p.table_blocks;
-    if (blocks == 0) return cudaSuccess;
+    const int64_t blocks = n + p.table_blocks;
     p.spacing = p.table_blocks > 0 ? (int32_t)(blocks / p.table_blocks) : 1;
     cudaError_t e = cudaSuccess;
     if (table) {

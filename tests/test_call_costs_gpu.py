@@ -1,0 +1,48 @@
+"""Calls whose cost must follow from their parts or their bytes, whatever their shape: limits that lie far from what is measured (half
+as much again and more) and far from what went wrong (ten times and more)."""
+import pytest
+
+from paper_2609_37626_b200 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def device_us(call, repeat=10):
+    """The best of five: one call on the device, out of `repeat` queued behind work that covers their launches."""
+    import torch
+    call()
+    best = float("inf")
+    cover = torch.empty(1 << 28, dtype=torch.uint8, device="cuda")
+    for _ in range(5):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        for _ in range(4):
+            cover.zero_()
+        a.record()
+        for _ in range(repeat):
+            call()
+        b.record()
+        b.synchronize()
+        best = min(best, a.elapsed_time(b) * 1e3 / repeat)
+    return best
+
+
+@pytest.mark.parametrize("kv_dtype", [0, 1])
+@pytest.mark.parametrize("lens", [[200], [200] * 4, [4000] * 8, [64] * 40])
+def test_a_migration_job_costs_what_its_parts_cost(kv_dtype, lens):
+    import torch
+    from paper_2609_37626_b200 import binding
+    w = W.make_workload("cost", 9500 + len(lens), lens, H=128, kv_dtype=kv_dtype)
+    dw = binding.DeviceWorkload(w)
+    n = 800
+    shape = (n, 64, 576)
+    src = torch.zeros(shape, dtype=torch.uint8 if kv_dtype else torch.bfloat16, device="cuda")
+    dst = torch.empty_like(src)
+    sc = [torch.zeros((n, 64), device="cuda") for _ in range(2)] if kv_dtype else [None, None]
+    ids = torch.randperm(n, device="cuda").to(torch.int32)
+    table = torch.arange(n, dtype=torch.int32, device="cuda")
+    ws = torch.empty(1 << 20, dtype=torch.uint8, device="cuda")
+    args = dict(src_scales=sc[0], dst_scales=sc[1], dst_id_base=n, workspace=ws)
+    job = binding.make_migrate_job(src, dst, ids, ids, table, **args)
+    parts = device_us(dw.decode) + device_us(lambda: binding.splash_kv_page_migrate(src, dst, ids, ids, table, **args))
+    both = device_us(lambda: dw.decode(migrate_job=job))
+    assert both <= 1.5 * parts + 10, (both, parts)
