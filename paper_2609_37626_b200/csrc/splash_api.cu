@@ -210,10 +210,10 @@ int check_migrate_job(const splash_migrate_job *job) {
                               job->workspace, job->workspace_bytes);
 }
 
-cudaError_t run_migrate_job(const splash_migrate_job *job, cudaStream_t stream) {
+cudaError_t run_migrate_job(const splash_migrate_job *job, int sm_count, cudaStream_t stream) {
     return launch_page_migrate(job->src_pool, job->src_scales, job->dst_pool, job->dst_scales, job->page_bytes, job->src_page_ids,
                                job->dst_page_ids, job->n, job->src_id_base, job->dst_id_base, job->max_page_id, job->block_table,
-                               job->num_table_entries, static_cast<int32_t *>(job->workspace), stream);
+                               job->num_table_entries, static_cast<int32_t *>(job->workspace), sm_count, stream);
 }
 
 // One decode call: plan, decode kernel, combine.  With a sparse stage, seq_lens are the list counts; the decode kernel gathers
@@ -235,7 +235,9 @@ int decode_dense(const splash_mla_shape *shape, const void *q, const void *kv_po
     const int B = shape->num_requests;
     if (B == 0 || head_end == head_begin) {     // idle rank: no attention to compute; its pages still move
         if (job != nullptr) {
-            cudaError_t e = run_migrate_job(job, static_cast<cudaStream_t>(stream_));
+            DeviceInfo dev;
+            if (!current_device_info(dev)) return SPLASH_CUDA_ERROR;
+            cudaError_t e = run_migrate_job(job, dev.sm_count, static_cast<cudaStream_t>(stream_));
             if (e != cudaSuccess) { set_error("CUDA error: %s", cudaGetErrorString(e)); return SPLASH_CUDA_ERROR; }
         }
         return SPLASH_OK;
@@ -267,7 +269,7 @@ int decode_dense(const splash_mla_shape *shape, const void *q, const void *kv_po
     // the idle issuer warps of the CTA pairs, under the decode, is not the faster one: the pages and the cache share the DRAM, and two
     // warps a pair stay far below its rate.  10,000 pages beside 16 contexts of 32,768 tokens on 128 heads over e4m3: 463 us, 246 this
     // way; 2,000 beside one of 262,144 over bf16: 188 and 122; with four and six such warps a pair they had been 367 and 140.)
-    if (job != nullptr) e = run_migrate_job(job, stream);
+    if (job != nullptr) e = run_migrate_job(job, dev.sm_count, stream);
     Tiling t = choose_tiling(shape, h, dev.sm_count, simt);
     // where the work partition comes from (splash_common.cuh): a batch of up to 32 requests is planned by the decode kernel
     // itself; if its contexts are short besides, no request is cut and the combine kernel is left out
@@ -476,9 +478,11 @@ int splash_kv_page_migrate(const void *src_pool, const float *src_scales, void *
     const int rc = check_migrate_args(src_pool, src_scales, dst_pool, dst_scales, page_bytes, src_page_ids, dst_page_ids, n,
                                       max_page_id, block_table, num_table_entries, workspace, workspace_bytes);
     if (rc != SPLASH_OK || n == 0) return rc;
+    DeviceInfo dev;
+    if (!current_device_info(dev)) return SPLASH_CUDA_ERROR;
     cudaError_t e = launch_page_migrate(src_pool, src_scales, dst_pool, dst_scales, page_bytes, src_page_ids,
                                         dst_page_ids, n, src_id_base, dst_id_base, max_page_id, block_table,
-                                        num_table_entries, static_cast<int32_t *>(workspace),
+                                        num_table_entries, static_cast<int32_t *>(workspace), dev.sm_count,
                                         static_cast<cudaStream_t>(stream_));
     if (e != cudaSuccess) { set_error("CUDA error: %s", cudaGetErrorString(e)); return SPLASH_CUDA_ERROR; }
     return SPLASH_OK;
@@ -505,11 +509,13 @@ int splash_kv_page_migrate_static(const void *src_pool, const float *src_scales,
         set_error("misaligned pointer (pools, scales: 16 B)"); return SPLASH_INVALID_ARG;
     }
     if (n > 0x7fffffffLL) { set_error("too many pages"); return SPLASH_INVALID_ARG; }
+    DeviceInfo dev;
+    if (!current_device_info(dev)) return SPLASH_CUDA_ERROR;
     int32_t *remap = nullptr;
     cudaError_t e = static_remap_address(&remap);      // first call on a device looks the symbol up
     if (e != cudaSuccess) { set_error("cudaGetSymbolAddress failed: %s", cudaGetErrorString(e)); return SPLASH_CUDA_ERROR; }
     e = launch_page_migrate(src_pool, src_scales, dst_pool, dst_scales, page_bytes, src_page_ids, dst_page_ids, n,
-                            src_id_base, dst_id_base, max_page_id, block_table, num_table_entries, remap,
+                            src_id_base, dst_id_base, max_page_id, block_table, num_table_entries, remap, dev.sm_count,
                             static_cast<cudaStream_t>(stream_));
     if (e != cudaSuccess) { set_error("CUDA error: %s", cudaGetErrorString(e)); return SPLASH_CUDA_ERROR; }
     return SPLASH_OK;
@@ -559,8 +565,10 @@ int splash_dop_pack_rows(const void *a, int64_t a_part_bytes, int64_t a_row_pitc
     }
     if (a_head_pitch < a_part_bytes || (b && b_head_pitch < b_part_bytes)) { set_error("head pitch smaller than the part"); return SPLASH_INVALID_ARG; }
     if (n > 0x7fffffffLL) { set_error("too many rows"); return SPLASH_INVALID_ARG; }
+    DeviceInfo dev;
+    if (!current_device_info(dev)) return SPLASH_CUDA_ERROR;
     cudaError_t e = launch_dop_pack_rows(a, b, send, send_row, n, h, a_part_bytes, b_part_bytes, a_row_pitch, a_head_pitch,
-                                         b_row_pitch, b_head_pitch, static_cast<cudaStream_t>(stream_));
+                                         b_row_pitch, b_head_pitch, dev.sm_count, static_cast<cudaStream_t>(stream_));
     if (e != cudaSuccess) { set_error("CUDA error: %s", cudaGetErrorString(e)); return SPLASH_CUDA_ERROR; }
     return SPLASH_OK;
 }
@@ -575,7 +583,9 @@ int splash_dop_swap_outer(const void *in, int64_t A, int64_t B, int64_t inner_by
         const int64_t bytes = A * B * inner_bytes;
         if (po < pi + bytes && pi < po + bytes) { set_error("out overlaps in"); return SPLASH_INVALID_ARG; }
     }
-    cudaError_t e = launch_dop_swap_outer(in, out, A, B, inner_bytes, static_cast<cudaStream_t>(stream_));
+    DeviceInfo dev;
+    if (!current_device_info(dev)) return SPLASH_CUDA_ERROR;
+    cudaError_t e = launch_dop_swap_outer(in, out, A, B, inner_bytes, dev.sm_count, static_cast<cudaStream_t>(stream_));
     if (e != cudaSuccess) { set_error("CUDA error: %s", cudaGetErrorString(e)); return SPLASH_CUDA_ERROR; }
     return SPLASH_OK;
 }
@@ -589,7 +599,9 @@ int splash_dop_unpack_rows(const void *recv, const int32_t *send_row, int64_t n,
         set_error("a required pointer is NULL or misaligned"); return SPLASH_INVALID_ARG;
     }
     if (out_row_pitch < row_bytes) { set_error("out_row_pitch smaller than a row"); return SPLASH_INVALID_ARG; }
-    cudaError_t e = launch_dop_unpack_rows(recv, out, send_row, n, row_bytes, out_row_pitch,
+    DeviceInfo dev;
+    if (!current_device_info(dev)) return SPLASH_CUDA_ERROR;
+    cudaError_t e = launch_dop_unpack_rows(recv, out, send_row, n, row_bytes, out_row_pitch, dev.sm_count,
                                            static_cast<cudaStream_t>(stream_));
     if (e != cudaSuccess) { set_error("CUDA error: %s", cudaGetErrorString(e)); return SPLASH_CUDA_ERROR; }
     return SPLASH_OK;

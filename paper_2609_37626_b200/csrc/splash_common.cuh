@@ -477,10 +477,10 @@ cudaError_t launch_sparse_gather(int B, int max_sel, int pages_per_request, cons
                                  int32_t *dense_table, int sm_count, cudaStream_t stream);
 cudaError_t launch_dop_pack_rows(const void *a, const void *b, void *out, const int32_t *send_row, int64_t n, int h,
                                  int64_t a_bytes, int64_t b_bytes, int64_t a_row_pitch, int64_t a_head_pitch,
-                                 int64_t b_row_pitch, int64_t b_head_pitch, cudaStream_t stream);
+                                 int64_t b_row_pitch, int64_t b_head_pitch, int sm_count, cudaStream_t stream);
 cudaError_t launch_dop_unpack_rows(const void *recv, void *out, const int32_t *send_row, int64_t n, int64_t row_bytes,
-                                   int64_t out_row_pitch, cudaStream_t stream);
-cudaError_t launch_dop_swap_outer(const void *in, void *out, int64_t A, int64_t Bn, int64_t inner_bytes, cudaStream_t stream);
+                                   int64_t out_row_pitch, int sm_count, cudaStream_t stream);
+cudaError_t launch_dop_swap_outer(const void *in, void *out, int64_t A, int64_t Bn, int64_t inner_bytes, int sm_count, cudaStream_t stream);
 cudaError_t launch_decode_simt(const DecodeParams &p, int kv_dtype, cudaStream_t stream);
 int simt_heads_per_group();
 // tcgen05 kernel: how it cuts a head slice of width h into CTAs, and its launcher
@@ -497,7 +497,7 @@ cudaError_t launch_page_migrate(const void *src_pool, const float *src_scales, v
                                 float *dst_scales, int64_t page_bytes, const int32_t *src_ids,
                                 const int32_t *dst_ids, int64_t n, int32_t src_base, int32_t dst_base,
                                 int32_t max_page_id, int32_t *block_table, int64_t num_entries,
-                                int32_t *remap, cudaStream_t stream);
+                                int32_t *remap, int sm_count, cudaStream_t stream);
 
 cudaError_t static_remap_address(int32_t **ptr);
 

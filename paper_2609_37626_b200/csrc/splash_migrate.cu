@@ -31,10 +31,12 @@ struct MigrateParams {
     int64_t page_bytes;
     const int32_t *src_ids, *dst_ids;
     int32_t n, src_base, dst_base, max_page_id;
+    int32_t parts;                   // blocks per page, `per` vectors each
+    int64_t vecs, per;
     int32_t *table;
     const int32_t *remap;
     int64_t num_entries;
-    int32_t table_blocks, spacing;   // block r * spacing, r < table_blocks, rewrites a piece of the table, the others copy a page
+    int32_t table_blocks, spacing;   // block r * spacing, r < table_blocks, rewrites a piece of the table, the others copy pages
     int32_t after_scatter;           // 1: a remap_scatter_kernel, which has waited for the work before it, comes before this grid
 };
 
@@ -59,7 +61,7 @@ __device__ __forceinline__ void rewrite_entries(const MigrateParams &p, int64_t 
     }
 }
 
-// One block per page, with its scale page, and the table's rewrite in blocks spread evenly between them.  Bound by HBM.
+// One block per page, several for a large one (RowSplit), the first with its scale page, and the table's rewrite in blocks spread evenly between them.  Bound by HBM.
 template <typename Vec>
 __global__ void __launch_bounds__(kCopyThreads, 4)
 page_migrate_kernel(const __grid_constant__ MigrateParams p) {
@@ -72,12 +74,14 @@ page_migrate_kernel(const __grid_constant__ MigrateParams p) {
         rewrite_entries(p, b / p.spacing);
         return;
     }
-    const int j = b - before;
+    const int x = b - before, j = p.parts == 1 ? x : x / p.parts;
+    const int64_t first = p.parts == 1 ? 0 : (x - j * p.parts) * p.per;
     const int64_t s = p.src_ids[j], d = p.dst_ids[j];
-    const int vecs = (int)(p.page_bytes / (int64_t)sizeof(Vec));
-    const Vec *src = reinterpret_cast<const Vec *>(static_cast<const char *>(p.src_pool) + s * p.page_bytes);
-    Vec *dst = reinterpret_cast<Vec *>(static_cast<char *>(p.dst_pool) + d * p.page_bytes);
-    copy_row(dst, vecs, [&](int c) { return src + c; });
+    const Vec *src = reinterpret_cast<const Vec *>(static_cast<const char *>(p.src_pool) + s * p.page_bytes) + first;
+    Vec *dst = reinterpret_cast<Vec *>(static_cast<char *>(p.dst_pool) + d * p.page_bytes) + first;
+    const int count = p.parts == 1 ? (int)p.vecs : (int)min(p.per, p.vecs - first);      // (none at the end of some)
+    copy_row<true>(dst, count, kCopyThreads, [&](int c) { return src + c; });
+    if (first > 0) return;
     if (p.src_scales != nullptr && threadIdx.x < kScaleVecs)
         p.dst_scales[d * kScaleVecs + threadIdx.x] = __ldg(p.src_scales + s * kScaleVecs + threadIdx.x);
 }
@@ -115,7 +119,7 @@ cudaError_t launch_page_migrate(const void *src_pool, const float *src_scales, v
                                 float *dst_scales, int64_t page_bytes, const int32_t *src_ids,
                                 const int32_t *dst_ids, int64_t n, int32_t src_base, int32_t dst_base,
                                 int32_t max_page_id, int32_t *block_table, int64_t num_entries,
-                                int32_t *remap, cudaStream_t stream) {
+                                int32_t *remap, int sm_count, cudaStream_t stream) {
     MigrateParams p;
     p.src_pool = src_pool; p.dst_pool = dst_pool;
     p.src_scales = reinterpret_cast<const uint4 *>(src_scales); p.dst_scales = reinterpret_cast<uint4 *>(dst_scales);
@@ -125,7 +129,11 @@ cudaError_t launch_page_migrate(const void *src_pool, const float *src_scales, v
     const bool table = num_entries > 0 && max_page_id > 0;
     p.table_blocks = table ? (int32_t)((num_entries + kEntriesPerBlock - 1) / kEntriesPerBlock) : 0;
     p.after_scatter = table ? 1 : 0;
-    const int64_t blocks = n + p.table_blocks;
+    // (in 32-byte vectors where the pages lie on 32-byte boundaries: they do in every pool of whole pages whose base does)
+    const bool wide = copy_width(address_bits(src_pool) | address_bits(dst_pool) | (uint64_t)page_bytes) == 32;
+    const RowSplit split(n, page_bytes / (wide ? 32 : 16), wide ? 32 : 16, sm_count);
+    p.parts = split.parts; p.vecs = split.vecs; p.per = split.per;
+    const int64_t blocks = n * p.parts + p.table_blocks;
     p.spacing = p.table_blocks > 0 ? (int32_t)(blocks / p.table_blocks) : 1;
     cudaError_t e = cudaSuccess;
     if (table) {
@@ -134,8 +142,6 @@ cudaError_t launch_page_migrate(const void *src_pool, const float *src_scales, v
         count_launch();
         if (e != cudaSuccess) return e;
     }
-    // 32-byte accesses where the pages lie on 32-byte boundaries (they do in every pool of whole pages whose base does)
-    const bool wide = copy_width(address_bits(src_pool) | address_bits(dst_pool) | (uint64_t)page_bytes) == 32;
     e = launch_dependent(wide ? page_migrate_kernel<Vec32> : page_migrate_kernel<uint4>, dim3((unsigned)blocks), dim3(kCopyThreads), 0, stream, p);
     count_launch();
     return e;

@@ -46,3 +46,33 @@ def test_a_migration_job_costs_what_its_parts_cost(kv_dtype, lens):
     parts = device_us(dw.decode) + device_us(lambda: binding.splash_kv_page_migrate(src, dst, ids, ids, table, **args))
     both = device_us(lambda: dw.decode(migrate_job=job))
     assert both <= 1.5 * parts + 10, (both, parts)
+
+
+@pytest.mark.parametrize("n,h,d", [(16384, 1, 576), (65536, 1, 144), (24, 1, 393216)])
+def test_rows_of_any_length_move_at_one_rate(n, h, d):
+    """The same 19 MB as 1,024 positions of 16 heads."""
+    import torch
+    from paper_2609_37626_b200 import binding
+
+    def us(n, h, d):
+        a = torch.zeros((n, h, d), dtype=torch.bfloat16, device="cuda")
+        out = torch.empty_like(a)
+        row = torch.randperm(n, device="cuda").to(torch.int32)
+        return (device_us(lambda: binding.splash_dop_pack_rows(a, None, row, out)), device_us(lambda: binding.splash_dop_unpack_rows(a, row, out)),
+                device_us(lambda: binding.splash_dop_swap_outer(a.view(8, n // 8, h, d), out.view(n // 8, 8, h, d))))
+
+    for got, usual in zip(us(n, h, d), us(1024, 16, 576)):
+        assert got <= 2 * usual + 3, (got, usual)
+
+
+def test_large_pages_move_at_the_rate_of_many_small_ones():
+    import torch
+    from paper_2609_37626_b200 import binding
+
+    def us(n, page):
+        src = torch.zeros((n, 16, page // 16), dtype=torch.uint8, device="cuda")
+        dst, ids, table = torch.empty_like(src), torch.randperm(n, device="cuda").to(torch.int32), torch.arange(n, dtype=torch.int32, device="cuda")
+        return device_us(lambda: binding.splash_kv_page_migrate(src, dst, ids, ids, table, dst_id_base=n))
+
+    large, small = us(8, 1 << 20), us(228, 36864)
+    assert large <= 2 * small + 3, (large, small)

@@ -55,3 +55,18 @@ def test_migrate_pages_and_table(page_bytes, entries):
     assert np.array_equal(dst.cpu().numpy(), want)
     move = {int(a): n_src + int(b) for a, b in zip(src_ids, dst_ids)}
     assert np.array_equal(t.cpu().numpy(), np.array([move.get(int(e), int(e)) for e in table], np.int32))
+
+
+def test_a_position_of_more_vectors_than_an_int_counts():
+    """2^31 and some 2-byte vectors in one position (odd addresses: no wider path), 4 GiB in and as much out."""
+    import torch
+    from paper_2609_37626_b200 import binding
+    d, h = (1 << 20) + 1, 2049                     # h * d = 2^31 + 2^20 + 2049
+    a = torch.empty((1, h, d), dtype=torch.int16, device="cuda")
+    a.view(-1)[:1 << 20] = torch.arange(1 << 20, device="cuda").to(torch.int16)
+    a.view(-1)[1 << 20:] = 17
+    a[0, :, 0] = torch.arange(h, device="cuda").to(torch.int16)
+    a[0, :, -1] = -torch.arange(h, device="cuda").to(torch.int16)
+    out = torch.zeros_like(a)
+    binding.splash_dop_pack_rows(a, None, torch.zeros(1, dtype=torch.int32, device="cuda"), out)
+    assert torch.equal(out, a)
