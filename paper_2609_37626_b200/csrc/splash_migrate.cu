@@ -15,7 +15,7 @@ constexpr int kScaleVecs = kPage * 4 / 16;  // 16-byte vectors of a scale page
 __global__ void __launch_bounds__(kCopyThreads)
 remap_scatter_kernel(int32_t *remap, const int32_t *__restrict__ src_ids, int64_t n, int32_t src_base, int32_t max_page_id) {
     grid_dependency_wait();         // launched while the work before it on the stream still runs
-    grid_launch_dependents();       // the pages may be copied meanwhile; the table's blocks wait for this grid
+    grid_launch_dependents();       // the copy's blocks may come in; they wait for this grid
     const int64_t j = (int64_t)blockIdx.x * kCopyThreads + threadIdx.x;
     if (j < n) {
         const int32_t s = src_base + src_ids[j];
@@ -37,7 +37,6 @@ struct MigrateParams {
     const int32_t *remap;
     int64_t num_entries;
     int32_t table_blocks, spacing;   // block r * spacing, r < table_blocks, rewrites a piece of the table, the others copy pages
-    int32_t after_scatter;           // 1: a remap_scatter_kernel, which has waited for the work before it, comes before this grid
 };
 
 constexpr int kEntriesPerBlock = kCopyThreads * 4;
@@ -65,12 +64,12 @@ __device__ __forceinline__ void rewrite_entries(const MigrateParams &p, int64_t 
 template <typename Vec>
 __global__ void __launch_bounds__(kCopyThreads, 4)
 page_migrate_kernel(const __grid_constant__ MigrateParams p) {
-    if (!p.after_scatter) grid_dependency_wait();
+    // Every block, those that copy too: that the scatter kernel has waited for the work in front says nothing to a block that does not.
+    grid_dependency_wait();
     grid_launch_dependents();
     const int b = blockIdx.x;
     const int before = min(p.table_blocks, b / p.spacing + 1);     // table blocks up to and including this place
     if (b % p.spacing == 0 && b / p.spacing < p.table_blocks) {
-        if (p.after_scatter) grid_dependency_wait();
         rewrite_entries(p, b / p.spacing);
         return;
     }
@@ -128,7 +127,6 @@ cudaError_t launch_page_migrate(const void *src_pool, const float *src_scales, v
     p.table = block_table; p.remap = remap; p.num_entries = num_entries;
     const bool table = num_entries > 0 && max_page_id > 0;
     p.table_blocks = table ? (int32_t)((num_entries + kEntriesPerBlock - 1) / kEntriesPerBlock) : 0;
-    p.after_scatter = table ? 1 : 0;
     // (in 32-byte vectors where the pages lie on 32-byte boundaries: they do in every pool of whole pages whose base does)
     const bool wide = copy_width(address_bits(src_pool) | address_bits(dst_pool) | (uint64_t)page_bytes) == 32;
     const RowSplit split(n, page_bytes / (wide ? 32 : 16), wide ? 32 : 16, sm_count);
