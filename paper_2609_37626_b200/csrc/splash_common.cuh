@@ -155,6 +155,15 @@ struct Segment {
 // own set-up (barriers, tensor memory), and blocks in grid_dependency_wait() before it
 // touches anything the predecessor wrote.
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// What a kernel reads behind its wait may have been written while it was already resident, by the kernel in front of it.  So it is
+// never read through the read-only path (__ldg, const __restrict__ parameters): such data counts as unchanged for the kernel's
+// lifetime, and a load of it may be moved over the wait.  Plain loads may not; nor these, which go to L2 past a line that a read
+// before the wait has left in L1, and are not merged with that read.
+__device__ __forceinline__ int32_t load_l2(const int32_t *ptr) {
+    int32_t v;
+    asm volatile("ld.global.cg.b32 %0, [%1];" : "=r"(v) : "l"(ptr) : "memory");
+    return v;
+}
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Where a decode kernel's partition comes from.  Workspace: the plan kernel wrote it.  Inline: a batch of at most 32
@@ -173,8 +182,8 @@ constexpr uint32_t kInlinePlanBytes = ((3 * kInlinePlanRequests + 4) * 4 + 15) /
 // Effective range of request i (the rule of the plan kernel).
 __device__ __forceinline__ void effective_range(int s, const int32_t *kv_begin, const int32_t *kv_end, int i, int len_cap, int &lo, int &hi) {
     if (len_cap >= 0 && (s < 0 || s > len_cap)) s = 1;     // a list count out of bounds: one (poisoned) row
-    lo = kv_begin ? __ldcg(kv_begin + i) : 0;
-    hi = kv_end ? __ldcg(kv_end + i) : s;
+    lo = kv_begin ? load_l2(kv_begin + i) : 0;
+    hi = kv_end ? load_l2(kv_end + i) : s;
     if (lo < 0) lo = 0;
     if (hi > s) hi = s;
     if (hi < lo) hi = lo;
@@ -189,7 +198,7 @@ __device__ __forceinline__ int cost_target(int total, int w, int W) {
 // The lengths of a batch of at most 32 requests, a request per lane: its effective range.
 __device__ __forceinline__ void lane_range(const DecodeParams &p, int lane, int &lo, int &hi) {
     lo = hi = 0;
-    if (lane < p.B) effective_range(__ldcg(p.seq_lens + lane), p.kv_begin, p.kv_end, lane, p.len_cap, lo, hi);
+    if (lane < p.B) effective_range(load_l2(p.seq_lens + lane), p.kv_begin, p.kv_end, lane, p.len_cap, lo, hi);
 }
 
 // One warp of a CTA: the plan, as far as worker `worker` needs it, from the lanes' ranges.
@@ -245,7 +254,7 @@ static __device__ __noinline__ void plan_ahead(const DecodeParams &p, int worker
         while (r + 1 < B && sp[r + 1] <= x) ++r;
         const int64_t idx = (int64_t)sp[B + 1 + r] / kPage + (x - sp[r]);
         if (idx >= 0 && idx < p.table_stride) {
-            const int page = __ldcg(p.block_table + (int64_t)r * p.table_stride + idx);
+            const int page = load_l2(p.block_table + (int64_t)r * p.table_stride + idx);
             if (page >= 0 && page < p.num_pool_pages) {
                 asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;"
                              ::"l"(static_cast<const uint8_t *>(p.kv_pool) + (size_t)page * f.page_bytes + f.offset), "r"(f.bytes) : "memory");

@@ -15,15 +15,15 @@ constexpr int kCopyDepth = 5;               // loads in flight per thread
 struct alignas(32) Vec32 { uint32_t v[8]; };
 
 __device__ __forceinline__ void load_stream(Vec32 &x, const Vec32 *ptr) {
-    asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                 : "=r"(x.v[0]), "=r"(x.v[1]), "=r"(x.v[2]), "=r"(x.v[3]), "=r"(x.v[4]), "=r"(x.v[5]), "=r"(x.v[6]), "=r"(x.v[7]) : "l"(ptr));
+    asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(x.v[0]), "=r"(x.v[1]), "=r"(x.v[2]), "=r"(x.v[3]), "=r"(x.v[4]), "=r"(x.v[5]), "=r"(x.v[6]), "=r"(x.v[7]) : "l"(ptr) : "memory");
 }
 __device__ __forceinline__ void store_stream(Vec32 *ptr, const Vec32 &x) {
     asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
                  ::"l"(ptr), "r"(x.v[0]), "r"(x.v[1]), "r"(x.v[2]), "r"(x.v[3]), "r"(x.v[4]), "r"(x.v[5]), "r"(x.v[6]), "r"(x.v[7]) : "memory");
 }
 template <typename Vec>
-__device__ __forceinline__ void load_stream(Vec &x, const Vec *ptr) { x = __ldg(ptr); }
+__device__ __forceinline__ void load_stream(Vec &x, const Vec *ptr) { x = *ptr; }
 template <typename Vec>
 __device__ __forceinline__ void store_stream(Vec *ptr, const Vec &x) { *ptr = x; }
 

@@ -286,7 +286,7 @@ decode_umma_fp8_kernel(const __grid_constant__ DecodeParams p, const __grid_cons
                 if (live) {
 #pragma unroll 6
                     for (int v = 0; v < 36; ++v) {
-                        uint4 x = __ldg(src + v);
+                        uint4 x = src[v];
                         const uint32_t w[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
                         for (int k = 0; k < 4; ++k) {
@@ -301,7 +301,7 @@ decode_umma_fp8_kernel(const __grid_constant__ DecodeParams p, const __grid_cons
                 if (part == 0) qs_s[(seg_it & 3) * kN + hd] = qs;
 #pragma unroll 2
                 for (int v = 0; v < 36; ++v) {
-                    uint4 x = live ? __ldg(src + v) : make_uint4(0u, 0u, 0u, 0u);
+                    uint4 x = live ? src[v] : make_uint4(0u, 0u, 0u, 0u);
                     const uint32_t w[4] = {x.x, x.y, x.z, x.w};
                     uint16_t hi[4], lo[4];
 #pragma unroll

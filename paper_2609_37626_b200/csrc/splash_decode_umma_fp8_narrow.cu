@@ -317,7 +317,7 @@ decode_umma_fp8_narrow_kernel(const __grid_constant__ DecodeParams p, const __gr
                 uint4 x[kVecs];
                 float amax = 0.f;
 #pragma unroll
-                for (int v = 0; v < kVecs; ++v) x[v] = live ? __ldg(src + v) : make_uint4(0u, 0u, 0u, 0u);
+                for (int v = 0; v < kVecs; ++v) x[v] = live ? src[v] : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
                 for (int v = 0; v < kVecs; ++v) {
                     const uint32_t w[4] = {x[v].x, x[v].y, x[v].z, x[v].w};

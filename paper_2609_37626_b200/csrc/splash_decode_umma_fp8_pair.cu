@@ -376,7 +376,7 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
                     for (int v0 = 0; v0 < kVecs; v0 += kVecs / 3) {
                         uint4 x[kVecs / 3];
 #pragma unroll
-                        for (int i = 0; i < kVecs / 3; ++i) x[i] = __ldg(src + v0 + i);
+                        for (int i = 0; i < kVecs / 3; ++i) x[i] = src[v0 + i];
 #pragma unroll
                         for (int i = 0; i < kVecs / 3; ++i) {
                             const uint32_t w[4] = {x[i].x, x[i].y, x[i].z, x[i].w};
@@ -399,7 +399,7 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
                 uint4 xa[9], xb[9];
                 auto load_batch = [&](uint4 (&x)[9], int v0) {
 #pragma unroll
-                    for (int i = 0; i < 9; ++i) x[i] = live ? __ldg(src + v0 + i) : make_uint4(0u, 0u, 0u, 0u);
+                    for (int i = 0; i < 9; ++i) x[i] = live ? src[v0 + i] : make_uint4(0u, 0u, 0u, 0u);
                 };
                 auto convert_batch = [&](const uint4 (&x)[9], int v0) {
 #pragma unroll

@@ -22,7 +22,7 @@ namespace {
 // A position: h rows of va + vb vectors.
 template <typename Vec, bool kBlock>
 __global__ void __launch_bounds__(kCopyThreads, 4)
-pack_rows_kernel(const Vec *__restrict__ a, const Vec *__restrict__ b, Vec *__restrict__ out, const int32_t *__restrict__ send_row, int64_t n,
+pack_rows_kernel(const Vec *a, const Vec *b, Vec *out, const int32_t *send_row, int64_t n,
                  const RowSplit split, int va, int vb, int64_t a_row_pitch, int64_t a_head_pitch, int64_t b_row_pitch, int64_t b_head_pitch) {
     grid_dependency_wait();       // launched while the work before it on the stream still runs
     grid_launch_dependents();
@@ -41,7 +41,7 @@ pack_rows_kernel(const Vec *__restrict__ a, const Vec *__restrict__ b, Vec *__re
 
 template <typename Vec, bool kBlock>
 __global__ void __launch_bounds__(kCopyThreads, 4)
-unpack_rows_kernel(const Vec *__restrict__ recv, Vec *__restrict__ out, const int32_t *__restrict__ send_row, int64_t n, const RowSplit split,
+unpack_rows_kernel(const Vec *recv, Vec *out, const int32_t *send_row, int64_t n, const RowSplit split,
                    int64_t out_row_pitch) {
     grid_dependency_wait();
     grid_launch_dependents();
@@ -54,7 +54,7 @@ unpack_rows_kernel(const Vec *__restrict__ recv, Vec *__restrict__ out, const in
 // block (s, r) of `split.vecs` vectors moves from in[s][r] to out[r][s]
 template <typename Vec, bool kBlock>
 __global__ void __launch_bounds__(kCopyThreads, 4)
-swap_outer_kernel(const Vec *__restrict__ in, Vec *__restrict__ out, int64_t A, int64_t Bn, const RowSplit split) {
+swap_outer_kernel(const Vec *in, Vec *out, int64_t A, int64_t Bn, const RowSplit split) {
     grid_dependency_wait();
     grid_launch_dependents();
     own_row<kBlock>(split, A * Bn, [&](int64_t blk, int64_t first, int vecs) {

@@ -26,9 +26,16 @@ namespace gather {
 // What a lane knows about a row: its address, or one of these
 constexpr unsigned long long kSkip = 0, kPoison = 1;           // no such row (zeros); a bad list entry, page id or count (NaN)
 
+// 16 bytes at a global address (a plain load of an address made from an integer would be a generic one)
+__device__ __forceinline__ uint4 load_global16(unsigned long long at) {
+    uint4 v;
+    asm volatile("ld.global.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(at) : "memory");
+    return v;
+}
+
 // 16 codes of a row or 16 bytes of its rope part
 __device__ __forceinline__ uint4 load16(unsigned long long row, uint32_t offset, uint32_t poison) {
-    if (row > kPoison) return __ldg(reinterpret_cast<const uint4 *>(row + offset));
+    if (row > kPoison) return load_global16(row + offset);
     const uint32_t fill = row == kPoison ? poison : 0u;
     return make_uint4(fill, fill, fill, fill);
 }
@@ -95,16 +102,16 @@ struct Resolver {
         bool any = row[0] != kSkip;
         if constexpr (kPeer) any |= row[1] != kSkip;
         if (!any) return;
-        if (step == 0) { cnt = __ldg(p.seq_lens + req); len = __ldg(p.ctx_lens + req); }
+        if (step == 0) { cnt = p.seq_lens[req]; len = p.ctx_lens[req]; }
 #pragma unroll
         for (int s = 0; s < kSets; ++s) {
             if (row[s] == kSkip) continue;
             if (step == 0) {
-                tok[s] = idx[s] < p.len_cap ? __ldg(p.sel + (int64_t)req * p.sel_stride + idx[s]) : -1;
+                tok[s] = idx[s] < p.len_cap ? p.sel[(int64_t)req * p.sel_stride + idx[s]] : -1;
             } else if (step == 1) {
                 // (a count outside [0, len_cap] stands for one poisoned row)
                 if (cnt < 0 || cnt > p.len_cap || tok[s] >= len) tok[s] = -1;
-                page[s] = tok[s] >= 0 ? __ldg(p.block_table + (int64_t)req * p.table_stride + tok[s] / kPage) : -1;
+                page[s] = tok[s] >= 0 ? p.block_table[(int64_t)req * p.table_stride + tok[s] / kPage] : -1;
             } else {
                 row[s] = page[s] < 0 || page[s] >= p.num_pool_pages ? kPoison
                     : reinterpret_cast<unsigned long long>(p.kv_pool) + (unsigned long long)((int64_t)page[s] * kPage + tok[s] % kPage) * kSparseRowBytes;
@@ -144,13 +151,15 @@ __device__ __forceinline__ void gather_tiles(const DecodeParams &p, const Iter &
     float4 scale;
     float peer_scale[2];
     auto load_scales = [](unsigned long long row) {
-        return row > kPoison ? __ldg(reinterpret_cast<const float4 *>(row + kDLatent)) : make_float4(1.f, 1.f, 1.f, 1.f);
+        const uint4 s = row > kPoison ? load_global16(row + kDLatent) : make_uint4(0x3f800000u, 0x3f800000u, 0x3f800000u, 0x3f800000u);
+        return make_float4(__uint_as_float(s.x), __uint_as_float(s.y), __uint_as_float(s.z), __uint_as_float(s.w));
     };
     auto load_peer = [&](unsigned long long row) {
 #pragma unroll
         for (int n = 0; n < 2; ++n) {
             peer_codes[n] = load16(row, (2 * n + rank) * 128 + 16 * x, kPoisonCodes);
-            peer_scale[n] = row > kPoison ? __ldg(reinterpret_cast<const float *>(row + kDLatent) + 2 * n + rank) : 1.f;
+            peer_scale[n] = 1.f;
+            if (row > kPoison) asm volatile("ld.global.f32 %0, [%1];" : "=f"(peer_scale[n]) : "l"(row + kDLatent + (2 * n + rank) * 4) : "memory");
         }
     };
     {

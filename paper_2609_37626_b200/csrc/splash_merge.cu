@@ -24,8 +24,7 @@ __device__ __forceinline__ float reference_max(float m) { return m == -INFINITY 
 // than the SMs hold at a time, four loads each and twelve blocks to an SM instead of eight.
 template <int kDepth>
 __global__ void __launch_bounds__(kMergeThreads, kDepth == 8 ? 8 : 12)
-lse_merge_kernel(int num_parts, int64_t rows, int d_v, const float *__restrict__ part_out,
-                 const float *__restrict__ part_lse, float *__restrict__ out, float *__restrict__ lse) {
+lse_merge_kernel(int num_parts, int64_t rows, int d_v, const float *part_out, const float *part_lse, float *out, float *lse) {
     __shared__ float w_s[kMergeThreads], red_s[2][kMergeThreads / 32];
     grid_launch_dependents();
     grid_dependency_wait();       // launched while the work before it on the stream still runs
@@ -92,7 +91,7 @@ constexpr int kMaxParts = 512;     // >= number of workers of any launch (one pe
 // the kernel is how many of them an SM holds at a time.
 template <bool kF16, bool kLean>
 __global__ void __launch_bounds__(kMergeThreads, kLean ? 16 : 8)
-split_combine_kernel(const DecodeParams p, const int4 *__restrict__ split_rec) {
+split_combine_kernel(const DecodeParams p, const int4 *split_rec) {
     __shared__ float w_s[kMaxParts];
     __shared__ float sc_s[kF16 ? kMaxParts : 1];      // f16 pieces: the power of two each row was divided by
     __shared__ int slot_s[kMaxParts];
@@ -217,7 +216,7 @@ split_combine_kernel(const DecodeParams p, const int4 *__restrict__ split_rec) {
 constexpr int kGroupedParts = 160, kCombineGroups = 4;
 template <bool kF16>
 __global__ void __launch_bounds__(kCombineGroups * kMergeThreads, 4)
-grouped_combine_kernel(const DecodeParams p, const int4 *__restrict__ split_rec) {
+grouped_combine_kernel(const DecodeParams p, const int4 *split_rec) {
     constexpr int kThreads = kCombineGroups * kMergeThreads, kDepth = 4;
     // weights, slots and (f16 pieces) the power of two each row was divided by; then the groups' sums
     constexpr int kFloats = (kF16 ? 3 : 2) * kGroupedParts;

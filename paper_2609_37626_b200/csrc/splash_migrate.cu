@@ -13,7 +13,7 @@ constexpr int kScaleVecs = kPage * 4 / 16;  // 16-byte vectors of a scale page
 // its own): an entry nobody wrote in this call holds anything, and the rewrite believes an entry only if the page that it
 // names does have that id.
 __global__ void __launch_bounds__(kCopyThreads)
-remap_scatter_kernel(int32_t *remap, const int32_t *__restrict__ src_ids, int64_t n, int32_t src_base, int32_t max_page_id) {
+remap_scatter_kernel(int32_t *remap, const int32_t *src_ids, int64_t n, int32_t src_base, int32_t max_page_id) {
     grid_dependency_wait();         // launched while the work before it on the stream still runs
     grid_launch_dependents();       // the copy's blocks may come in; they wait for this grid
     const int64_t j = (int64_t)blockIdx.x * kCopyThreads + threadIdx.x;
@@ -82,7 +82,7 @@ page_migrate_kernel(const __grid_constant__ MigrateParams p) {
     copy_row<true>(dst, count, kCopyThreads, [&](int c) { return src + c; });
     if (first > 0) return;
     if (p.src_scales != nullptr && threadIdx.x < kScaleVecs)
-        p.dst_scales[d * kScaleVecs + threadIdx.x] = __ldg(p.src_scales + s * kScaleVecs + threadIdx.x);
+        p.dst_scales[d * kScaleVecs + threadIdx.x] = p.src_scales[s * kScaleVecs + threadIdx.x];
 }
 
 // Remap table of the allocation-free entry point: lives in the library's device image,

@@ -24,8 +24,8 @@ constexpr int kPlanSmemWorkers = 512;
 // bisections, the stores) and comes on top of every call of more than 32 requests.  As many threads as there are requests
 // or workers, one barrier per 1,024 requests in the scan, 32-bit arithmetic.
 __global__ void __launch_bounds__(kPlanThreads)
-plan_kernel(int B, int W, int overhead, int len_cap, const int32_t *__restrict__ seq_lens, const int32_t *__restrict__ kv_begin,
-            const int32_t *__restrict__ kv_end, int32_t *tile_start,
+plan_kernel(int B, int W, int overhead, int len_cap, const int32_t *seq_lens, const int32_t *kv_begin,
+            const int32_t *kv_end, int32_t *tile_start,
             int32_t *__restrict__ req_lo, int32_t *__restrict__ req_hi,
             int32_t *__restrict__ req_wfirst, int32_t *__restrict__ req_wlast,
             int32_t *cost_start, int32_t *worker_begin, int32_t *__restrict__ split_list, int32_t *__restrict__ worker_req,

@@ -331,7 +331,7 @@ __device__ __forceinline__ void fill_rows_by_hand(uint8_t *slabs, uint32_t slab_
         const int t = tok_first + r;
         uint4 v = make_uint4(0u, 0u, 0u, 0u);
         if (page != nullptr && t >= a && t < b)
-            v = __ldg(reinterpret_cast<const uint4 *>(page + (size_t)t * (9 * kChunkBytes) + (size_t)(src_chunk0 + c) * kChunkBytes + j * 16));
+            v = *reinterpret_cast<const uint4 *>(page + (size_t)t * (9 * kChunkBytes) + (size_t)(src_chunk0 + c) * kChunkBytes + j * 16);
         const int sw = kChunkBytes == 128 ? (r & 7) : ((r >> 1) & 3);
         *reinterpret_cast<uint4 *>(slabs + (size_t)(dst_slot0 + c) * slab_bytes + (size_t)r * kChunkBytes + ((j ^ sw) << 4)) = v;
     }
