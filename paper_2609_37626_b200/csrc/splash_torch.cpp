@@ -467,9 +467,10 @@ PyObject *dop_unpack_rows(PyObject *, PyObject *const *args, Py_ssize_t nargs, P
     if (!(recv = tensor(v[0], "recv")) || !(row = tensor(v[1], "send_row")) || !(out = tensor(v[2], "out"))) return nullptr;
     SPLASH_ASSERT(recv->is_contiguous() && row->scalar_type() == at::kInt && row->is_contiguous());
     if (out->size(0) > 0) {
-        SPLASH_ASSERT(recv->sizes().slice(1) == out->sizes().slice(1));
-        int64_t dense = 1;                          // every row of out is dense (the rows themselves may lie apart)
-        for (int64_t k = out->dim() - 1; k >= 1; --k) {
+        auto of_a_row = [](const at::Tensor &t) { return t.dim() > 0 ? t.sizes().slice(1) : at::IntArrayRef(); };
+        SPLASH_ASSERT(of_a_row(*recv) == of_a_row(*out));
+        int64_t dense = 1;                          // every row of out is dense (the rows themselves may lie apart, and one without elements is)
+        for (int64_t k = out->dim() - 1; k >= 1 && out->numel() > 0; --k) {
             SPLASH_ASSERT(out->size(k) == 1 || out->stride(k) == dense);
             dense *= out->size(k);
         }
