@@ -11,11 +11,14 @@ C++; the rest goes through ctypes.
 from __future__ import annotations
 
 import ctypes
-import importlib
+import importlib.util
 import os
+import sys
 from typing import Optional
 
 import torch
+
+from . import build as _build
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libsplash_mla.so")
@@ -188,11 +191,18 @@ def _load_ext():
     """Import ``_splash_torch`` and put its functions in this module's namespace (raises if it has not been built)."""
     global _ext
     load()
-    try:
-        _ext = importlib.import_module("._splash_torch", __package__)
-    except ImportError as e:
-        raise ImportError(f"{__package__}._splash_torch does not load ({e}): build it with `python -m {__package__}.build` "
-                          "(there is no fallback)") from e
+    name, path = f"{__package__}._splash_torch", _build.torch_ext_path()
+    ext = sys.modules.get(name)
+    if ext is None:
+        try:
+            spec = importlib.util.spec_from_file_location(name, path)
+            ext = importlib.util.module_from_spec(spec)
+            spec.loader.exec_module(ext)
+        except ImportError as e:
+            raise ImportError(f"{path} does not load ({e}): build it for torch {torch.__version__} with "
+                              f"`python -m {__package__}.build` (there is no fallback)") from e
+        sys.modules[name] = ext
+    _ext = ext
     _ext.set_error_class(SplashError)
     for name in _NATIVE:
         globals()[name] = getattr(_ext, name)
@@ -205,7 +215,7 @@ def __getattr__(name):     # first use of a native function where the module was
     raise AttributeError(f"module {__name__!r} has no attribute {name!r}")
 
 
-if os.path.exists(LIB_PATH) and os.path.exists(os.path.join(_HERE, "_splash_torch.so")):
+if os.path.exists(LIB_PATH) and os.path.exists(_build.torch_ext_path()):
     _load_ext()
 
 
