@@ -128,9 +128,10 @@ decode_umma_pair_kernel(const __grid_constant__ DecodeParams p, const __grid_con
     if (tid == 0) {
         // barriers the leader's issuers wait on count the warps of both CTAs (the peer's copies are unused)
         for (int s = 0; s < kStages; ++s) {
-            constexpr int kFilled = kSparse ? 2 * kGatherWarps : 1;       // by the gathering warps of both CTAs, or by bytes
-            mbar_init(bar(kBarKFull + s), kFilled); mbar_init(bar(kBarQkDone + s), 1);
-            mbar_init(bar(kBarVFull + s), kFilled); mbar_init(bar(kBarStageEmpty + s), 1);
+            // by the gathering warps (the leader's also by the peer's relay, see there), or by bytes
+            const int filled = kSparse ? kGatherWarps + (rank == 0 ? 1 : 0) : 1;
+            mbar_init(bar(kBarKFull + s), filled); mbar_init(bar(kBarQkDone + s), 1);
+            mbar_init(bar(kBarVFull + s), filled); mbar_init(bar(kBarStageEmpty + s), 1);
         }
         mbar_init(bar(kBarQFull), 1); mbar_init(bar(kBarQEmpty), 1);
         for (int b = 0; b < 2; ++b) {
@@ -305,7 +306,17 @@ decode_umma_pair_kernel(const __grid_constant__ DecodeParams p, const __grid_con
             ++seg_it;
         }
     } else if (warp >= kWarpQk && warp < kWarpSoftmax) {
-        // (the issuer warps of the peer CTA have nothing to do)
+        // the issuer warps of the peer CTA.  Sparse: they report to the leader that the gathering warps of this CTA have filled a stage
+        // (kWarpQk) and the other half's slots of it (kWarpPv).  What was written with plain stores is announced with a release at
+        // cluster scope; from a gathering warp that would wait for the row loads it has in flight (64 requests x 2,048 tokens on 128
+        // heads: 118 us a call against 81).
+        if constexpr (kSparse) {
+            const int full = warp == kWarpQk ? kBarKFull : kBarVFull;
+            for (int t = 0; t < it.end - it.x; ++t) {
+                mbar_wait(ctx, bar(full + t % kStages), (t / kStages) & 1, full + t % kStages);
+                if (lane == 0) mbar_arrive_cluster_release(leader_bar(full + t % kStages));
+            }
+        }
     } else if (kSparse && warp > kWarpVProducer) {
         // ===================================================== sparse decode: rows into the stages, in place of the TMA producers
         if constexpr (kSparse)
@@ -315,13 +326,13 @@ decode_umma_pair_kernel(const __grid_constant__ DecodeParams p, const __grid_con
                 [&](uint32_t t) {
                     fence_proxy_async();
                     __syncwarp();
-                    if (lane == 0) arrive_on_leader(kBarKFull + t % kStages);
+                    if (lane == 0) mbar_arrive(bar(kBarKFull + t % kStages));
                 },
                 [&](uint32_t t) { mbar_wait(ctx, bar(kBarQkDone + t % kStages), (t / kStages) & 1, kBarQkDone); },
                 [&](uint32_t t) {
                     fence_proxy_async();
                     __syncwarp();
-                    if (lane == 0) arrive_on_leader(kBarVFull + t % kStages);
+                    if (lane == 0) mbar_arrive(bar(kBarVFull + t % kStages));
                 });
     } else {
         // ===================================================== softmax + epilogue warps
