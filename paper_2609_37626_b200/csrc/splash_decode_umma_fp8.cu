@@ -116,7 +116,7 @@ decode_umma_fp8_kernel(const __grid_constant__ DecodeParams p, const __grid_cons
     tcgen05_fence_after();
     const uint32_t tmem_base = misc[0];
     SegmentIter<kOffPlan> it;
-    start_plan<false>(p, worker, kThreads / 32 - 1, it, FirstLoads{kStageBytes, 0u, kStageBytes, kStages, head0, kN});
+    start_plan<false>(p, worker, blockIdx.x % p.num_groups == 0, kThreads / 32 - 1, it, FirstLoads{kStageBytes, 0u, kStageBytes, kStages, head0, kN});
     const long long t_start = clock64();
 
     Segment seg;

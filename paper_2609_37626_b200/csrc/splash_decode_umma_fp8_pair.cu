@@ -172,7 +172,7 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
     tcgen05_fence_after();
     const uint32_t tmem_base = misc[0];
     SegmentIter<kInline ? L::kOffPlan : kPlanInWorkspace> it;
-    start_plan<false>(p, worker, kThreads / 32 - 1, it, FirstLoads{kPageBytes, 0u, kPageBytes, kStages, head0, H});
+    start_plan<false>(p, worker, rank == 0 && pair_id == worker * p.pair_groups, kThreads / 32 - 1, it, FirstLoads{kPageBytes, 0u, kPageBytes, kStages, head0, H});
     const long long t_start = clock64();
     const unsigned long long ns_start = global_timer_ns();
 
