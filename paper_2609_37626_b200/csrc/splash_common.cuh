@@ -134,6 +134,8 @@ struct DecodeParams {
     int32_t num_workers;
     int32_t request_overhead_tiles;   // per-request cost the plan adds to the tile count
     int32_t plan_mode;                // kPlanWorkspace, kPlanInline or kPlanWhole
+    int32_t plan_workers;             // > 0: an inline plan is left in the workspace in full, as one for that many workers, for a
+                                      // later call that takes it over and reads it there
     int32_t clear_status;             // 1: no plan kernel ran (its partition is taken again): block 0 clears the error words
     const int32_t *kv_begin, *kv_end; // the inline modes read the ranges themselves
     int4 *split_rec;                  // kPlanInline: where block 0 leaves the combine kernel's records
@@ -278,6 +280,16 @@ static __device__ __noinline__ void plan_ahead(const DecodeParams &p, int worker
 // late by microseconds at many requests: 32 of 2,048 tokens, 16 heads over e4m3, 23.7 us a call, now 20.2.)
 static __device__ __noinline__ void publish_inline_plan(const DecodeParams &p, const int32_t *ts, int lane) {
     const int B = p.B, W = p.num_workers, overhead = p.request_overhead_tiles;
+    if (p.plan_workers > 0) {
+        for (int i = lane; i <= B; i += 32) const_cast<int32_t *>(p.tile_start)[i] = ts[i];
+        if (lane < B) { const_cast<int32_t *>(p.req_lo)[lane] = ts[B + 1 + lane]; const_cast<int32_t *>(p.req_hi)[lane] = ts[2 * B + 1 + lane]; }
+        if (p.plan_mode == kPlanWhole) {       // a request each, nothing for the other workers
+            for (int w = lane; w <= p.plan_workers; w += 32) {
+                const_cast<int32_t *>(p.worker_begin)[w] = ts[min(w, B)];
+                const_cast<int32_t *>(p.worker_req)[w] = min(w, B - 1);
+            }
+        }
+    }
     int split = 0;
     if (p.plan_mode == kPlanInline) {
         const int rs = lane < B ? ts[lane] : ts[B], n = lane < B ? ts[lane + 1] - rs : 0;
@@ -400,6 +412,7 @@ __device__ __forceinline__ void start_plan(const DecodeParams &p, int worker, bo
                 int32_t *const begin = const_cast<int32_t *>(p.worker_begin) + worker;
                 begin[0] = sp[3 * p.B + 1];
                 if (worker == p.num_workers - 1) begin[1] = sp[p.B];
+                if (p.plan_workers > 0) const_cast<int32_t *>(p.worker_req)[worker] = sp[3 * p.B + 3];
             }
             if (blockIdx.x == 0 && warp == plan_warp) publish_inline_plan(p, sp, lane);
             it.init(p, worker);
