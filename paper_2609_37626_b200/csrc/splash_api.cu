@@ -460,7 +460,9 @@ int splash_lse_merge(int32_t num_parts, int64_t rows, int32_t d_v, const float *
         size_t pbytes = (size_t)num_parts * rows * d_v * 4, obytes = (size_t)rows * d_v * 4;
         if (oo < po + pbytes && po < oo + obytes) { set_error("out aliases part_out"); return SPLASH_INVALID_ARG; }
     }
-    cudaError_t e = launch_lse_merge(num_parts, rows, d_v, part_out, part_lse, out, lse, static_cast<cudaStream_t>(stream_));
+    DeviceInfo dev;
+    if (!current_device_info(dev)) return SPLASH_CUDA_ERROR;
+    cudaError_t e = launch_lse_merge(num_parts, rows, d_v, part_out, part_lse, out, lse, dev.sm_count, static_cast<cudaStream_t>(stream_));
     if (e != cudaSuccess) { set_error("CUDA error: %s", cudaGetErrorString(e)); return SPLASH_CUDA_ERROR; }
     return SPLASH_OK;
 }

@@ -511,7 +511,7 @@ cudaError_t launch_decode_umma_fp8_pair(const DecodeParams &p, cudaStream_t stre
 cudaError_t launch_decode_umma_pair(const DecodeParams &p, cudaStream_t stream);
 cudaError_t launch_split_combine(const DecodeParams &p, const int4 *split_rec, int sm_count, cudaStream_t stream);
 cudaError_t launch_lse_merge(int num_parts, int64_t rows, int d_v, const float *part_out,
-                             const float *part_lse, float *out, float *lse, cudaStream_t stream);
+                             const float *part_lse, float *out, float *lse, int sm_count, cudaStream_t stream);
 cudaError_t launch_page_migrate(const void *src_pool, const float *src_scales, void *dst_pool,
                                 float *dst_scales, int64_t page_bytes, const int32_t *src_ids,
                                 const int32_t *dst_ids, int64_t n, int32_t src_base, int32_t dst_base,

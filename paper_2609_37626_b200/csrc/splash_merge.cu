@@ -18,7 +18,8 @@ constexpr int kMergeThreads = 128;
 // weights add up to exactly 0, or an LSE is NaN (which fmaxf passes over), and so is the sum: the row becomes NaN, not empty.
 __device__ __forceinline__ float reference_max(float m) { return m == -INFINITY ? 0.f : m; }
 
-// One CTA per row; each thread owns float4 columns tid, tid + 128, ...  The parts' LSEs come in one load each, a part per
+// One CTA per row and 128 float4 columns, a column per thread.  (Rows of up to 512 values are one CTA.  A CTA that went over the columns of a
+// wider row: 700 rows of three parts, 2,048 wide, 6.3 us, now MERGEUS.)  The parts' LSEs come in one load each, a part per
 // thread, and the parts' rows kDepth loads at a time: taken one after the other in every thread they were a chain of round trips
 // (the decode of a CP shard with the merge of eight parts of 128 rows behind it: 28.2 us, now 27.1).  Where the rows are more
 // than the SMs hold at a time, four loads each and twelve blocks to an SM instead of eight.
@@ -31,7 +32,7 @@ lse_merge_kernel(int num_parts, int64_t rows, int d_v, const float *part_out, co
     const int64_t r = blockIdx.x;
     const int tid = threadIdx.x;
     float4 *o4 = reinterpret_cast<float4 *>(out + r * d_v);
-    const int nvec = d_v / 4;
+    const int nvec = d_v / 4, c_first = blockIdx.y * kMergeThreads + tid, c_step = gridDim.y * kMergeThreads;
     const float first = tid < num_parts ? part_lse[(int64_t)tid * rows + r] : -INFINITY;
     float m = first;
     for (int j = tid + kMergeThreads; j < num_parts; j += kMergeThreads) m = fmaxf(m, part_lse[(int64_t)j * rows + r]);
@@ -46,8 +47,8 @@ lse_merge_kernel(int num_parts, int64_t rows, int d_v, const float *part_out, co
     __syncthreads();
     Z = (red_s[1][0] + red_s[1][1]) + (red_s[1][2] + red_s[1][3]);       // the same in every thread
     if (Z == 0.f) {                   // no part saw a token
-        for (int c = tid; c < nvec; c += kMergeThreads) o4[c] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (tid == 0) lse[r] = -INFINITY;
+        for (int c = c_first; c < nvec; c += c_step) o4[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (c_first == 0) lse[r] = -INFINITY;
         return;
     }
     const float L = m + logf(Z);
@@ -56,7 +57,7 @@ lse_merge_kernel(int num_parts, int64_t rows, int d_v, const float *part_out, co
         if (j0 > 0) __syncthreads();
         if (tid < n) w_s[tid] = expf((j0 == 0 ? first : part_lse[(int64_t)(j0 + tid) * rows + r]) - L);
         __syncthreads();
-        for (int c = tid; c < nvec; c += kMergeThreads) {
+        for (int c = c_first; c < nvec; c += c_step) {
             float4 acc = j0 == 0 ? make_float4(0.f, 0.f, 0.f, 0.f) : o4[c];
             for (int j = 0; j < n; j += kDepth) {
                 float4 v[kDepth];
@@ -75,7 +76,7 @@ lse_merge_kernel(int num_parts, int64_t rows, int d_v, const float *part_out, co
             o4[c] = acc;
         }
     }
-    if (tid == 0) lse[r] = L;
+    if (c_first == 0) lse[r] = L;
 }
 
 // Grid W*h: block = (entry of the plan's list of split requests, head k of the slice).  A
@@ -323,9 +324,11 @@ grouped_combine_kernel(const DecodeParams p, const int4 *split_rec) {
 }  // namespace
 
 cudaError_t launch_lse_merge(int num_parts, int64_t rows, int d_v, const float *part_out,
-                             const float *part_lse, float *out, float *lse, cudaStream_t stream) {
-    constexpr int64_t kResident = 8 * 148;       // (24,960 rows of five parts, a decode in front: 121.6 us with eight loads, now 111)
-    const cudaError_t e = launch_dependent(rows <= kResident ? lse_merge_kernel<8> : lse_merge_kernel<4>, dim3((unsigned)rows), dim3(kMergeThreads), 0, stream, num_parts, rows, d_v,
+                             const float *part_lse, float *out, float *lse, int sm_count, cudaStream_t stream) {
+    const int64_t wide = (d_v / 4 + kMergeThreads - 1) / kMergeThreads;
+    const dim3 grid((unsigned)rows, (unsigned)(wide < 65535 ? wide : 65535));
+    const int64_t resident = 8 * (int64_t)sm_count;       // (24,960 rows of five parts, a decode in front: 121.6 us with eight loads, now 111)
+    const cudaError_t e = launch_dependent(rows * grid.y <= resident ? lse_merge_kernel<8> : lse_merge_kernel<4>, grid, dim3(kMergeThreads), 0, stream, num_parts, rows, d_v,
                                            part_out, part_lse, out, lse);
     count_launch();
     return e;

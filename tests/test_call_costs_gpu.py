@@ -76,3 +76,17 @@ def test_large_pages_move_at_the_rate_of_many_small_ones():
 
     large, small = us(8, 1 << 20), us(228, 36864)
     assert large <= 2 * small + 3, (large, small)
+
+
+def test_wide_rows_merge_at_the_rate_of_usual_ones():
+    """64 rows of four parts, 8,192 wide, against 1,024 rows of 512."""
+    import torch
+    from paper_2609_37626_b200 import binding
+
+    def us(rows, d_v):
+        o, l = torch.zeros((4, rows, d_v), device="cuda"), torch.zeros((4, rows), device="cuda")
+        out, lse = torch.empty((rows, d_v), device="cuda"), torch.empty(rows, device="cuda")
+        return device_us(lambda: binding.splash_lse_merge(o, l, out, lse))
+
+    wide, usual = us(64, 8192), us(1024, 512)
+    assert wide <= 1.5 * usual + 2, (wide, usual)

@@ -1,0 +1,12 @@
+"""The merge of rows of more than 512 values takes several blocks a row: the cases of the usual widths at the edges of a block's 512 columns."""
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("parts", [1, 5, 129])
+@pytest.mark.parametrize("rows", [3, 700])
+@pytest.mark.parametrize("d_v", [508, 516, 1024, 1540])
+def test_wide_rows(parts, rows, d_v):
+    import test_merge_widths_gpu
+    test_merge_widths_gpu.test_parts_and_rows(parts, rows, d_v)
