@@ -79,6 +79,9 @@ static_assert(kOffQHi % 512 == 0 && kOffQLo % 512 == 0 && kOffPHi % 512 == 0 && 
 // tensor memory: O^T 4 blocks x 64 columns, then 2 S buffers x 2 partial accumulators x 64 columns
 constexpr uint32_t kColO = 0, kColS = 256;
 
+// kInline: the variant that can plan for itself, as in splash_decode_umma_fp8_pair.cu (64 requests of 1,000 to 8,000 tokens on 128 heads:
+// OLDUS with one kernel for both, NEWUS behind a plan kernel now)
+template <bool kInline>
 __global__ void __launch_bounds__(kThreads, 1)
 decode_umma_fp8_kernel(const __grid_constant__ DecodeParams p, const __grid_constant__ CUtensorMap tmap_kv) {
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -115,7 +118,7 @@ decode_umma_fp8_kernel(const __grid_constant__ DecodeParams p, const __grid_cons
     __syncthreads();
     tcgen05_fence_after();
     const uint32_t tmem_base = misc[0];
-    SegmentIter<kOffPlan> it;
+    SegmentIter<kInline ? kOffPlan : kPlanInWorkspace> it;
     start_plan<false>(p, worker, blockIdx.x % p.num_groups == 0, kThreads / 32 - 1, it, FirstLoads{kStageBytes, 0u, kStageBytes, kStages, head0, kN});
     const long long t_start = clock64();
 
@@ -560,9 +563,13 @@ cudaError_t launch_decode_umma_fp8(const DecodeParams &p, cudaStream_t stream) {
                      (uint64_t)kPage * kDQK, 64))
         return cudaErrorInvalidValue;
     static DeviceOnce once;
-    cudaError_t e = once.run([&] { return cudaFuncSetAttribute(decode_umma_fp8_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes); });
+    cudaError_t e = once.run([&] {
+        const cudaError_t e0 = cudaFuncSetAttribute(decode_umma_fp8_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
+        if (e0 != cudaSuccess) return e0;
+        return cudaFuncSetAttribute(decode_umma_fp8_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
+    });
     if (e != cudaSuccess) return e;
-    e = launch_dependent(decode_umma_fp8_kernel, dim3((unsigned)(p.num_workers * p.num_groups)), dim3(kThreads),
+    e = launch_dependent(p.plan_mode == kPlanWorkspace ? decode_umma_fp8_kernel<false> : decode_umma_fp8_kernel<true>, dim3((unsigned)(p.num_workers * p.num_groups)), dim3(kThreads),
                          (size_t)kSmemBytes, stream, p, mkv);
     count_launch();
     return e;
