@@ -210,15 +210,15 @@ SPLASH_API size_t splash_mla_decode_workspace_bytes(const splash_mla_shape *shap
  *   sel_tokens   int32; entry j of request i at sel_tokens[i * sel_stride + j]; entries at or
  *                beyond sel_count[i] are never read
  *   sel_count    [num_requests] int32, each in [0, max_selected]
- *   max_selected bound on sel_count (the indexer's k, e.g. 2048); sizes the workspace
+ *   max_selected bound on sel_count (the indexer's k, e.g. 2048)
  *   workspace    at least splash_mla_decode_sparse_workspace_bytes() bytes, 256-byte aligned
  *
  * All pointers are device pointers.  A list entry outside [0, seq_lens[i]), a page id outside
  * the pool or a count outside [0, max_selected] is never dereferenced; the outputs of that
- * request are then NaN.  Two stages on the device: the listed rows are gathered and dequantised
- * (code times block scale, rounded to bf16) into a dense bf16 cache inside the workspace, then
- * the dense decode kernels run over it (launch order: plan over the list counts, gather,
- * decode kernel, combine).
+ * request are then NaN.  The CTAs of the decode kernel gather the listed rows of their own work
+ * and dequantise them (code times block scale, rounded to bf16) straight into shared memory.
+ * (With SPLASH_FLAG_SIMT a kernel in front gathers them into a dense bf16 cache inside the
+ * workspace, which is larger by 1,152 bytes per listable token then.)
  */
 SPLASH_API int splash_mla_decode_sparse(const splash_mla_shape *shape, const void *q, const void *kv_pool,
                              const int32_t *block_table, const int32_t *seq_lens,
@@ -226,7 +226,7 @@ SPLASH_API int splash_mla_decode_sparse(const splash_mla_shape *shape, const voi
                              int32_t max_selected, int32_t head_begin, int32_t head_end,
                              float *out, float *lse, void *workspace, size_t workspace_bytes, void *stream);
 
-/* Workspace size for splash_mla_decode_sparse (host computation).  Returns 0 on invalid arguments. */
+/* Workspace size for splash_mla_decode_sparse with these shape.flags (host computation).  Returns 0 on invalid arguments. */
 SPLASH_API size_t splash_mla_decode_sparse_workspace_bytes(const splash_mla_shape *shape, int32_t max_selected,
                                                 int32_t head_begin, int32_t head_end);
 
@@ -397,7 +397,7 @@ SPLASH_API int splash_last_launch_count(void);
  * splash_get_kernel_timing() synchronises on the last call's final event and returns
  * the three durations in milliseconds (host pointers, each may be NULL).  Off by
  * default; enabling it adds four event records per call and nothing else.  For
- * splash_mla_decode_sparse the decode figure covers the gather kernel and the decode kernel.
+ * splash_mla_decode_sparse the decode figure covers the gathering, in that kernel or, with SPLASH_FLAG_SIMT, in front of it.
  */
 SPLASH_API int splash_set_kernel_timing(int enable);
 SPLASH_API int splash_get_kernel_timing(float *plan_ms, float *decode_ms, float *combine_ms);

@@ -375,9 +375,10 @@ int splash_mla_decode_migrating(const splash_mla_shape *shape, const void *q, co
 
 namespace {
 
-// Workspace of a sparse call: [dense decode workspace][dense table B * ppr][dense cache].
+// Workspace of a sparse call: [dense decode workspace], on the fp32 kernel also [dense table B * ppr][dense cache].
 struct SparseView {
-    splash_mla_shape dense;        // the shape of the dense call over the gathered cache
+    splash_mla_shape dense;        // the shape of the dense call over the listed rows
+    bool gathered;                 // they are gathered into the workspace
     int pages_per_request;
     size_t inner_bytes, off_table, off_pool, bytes;
 };
@@ -398,9 +399,12 @@ bool make_sparse_view(const splash_mla_shape *shape, int32_t max_selected, int32
     v.inner_bytes = splash_mla_decode_workspace_bytes(&v.dense, head_begin, head_end);
     if (v.inner_bytes == 0) return false;
     size_t off = align_up(v.inner_bytes, 256);
-    v.off_table = off; off = align_up(off + sizeof(int32_t) * (size_t)pages, 256);
-    v.off_pool = off; off += (size_t)pages * kPage * kDQK * 2;
-    v.bytes = align_up(off, 256);
+    v.gathered = (shape->flags & SPLASH_FLAG_SIMT) != 0;
+    if (v.gathered) {
+        v.off_table = off; off = align_up(off + sizeof(int32_t) * (size_t)pages, 256);
+        v.off_pool = off; off = align_up(off + (size_t)pages * kPage * kDQK * 2, 256);
+    }
+    v.bytes = off;
     return true;
 }
 
@@ -438,9 +442,9 @@ int splash_mla_decode_sparse(const splash_mla_shape *shape, const void *q, const
     st.pool656 = kv_pool; st.num_pool_pages = shape->num_pool_pages; st.block_table = block_table;
     st.table_stride = shape->block_table_stride; st.ctx_lens = seq_lens; st.sel = sel_tokens; st.sel_count = sel_count;
     st.sel_stride = sel_stride; st.max_selected = max_selected; st.pages_per_request = v.pages_per_request;
-    st.dense_table = reinterpret_cast<int32_t *>(ws + v.off_table);
+    st.dense_table = v.gathered ? reinterpret_cast<int32_t *>(ws + v.off_table) : nullptr;
     // plan (over the list counts) -> decode kernel, whose CTAs gather the rows of their own tiles -> combine
-    return decode_dense(&v.dense, q, ws + v.off_pool, nullptr, st.dense_table, sel_count, head_begin, head_end, nullptr, nullptr,
+    return decode_dense(&v.dense, q, v.gathered ? ws + v.off_pool : kv_pool, nullptr, v.gathered ? st.dense_table : block_table, sel_count, head_begin, head_end, nullptr, nullptr,
                         out, lse, workspace, v.inner_bytes, stream_, &st);
 }
 
