@@ -76,7 +76,7 @@ enum {
     /* Run the plain SIMT (fp32 CUDA-core) decode kernel instead of the tcgen05 one.
      * A diagnostic path: same plan, same partial slots, same combine; slow. */
     SPLASH_FLAG_SIMT = 1u,
-    /* slices of 65..128 heads: use two independent 64-head CTAs per KV worker instead of a CTA
+    /* slices of 65..128 heads, over e4m3 of 33..128: use independent CTAs of 64 heads, one or two per KV worker, instead of a CTA
      * pair issuing cta_group::2 MMAs.  A diagnostic path. */
     SPLASH_FLAG_NO_PAIR = 2u,
     /* splash_mla_decode_sparse only: accepted, without effect.  (It asked for one kernel that gathers, dequantises and
@@ -94,8 +94,8 @@ enum {
      * the shape (num_requests, q_rows, kv_dtype, the other flag bits) and the device only -- not of q, the cache, the
      * scales or the block table -- and a decode step runs the same batch through every layer of the model: the first
      * layer's call plans, the others pass this bit.  The caller asserts that those arguments are what they were in the
-     * last call WITHOUT this bit on the same workspace (nothing checks it; a different batch would be cut along the old
-     * batch's boundaries and give wrong results, within bounds).  The error words of the status block are cleared as in
+     * last call WITHOUT this bit on the same workspace (nothing checks it; a different batch may be cut along the old
+     * batch's boundaries and give wrong results, within bounds).  The layers' block tables may be of different widths.  The error words of the status block are cleared as in
      * any call.  Ignored by the sparse entry point and together with SPLASH_FLAG_VALIDATE (which needs the plan's pass). */
     SPLASH_FLAG_REUSE_PLAN = 16u
 };
@@ -274,10 +274,9 @@ SPLASH_API int splash_kv_page_migrate(const void *src_pool, const float *src_sca
 SPLASH_API size_t splash_kv_page_migrate_workspace_bytes(int32_t max_page_id);
 
 /*
- * A decode call that carries a page migration with it: the overlapped transfer of a layout
- * switch, in which one layer's state moves while another layer computes, so that about one
- * layer's transfer stays exposed (Sec. 4.1 "Overlapped transfer", the exposed-cost equation of
- * Sec. 4.2).  The effect is that of
+ * A decode call that carries a page migration with it: the layer-by-layer transfer of a layout
+ * switch, in which one layer's state moves with the call that computes another (Sec. 4.1
+ * "Overlapped transfer").  The effect is that of
  *     splash_kv_page_migrate(job...)  and  splash_mla_decode(...)
  * issued on `stream` in either order; the two must therefore be independent: the decode reads
  * none of the job's destination pages and not the job's block table (the usual case: the job
@@ -392,8 +391,9 @@ SPLASH_API int splash_last_launch_count(void);
 
 /*
  * Per-kernel timing of splash_mla_decode, for benchmarks.  While enabled (per host
- * thread), every decode call records CUDA events on its stream around its three
- * kernels (plan, decode, split combine); the events are created on first use.
+ * thread), every decode call records CUDA events on its stream around its
+ * kernels (plan, decode, split combine; about zero for one that the call does
+ * without); the events are created on first use.
  * splash_get_kernel_timing() synchronises on the last call's final event and returns
  * the three durations in milliseconds (host pointers, each may be NULL).  Off by
  * default; enabling it adds four event records per call and nothing else.  For

@@ -18,10 +18,10 @@ constexpr int kMergeThreads = 128;
 // weights add up to exactly 0, or an LSE is NaN (which fmaxf passes over), and so is the sum: the row becomes NaN, not empty.
 __device__ __forceinline__ float reference_max(float m) { return m == -INFINITY ? 0.f : m; }
 
-// One CTA per row and 128 float4 columns, a column per thread.  (Rows of up to 512 values are one CTA.  A CTA that went over the columns of a
-// wider row: 700 rows of three parts, 2,048 wide, 6.3 us, now MERGEUS.)  The parts' LSEs come in one load each, a part per
+// One CTA per row and 128 float4 columns, a column per thread.  (Rows of up to 512 values are one CTA.  A CTA that goes over the columns of a
+// wider row has too few loads in flight: 64 rows of four parts, 8,192 wide, 11.3 us.)  The parts' LSEs come in one load each, a part per
 // thread, and the parts' rows kDepth loads at a time: taken one after the other in every thread they were a chain of round trips
-// (the decode of a CP shard with the merge of eight parts of 128 rows behind it: 28.2 us, now 27.1).  Where the rows are more
+// (128 rows of eight parts: 3.0 us, now 2.6; 24,960 of five: 77.5, now 55.4).  Where the rows are more
 // than the SMs hold at a time, four loads each and twelve blocks to an SM instead of eight.
 template <int kDepth>
 __global__ void __launch_bounds__(kMergeThreads, kDepth == 8 ? 8 : 12)

@@ -15,36 +15,34 @@ pytestmark = pytest.mark.gpu
 def test_lengths_ranges_and_table_change_under_the_call_before(kv_dtype, H, lens):
     import torch
     from paper_2609_37626_b200 import binding
+    from test_inputs_written_in_front_gpu import Arena, ints
     w = W.make_workload("ahead", 8300 + H + len(lens), lens, H=H, kv_dtype=kv_dtype)
     dw = binding.DeviceWorkload(w)
     rng = np.random.default_rng(7)
-    variants = []
+    versions = []
     for v in range(4):
         keep = np.array([rng.integers(0, n + 1) for n in lens], np.int32) if v else np.array(lens, np.int32)
         begin = np.array([rng.integers(0, max(1, k // 2)) for k in keep], np.int32) if v else np.zeros(len(lens), np.int32)
-        variants.append((torch.from_numpy(keep).cuda(), torch.from_numpy(begin).cuda()))
-    good = dw.block_table.clone()
-    begin = variants[0][1].clone()
-    call = lambda: dw.decode(kv_begin=begin)
+        versions.append(dict(lens=ints(keep), begin=ints(begin), table=dw.block_table))
+    versions.append(dict(versions[0], table=torch.full_like(dw.block_table, -1)))       # what a call that plans ahead may find
+    a = Arena(versions)
+    call = lambda: binding.splash_mla_decode(dw.q, dw.kv_pool, a.view("table"), a.view("lens"), softmax_scale=w.softmax_scale,
+                                             kv_scales=dw.kv_scales, kv_begin=a.view("begin"))
     want = []
-    for keep, b in variants:
-        dw.seq_lens.copy_(keep)
-        begin.copy_(b)
+    for v in range(4):
+        a.put(v)
         torch.cuda.synchronize()
         want.append([t.clone() for t in call()])
     torch.cuda.synchronize()
     got = []
     for r in range(12):
-        dw.block_table.fill_(-1)            # what a call that plans ahead may find
+        a.put(4)
         call()
-        dw.seq_lens.copy_(variants[r % 4][0])
-        begin.copy_(variants[r % 4][1])
-        dw.block_table.copy_(good)
+        a.put(r % 4)            # the library's own move: it lets the next call in before its last stores, which are these
         got.append([t.clone() for t in call()])
     torch.cuda.synchronize()
     for r, (o, l) in enumerate(got):
         assert torch.equal(o, want[r % 4][0]) and torch.equal(l, want[r % 4][1]), r
-    dw.seq_lens.copy_(variants[0][0])
 
 
 @pytest.mark.parametrize("kv_dtype,H", [(0, 16), (1, 16), (0, 128), (1, 74), (0, 74)])      # one row per SM is 148

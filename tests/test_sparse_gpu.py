@@ -15,8 +15,8 @@ TOL_O = TOL[1]["abs_o"]
 TOL_LSE = TOL[1]["lse"]
 
 
-# 0: the gather kernel followed by the dense kernels; 4: the fused kernel (gather + dequantise + attention on CTA pairs)
-PATHS = {"two_stage": 0, "fused": 4}
+# 4: SPLASH_FLAG_SPARSE_FUSED, accepted without effect (every sparse call gathers in the decode CTAs)
+PATHS = {"plain": 0, "fused_flag": 4}
 
 
 @pytest.fixture(params=list(PATHS))
