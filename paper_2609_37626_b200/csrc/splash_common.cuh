@@ -175,6 +175,8 @@ __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddep
 // i -- so that there is nothing to combine either.
 enum { kPlanWorkspace = 0, kPlanInline = 1, kPlanWhole = 2 };
 constexpr int kInlinePlanRequests = 32;
+// (contexts of at most this many pages: 4 requests in a table as wide as they are against one of 2,048 columns, whose requests are cut and
+// combined: 16 heads 11.9 against 15 to 16 us, 128 heads 11.1 against 13.8, e4m3 9.1 against 12.8 and 16.9 against 21.4)
 constexpr int kWholeRequestPages = 4;
 constexpr int kInlinePairPages = 8192;
 // shared-memory copy of an inline plan: tile_start[B + 1], lo[B], hi[B] (as in the workspace), then the worker's first
