@@ -18,8 +18,8 @@ constexpr int kMergeThreads = 128;
 // weights add up to exactly 0, or an LSE is NaN (which fmaxf passes over), and so is the sum: the row becomes NaN, not empty.
 __device__ __forceinline__ float reference_max(float m) { return m == -INFINITY ? 0.f : m; }
 
-// One CTA per row and 128 float4 columns, a column per thread.  (Rows of up to 512 values are one CTA.  A CTA that goes over the columns of a
-// wider row has too few loads in flight: 64 rows of four parts, 8,192 wide, 11.3 us.)  The parts' LSEs come in one load each, a part per
+// One CTA per row and 128 float4 columns, a column per thread, where the rows are few (launch_lse_merge).  (A CTA that goes over all columns of a
+// wide row has too few loads in flight then: 64 rows of four parts, 8,192 wide, 11.5 us, now 3.8.)  The parts' LSEs come in one load each, a part per
 // thread, and the parts' rows kDepth loads at a time: taken one after the other in every thread they were a chain of round trips
 // (128 rows of eight parts: 3.0 us, now 2.6; 24,960 of five: 77.5, now 55.4).  Where the rows are more
 // than the SMs hold at a time, four loads each and twelve blocks to an SM instead of eight.
@@ -326,8 +326,11 @@ grouped_combine_kernel(const DecodeParams p, const int4 *split_rec) {
 cudaError_t launch_lse_merge(int num_parts, int64_t rows, int d_v, const float *part_out,
                              const float *part_lse, float *out, float *lse, int sm_count, cudaStream_t stream) {
     const int64_t wide = (d_v / 4 + kMergeThreads - 1) / kMergeThreads;
-    const dim3 grid((unsigned)rows, (unsigned)(wide < 65535 ? wide : 65535));
     const int64_t resident = 8 * (int64_t)sm_count;       // (24,960 rows of five parts, a decode in front: 121.6 us with eight loads, now 111)
+    // Rows are cut while there are too few of them to fill the SMs, into about two blocks for each place.  More rows than places gain
+    // nothing from it and each block starts with the row's weights: 3,000 rows of two parts, 1,536 wide, 7.9 us whole and 12.1 cut.
+    const int64_t cut = rows > 0 && rows <= resident ? (2 * resident + rows - 1) / rows : 1;
+    const dim3 grid((unsigned)rows, (unsigned)(cut < wide ? cut : wide));
     const cudaError_t e = launch_dependent(rows * grid.y <= resident ? lse_merge_kernel<8> : lse_merge_kernel<4>, grid, dim3(kMergeThreads), 0, stream, num_parts, rows, d_v,
                                            part_out, part_lse, out, lse);
     count_launch();
