@@ -574,6 +574,9 @@ decode_umma_fp8_narrow_kernel(const __grid_constant__ DecodeParams p, const __gr
 #pragma unroll 1
                 for (int half = 0; half < 2; ++half) {
                     const int row = 8 * (sw >> 2), n0 = half * (N / 2) + row;       // this warp's eight heads
+                    float inv[8];                           // (read here: a load after a store waits for it, since they might overlap: 0.9 us a request)
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) inv[k] = l_s[n0 + k];
 #pragma unroll
                     for (int j = 0; j < 4; j += 2) {
                         float o[2][8], o_lo[2][8];
@@ -587,7 +590,7 @@ decode_umma_fp8_narrow_kernel(const __grid_constant__ DecodeParams p, const __gr
                         for (int jj = 0; jj < 2; ++jj)
 #pragma unroll
                             for (int k = 0; k < 8; ++k)
-                                stg[(row + k) * kDV + 128 * (j + jj) + 32 * q4 + lane] = fmaf(o_lo[jj][k], 0.0625f, o[jj][k]) * l_s[n0 + k];
+                                stg[(row + k) * kDV + 128 * (j + jj) + 32 * q4 + lane] = fmaf(o_lo[jj][k], 0.0625f, o[jj][k]) * inv[k];
                     }
                     fence_proxy_async();
                     named_bar_sync<1, kSoftmaxThreads>();
