@@ -51,7 +51,7 @@ struct PlanView {
     int32_t *worker_begin;  // [W+1] global tile index where each worker starts
     int32_t *split_list;    // [W+1] requests computed in more than one piece (count in status[8])
     int32_t *worker_req;    // [W+1] the request that holds a worker's first tile (what the kernels would bisect for)
-    int4 *split_rec;        // [W+1] per entry of split_list: (request, first worker, last worker, first tile of the request)
+    int4 *split_rec;        // [W+1] per entry of split_list: (request, first worker, last worker, SplitFlags)
     float *partial_lse;     // [2W][h]
     float *partial_scale;   // [2W][h]
     float *partial_out;     // [2W][h][512]
@@ -89,6 +89,11 @@ inline __host__ PlanView make_plan_view(void *workspace, int B, int W, int h) {
     v.bytes = off;
     return v;
 }
+
+// What a record says of a cut request's slots: a worker's piece lies in slot 2 w, the first worker's in 2 w + 1 if an earlier request's
+// piece came before it; and whether there may be workers among them whose start fell on the same tile as the next one's, so
+// that they hold nothing (the plan kernel's, where all the work costs less than there are workers).
+enum SplitFlags { kSplitSecondSlot = 1, kSplitGaps = 2 };
 
 // Arguments common to the decode kernels.
 struct DecodeParams {
@@ -205,9 +210,12 @@ __device__ __forceinline__ void lane_range(const DecodeParams &p, int lane, int 
     if (lane < p.B) effective_range(load_l2(p.seq_lens + lane), p.kv_begin, p.kv_end, lane, p.len_cap, lo, hi);
 }
 
+// Workers that an inline plan cuts the work for: no more than it costs tiles, or some would start where the next one does.
+__device__ __forceinline__ int cut_workers(const DecodeParams &p, int cost) { return min(p.num_workers, cost); }
+
 // One warp of a CTA: the plan, as far as worker `worker` needs it, from the lanes' ranges.
 static __device__ __noinline__ void build_inline_plan(const DecodeParams &p, int worker, int32_t *sp, int lane, int lo, int hi) {
-    const int B = p.B, W = p.num_workers, overhead = p.request_overhead_tiles;
+    const int B = p.B, overhead = p.request_overhead_tiles;
     const int n = hi > lo ? (hi + kPage - 1) / kPage - lo / kPage : 0;
     const int c = n > 0 ? n + overhead : 0;
     int sn = n, sc = c;
@@ -222,12 +230,12 @@ static __device__ __noinline__ void build_inline_plan(const DecodeParams &p, int
         if (lane == worker) { sp[3 * B + 1] = sn - n; sp[3 * B + 2] = sn; sp[3 * B + 3] = worker; }
         return;
     }
-    const int tiles = __shfl_sync(0xffffffffu, sn, 31), cost = __shfl_sync(0xffffffffu, sc, 31);
+    const int tiles = __shfl_sync(0xffffffffu, sn, 31), cost = __shfl_sync(0xffffffffu, sc, 31), W = cut_workers(p, cost);
     // first tile of worker w (the same w in all lanes) and the request that holds it: as many requests lie before it as
     // end at or before its share of the cost
     auto start = [&](int w, int &req) {
         req = 0;
-        if (w >= W || cost == 0) return tiles;
+        if (w >= W) return tiles;
         const int target = cost_target(cost, w, W);
         req = __popc(__ballot_sync(0xffffffffu, sc <= target));
         const int off = target - __shfl_sync(0xffffffffu, sc - c, req) - overhead;
@@ -281,7 +289,7 @@ static __device__ __noinline__ void plan_ahead(const DecodeParams &p, int worker
 // so the last such worker is floor(((c + overhead + t + 1) W - 1) / cost).  (Block 0 going through all workers for every request was
 // late by microseconds at many requests: 32 of 2,048 tokens, 16 heads over e4m3, 23.7 us a call, now 20.2.)
 static __device__ __noinline__ void publish_inline_plan(const DecodeParams &p, const int32_t *ts, int lane) {
-    const int B = p.B, W = p.num_workers, overhead = p.request_overhead_tiles;
+    const int B = p.B, overhead = p.request_overhead_tiles;
     if (p.plan_workers > 0) {
         for (int i = lane; i <= B; i += 32) const_cast<int32_t *>(p.tile_start)[i] = ts[i];
         if (lane < B) { const_cast<int32_t *>(p.req_lo)[lane] = ts[B + 1 + lane]; const_cast<int32_t *>(p.req_hi)[lane] = ts[2 * B + 1 + lane]; }
@@ -294,14 +302,14 @@ static __device__ __noinline__ void publish_inline_plan(const DecodeParams &p, c
     }
     int split = 0;
     if (p.plan_mode == kPlanInline) {
-        const int rs = lane < B ? ts[lane] : ts[B], n = lane < B ? ts[lane + 1] - rs : 0;
+        const int n = lane < B ? ts[lane + 1] - ts[lane] : 0;
         int sc = n > 0 ? n + overhead : 0;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const int b = __shfl_up_sync(0xffffffffu, sc, o);
             if (lane >= o) sc += b;
         }
-        const int cost = __shfl_sync(0xffffffffu, sc, 31);
+        const int cost = __shfl_sync(0xffffffffu, sc, 31), W = cut_workers(p, cost);
         int wf = 0, wl = 0;
         if (n > 0) {
             auto worker_before = [&](int c) { return min(W - 1, (int)(((unsigned long long)(unsigned)c * (unsigned)W - 1) / (unsigned)cost)); };
@@ -310,7 +318,7 @@ static __device__ __noinline__ void publish_inline_plan(const DecodeParams &p, c
         }
         const unsigned cut = __ballot_sync(0xffffffffu, wf != wl);
         split = __popc(cut);
-        if ((cut >> lane) & 1u) p.split_rec[__popc(cut & ((1u << lane) - 1u))] = make_int4(lane, wf, wl, rs);
+        if ((cut >> lane) & 1u) p.split_rec[__popc(cut & ((1u << lane) - 1u))] = make_int4(lane, wf, wl, (long long)wf * cost < (long long)(sc - n - overhead) * W ? kSplitSecondSlot : 0);      // (its share starts in front of the request's)
     }
     if (lane < 16) p.status[lane] = lane == 8 ? split : 0;
 }

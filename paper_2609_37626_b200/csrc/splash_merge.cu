@@ -79,180 +79,210 @@ lse_merge_kernel(int num_parts, int64_t rows, int d_v, const float *part_out, co
     if (c_first == 0) lse[r] = L;
 }
 
-// Grid W*h: block = (entry of the plan's list of split requests, head k of the slice).  A
-// request computed in one piece and an empty one were written by the decode kernel itself; a
-// split request is merged from the slots of its workers in worker order.  The weights are
-// computed once per block (thread j takes worker wf + j), then every thread streams its
-// float4 column over the parts with several loads in flight.
+// The combine kernels: block = (entry of the plan's list of split requests, head k of the slice).  A request computed in one
+// piece and an empty one were written by the decode kernel itself; a split request is merged from the slots of its workers in
+// worker order.  What bounds them is round trips to L2 and DRAM: the list's length and the entry's record come in the first, and the
+// record says where the pieces lie, so that their LSEs and their rows come in the second.
 constexpr int kMaxParts = 512;     // >= number of workers of any launch (one per SM at most)
+
+// Where a cut request's pieces lie.
+struct Pieces {
+    int request, first_worker, n, flags;
+    __device__ __forceinline__ explicit Pieces(const int4 &rec) : request(rec.x), first_worker(rec.y), n(rec.z - rec.y + 1), flags(rec.w) {}
+    __device__ __forceinline__ uint32_t row(int j, int h, int k) const {
+        return (uint32_t)(2 * (first_worker + j) + (j == 0 ? flags & kSplitSecondSlot : 0)) * h + k;
+    }
+    // (a slot nobody wrote holds stale bytes)
+    __device__ __forceinline__ bool live(const DecodeParams &p, int j) const {
+        return !(flags & kSplitGaps) || p.worker_begin[first_worker + j + 1] > p.worker_begin[first_worker + j];
+    }
+};
+
+// Four columns of a slot's row as they lie in memory.  (Loads first, conversions with the arithmetic: a conversion next to its load would
+// make every load wait for the one before it.)
+template <bool kF16>
+struct PartRow {
+    using Raw = typename std::conditional<kF16, uint2, float4>::type;
+    static __device__ __forceinline__ Raw load(const DecodeParams &p, uint32_t row, int c) {      // (at most 2 W h rows, of 128 fours)
+        return reinterpret_cast<const Raw *>(p.partial_out)[row * (kDV / 4) + c];
+    }
+    static __device__ __forceinline__ void add(float4 &acc, const Raw &raw, float w) {
+        float4 v;
+        if constexpr (kF16) {
+            const float2 a = __half22float2(*reinterpret_cast<const __half2 *>(&raw.x)), b = __half22float2(*reinterpret_cast<const __half2 *>(&raw.y));
+            v = make_float4(a.x, a.y, b.x, b.y);
+        } else {
+            v = raw;
+        }
+        acc.x = fmaf(w, v.x, acc.x); acc.y = fmaf(w, v.y, acc.y);
+        acc.z = fmaf(w, v.z, acc.z); acc.w = fmaf(w, v.w, acc.w);
+    }
+};
 
 // kF16: the partial outputs are f16 (rows of 512 halves) or fp32.  kLean: a variant for launches whose requests are cut
 // into few pieces each (many requests per worker): at most four part loads in flight, few enough registers for sixteen
-// resident blocks per SM instead of eight -- its blocks are short chains of round trips to DRAM, and what bounds
+// resident blocks per SM instead of eight -- its blocks are short chains of round trips, and what bounds
 // the kernel is how many of them an SM holds at a time.
 template <bool kF16, bool kLean>
 __global__ void __launch_bounds__(kMergeThreads, kLean ? 16 : 8)
 split_combine_kernel(const DecodeParams p, const int4 *split_rec) {
+    using Row = PartRow<kF16>;
     __shared__ float w_s[kMaxParts];
     __shared__ float sc_s[kF16 ? kMaxParts : 1];      // f16 pieces: the power of two each row was divided by
-    __shared__ int slot_s[kMaxParts];
-    __shared__ float red_s[kMergeThreads / 32];
+    __shared__ float red_s[kMergeThreads / 32], sum_s[kMergeThreads / 32];
     const int h = p.head_end - p.head_begin;
     const int k = blockIdx.x % h, entry = blockIdx.x / h;
     const int g = p.head_begin + k;
     grid_launch_dependents();     // a next call's first kernel may come in once every block of this grid has started
     grid_dependency_wait();       // the decode kernel's partial slots (and the plan) are read from here on
-    // Three rounds of loads, each independent within itself (the plan's arrays have long left L2 by now, so every
-    // dependent load is a trip to DRAM): the list length and this entry's record; then the worker boundaries and the
-    // LSE of every candidate slot; then the partial outputs.
     const int n_entries = p.status[8];
-    const int4 rec = split_rec[entry];             // (request, first worker, last worker, first tile); unused past the list's end
+    const Pieces pieces(split_rec[entry]);             // (unused past the list's end)
     if (entry >= n_entries) return;
-    const int i = rec.x, wf = rec.y, wl = rec.z;
+    const int i = pieces.request, nparts = pieces.n;
     float4 *o4 = reinterpret_cast<float4 *>(p.out + (int64_t)i * p.out_stride_request + (int64_t)g * p.out_stride_head);
     float *lse = p.lse + (int64_t)i * p.lse_stride_request + g;
     const int c = threadIdx.x;             // 128 threads x float4 = 512 columns
-    // workers between the first and the last may own no tiles at all (their start snapped to
-    // the same tile as their successor's): they wrote no slot and get weight 0
-    const int rs = rec.w;
-    const int nparts = wl - wf + 1;
+    if (kLean && nparts <= 4 && !(pieces.flags & kSplitGaps)) {
+        // few pieces, as nearly all requests of such a launch: every thread has all their LSEs, and nothing is exchanged
+        typename Row::Raw raw[4];
+        float L[4], scale[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            L[j] = -INFINITY; scale[j] = 1.f;
+            if (j < nparts) {
+                const uint32_t row = pieces.row(j, h, k);
+                L[j] = p.partial_lse[row];
+                if constexpr (kF16) scale[j] = p.partial_scale[row];
+                raw[j] = Row::load(p, row, c);
+            }
+        }
+        const float m = reference_max(fmaxf(fmaxf(L[0], L[1]), fmaxf(L[2], L[3])));
+        float Z = 0.f;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) { L[j] = expf(L[j] - m); Z += L[j]; }      // (0 for a piece that is not there)
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (Z != 0.f) {
+            const float inv_z = 1.f / Z;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float w = L[j] * inv_z;
+                if (w != 0.f) Row::add(acc, raw[j], kF16 ? w * scale[j] : w);
+            }
+        }
+        o4[c] = acc;
+        if (c == 0) *lse = Z == 0.f ? -INFINITY : m + logf(Z);
+        return;
+    }
+    // the first pieces' rows, beside the LSEs
+    constexpr int kFirst = kLean ? 0 : kF16 ? 16 : 8;
+    typename Row::Raw first[kFirst + 1];
+#pragma unroll
+    for (int u = 0; u < kFirst; ++u)
+        if (u < nparts) first[u] = Row::load(p, pieces.row(u, h, k), c);
     float m = -INFINITY;
     for (int j = c; j < nparts; j += kMergeThreads) {
-        const int w = wf + j;
-        // slot 2 w + 1 can only be the first worker's (the request starts inside its run); both candidates' LSEs are
-        // fetched beside the boundaries that decide between them (a slot nobody wrote holds stale bytes: not used)
-        const int wb0 = p.worker_begin[w], wb1 = p.worker_begin[w + 1];
-        const float L0 = p.partial_lse[(int64_t)(2 * w) * h + k];
-        const float L1 = j == 0 ? p.partial_lse[(int64_t)(2 * w + 1) * h + k] : 0.f;
-        float S0 = 1.f, S1 = 1.f;
-        if constexpr (kF16) {
-            S0 = p.partial_scale[(int64_t)(2 * w) * h + k];
-            if (j == 0) S1 = p.partial_scale[(int64_t)(2 * w + 1) * h + k];
-        }
-        const bool live = wb1 > wb0;
-        const int slot = 2 * w + (rs <= wb0 ? 0 : 1);
-        const float L = live ? ((slot & 1) ? L1 : L0) : -INFINITY;
-        if constexpr (kF16) sc_s[j] = (slot & 1) ? S1 : S0;
-        slot_s[j] = slot;
-        w_s[j] = L;
-        m = fmaxf(m, L);
+        const uint32_t row = pieces.row(j, h, k);
+        const float L = p.partial_lse[row];
+        if constexpr (kF16) sc_s[j] = p.partial_scale[row];
+        w_s[j] = pieces.live(p, j) ? L : -INFINITY;
+        m = fmaxf(m, w_s[j]);
     }
     for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
     if ((c & 31) == 0) red_s[c >> 5] = m;
     __syncthreads();
     m = reference_max(fmaxf(fmaxf(red_s[0], red_s[1]), fmaxf(red_s[2], red_s[3])));
-    for (int j = c; j < nparts; j += kMergeThreads) w_s[j] = expf(w_s[j] - m);     // 0 for dead workers
-    __syncthreads();
     float Z = 0.f;
-    for (int j = 0; j < nparts; ++j) Z += w_s[j];          // same order in every thread: one value of Z
+    for (int j = c; j < nparts; j += kMergeThreads) { w_s[j] = expf(w_s[j] - m); Z += w_s[j]; }     // 0 for dead workers
+    for (int o = 16; o; o >>= 1) Z += __shfl_xor_sync(0xffffffffu, Z, o);
+    if ((c & 31) == 0) sum_s[c >> 5] = Z;
+    __syncthreads();
+    Z = (sum_s[0] + sum_s[1]) + (sum_s[2] + sum_s[3]);     // the same in every thread
     if (Z == 0.f) {                        // no piece saw a token (a query row whose causal range is empty)
         o4[c] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (c == 0) *lse = -INFINITY;
         return;
     }
-    const float L = m + logf(Z);
     const float inv_z = 1.f / Z;
-    // this thread's four columns of a slot's row as they lie in memory (loads first, conversions with the arithmetic:
-    // a conversion next to its load would make every load wait for the one before it)
-    using Raw = typename std::conditional<kF16, uint2, float4>::type;
-    auto load_part = [&](int slot) -> Raw {
-        const int64_t row = (int64_t)slot * h + k;
-        if constexpr (kF16) return reinterpret_cast<const uint2 *>(reinterpret_cast<const __half *>(p.partial_out) + row * kDV)[c];
-        else return reinterpret_cast<const float4 *>(p.partial_out + row * kDV)[c];
-    };
-    auto widen = [](const Raw &r) -> float4 {
-        if constexpr (kF16) {
-            const float2 a = __half22float2(*reinterpret_cast<const __half2 *>(&r.x)), b = __half22float2(*reinterpret_cast<const __half2 *>(&r.y));
-            return make_float4(a.x, a.y, b.x, b.y);
-        } else {
-            return r;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    auto add = [&](int j, const typename Row::Raw &raw) {
+        float w = w_s[j] * inv_z;
+        if (w != 0.f) {                    // a dead worker's slot holds stale bytes
+            if constexpr (kF16) w *= sc_s[j];
+            Row::add(acc, raw, w);
         }
     };
-    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    int j = 0;
+#pragma unroll
+    for (int u = 0; u < kFirst; ++u)
+        if (u < nparts) add(u, first[u]);
+    int j = kFirst;
     // sixteen, then (up to) four part loads in flight per thread: one long context cut into a piece per worker is merged by
     // one block per head, and the part loop is a chain of round trips to L2 / HBM
     for (; !kLean && j + 16 <= nparts; j += 16) {
-        Raw raw[16];
+        typename Row::Raw raw[16];
 #pragma unroll
-        for (int u = 0; u < 16; ++u)
-            raw[u] = load_part(slot_s[j + u]);
+        for (int u = 0; u < 16; ++u) raw[u] = Row::load(p, pieces.row(j + u, h, k), c);
 #pragma unroll
-        for (int u = 0; u < 16; ++u) {
-            float wgt = w_s[j + u] * inv_z;
-            if (wgt != 0.f) {          // a dead worker's slot holds stale bytes
-                if constexpr (kF16) wgt *= sc_s[j + u];
-                const float4 v = widen(raw[u]);
-                acc.x = fmaf(wgt, v.x, acc.x); acc.y = fmaf(wgt, v.y, acc.y);
-                acc.z = fmaf(wgt, v.z, acc.z); acc.w = fmaf(wgt, v.w, acc.w);
-            }
-        }
+        for (int u = 0; u < 16; ++u) add(j + u, raw[u]);
     }
-    // the rest four at a time as well, loads first: taken one by one, each part's load would wait for the previous
-    // part's arithmetic, and a request cut into two or three pieces (the usual case) would pay a round trip per piece
+    // (loads first: a request cut into two or three pieces, the usual case, would pay a round trip per piece)
     for (; j < nparts; j += 4) {
-        Raw raw[4];
+        typename Row::Raw raw[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u)
-            if (j + u < nparts) raw[u] = load_part(slot_s[j + u]);
+            if (j + u < nparts) raw[u] = Row::load(p, pieces.row(j + u, h, k), c);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            float wgt = j + u < nparts ? w_s[j + u] * inv_z : 0.f;
-            if (wgt != 0.f) {          // a dead worker's slot holds stale bytes
-                if constexpr (kF16) wgt *= sc_s[j + u];
-                const float4 v = widen(raw[u]);
-                acc.x = fmaf(wgt, v.x, acc.x); acc.y = fmaf(wgt, v.y, acc.y);
-                acc.z = fmaf(wgt, v.z, acc.z); acc.w = fmaf(wgt, v.w, acc.w);
-            }
-        }
+        for (int u = 0; u < 4; ++u)
+            if (j + u < nparts) add(j + u, raw[u]);
     }
     o4[c] = acc;
-    if (c == 0) *lse = L;
+    if (c == 0) *lse = m + logf(Z);
 }
 
 // The same for launches of no more rows than SMs (a small batch): four groups of 128 threads take every fourth piece and add
-// their sums in shared memory.  2 KB of that and 32 registers, so that a block fits beside a decode CTA of 16 heads:
-// the next call's CTAs come in, plan and prefetch while this kernel runs (eight layers of 8 requests: with the kernel above, 6 KB
-// a block, they came in 1.6 to 4.4 us later, one by one as its blocks left).
+// their sums in shared memory.  Behind the kernels of 16 and 32 heads 2 KB of shared memory and 32 registers, so that a block fits
+// beside a decode CTA of 16 heads: the next call's CTAs come in, plan and prefetch while this kernel runs (eight layers of 8 requests:
+// with the kernel above, 6 KB a block, they came in 1.6 to 4.4 us later, one by one as its blocks left; with 40 registers too).  Behind the
+// others (kDeep), which leave no room for that anyway, more loads are in flight, the first of them beside those of the LSEs: 74
+// pieces on 128 heads 5.4 us, now 4.5.  (A warp for itself with 32 columns of a row and no barriers: 10 us, every warp loads all LSEs then.)
 constexpr int kGroupedParts = 160, kCombineGroups = 4;
-template <bool kF16>
-__global__ void __launch_bounds__(kCombineGroups * kMergeThreads, 4)
+template <bool kF16, bool kDeep>
+__global__ void __launch_bounds__(kCombineGroups * kMergeThreads, kDeep ? 2 : 4)
 grouped_combine_kernel(const DecodeParams p, const int4 *split_rec) {
-    constexpr int kThreads = kCombineGroups * kMergeThreads, kDepth = 4;
-    // weights, slots and (f16 pieces) the power of two each row was divided by; then the groups' sums
-    constexpr int kFloats = (kF16 ? 3 : 2) * kGroupedParts;
-    __shared__ __align__(16) float smem_f[kFloats > 4 * kMergeThreads ? kFloats : 4 * kMergeThreads];
+    using Row = PartRow<kF16>;
+    constexpr int kThreads = kCombineGroups * kMergeThreads, kDepth = !kDeep ? 4 : kF16 ? 16 : 8;
+    // weights (f16 pieces: times the power of two each row was divided by); then the groups' sums
+    __shared__ __align__(16) float smem_f[4 * kMergeThreads];
+    static_assert(kGroupedParts <= 4 * kMergeThreads && kGroupedParts <= kThreads, "a piece per thread");
     __shared__ float max_s[kThreads / 32], sum_s[kThreads / 32];
-    float *const w_s = smem_f, *const sc_s = smem_f + 2 * kGroupedParts;
-    int *const slot_s = reinterpret_cast<int *>(smem_f + kGroupedParts);
+    float *const w_s = smem_f;
     const int h = p.head_end - p.head_begin;
     const int k = blockIdx.x % h, entry = blockIdx.x / h;
     const int g = p.head_begin + k;
     grid_launch_dependents();
     grid_dependency_wait();
     const int n_entries = p.status[8];
-    const int4 rec = split_rec[entry];
+    const Pieces pieces(split_rec[entry]);
     if (entry >= n_entries) return;
-    const int i = rec.x, wf = rec.y, nparts = rec.z - rec.y + 1, rs = rec.w;
+    const int i = pieces.request, nparts = pieces.n;
     float4 *o4 = reinterpret_cast<float4 *>(p.out + (int64_t)i * p.out_stride_request + (int64_t)g * p.out_stride_head);
     float *lse = p.lse + (int64_t)i * p.lse_stride_request + g;
     const int tid = threadIdx.x, c = tid % kMergeThreads, group = tid / kMergeThreads;
-    float L = -INFINITY;
-    if (tid < nparts) {                    // (kThreads >= kGroupedParts: a piece per thread)
-        const int w = wf + tid;
-        const int wb0 = p.worker_begin[w], wb1 = p.worker_begin[w + 1];
-        const float L0 = p.partial_lse[(int64_t)(2 * w) * h + k];
-        const float L1 = tid == 0 ? p.partial_lse[(int64_t)(2 * w + 1) * h + k] : 0.f;
-        float S0 = 1.f, S1 = 1.f;
-        if constexpr (kF16) {
-            S0 = p.partial_scale[(int64_t)(2 * w) * h + k];
-            if (tid == 0) S1 = p.partial_scale[(int64_t)(2 * w + 1) * h + k];
-        }
-        const int slot = 2 * w + (rs <= wb0 ? 0 : 1);
-        if (wb1 > wb0) L = (slot & 1) ? L1 : L0;
-        if constexpr (kF16) sc_s[tid] = (slot & 1) ? S1 : S0;
-        slot_s[tid] = slot;
+    float L = -INFINITY, scale = 1.f;
+    if (tid < nparts) {
+        const uint32_t row = pieces.row(tid, h, k);
+        L = p.partial_lse[row];
+        if constexpr (kF16) scale = p.partial_scale[row];
+        if (!pieces.live(p, tid)) L = -INFINITY;
     }
+    typename Row::Raw raw[kDepth];
+    auto load = [&](int j0) {
+#pragma unroll
+        for (int u = 0; u < kDepth; ++u) {
+            const int j = j0 + u * kCombineGroups;
+            if (j < nparts) raw[u] = Row::load(p, pieces.row(j, h, k), c);
+        }
+    };
+    if constexpr (kDeep) load(group);
     float m = L;
     for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
     if ((tid & 31) == 0) max_s[tid >> 5] = m;
@@ -262,7 +292,7 @@ grouped_combine_kernel(const DecodeParams p, const int4 *split_rec) {
     for (int x = 1; x < kThreads / 32; ++x) m = fmaxf(m, max_s[x]);
     m = reference_max(m);
     float Z = tid < nparts ? expf(L - m) : 0.f;
-    if (tid < nparts) w_s[tid] = Z;
+    if (tid < nparts) w_s[tid] = Z == 0.f ? 0.f : Z * scale;       // (a slot nobody wrote holds any scale)
     for (int o = 16; o; o >>= 1) Z += __shfl_xor_sync(0xffffffffu, Z, o);
     if ((tid & 31) == 0) sum_s[tid >> 5] = Z;
     __syncthreads();
@@ -275,33 +305,14 @@ grouped_combine_kernel(const DecodeParams p, const int4 *split_rec) {
         return;
     }
     const float inv_z = 1.f / Z;
-    using Raw = typename std::conditional<kF16, uint2, float4>::type;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int j0 = group; j0 < nparts; j0 += kCombineGroups * kDepth) {
-        Raw raw[kDepth];
-#pragma unroll
-        for (int u = 0; u < kDepth; ++u)
-            if (j0 + u * kCombineGroups < nparts) {
-                const int64_t row = (int64_t)slot_s[j0 + u * kCombineGroups] * h + k;
-                if constexpr (kF16) raw[u] = reinterpret_cast<const uint2 *>(reinterpret_cast<const __half *>(p.partial_out) + row * kDV)[c];
-                else raw[u] = reinterpret_cast<const float4 *>(p.partial_out + row * kDV)[c];
-            }
+        if (!kDeep || j0 != group) load(j0);
 #pragma unroll
         for (int u = 0; u < kDepth; ++u) {
             const int j = j0 + u * kCombineGroups;
-            float wgt = j < nparts ? w_s[j] * inv_z : 0.f;
-            if (wgt != 0.f) {              // a dead worker's slot holds stale bytes
-                float4 v;
-                if constexpr (kF16) {
-                    wgt *= sc_s[j];
-                    const float2 a = __half22float2(*reinterpret_cast<const __half2 *>(&raw[u].x)), b = __half22float2(*reinterpret_cast<const __half2 *>(&raw[u].y));
-                    v = make_float4(a.x, a.y, b.x, b.y);
-                } else {
-                    v = raw[u];
-                }
-                acc.x = fmaf(wgt, v.x, acc.x); acc.y = fmaf(wgt, v.y, acc.y);
-                acc.z = fmaf(wgt, v.z, acc.z); acc.w = fmaf(wgt, v.w, acc.w);
-            }
+            const float w = j < nparts ? w_s[j] * inv_z : 0.f;
+            if (w != 0.f) Row::add(acc, raw[u], w);              // a dead worker's slot holds stale bytes
         }
     }
     float4 *const total = reinterpret_cast<float4 *>(smem_f);
@@ -347,14 +358,18 @@ cudaError_t launch_split_combine(const DecodeParams &p, const int4 *split_rec, i
         cudaFuncSetAttribute(split_combine_kernel<true, false>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
         cudaFuncSetAttribute(split_combine_kernel<false, true>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
         cudaFuncSetAttribute(split_combine_kernel<true, true>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-        cudaFuncSetAttribute(grouped_combine_kernel<false>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-        cudaFuncSetAttribute(grouped_combine_kernel<true>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+        cudaFuncSetAttribute(grouped_combine_kernel<false, false>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+        cudaFuncSetAttribute(grouped_combine_kernel<false, true>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+        cudaFuncSetAttribute(grouped_combine_kernel<true, true>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
         return cudaSuccess;
     });
     // many requests per worker: every request is cut into a few pieces at most
     const bool lean = (int64_t)p.B * 4 >= p.num_workers;
-    const bool grouped = !lean && grid.x <= (unsigned)sm_count && p.num_workers <= kGroupedParts;
-    auto kernel = grouped ? (p.partial_f16 ? grouped_combine_kernel<true> : grouped_combine_kernel<false>) : p.partial_f16 ? (lean ? split_combine_kernel<true, true> : split_combine_kernel<true, false>)
+    const bool room = p.heads_per_group <= 32 && p.num_groups == 1;       // for a block beside a decode CTA
+    // as many rows as are resident at once (room: one beside each CTA): two requests on 128 heads 17.8 us, now 16.1; with 384 rows 18.0 against 17.4
+    const bool grouped = !lean && grid.x <= (room ? 1u : 2u) * (unsigned)sm_count && p.num_workers <= kGroupedParts;
+    auto kernel = grouped ? (p.partial_f16 ? grouped_combine_kernel<true, true> : room ? grouped_combine_kernel<false, false> : grouped_combine_kernel<false, true>)
+                : p.partial_f16 ? (lean ? split_combine_kernel<true, true> : split_combine_kernel<true, false>)
                                 : (lean ? split_combine_kernel<false, true> : split_combine_kernel<false, false>);
     cudaError_t e = launch_dependent(kernel, grid, dim3(grouped ? kCombineGroups * kMergeThreads : kMergeThreads), 0, stream, p, split_rec);
     count_launch();
