@@ -275,14 +275,9 @@ int decode_dense(const splash_mla_shape *shape, const void *q, const void *kv_po
     // itself; if its contexts are short besides, no request is cut and the combine kernel is left out
     int plan_mode = kPlanWorkspace;
     const int plan_workers = t.num_workers;
-    bool e4m3_pairs = false;
     if (!simt && !(shape->flags & SPLASH_FLAG_VALIDATE) && B <= kInlinePlanRequests) {
         const int pages = sparse ? sparse->pages_per_request : shape->block_table_stride;
-        // (the e4m3 pair kernel's own plan saves 4 us and costs 2.6 % of its main loop: long contexts keep the plan kernel; and a call
-        // that takes a partition over finds it in the workspace, whoever has made it)
-        e4m3_pairs = shape->kv_dtype == SPLASH_KV_E4M3_TOKEN_SCALE && t.num_groups == 2 && !(shape->flags & SPLASH_FLAG_NO_PAIR);
-        if (!e4m3_pairs || (int64_t)B * pages * t.pair_groups <= kInlinePairPages)
-            plan_mode = pages <= kWholeRequestPages && B <= t.num_workers ? kPlanWhole : kPlanInline;
+        plan_mode = pages <= kWholeRequestPages && B <= t.num_workers ? kPlanWhole : kPlanInline;
         if (plan_mode == kPlanWhole) t.num_workers = B;
     }
     PlanView v = make_plan_view(workspace, B, plan_workers, h);
@@ -304,7 +299,7 @@ int decode_dense(const splash_mla_shape *shape, const void *q, const void *kv_po
     p.softmax_scale = shape->softmax_scale;
     p.tile_start = v.tile_start; p.req_lo = v.req_lo; p.req_hi = v.req_hi; p.worker_begin = v.worker_begin;
     p.worker_req = v.worker_req; p.split_rec = v.split_rec;
-    p.plan_mode = plan_mode; p.plan_workers = e4m3_pairs ? plan_workers : 0; p.kv_begin = kv_begin; p.kv_end = kv_end;
+    p.plan_mode = plan_mode; p.kv_begin = kv_begin; p.kv_end = kv_end;
     p.status = v.status; p.partial_lse = v.partial_lse; p.partial_out = v.partial_out; p.partial_scale = v.partial_scale;
     p.trace = g_trace;
     p.len_cap = sparse ? sparse->max_selected : -1;

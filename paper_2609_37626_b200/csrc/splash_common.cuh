@@ -139,8 +139,7 @@ struct DecodeParams {
     int32_t num_workers;
     int32_t request_overhead_tiles;   // per-request cost the plan adds to the tile count
     int32_t plan_mode;                // kPlanWorkspace, kPlanInline or kPlanWhole
-    int32_t plan_workers;             // > 0: an inline plan is left in the workspace in full, as one for that many workers, for a
-                                      // later call that takes it over and reads it there
+    int32_t q_by_hand;                // e4m3 kernels: the query rows come by plain loads (strides that a tensor map cannot state)
     int32_t clear_status;             // 1: no plan kernel ran (its partition is taken again): block 0 clears the error words
     const int32_t *kv_begin, *kv_end; // the inline modes read the ranges themselves
     int4 *split_rec;                  // kPlanInline: where block 0 leaves the combine kernel's records
@@ -183,7 +182,6 @@ constexpr int kInlinePlanRequests = 32;
 // (contexts of at most this many pages: 4 requests in a table as wide as they are against one of 2,048 columns, whose requests are cut and
 // combined: 16 heads 11.9 against 15 to 16 us, 128 heads 11.1 against 13.8, e4m3 9.1 against 12.8 and 16.9 against 21.4)
 constexpr int kWholeRequestPages = 4;
-constexpr int kInlinePairPages = 8192;
 // shared-memory copy of an inline plan: tile_start[B + 1], lo[B], hi[B] (as in the workspace), then the worker's first
 // tile, its end, and the request that holds the first
 constexpr uint32_t kInlinePlanBytes = ((3 * kInlinePlanRequests + 4) * 4 + 15) / 16 * 16;
@@ -282,24 +280,14 @@ static __device__ __noinline__ void plan_ahead(const DecodeParams &p, int worker
     for (int i = lane; i < rows * 9; i += 32) asm volatile("prefetch.global.L2 [%0];" ::"l"(q + (int64_t)(i / 9) * p.q_stride_head * 2 + (i % 9) * 128));
 }
 
-// What the combine kernel reads.  The first CTA of every worker leaves its own first tile (start_plan); the same warp of block 0, once its
-// CTA is under way, the list of the requests that were cut, and clears the status block (this cannot wipe another CTA's report: the first
+// What the combine kernel reads: the plan's warp of block 0 leaves the list of the requests that were cut, once its CTA is under way, and clears
+// the status block (this cannot wipe another CTA's report: the first
 // one a CTA can make is the end of a bounded wait, seconds after this).  A lane knows the first and the last worker of its request
 // from the costs alone: worker w starts at or before tile t of a request whose cost begins at c iff floor(w cost / W) <= c + overhead + t,
 // so the last such worker is floor(((c + overhead + t + 1) W - 1) / cost).  (Block 0 going through all workers for every request was
 // late by microseconds at many requests: 32 of 2,048 tokens, 16 heads over e4m3, 23.7 us a call, now 20.2.)
 static __device__ __noinline__ void publish_inline_plan(const DecodeParams &p, const int32_t *ts, int lane) {
     const int B = p.B, overhead = p.request_overhead_tiles;
-    if (p.plan_workers > 0) {
-        for (int i = lane; i <= B; i += 32) const_cast<int32_t *>(p.tile_start)[i] = ts[i];
-        if (lane < B) { const_cast<int32_t *>(p.req_lo)[lane] = ts[B + 1 + lane]; const_cast<int32_t *>(p.req_hi)[lane] = ts[2 * B + 1 + lane]; }
-        if (p.plan_mode == kPlanWhole) {       // a request each, nothing for the other workers
-            for (int w = lane; w <= p.plan_workers; w += 32) {
-                const_cast<int32_t *>(p.worker_begin)[w] = ts[min(w, B)];
-                const_cast<int32_t *>(p.worker_req)[w] = min(w, B - 1);
-            }
-        }
-    }
     int split = 0;
     if (p.plan_mode == kPlanInline) {
         const int n = lane < B ? ts[lane + 1] - ts[lane] : 0;
@@ -397,11 +385,11 @@ struct SegmentIter<kPlanInWorkspace> {
 };
 
 // The beginning of a decode kernel, all threads, around its grid_dependency_wait: the plan's origin by the call's mode.
-// `first_cta`: the first of its worker's CTAs.  `plan_warp`: a warp that is not needed at once.  kAhead: the kernel leaves a combine block room beside its CTA, so its CTAs are
+// `plan_warp`: a warp that is not needed at once.  kAhead: the kernel leaves a combine block room beside its CTA, so its CTAs are
 // there well before the wait ends and may plan ahead; where they come in only as the blocks before them leave, planning twice
 // is time lost (1 us of a call).  A call that cuts no request has no combine kernel in front of the next one: always ahead.
 template <bool kAhead, uint32_t kPlanOffset>
-__device__ __forceinline__ void start_plan(const DecodeParams &p, int worker, bool first_cta, int plan_warp, SegmentIter<kPlanOffset> &it, const FirstLoads &f) {
+__device__ __forceinline__ void start_plan(const DecodeParams &p, int worker, int plan_warp, SegmentIter<kPlanOffset> &it, const FirstLoads &f) {
     if constexpr (kPlanOffset != kPlanInWorkspace) {
         if (p.plan_mode != kPlanWorkspace) {
             const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -418,12 +406,6 @@ __device__ __forceinline__ void start_plan(const DecodeParams &p, int worker, bo
                 if (!ahead || __any_sync(0xffffffffu, lo2 != lo || hi2 != hi)) build_inline_plan(p, worker, sp, lane, lo2, hi2);
             }
             __syncthreads();
-            if (first_cta && warp == plan_warp && lane == 0 && p.plan_mode == kPlanInline) {
-                int32_t *const begin = const_cast<int32_t *>(p.worker_begin) + worker;
-                begin[0] = sp[3 * p.B + 1];
-                if (worker == p.num_workers - 1) begin[1] = sp[p.B];
-                if (p.plan_workers > 0) const_cast<int32_t *>(p.worker_req)[worker] = sp[3 * p.B + 3];
-            }
             if (blockIdx.x == 0 && warp == plan_warp) publish_inline_plan(p, sp, lane);
             it.init(p, worker);
             return;

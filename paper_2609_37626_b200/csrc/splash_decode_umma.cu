@@ -134,7 +134,7 @@ decode_umma_kernel(const __grid_constant__ DecodeParams p, const __grid_constant
     tcgen05_fence_after();
     const uint32_t tmem_base = misc[0];
     SegmentIter<L::kOffPlan> it;
-    start_plan<N < 64>(p, worker, group == 0, kWarpGather - 1, it, FirstLoads{kStageBytes, 0u, kStageBytes, kStages + 1, head0, N});
+    start_plan<N < 64>(p, worker, kWarpGather - 1, it, FirstLoads{kStageBytes, 0u, kStageBytes, kStages + 1, head0, N});
     const long long t_start = clock64();
 
     Segment seg;

@@ -79,7 +79,7 @@ static_assert(kOffQHi % 512 == 0 && kOffQLo % 512 == 0 && kOffPHi % 512 == 0 && 
 // tensor memory: O^T 4 blocks x 64 columns, then 2 S buffers x 2 partial accumulators x 64 columns
 constexpr uint32_t kColO = 0, kColS = 256;
 
-// kInline: the variant that can plan for itself, as in splash_decode_umma_fp8_pair.cu (64 requests of 1,000 to 8,000 tokens on 128 heads:
+// kInline: the variant that can plan for itself (the kernel sits at its register cap: 64 requests of 1,000 to 8,000 tokens on 128 heads:
 // 142.3 us with one kernel for both, 139.5 before it could)
 template <bool kInline>
 __global__ void __launch_bounds__(kThreads, 1)
@@ -119,7 +119,7 @@ decode_umma_fp8_kernel(const __grid_constant__ DecodeParams p, const __grid_cons
     tcgen05_fence_after();
     const uint32_t tmem_base = misc[0];
     SegmentIter<kInline ? kOffPlan : kPlanInWorkspace> it;
-    start_plan<false>(p, worker, blockIdx.x % p.num_groups == 0, kThreads / 32 - 1, it, FirstLoads{kStageBytes, 0u, kStageBytes, kStages, head0, kN});
+    start_plan<false>(p, worker, kThreads / 32 - 1, it, FirstLoads{kStageBytes, 0u, kStageBytes, kStages, head0, kN});
     const long long t_start = clock64();
 
     Segment seg;

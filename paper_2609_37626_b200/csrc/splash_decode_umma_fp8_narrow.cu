@@ -142,7 +142,7 @@ decode_umma_fp8_narrow_kernel(const __grid_constant__ DecodeParams p, const __gr
     tcgen05_fence_after();
     const uint32_t tmem_base = misc[0];
     SegmentIter<L::kOffPlan> it;
-    start_plan<N == 16>(p, worker, group == 0, kThreads / 32 - 1, it, FirstLoads{kStageBytes, 0u, kStageBytes, kStages, head0, N});
+    start_plan<N == 16>(p, worker, kThreads / 32 - 1, it, FirstLoads{kStageBytes, 0u, kStageBytes, kStages, head0, N});
     const long long t_start = clock64();
 
     Segment seg;

@@ -36,6 +36,7 @@
 // Barriers that the issuers wait on live in the leader; the peer's warps arrive on them across
 // the cluster (relaxed arrivals: what they announce is already in place on the peer's SM), and
 // TMA loads of the peer complete on them too.
+// The query rows come by TMA once the last QK^T of the request before has read their predecessors, and are split in place.
 #include "splash_fp8.cuh"
 #include "splash_pair.cuh"
 
@@ -72,7 +73,8 @@ struct Layout {
         kBarStageEmpty = kBarVFull + kStages, // [stages] P.V of the stage retired (multicast commit): stage, its scales and
                                               //     the P buffer are free, O is up to date
         kBarScFull = kBarStageEmpty + kStages,// [stages] local: scale pages of the stage landed
-        kBarQFull = kBarScFull + kStages,     // leader: query operands of both CTAs written
+        kBarQRaw = kBarScFull + kStages,      // local: the request's query rows landed
+        kBarQFull,                            // leader: query operands of both CTAs written
         kBarQLocal,                           // local: this CTA's query scales written
         kBarQEmpty,                           // last QK^T of the request retired (multicast commit)
         kBarQsRead,                           // local: the softmax warps have picked up the request's query scales
@@ -83,9 +85,10 @@ struct Layout {
         kBarOEmpty,                           // O drained (leader: by both CTAs)
         kNumBarriers
     };
-    // query operand: 9 chunk slabs of 64 rows x 64 B for q hi and as many for q lo (H = 64), or both as rows of one (H = 32)
-    static constexpr uint32_t kQTerm = H == 64 ? 9 * kSlab : 16 * 64;        // from a head's hi row to its lo row
-    static constexpr uint32_t kPTerm = H == 64 ? 2 * kSlab : 16 * 64;        // the same in P
+    // query operand: 9 chunk slabs of 2 H rows x 64 B, eight hi rows and the same heads' eight lo rows in turn (QueryRows).  H = 64: two
+    // operands, 1,024 bytes from one group of eight rows to the next; H = 32: one
+    static constexpr uint32_t kQSlab = 2 * H * 64;
+    static constexpr uint32_t kPTerm = H == 64 ? 2 * kSlab : 16 * 64;        // from a head's hi row of P to its lo row
     static constexpr uint32_t kPBuf = H == 64 ? 4 * kSlab : 2 * kSlab;
     static constexpr uint32_t kOffK = 0;                            // [stages] 9 chunk slots
     static constexpr uint32_t kOffQ = kOffK + kStages * kPageBytes;
@@ -107,23 +110,27 @@ struct Layout {
     static constexpr uint32_t kColO = 0, kColS = 256;
 };
 
-// Issued by the elected lane of a converged warp; the operands are uniform.
-__device__ __forceinline__ void umma_e4m3_pair(uint32_t elected, uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+// Issued by the elected lane of a converged warp; the operands are uniform.  `a_at`, `b_at`: 16-byte units added to the descriptors'
+// addresses.  Only the low words of the descriptors move with them, and what they start from is said to be uniform: with 64-bit sums, and
+// addresses that only happen to be the same in all lanes, an issuer is slower than the tensor pipe (128 heads: 150 requests of 6,000 tokens
+// 288 us, now 266; the rollout batch 680 and 627).
+__device__ __forceinline__ void umma_e4m3_pair(uint32_t elected, uint32_t d_tmem, uint64_t a_desc, uint32_t a_at, uint64_t b_desc, uint32_t b_at, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "setp.ne.b32 q, %5, 0;\n\t"
-        "@q tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(elected) : "memory");
+        "{\n\t.reg .pred p, q;\n\t.reg .b64 a, b;\n\t"
+        "setp.ne.b32 p, %6, 0;\n\t"
+        "setp.ne.b32 q, %7, 0;\n\t"
+        "mov.b64 a, {%1, %2};\n\t"
+        "mov.b64 b, {%3, %4};\n\t"
+        "@q tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], a, b, %5, p;\n\t}"
+        ::"r"(d_tmem), "r"((uint32_t)a_desc + a_at), "r"((uint32_t)(a_desc >> 32)), "r"((uint32_t)b_desc + b_at), "r"((uint32_t)(b_desc >> 32)),
+          "r"(idesc), "r"(accumulate), "r"(elected) : "memory");
 }
 
-// kInline: the variant that can plan for itself.  The kernel sits at its register cap, and a walk over the segments that
-// can read either plan costs the main loop 0.6 to 2.4 % of its cycles: calls behind a plan kernel have their own variant.
-template <int H, bool kInline>
+template <int H>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid_constant__ CUtensorMap tmap_page,
                             const __grid_constant__ CUtensorMap tmap_pair, const __grid_constant__ CUtensorMap tmap_out,
-                            const __grid_constant__ CUtensorMap tmap_part) {
+                            const __grid_constant__ CUtensorMap tmap_part, const __grid_constant__ CUtensorMap tmap_q) {
     using L = Layout<H>;
     constexpr int kStages = L::kStages;
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -152,6 +159,7 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
             mbar_init(bar(L::kBarVFull + s), 1); mbar_init(bar(L::kBarStageEmpty + s), 1);
             mbar_init(bar(L::kBarScFull + s), 1);
         }
+        mbar_init(bar(L::kBarQRaw), 1);
         mbar_init(bar(L::kBarQFull), 2 * kConvertWarps); mbar_init(bar(L::kBarQLocal), kConvertWarps); mbar_init(bar(L::kBarQEmpty), 1);
         mbar_init(bar(L::kBarQsRead), kSoftmaxWarps);
         for (int b = 0; b < 2; ++b) {
@@ -171,8 +179,8 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
     cluster_sync_all();                                   // barriers of both CTAs exist before anyone signals them
     tcgen05_fence_after();
     const uint32_t tmem_base = misc[0];
-    SegmentIter<kInline ? L::kOffPlan : kPlanInWorkspace> it;
-    start_plan<false>(p, worker, rank == 0 && pair_id == worker * p.pair_groups, kThreads / 32 - 1, it, FirstLoads{kPageBytes, 0u, kPageBytes, kStages, head0, H});
+    SegmentIter<L::kOffPlan> it;
+    start_plan<false>(p, worker, kThreads / 32 - 1, it, FirstLoads{kPageBytes, 0u, kPageBytes, kStages, head0, H});
     const long long t_start = clock64();
     const unsigned long long ns_start = global_timer_ns();
 
@@ -293,14 +301,14 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 tcgen05_fence_after();
-                const uint32_t d = tmem_u + L::kColS + b * 64;
-                const uint64_t dq = make_desc_sw64(sbase + L::kOffQ, 16, 512);                            // A: 2 x 64 rows x 32
-                const uint64_t dk = make_desc_sw64(sbase + L::kOffK + stage * kPageBytes, 16, 512);       // B: 2 x 64 tokens x 32
+                const uint32_t d = uniform(tmem_u + L::kColS + b * 64);
+                const uint64_t dq = make_desc_sw64(uniform(sbase + L::kOffQ), 16, H == 64 ? 1024 : 512);           // A: 2 x 64 rows x 32
+                const uint64_t dk = make_desc_sw64(uniform(sbase + L::kOffK + stage * kPageBytes), 16, 512);       // B: 2 x 64 tokens x 32
                 // 18 K = 32 steps, for H = 64 with q hi and then with q lo
 #pragma unroll
                 for (int t = 0; t < (H == 64 ? 36 : 18); ++t) {
-                    const uint32_t ks = t % 18, at = (ks >> 1) * kSlab + (ks & 1) * 32;
-                    umma_e4m3_pair(elected, d, dq + (((t / 18) * L::kQTerm + at) >> 4), dk + (at >> 4), kIdescQK, t != 0);
+                    const uint32_t ks = t % 18, at = (ks >> 1) * kSlab + (ks & 1) * 32, at_q = (ks >> 1) * L::kQSlab + (ks & 1) * 32;
+                    umma_e4m3_pair(elected, d, dq, ((t / 18) * 512 + at_q) >> 4, dk, at >> 4, kIdescQK, t != 0);
                 }
                 if (elected) { umma_commit_pair(bar(L::kBarSFull + b)); umma_commit_pair(bar(L::kBarQkDone + stage)); }
                 __syncwarp();
@@ -329,8 +337,8 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
                 tcgen05_fence_after();
                 const int pages = 2 * s + 1 < ntiles ? 2 : 1;     // page B's MMAs are skipped when it does not exist
                 // A: P rows, slab = page, 32 tokens; B: slots 4n + 2 page, + 1 (two 64-wide dv chunks, LBO), 32 tokens
-                const uint64_t da = make_desc_sw64(sbase + L::kOffP + pb * L::kPBuf, 16, 512);
-                const uint64_t db = make_desc_sw64(sbase + L::kOffK + stage * kPageBytes, kSlab, 512);
+                const uint64_t da = make_desc_sw64(uniform(sbase + L::kOffP + pb * L::kPBuf), 16, 512);
+                const uint64_t db = make_desc_sw64(uniform(sbase + L::kOffK + stage * kPageBytes), kSlab, 512);
 #pragma unroll
                 for (int hl = 0; hl < (H == 64 ? 2 : 1); ++hl) {
                     for (int pg = 0; pg < pages; ++pg) {
@@ -338,8 +346,8 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
                         for (int k = 0; k < 2; ++k) {
 #pragma unroll
                             for (int n = 0; n < 2; ++n)           // dv half: columns [256 n, 256 n + 256)
-                                umma_e4m3_pair(elected, tmem_u + L::kColO + n * 128, da + ((hl * L::kPTerm + pg * kSlab + k * 32) >> 4),
-                                               db + (((4 * n + 2 * pg) * kSlab + k * 2048) >> 4), hl ? kIdescPVLo : kIdescPV,
+                                umma_e4m3_pair(elected, tmem_u + L::kColO + n * 128, da, (hl * L::kPTerm + pg * kSlab + k * 32) >> 4,
+                                               db, ((4 * n + 2 * pg) * kSlab + k * 2048) >> 4, hl ? kIdescPVLo : kIdescPV,
                                                (uint32_t)s | (uint32_t)(hl | pg | k));
                         }
                     }
@@ -356,81 +364,38 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
         // (the issuer warps of the peer CTA have nothing to do)
     } else if (warp >= kWarpConvert && warp < kWarpConvert + kConvertWarps) {
         // ===================================================== query converters (this CTA's heads)
-        const int ct = (warp - kWarpConvert) * 32 + lane;   // 0..127
+        using Rows = QueryRows<H, kConvertWarps>;
+        const int cw = warp - kWarpConvert;
         float *qs_s = reinterpret_cast<float *>(smem + L::kOffQs);
         uint32_t seg_it = 0;
         bool ok = true;
         while (ok && it.next(p, seg)) {
             {
-                constexpr int kParts = 128 / H, kVecs = 72 / kParts;      // threads per head, 16-byte loads per thread
-                const int hd = ct / kParts, part = ct % kParts;
-                const int gh = head0 + hd;
-                const bool live = gh < p.head_end;
-                const uint4 *src = reinterpret_cast<const uint4 *>(
-                    static_cast<const __nv_bfloat16 *>(p.q) + (int64_t)seg.request * p.q_stride_request +
-                    (int64_t)(live ? gh : p.head_begin) * p.q_stride_head + part * (kVecs * 8));
-                // first pass (row maximum) while the previous request is still being multiplied
-                float amax = 0.f;
-                if (live) {
-#pragma unroll 1
-                    for (int v0 = 0; v0 < kVecs; v0 += kVecs / 3) {
-                        uint4 x[kVecs / 3];
-#pragma unroll
-                        for (int i = 0; i < kVecs / 3; ++i) x[i] = src[v0 + i];
-#pragma unroll
-                        for (int i = 0; i < kVecs / 3; ++i) {
-                            const uint32_t w[4] = {x[i].x, x[i].y, x[i].z, x[i].w};
-#pragma unroll
-                            for (int k = 0; k < 4; ++k) {
-                                amax = fmaxf(amax, fabsf(__uint_as_float(w[k] << 16)));
-                                amax = fmaxf(amax, fabsf(__uint_as_float(w[k] & 0xffff0000u)));
+                // the operand buffer is free once the last QK^T of the previous request has retired
+                Rows rows(smem + L::kOffQ, cw, lane);
+                const int gh = head0 + rows.row;
+                if (p.q_by_hand) {
+                    ok = warp_wait(ctx, bar(L::kBarQEmpty), (seg_it & 1) ^ 1, L::kBarQEmpty);
+                    if (!ok) break;
+                    rows.by_hand(static_cast<const __nv_bfloat16 *>(p.q) + (int64_t)seg.request * p.q_stride_request + (int64_t)gh * p.q_stride_head, gh < p.head_end);
+                } else {
+                    if (cw == 0) {
+                        if (lane == 0) {
+                            ok = mbar_wait(ctx, bar(L::kBarQEmpty), (seg_it & 1) ^ 1, L::kBarQEmpty);
+                            if (ok) {
+                                mbar_expect_tx(bar(L::kBarQRaw), Rows::kBytes);
+                                tma_load_4d(sbase + L::kOffQ, &tmap_q, bar(L::kBarQRaw), 0, head0, 0, seg.request);
                             }
                         }
+                        ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+                        if (!ok) break;
                     }
+                    ok = warp_wait(ctx, bar(L::kBarQRaw), seg_it & 1, L::kBarQRaw);
+                    if (!ok) break;
                 }
-#pragma unroll
-                for (int o = 1; o < kParts; o <<= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-                const float qs = amax > 0.f ? amax * (1.0f / 448.0f) : 1.0f;
-                const float inv = amax > 0.f ? 448.0f / amax : 1.0f;
-                if (part == 0) qs_s[(seg_it & 3) * H + hd] = qs;
-                // second pass in batches of nine 16-byte loads, a batch ahead: the first batch is in
-                // flight while this warp waits for the operand buffers, which are free once the last
-                // QK^T of the previous request has retired
-                uint4 xa[9], xb[9];
-                auto load_batch = [&](uint4 (&x)[9], int v0) {
-#pragma unroll
-                    for (int i = 0; i < 9; ++i) x[i] = live ? src[v0 + i] : make_uint4(0u, 0u, 0u, 0u);
-                };
-                auto convert_batch = [&](const uint4 (&x)[9], int v0) {
-#pragma unroll
-                    for (int i = 0; i < 9; ++i) {
-                        const uint32_t w[4] = {x[i].x, x[i].y, x[i].z, x[i].w};
-                        uint16_t hi[4], lo[4];
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            const float e0 = __uint_as_float(w[k] << 16) * inv, e1 = __uint_as_float(w[k] & 0xffff0000u) * inv;
-                            split_e4m3_e4m3_x2(e0, e1, hi[k], lo[k]);      // packed f16 arithmetic: half the instructions
-                        }
-                        const uint32_t d = (uint32_t)(part * (kVecs * 8) + (v0 + i) * 8);
-                        const uint32_t row = H == 64 ? hd : 2 * hd - (hd & 15);      // H = 32: 32 (hd / 16) + hd mod 16
-                        const uint32_t off = (d >> 6) * kSlab + sw64(row, d & 63);
-                        *reinterpret_cast<uint2 *>(smem + L::kOffQ + off) =
-                            make_uint2((uint32_t)hi[0] | ((uint32_t)hi[1] << 16), (uint32_t)hi[2] | ((uint32_t)hi[3] << 16));
-                        *reinterpret_cast<uint2 *>(smem + L::kOffQ + L::kQTerm + off) =
-                            make_uint2((uint32_t)lo[0] | ((uint32_t)lo[1] << 16), (uint32_t)lo[2] | ((uint32_t)lo[3] << 16));
-                    }
-                };
-                load_batch(xa, 0);
-                ok = warp_wait(ctx, bar(L::kBarQEmpty), (seg_it & 1) ^ 1, L::kBarQEmpty);
-                if (!ok) break;
-                load_batch(xb, 9);  convert_batch(xa, 0);
-                if constexpr (H == 64) {
-                    load_batch(xa, 18); convert_batch(xb, 9);
-                    load_batch(xb, 27); convert_batch(xa, 18);
-                    convert_batch(xb, 27);
-                } else {
-                    convert_batch(xb, 9);
-                }
+                const float amax = rows.largest();
+                if (rows.part == 0) qs_s[(seg_it & 3) * H + rows.row] = amax > 0.f ? amax * (1.0f / 448.0f) : 1.0f;
+                rows.split(amax > 0.f ? 448.0f / amax : 1.0f);
                 fence_proxy_async();
                 __syncwarp();
                 // The softmax warps wait on QLocal by phase parity, so it must never complete two phases
@@ -711,10 +676,11 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
                 tcgen05_fence_after();
                 float sv[16];                     // [4 k + e]: head hA, token 8 k + 2 tq + e; [4 k + 2 + e]: head hA + 8
                 {
-                    float part[16];
+                    // a load has eight heads' hi rows and their lo rows
+                    float xa[16], xb[16];
                     const uint32_t sb = tmem_base + lane_addr + L::kColS + b * 64 + 32 * cf;
-                    tmem_ld_frag<32>(sb, sv);
-                    tmem_ld_frag<32>(sb + (16u << 16), part);
+                    tmem_ld_frag<32>(sb, xa);
+                    tmem_ld_frag<32>(sb + (16u << 16), xb);
                     // meanwhile: lane j prepares token 32 cf + j.  A token outside the range gets scale 0 and
                     // log2 scale -inf; its row of K may hold anything, so its logit is also forced below.
                     const int r = 32 * cf + lane;
@@ -724,7 +690,9 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
                     tok_r[lane] = v ? fast_rcp(ts) : 0.f;
                     tmem_wait_ld();
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) sv[j] += part[j];
+                    for (int k = 0; k < 4; ++k)
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) { sv[4 * k + e] = xa[4 * k + e] + xa[4 * k + 2 + e]; sv[4 * k + 2 + e] = xb[4 * k + e] + xb[4 * k + 2 + e]; }
                 }
                 tcgen05_fence_before();
                 __syncwarp();
@@ -927,7 +895,7 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
 
 template <int H>
 cudaError_t launch_pair(const DecodeParams &p, cudaStream_t stream) {
-    alignas(64) CUtensorMap mpage, mpair;
+    alignas(64) CUtensorMap mpage, mpair, mq;
     const uint64_t pages = (uint64_t)(p.num_pool_pages > 0 ? p.num_pool_pages : 1);
     if (!make_map_4d(&mpage, CU_TENSOR_MAP_DATA_TYPE_UINT8, CU_TENSOR_MAP_SWIZZLE_64B, p.kv_pool, kPage, pages,
                      (uint64_t)kDQK, 64, (uint64_t)kPage * kDQK, 64, 9))
@@ -945,17 +913,18 @@ cudaError_t launch_pair(const DecodeParams &p, cudaStream_t stream) {
     const uint64_t h = (uint64_t)(p.head_end - p.head_begin);
     if (!make_store_map_3d(&mpart, p.partial_out, kDV, h, (uint64_t)2 * p.num_workers, (uint64_t)kDV * 4, h * kDV * 4, H / 2))
         return cudaErrorInvalidValue;
+    DecodeParams args = p;
+    args.q_by_hand = make_query_map(&mq, p, H) ? 0 : 1;
+    if (args.q_by_hand) mq = mpage;
     const int smem = (int)Layout<H>::kSmemBytes;
     static DeviceOnce once;
     cudaError_t e = once.run([&] {
-        const cudaError_t e0 = cudaFuncSetAttribute(decode_umma_fp8_pair_kernel<H, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e0 != cudaSuccess) return e0;
-        return cudaFuncSetAttribute(decode_umma_fp8_pair_kernel<H, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        return cudaFuncSetAttribute(decode_umma_fp8_pair_kernel<H>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     });
     if (e != cudaSuccess) return e;
     // (the cluster shape is part of the kernel's declaration)
-    e = launch_dependent(p.plan_mode == kPlanWorkspace ? decode_umma_fp8_pair_kernel<H, false> : decode_umma_fp8_pair_kernel<H, true>,
-                         dim3((unsigned)(p.num_workers * p.pair_groups * 2)), dim3(kThreads), (size_t)smem, stream, p, mpage, mpair, mout, mpart);
+    e = launch_dependent(decode_umma_fp8_pair_kernel<H>,
+                         dim3((unsigned)(p.num_workers * p.pair_groups * 2)), dim3(kThreads), (size_t)smem, stream, args, mpage, mpair, mout, mpart, mq);
     count_launch();
     return e;
 }

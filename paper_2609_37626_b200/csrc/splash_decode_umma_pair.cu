@@ -152,7 +152,7 @@ decode_umma_pair_kernel(const __grid_constant__ DecodeParams p, const __grid_con
     tcgen05_fence_after();
     const uint32_t tmem_base = misc[0];
     SegmentIter<kOffPlan> it;
-    start_plan<false>(p, worker, rank == 0 && pair_id == worker * p.pair_groups, kWarpVProducer, it, FirstLoads{2 * kStageBytes, rank * kStageBytes, kStageBytes, kStages, head0, kN});
+    start_plan<false>(p, worker, kWarpVProducer, it, FirstLoads{2 * kStageBytes, rank * kStageBytes, kStageBytes, kStages, head0, kN});
     const long long t_start = clock64();
     const unsigned long long ns_start = global_timer_ns();
 

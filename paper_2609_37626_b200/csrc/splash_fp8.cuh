@@ -91,5 +91,95 @@ __device__ __forceinline__ float fast_rcp(float x) {
     return y;
 }
 
+// ---- query operands ---------------------------------------------------------------
+// The rows of kHeads heads arrive by one TMA load as bf16, [9 chunks][kHeads rows][128 B] in the 128-byte swizzle, and become the two
+// 8-bit terms in place: the 1,024 bytes of eight rows of a chunk are then eight rows of 64 hi bytes and eight of 64 lo bytes in
+// the 64-byte swizzle.  A converter warp has kHeads / kWarps rows, whole groups of eight, so that what it overwrites is its own; a lane has a
+// row and every kParts-th chunk, eight neighbouring lanes eight neighbouring rows (no bank conflicts).
+// (The rows were loaded from global memory into registers, twice over, for the maximum and for the conversion, in seven round trips where the
+// registers of 128 threads hold a quarter of them: 6.4 us from the plan to the operands of a call's first request on 128 heads, now 4.2.  For 16 or 32
+// heads, whose rows fit those registers at once, that is the faster way: eight layers of 8 requests 123 us, 127 this way.)
+template <int kHeads, int kWarps>
+struct QueryRows {
+    static constexpr int kRows = kHeads / kWarps, kParts = 32 / kRows;
+    static constexpr uint32_t kBytes = kHeads * kDQK * 2;
+    static_assert(kRows % 8 == 0 && 32 % kRows == 0, "whole groups of eight rows");
+    const uint8_t *src;          // the row: in shared memory, or (by hand) in global memory
+    uint8_t *dst;                // its hi bytes
+    uint32_t chunk_stride, swizzle;
+    int row, part;
+    bool live;                   // (by hand: a row outside the slice reads as zeros, as the TMA unit fills it)
+    __device__ __forceinline__ QueryRows(uint8_t *operand, int warp, int lane) {
+        row = warp * kRows + lane % kRows; part = lane / kRows;
+        src = operand + row * 128; chunk_stride = kHeads * 128; swizzle = row & 7; live = true;
+        dst = operand + (row >> 3) * 1024 + (row & 7) * 64;
+    }
+    __device__ __forceinline__ void by_hand(const void *global_row, bool in_slice) {
+        src = static_cast<const uint8_t *>(global_row); chunk_stride = 128; swizzle = 0; live = in_slice;
+    }
+    __device__ __forceinline__ void load(uint4 (&x)[8], int c) const {
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            x[j] = live ? *reinterpret_cast<const uint4 *>(src + c * chunk_stride + ((j ^ swizzle) << 4)) : make_uint4(0u, 0u, 0u, 0u);
+    }
+    // largest magnitude of the row (a NaN is passed over), the same in the lanes that share it.
+    __device__ __forceinline__ float largest() const {
+        uint32_t m = 0;
+#pragma unroll 1
+        for (int c = part; c < 9; c += kParts) {
+            uint4 x[8];
+            load(x, c);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const uint32_t w[4] = {x[j].x, x[j].y, x[j].z, x[j].w};
+#pragma unroll
+                for (int k = 0; k < 4; ++k) asm("max.bf16x2 %0, %0, %1;" : "+r"(m) : "r"(w[k] & 0x7fff7fffu));
+            }
+        }
+        float v = fmaxf(__uint_as_float(m << 16), __uint_as_float(m & 0xffff0000u));
+#pragma unroll
+        for (int o = kRows; o < 32; o <<= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+        return v;
+    }
+    __device__ __forceinline__ void split(float inv) const {
+#pragma unroll 1
+        for (int i = 0; i < (9 + kParts - 1) / kParts; ++i) {
+            const int c = part + i * kParts;
+            uint4 x[8];
+            if (c < 9) load(x, c);
+            __syncwarp();                 // the eight rows have been read
+            if (c < 9) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    uint32_t hi[4], lo[4];
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const uint4 v = x[2 * j + e];
+                        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+                        uint16_t h[4], l[4];
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)
+                            split_e4m3_e4m3_x2(__uint_as_float(w[k] << 16) * inv, __uint_as_float(w[k] & 0xffff0000u) * inv, h[k], l[k]);
+                        hi[2 * e] = (uint32_t)h[0] | ((uint32_t)h[1] << 16); hi[2 * e + 1] = (uint32_t)h[2] | ((uint32_t)h[3] << 16);
+                        lo[2 * e] = (uint32_t)l[0] | ((uint32_t)l[1] << 16); lo[2 * e + 1] = (uint32_t)l[2] | ((uint32_t)l[3] << 16);
+                    }
+                    uint8_t *const at = dst + c * (kHeads * 128) + (((j ^ (row >> 1)) & 3) << 4);
+                    *reinterpret_cast<uint4 *>(at) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+                    *reinterpret_cast<uint4 *>(at + 512) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+                }
+            }
+        }
+    }
+};
+
+// The map of those loads, over the heads below head_end (a box reads zeros past them).  False where the strides are none that a map can
+// state: the kernel then loads the rows by hand.
+inline bool make_query_map(CUtensorMap *map, const DecodeParams &p, uint32_t heads) {
+    const int64_t limit = (int64_t)1 << 39;          // in elements of two bytes
+    if (p.q_stride_head >= limit || (p.B > 1 && (p.q_stride_request <= 0 || p.q_stride_request >= limit))) return false;
+    return make_map_4d(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, CU_TENSOR_MAP_SWIZZLE_128B, p.q, (uint64_t)p.head_end, (uint64_t)p.B,
+                       (uint64_t)p.q_stride_head * 2, 128, (uint64_t)(p.B > 1 ? p.q_stride_request : p.q_stride_head * p.H) * 2, heads);
+}
+
 }  // namespace umma
 }  // namespace splash
