@@ -91,14 +91,20 @@ static_assert(kOffQ % 1024 == 0 && kOffP1 % 1024 == 0 && kSlab % 1024 == 0, "swi
 // tensor memory: O two halves of dv x 128 columns, then 2 S buffers x 32 columns
 constexpr uint32_t kColO = 0, kColS = 256;
 
-// Issued by the elected lane of a converged warp; the operands are uniform.
-__device__ __forceinline__ void umma_bf16_pair(uint32_t elected, uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+// Issued by the elected lane of a converged warp; the operands are uniform.  `a_at`, `b_at`: 16-byte units added to the descriptors'
+// addresses.  Only the low words of the descriptors move with them, and what they start from is said to be uniform: with 64-bit sums, and
+// addresses that only happen to be the same in all lanes, an issuer is slower than the tensor pipe (64 requests of 1,024 to 8,192
+// tokens 116.6 us, now 112.6; 48 requests with four query rows on 32 heads 88.8 and 85.7).
+__device__ __forceinline__ void umma_bf16_pair(uint32_t elected, uint32_t d_tmem, uint64_t a_desc, uint32_t a_at, uint64_t b_desc, uint32_t b_at, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "setp.ne.b32 q, %5, 0;\n\t"
-        "@q tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(elected) : "memory");
+        "{\n\t.reg .pred p, q;\n\t.reg .b64 a, b;\n\t"
+        "setp.ne.b32 p, %6, 0;\n\t"
+        "setp.ne.b32 q, %7, 0;\n\t"
+        "mov.b64 a, {%1, %2};\n\t"
+        "mov.b64 b, {%3, %4};\n\t"
+        "@q tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %5, p;\n\t}"
+        ::"r"(d_tmem), "r"((uint32_t)a_desc + a_at), "r"((uint32_t)(a_desc >> 32)), "r"((uint32_t)b_desc + b_at), "r"((uint32_t)(b_desc >> 32)),
+          "r"(idesc), "r"(accumulate), "r"(elected) : "memory");
 }
 
 template <bool kSparse>
@@ -255,12 +261,12 @@ decode_umma_pair_kernel(const __grid_constant__ DecodeParams p, const __grid_con
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 tcgen05_fence_after();
-                const uint32_t d = tmem_u + kColS + b * kHalf;
-                const uint64_t dq = make_desc(sbase + kOffQ, 16, 1024);                          // A: 2 x 64 heads x 16
-                const uint64_t dk = make_desc(sbase + kOffK + stage * kStageBytes, 16, 1024);    // B: 2 x 32 tokens x 16
+                const uint32_t d = uniform(tmem_u + kColS + b * kHalf);
+                const uint64_t dq = make_desc(uniform(sbase + kOffQ), 16, 1024);                          // A: 2 x 64 heads x 16
+                const uint64_t dk = make_desc(uniform(sbase + kOffK + stage * kStageBytes), 16, 1024);    // B: 2 x 32 tokens x 16
 #pragma unroll
                 for (int t = 0; t < 36; ++t)
-                    umma_bf16_pair(elected, d, dq + (((t >> 2) * kQSlab + (t & 3) * 32) >> 4), dk + (((t >> 2) * kSlab + (t & 3) * 32) >> 4), kIdescQK, t != 0);
+                    umma_bf16_pair(elected, d, dq, ((t >> 2) * kQSlab + (t & 3) * 32) >> 4, dk, ((t >> 2) * kSlab + (t & 3) * 32) >> 4, kIdescQK, t != 0);
                 if (elected) { umma_commit_pair(bar(kBarSFull + b)); umma_commit_pair(bar(kBarQkDone + stage)); }
                 __syncwarp();
             }
@@ -284,18 +290,18 @@ decode_umma_pair_kernel(const __grid_constant__ DecodeParams p, const __grid_con
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 tcgen05_fence_after();
-                const uint32_t k0 = sbase + kOffK + stage * kStageBytes;
+                const uint32_t k0 = uniform(sbase + kOffK + stage * kStageBytes);
                 // 16 tokens of half-page j / 2.  A: P rows (heads), 32 bytes of the 64-byte row (half-page 0: in the
                 // stage's rope slot, 1: in its own buffer);
                 // B: slots 4n + 2g, + 1 (two 64-wide dv chunks, LBO apart), 16 token rows, MN-major
-                const uint64_t da0 = make_desc_sw64(k0 + 8 * kSlab, 16, 512), da1 = make_desc_sw64(sbase + kOffP1 + pb * kPHalfBytes, 16, 512);
+                const uint64_t da0 = make_desc_sw64(k0 + 8 * kSlab, 16, 512), da1 = make_desc_sw64(uniform(sbase + kOffP1 + pb * kPHalfBytes), 16, 512);
                 const uint64_t db = make_desc(k0, kSlab, 1024);
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
 #pragma unroll
                     for (int n = 0; n < 2; ++n)                  // dv half: columns [256 n, 256 n + 256)
-                        umma_bf16_pair(elected, tmem_u + kColO + n * 128, (j < 2 ? da0 : da1) + (((j & 1) * 32) >> 4),
-                                       db + (((4 * n + 2 * (j >> 1)) * kSlab + (j & 1) * 2048) >> 4), kIdescPV, (uint32_t)i | (uint32_t)j);
+                        umma_bf16_pair(elected, tmem_u + kColO + n * 128, j < 2 ? da0 : da1, ((j & 1) * 32) >> 4,
+                                       db, ((4 * n + 2 * (j >> 1)) * kSlab + (j & 1) * 2048) >> 4, kIdescPV, (uint32_t)i | (uint32_t)j);
                 }
                 if (elected) {
                     umma_commit_pair(bar(kBarStageEmpty + stage));
