@@ -91,9 +91,9 @@ inline __host__ PlanView make_plan_view(void *workspace, int B, int W, int h) {
 }
 
 // What a record says of a cut request's slots: a worker's piece lies in slot 2 w, the first worker's in 2 w + 1 if an earlier request's
-// piece came before it; and whether there may be workers among them whose start fell on the same tile as the next one's, so
-// that they hold nothing (the plan kernel's, where all the work costs less than there are workers).
-enum SplitFlags { kSplitSecondSlot = 1, kSplitGaps = 2 };
+// piece came before it.  Where all the work costs less than there are workers, the plan kernel lets several workers start on one tile, of
+// which the last one has it: the cost stands above that bit then (else 0), and a combine kernel works out which they are.
+enum SplitFlags { kSplitSecondSlot = 1, kSplitCostShift = 1 };
 
 // Arguments common to the decode kernels.
 struct DecodeParams {

@@ -85,16 +85,20 @@ lse_merge_kernel(int num_parts, int64_t rows, int d_v, const float *part_out, co
 // record says where the pieces lie, so that their LSEs and their rows come in the second.
 constexpr int kMaxParts = 512;     // >= number of workers of any launch (one per SM at most)
 
-// Where a cut request's pieces lie.
+// Where a cut request's pieces lie.  Their numbers do not depend on who has made the plan, nor do the sums then: with less cost than workers
+// (kGaps: the plan kernel's plans, which may be such), cost unit u is a tile or overhead, and the last worker whose share starts
+// at it is number floor(((u + 1) W - 1) / cost).
+template <bool kGaps>
 struct Pieces {
-    int request, first_worker, n, flags;
-    __device__ __forceinline__ explicit Pieces(const int4 &rec) : request(rec.x), first_worker(rec.y), n(rec.z - rec.y + 1), flags(rec.w) {}
-    __device__ __forceinline__ uint32_t row(int j, int h, int k) const {
-        return (uint32_t)(2 * (first_worker + j) + (j == 0 ? flags & kSplitSecondSlot : 0)) * h + k;
+    int request, first, n, flags, cost, workers;
+    __device__ __forceinline__ Pieces(const DecodeParams &p, const int4 &rec)
+        : request(rec.x), first(rec.y), n(rec.z - rec.y + 1), flags(rec.w), cost(rec.w >> kSplitCostShift), workers(p.num_workers) {
+        if (kGaps && cost > 0) { first = rec.y * cost / workers; n = rec.z * cost / workers - first + 1; }
     }
-    // (a slot nobody wrote holds stale bytes)
-    __device__ __forceinline__ bool live(const DecodeParams &p, int j) const {
-        return !(flags & kSplitGaps) || p.worker_begin[first_worker + j + 1] > p.worker_begin[first_worker + j];
+    __device__ __forceinline__ uint32_t row(int j, int h, int k) const {
+        int w = first + j;
+        if (kGaps && cost > 0) w = ((w + 1) * workers - 1) / cost;
+        return (uint32_t)(2 * w + (j == 0 ? flags & kSplitSecondSlot : 0)) * h + k;
     }
 };
 
@@ -123,11 +127,12 @@ struct PartRow {
 // into few pieces each (many requests per worker): at most four part loads in flight, few enough registers for sixteen
 // resident blocks per SM instead of eight -- its blocks are short chains of round trips, and what bounds
 // the kernel is how many of them an SM holds at a time.
-template <bool kF16, bool kLean>
+template <bool kF16, bool kLean, bool kGaps>
 __global__ void __launch_bounds__(kMergeThreads, kLean ? 16 : 8)
 split_combine_kernel(const DecodeParams p, const int4 *split_rec) {
     using Row = PartRow<kF16>;
     __shared__ float w_s[kMaxParts];
+    __shared__ uint32_t row_s[kMaxParts];
     __shared__ float sc_s[kF16 ? kMaxParts : 1];      // f16 pieces: the power of two each row was divided by
     __shared__ float red_s[kMergeThreads / 32], sum_s[kMergeThreads / 32];
     const int h = p.head_end - p.head_begin;
@@ -136,13 +141,13 @@ split_combine_kernel(const DecodeParams p, const int4 *split_rec) {
     grid_launch_dependents();     // a next call's first kernel may come in once every block of this grid has started
     grid_dependency_wait();       // the decode kernel's partial slots (and the plan) are read from here on
     const int n_entries = p.status[8];
-    const Pieces pieces(split_rec[entry]);             // (unused past the list's end)
+    const Pieces<kGaps> pieces(p, split_rec[entry]);          // (unused past the list's end)
     if (entry >= n_entries) return;
     const int i = pieces.request, nparts = pieces.n;
     float4 *o4 = reinterpret_cast<float4 *>(p.out + (int64_t)i * p.out_stride_request + (int64_t)g * p.out_stride_head);
     float *lse = p.lse + (int64_t)i * p.lse_stride_request + g;
     const int c = threadIdx.x;             // 128 threads x float4 = 512 columns
-    if (kLean && nparts <= 4 && !(pieces.flags & kSplitGaps)) {
+    if (kLean && nparts <= 4) {
         // few pieces, as nearly all requests of such a launch: every thread has all their LSEs, and nothing is exchanged
         typename Row::Raw raw[4];
         float L[4], scale[4];
@@ -184,15 +189,15 @@ split_combine_kernel(const DecodeParams p, const int4 *split_rec) {
         const uint32_t row = pieces.row(j, h, k);
         const float L = p.partial_lse[row];
         if constexpr (kF16) sc_s[j] = p.partial_scale[row];
-        w_s[j] = pieces.live(p, j) ? L : -INFINITY;
-        m = fmaxf(m, w_s[j]);
+        w_s[j] = L; row_s[j] = row;
+        m = fmaxf(m, L);
     }
     for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
     if ((c & 31) == 0) red_s[c >> 5] = m;
     __syncthreads();
     m = reference_max(fmaxf(fmaxf(red_s[0], red_s[1]), fmaxf(red_s[2], red_s[3])));
     float Z = 0.f;
-    for (int j = c; j < nparts; j += kMergeThreads) { w_s[j] = expf(w_s[j] - m); Z += w_s[j]; }     // 0 for dead workers
+    for (int j = c; j < nparts; j += kMergeThreads) { w_s[j] = expf(w_s[j] - m); Z += w_s[j]; }     // (0 for a piece that saw no token)
     for (int o = 16; o; o >>= 1) Z += __shfl_xor_sync(0xffffffffu, Z, o);
     if ((c & 31) == 0) sum_s[c >> 5] = Z;
     __syncthreads();
@@ -206,7 +211,7 @@ split_combine_kernel(const DecodeParams p, const int4 *split_rec) {
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
     auto add = [&](int j, const typename Row::Raw &raw) {
         float w = w_s[j] * inv_z;
-        if (w != 0.f) {                    // a dead worker's slot holds stale bytes
+        if (w != 0.f) {                    // (0: a piece that saw no token)
             if constexpr (kF16) w *= sc_s[j];
             Row::add(acc, raw, w);
         }
@@ -220,7 +225,7 @@ split_combine_kernel(const DecodeParams p, const int4 *split_rec) {
     for (; !kLean && j + 16 <= nparts; j += 16) {
         typename Row::Raw raw[16];
 #pragma unroll
-        for (int u = 0; u < 16; ++u) raw[u] = Row::load(p, pieces.row(j + u, h, k), c);
+        for (int u = 0; u < 16; ++u) raw[u] = Row::load(p, row_s[j + u], c);
 #pragma unroll
         for (int u = 0; u < 16; ++u) add(j + u, raw[u]);
     }
@@ -229,7 +234,7 @@ split_combine_kernel(const DecodeParams p, const int4 *split_rec) {
         typename Row::Raw raw[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u)
-            if (j + u < nparts) raw[u] = Row::load(p, pieces.row(j + u, h, k), c);
+            if (j + u < nparts) raw[u] = Row::load(p, row_s[j + u], c);
 #pragma unroll
         for (int u = 0; u < 4; ++u)
             if (j + u < nparts) add(j + u, raw[u]);
@@ -245,7 +250,7 @@ split_combine_kernel(const DecodeParams p, const int4 *split_rec) {
 // others (kDeep), which leave no room for that anyway, more loads are in flight, the first of them beside those of the LSEs: 74
 // pieces on 128 heads 5.4 us, now 4.5.  (A warp for itself with 32 columns of a row and no barriers: 10 us, every warp loads all LSEs then.)
 constexpr int kGroupedParts = 160, kCombineGroups = 4;
-template <bool kF16, bool kDeep>
+template <bool kF16, bool kDeep, bool kGaps>
 __global__ void __launch_bounds__(kCombineGroups * kMergeThreads, kDeep ? 2 : 4)
 grouped_combine_kernel(const DecodeParams p, const int4 *split_rec) {
     using Row = PartRow<kF16>;
@@ -261,7 +266,7 @@ grouped_combine_kernel(const DecodeParams p, const int4 *split_rec) {
     grid_launch_dependents();
     grid_dependency_wait();
     const int n_entries = p.status[8];
-    const Pieces pieces(split_rec[entry]);
+    const Pieces<kGaps> pieces(p, split_rec[entry]);
     if (entry >= n_entries) return;
     const int i = pieces.request, nparts = pieces.n;
     float4 *o4 = reinterpret_cast<float4 *>(p.out + (int64_t)i * p.out_stride_request + (int64_t)g * p.out_stride_head);
@@ -272,7 +277,6 @@ grouped_combine_kernel(const DecodeParams p, const int4 *split_rec) {
         const uint32_t row = pieces.row(tid, h, k);
         L = p.partial_lse[row];
         if constexpr (kF16) scale = p.partial_scale[row];
-        if (!pieces.live(p, tid)) L = -INFINITY;
     }
     typename Row::Raw raw[kDepth];
     auto load = [&](int j0) {
@@ -292,7 +296,7 @@ grouped_combine_kernel(const DecodeParams p, const int4 *split_rec) {
     for (int x = 1; x < kThreads / 32; ++x) m = fmaxf(m, max_s[x]);
     m = reference_max(m);
     float Z = tid < nparts ? expf(L - m) : 0.f;
-    if (tid < nparts) w_s[tid] = Z == 0.f ? 0.f : Z * scale;       // (a slot nobody wrote holds any scale)
+    if (tid < nparts) w_s[tid] = Z * scale;
     for (int o = 16; o; o >>= 1) Z += __shfl_xor_sync(0xffffffffu, Z, o);
     if ((tid & 31) == 0) sum_s[tid >> 5] = Z;
     __syncthreads();
@@ -312,7 +316,7 @@ grouped_combine_kernel(const DecodeParams p, const int4 *split_rec) {
         for (int u = 0; u < kDepth; ++u) {
             const int j = j0 + u * kCombineGroups;
             const float w = j < nparts ? w_s[j] * inv_z : 0.f;
-            if (w != 0.f) Row::add(acc, raw[u], w);              // a dead worker's slot holds stale bytes
+            if (w != 0.f) Row::add(acc, raw[u], w);              // (0: a piece that saw no token)
         }
     }
     float4 *const total = reinterpret_cast<float4 *>(smem_f);
@@ -352,25 +356,25 @@ cudaError_t launch_split_combine(const DecodeParams &p, const int4 *split_rec, i
     // at most one request straddles each boundary between consecutive workers
     const int max_split = p.num_workers < p.B ? p.num_workers : p.B;
     dim3 grid((unsigned)((int64_t)(p.head_end - p.head_begin) * max_split));
-    static DeviceOnce once;
-    once.run([&] {   // keep the decode kernel's shared-memory carve-out (a preference: a failure is not an error)
-        cudaFuncSetAttribute(split_combine_kernel<false, false>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-        cudaFuncSetAttribute(split_combine_kernel<true, false>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-        cudaFuncSetAttribute(split_combine_kernel<false, true>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-        cudaFuncSetAttribute(split_combine_kernel<true, true>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-        cudaFuncSetAttribute(grouped_combine_kernel<false, false>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-        cudaFuncSetAttribute(grouped_combine_kernel<false, true>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-        cudaFuncSetAttribute(grouped_combine_kernel<true, true>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-        return cudaSuccess;
-    });
     // many requests per worker: every request is cut into a few pieces at most
     const bool lean = (int64_t)p.B * 4 >= p.num_workers;
     const bool room = p.heads_per_group <= 32 && p.num_groups == 1;       // for a block beside a decode CTA
     // as many rows as are resident at once (room: one beside each CTA): two requests on 128 heads 17.8 us, now 16.1; with 384 rows 18.0 against 17.4
     const bool grouped = !lean && grid.x <= (room ? 1u : 2u) * (unsigned)sm_count && p.num_workers <= kGroupedParts;
-    auto kernel = grouped ? (p.partial_f16 ? grouped_combine_kernel<true, true> : room ? grouped_combine_kernel<false, false> : grouped_combine_kernel<false, true>)
-                : p.partial_f16 ? (lean ? split_combine_kernel<true, true> : split_combine_kernel<true, false>)
-                                : (lean ? split_combine_kernel<false, true> : split_combine_kernel<false, false>);
+    auto choose = [&](auto gaps) {
+        constexpr bool kGaps = decltype(gaps)::value;
+        return grouped ? (p.partial_f16 ? grouped_combine_kernel<true, true, kGaps> : room ? grouped_combine_kernel<false, false, kGaps> : grouped_combine_kernel<false, true, kGaps>)
+             : p.partial_f16 ? (lean ? split_combine_kernel<true, true, kGaps> : split_combine_kernel<true, false, kGaps>)
+                             : (lean ? split_combine_kernel<false, true, kGaps> : split_combine_kernel<false, false, kGaps>);
+    };
+    const bool gaps = p.plan_mode == kPlanWorkspace;
+    auto kernel = gaps ? choose(std::true_type()) : choose(std::false_type());
+    // the decode kernel's shared-memory carve-out is kept (a preference: a failure is not an error)
+    static DeviceOnce once[2][2][2][2];
+    once[gaps][grouped][p.partial_f16 != 0][grouped ? room : lean].run([&] {
+        cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+        return cudaSuccess;
+    });
     cudaError_t e = launch_dependent(kernel, grid, dim3(grouped ? kCombineGroups * kMergeThreads : kMergeThreads), 0, stream, p, split_rec);
     count_launch();
     return e;

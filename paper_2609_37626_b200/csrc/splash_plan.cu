@@ -123,7 +123,7 @@ plan_kernel(int B, int W, int overhead, int len_cap, const int32_t *seq_lens, co
             const int e = atomicAdd(&n_split, 1);
             split_list[e] = i;
             // all the combine kernel needs to know about the request, in one load
-            split_rec[e] = make_int4(i, wf, wl, (worker_begin[wf] < rs ? kSplitSecondSlot : 0) | (total_cost < W ? kSplitGaps : 0));
+            split_rec[e] = make_int4(i, wf, wl, (worker_begin[wf] < rs ? kSplitSecondSlot : 0) | (total_cost < W ? total_cost << kSplitCostShift : 0));
         }
     }
     if (staged) {

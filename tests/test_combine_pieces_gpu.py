@@ -31,3 +31,15 @@ def test_many_requests_and_a_long_one(kv_dtype, H):
     for x in (lens, few):
         w = W.make_workload("pieces", 9400 + H, x, H=H, kv_dtype=kv_dtype)
         compare(*gpu_run(w), *oracle_run(w), kv_dtype=kv_dtype)
+
+
+@pytest.mark.parametrize("kv_dtype,H", [(0, 16), (0, 32), (0, 128), (1, 16), (1, 128)])
+@pytest.mark.parametrize("lens", [[64 * 7], [300, 700, 64, 1000], [64 * 20, 0, 1]])
+def test_the_planner_makes_no_difference(kv_dtype, H, lens):
+    """Less work than workers: the plan kernel (validation mode runs it) leaves workers without a piece between those with one, the
+    plan that a decode kernel makes for itself does not; the same pieces, merged in the same order."""
+    from paper_2609_37626_b200 import binding
+    w = W.make_workload("planner", 9450 + H + sum(lens), lens, H=H, kv_dtype=kv_dtype)
+    w.block_table = np.pad(w.block_table, ((0, 0), (0, 8)), constant_values=-1)      # wide enough for requests to be cut
+    a, b = gpu_run(w), gpu_run(w, flags=binding.SPLASH_FLAG_VALIDATE)
+    assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
