@@ -70,7 +70,7 @@ struct Layout {
     static constexpr uint32_t kOffQ = kOffKv + kStages * kStageBytes;
     static constexpr uint32_t kOffP = kOffQ + kQBytes;
     // output staging for the narrow groups, [16 heads][512 dv] floats: the finished tile leaves through the bulk-copy engine
-    // (64-head groups have no shared memory left for it and store from registers)
+    // (64-head groups have no shared memory left for it and turn their tile over in the P buffer)
     static constexpr uint32_t kOutBytes = N < 64 ? 16 * kDV * 4 : 0;
     static constexpr uint32_t kOffOut = kOffP + kPBytes;
     static constexpr uint32_t kOffRed = kOffOut + kOutBytes; // float [N][4]
