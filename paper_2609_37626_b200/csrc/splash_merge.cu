@@ -246,7 +246,9 @@ split_combine_kernel(const DecodeParams p, const int4 *split_rec) {
 // The same for launches of no more rows than SMs (a small batch): four groups of 128 threads take every fourth piece and add
 // their sums in shared memory.  Behind the kernels of 16 and 32 heads 2 KB of shared memory and 32 registers, so that a block fits
 // beside a decode CTA of 16 heads: the next call's CTAs come in, plan and prefetch while this kernel runs (eight layers of 8 requests:
-// with the kernel above, 6 KB a block, they came in 1.6 to 4.4 us later, one by one as its blocks left; with 40 registers too).  Behind the
+// with the kernel above, 6 KB a block, they came in 1.6 to 4.4 us later, one by one as its blocks left; with 40 registers too); the pieces' rows wait
+// in shared memory then (worked out where they are loaded, they did not fit those registers: one context of 16,384 tokens on 16 heads 18.4 us,
+// now 17.1; of 65,536 28.9 and 27.5).  Behind the
 // others (kDeep), which leave no room for that anyway, more loads are in flight, the first of them beside those of the LSEs: 74
 // pieces on 128 heads 5.4 us, now 4.5.  (A warp for itself with 32 columns of a row and no barriers: 10 us, every warp loads all LSEs then.)
 constexpr int kGroupedParts = 160, kCombineGroups = 4;
@@ -255,11 +257,12 @@ __global__ void __launch_bounds__(kCombineGroups * kMergeThreads, kDeep ? 2 : 4)
 grouped_combine_kernel(const DecodeParams p, const int4 *split_rec) {
     using Row = PartRow<kF16>;
     constexpr int kThreads = kCombineGroups * kMergeThreads, kDepth = !kDeep ? 4 : kF16 ? 16 : 8;
-    // weights (f16 pieces: times the power of two each row was divided by); then the groups' sums
+    // weights (f16 pieces: times the power of two each row was divided by) and (!kDeep) row numbers; then the groups' sums
     __shared__ __align__(16) float smem_f[4 * kMergeThreads];
-    static_assert(kGroupedParts <= 4 * kMergeThreads && kGroupedParts <= kThreads, "a piece per thread");
+    static_assert(2 * kGroupedParts <= 4 * kMergeThreads && kGroupedParts <= kThreads, "a piece per thread");
     __shared__ float max_s[kThreads / 32], sum_s[kThreads / 32];
     float *const w_s = smem_f;
+    uint32_t *const row_s = reinterpret_cast<uint32_t *>(smem_f + kGroupedParts);
     const int h = p.head_end - p.head_begin;
     const int k = blockIdx.x % h, entry = blockIdx.x / h;
     const int g = p.head_begin + k;
@@ -277,13 +280,14 @@ grouped_combine_kernel(const DecodeParams p, const int4 *split_rec) {
         const uint32_t row = pieces.row(tid, h, k);
         L = p.partial_lse[row];
         if constexpr (kF16) scale = p.partial_scale[row];
+        if constexpr (!kDeep) row_s[tid] = row;
     }
     typename Row::Raw raw[kDepth];
     auto load = [&](int j0) {
 #pragma unroll
         for (int u = 0; u < kDepth; ++u) {
             const int j = j0 + u * kCombineGroups;
-            if (j < nparts) raw[u] = Row::load(p, pieces.row(j, h, k), c);
+            if (j < nparts) raw[u] = Row::load(p, kDeep ? pieces.row(j, h, k) : row_s[j], c);
         }
     };
     if constexpr (kDeep) load(group);
