@@ -372,12 +372,13 @@ decode_umma_fp8_pair_kernel(const __grid_constant__ DecodeParams p, const __grid
         while (ok && it.next(p, seg)) {
             {
                 // the operand buffer is free once the last QK^T of the previous request has retired
+                // (the rows asked into L2 here, in front of the wait: 300 requests of 64 to 500 tokens 0.8 to 1.4 % slower, no call faster)
                 Rows rows(smem + L::kOffQ, cw, lane);
-                const int gh = head0 + rows.row;
                 if (p.q_by_hand) {
                     ok = warp_wait(ctx, bar(L::kBarQEmpty), (seg_it & 1) ^ 1, L::kBarQEmpty);
                     if (!ok) break;
-                    rows.by_hand(static_cast<const __nv_bfloat16 *>(p.q) + (int64_t)seg.request * p.q_stride_request + (int64_t)gh * p.q_stride_head, gh < p.head_end);
+                    rows.copy_by_hand(static_cast<const uint16_t *>(p.q) + (int64_t)seg.request * p.q_stride_request + (int64_t)head0 * p.q_stride_head,
+                                      p.q_stride_head, p.head_end - head0, lane);
                 } else {
                     if (cw == 0) {
                         if (lane == 0) {

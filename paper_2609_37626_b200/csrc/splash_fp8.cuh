@@ -104,23 +104,34 @@ struct QueryRows {
     static constexpr int kRows = kHeads / kWarps, kParts = 32 / kRows;
     static constexpr uint32_t kBytes = kHeads * kDQK * 2;
     static_assert(kRows % 8 == 0 && 32 % kRows == 0, "whole groups of eight rows");
-    const uint8_t *src;          // the row: in shared memory, or (by hand) in global memory
+    uint8_t *const operand;
+    const uint8_t *src;          // the row as it came
     uint8_t *dst;                // its hi bytes
-    uint32_t chunk_stride, swizzle;
     int row, part;
-    bool live;                   // (by hand: a row outside the slice reads as zeros, as the TMA unit fills it)
-    __device__ __forceinline__ QueryRows(uint8_t *operand, int warp, int lane) {
+    __device__ __forceinline__ QueryRows(uint8_t *operand_, int warp, int lane) : operand(operand_) {
         row = warp * kRows + lane % kRows; part = lane / kRows;
-        src = operand + row * 128; chunk_stride = kHeads * 128; swizzle = row & 7; live = true;
+        src = operand + row * 128;
         dst = operand + (row >> 3) * 1024 + (row & 7) * 64;
     }
-    __device__ __forceinline__ void by_hand(const void *global_row, bool in_slice) {
-        src = static_cast<const uint8_t *>(global_row); chunk_stride = 128; swizzle = 0; live = in_slice;
+    // What the TMA load delivers, this warp's rows of it, without a tensor map: row r of the slice's `live` rows at q + r * stride (elements),
+    // zeros behind them.  All of a lane's copies are in flight at once.  (Read into registers where they are used, for the maximum and
+    // again for the terms, the rows were ten round trips: 512 requests of 200 to 1,500 tokens with one query for all, 128 heads, 166 us, now 138.)
+    // Out of line, or the kernel's other roles pay for its registers: 8 requests on 128 heads 26.2 us instead of 25.8, whatever their rows come by.
+    __device__ __noinline__ void copy_by_hand(const uint16_t *q, int64_t stride, int live, int lane) const {
+        const int first = row - lane % kRows;
+#pragma unroll 4
+        for (int i = lane; i < kRows * 72; i += 32) {
+            const int r = first + i / 72, v = i % 72;
+            uint8_t *const to = operand + (v >> 3) * (kHeads * 128) + r * 128 + (((v ^ r) & 7) << 4);
+            if (r < live) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(to)), "l"(q + (int64_t)r * stride + v * 8) : "memory");
+            else *reinterpret_cast<uint4 *>(to) = make_uint4(0u, 0u, 0u, 0u);
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncwarp();
     }
     __device__ __forceinline__ void load(uint4 (&x)[8], int c) const {
 #pragma unroll
-        for (int j = 0; j < 8; ++j)
-            x[j] = live ? *reinterpret_cast<const uint4 *>(src + c * chunk_stride + ((j ^ swizzle) << 4)) : make_uint4(0u, 0u, 0u, 0u);
+        for (int j = 0; j < 8; ++j) x[j] = *reinterpret_cast<const uint4 *>(src + c * (kHeads * 128) + (((j ^ row) & 7) << 4));
     }
     // largest magnitude of the row (a NaN is passed over), the same in the lanes that share it.
     __device__ __forceinline__ float largest() const {

@@ -90,3 +90,17 @@ def test_wide_rows_merge_at_the_rate_of_usual_ones():
 
     wide, usual = us(64, 8192), us(1024, 512)
     assert wide <= 1.5 * usual + 2, (wide, usual)
+
+
+@pytest.mark.parametrize("H", [64, 128])
+def test_one_query_for_all_costs_what_a_query_each_costs(H):
+    """e4m3 over CTA pairs: query rows at a request stride of 0 come by other loads than those that a tensor map can state."""
+    import numpy as np
+    import torch
+    from paper_2609_37626_b200 import binding
+    w = W.make_workload("query", 9510 + H, np.random.default_rng(H).integers(200, 1500, size=512), H=H, kv_dtype=1)
+    dw = binding.DeviceWorkload(w)
+    apart = device_us(dw.decode)
+    dw.q = dw.q[:1].expand(512, H, 576)
+    shared = device_us(dw.decode)
+    assert shared <= 1.1 * apart, (shared, apart)

@@ -32,3 +32,21 @@ def test_one_query_for_all_requests(H, hb, he):
     w.q = apart.contiguous().view(torch.uint16).cpu().numpy()
     compare(np.pad(whole[0].cpu().numpy(), ((0, 0), (hb, H - he), (0, 0))), np.pad(whole[1].cpu().numpy(), ((0, 0), (hb, H - he))), *oracle_run(w),
             kv_dtype=1, rows=[(i, g) for i in range(len(lens)) for g in range(hb, he)])
+
+
+@pytest.mark.parametrize("H,hb,he,R", [(16, 0, 16, 3), (24, 5, 16, 5), (48, 0, 48, 8), (128, 0, 128, 2), (128, 3, 100, 5)])
+def test_several_rows_per_request(H, hb, he, R):
+    """Virtual heads, up to five CTA pairs a worker, the last of them with few heads or none in its second CTA."""
+    import torch
+    from paper_2609_37626_b200 import binding as B
+    lens = [70, R, 700, 64 * 9]
+    w = W.make_workload("qs_rows", 9600 + H + he, lens, H=H, head_begin=hb, head_end=he, kv_dtype=1)
+    dw = B.DeviceWorkload(w)
+    one = torch.randn((1, H, R, 576), generator=torch.Generator("cuda").manual_seed(he), device="cuda").to(torch.bfloat16)
+    apart = one.expand(len(lens), H, R, 576)
+    args = (dw.kv_pool, dw.block_table, dw.seq_lens)
+    kw = dict(softmax_scale=w.softmax_scale, kv_scales=dw.kv_scales, head_begin=hb, head_end=he)
+    whole = B.splash_mla_decode(apart.contiguous(), *args, **kw)
+    whole = (whole[0][:, hb:he].clone(), whole[1][:, hb:he].clone())
+    shared = B.splash_mla_decode(apart, *args, **kw)
+    assert torch.equal(whole[0], shared[0][:, hb:he]) and torch.equal(whole[1], shared[1][:, hb:he])
