@@ -184,12 +184,13 @@ struct QueryRows {
 };
 
 // The map of those loads, over the heads below head_end (a box reads zeros past them).  False where the strides are none that a map can
-// state: the kernel then loads the rows by hand.
+// state: the kernel then loads the rows by hand, and the call has not failed.
 inline bool make_query_map(CUtensorMap *map, const DecodeParams &p, uint32_t heads) {
     const int64_t limit = (int64_t)1 << 39;          // in elements of two bytes
     if (p.q_stride_head >= limit || (p.B > 1 && (p.q_stride_request <= 0 || p.q_stride_request >= limit))) return false;
-    return make_map_4d(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, CU_TENSOR_MAP_SWIZZLE_128B, p.q, (uint64_t)p.head_end, (uint64_t)p.B,
-                       (uint64_t)p.q_stride_head * 2, 128, (uint64_t)(p.B > 1 ? p.q_stride_request : p.q_stride_head * p.H) * 2, heads);
+    // (one request: any stride that a map takes)
+    return encode_map_4d(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, CU_TENSOR_MAP_SWIZZLE_128B, p.q, (uint64_t)p.head_end, (uint64_t)p.B,
+                         (uint64_t)p.q_stride_head * 2, 128, (uint64_t)(p.B > 1 ? p.q_stride_request : p.q_stride_head) * 2, heads, 9) == CUDA_SUCCESS;
 }
 
 }  // namespace umma

@@ -358,19 +358,25 @@ inline EncodeTiledFn encode_tiled() {
 // elements, so one box of (64, box_rows, 9, 1) lands in shared memory as [chunk][row][64
 // elements], each chunk slab in the swizzle the MMA descriptors expect (128 B for 16-bit
 // elements, 64 B for 8-bit ones).
-inline bool make_map_4d(CUtensorMap *map, CUtensorMapDataType dtype, CUtensorMapSwizzle swizzle, const void *base,
-                        uint64_t rows, uint64_t outer, uint64_t row_stride_bytes, uint64_t chunk_stride_bytes,
-                        uint64_t outer_stride_bytes, uint32_t box_rows, uint32_t box_chunks = 9) {
+inline CUresult encode_map_4d(CUtensorMap *map, CUtensorMapDataType dtype, CUtensorMapSwizzle swizzle, const void *base,
+                              uint64_t rows, uint64_t outer, uint64_t row_stride_bytes, uint64_t chunk_stride_bytes,
+                              uint64_t outer_stride_bytes, uint32_t box_rows, uint32_t box_chunks) {
     EncodeTiledFn fn = encode_tiled();
-    if (!fn) { set_error("cuTensorMapEncodeTiled is not available"); return false; }
+    if (!fn) return CUDA_ERROR_NOT_FOUND;
     cuuint64_t dims[4] = {64, rows, 9, outer};
     cuuint64_t strides[3] = {row_stride_bytes, chunk_stride_bytes, outer_stride_bytes};
     cuuint32_t box[4] = {64, box_rows, box_chunks, 1};
     cuuint32_t estr[4] = {1, 1, 1, 1};
-    CUresult r = fn(map, dtype, 4, const_cast<void *>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                    swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) { set_error("cuTensorMapEncodeTiled failed with CUresult %d", (int)r); return false; }
-    return true;
+    return fn(map, dtype, 4, const_cast<void *>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+              swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+}
+// The same where the call cannot go on without the map.
+inline bool make_map_4d(CUtensorMap *map, CUtensorMapDataType dtype, CUtensorMapSwizzle swizzle, const void *base,
+                        uint64_t rows, uint64_t outer, uint64_t row_stride_bytes, uint64_t chunk_stride_bytes,
+                        uint64_t outer_stride_bytes, uint32_t box_rows, uint32_t box_chunks = 9) {
+    const CUresult r = encode_map_4d(map, dtype, swizzle, base, rows, outer, row_stride_bytes, chunk_stride_bytes, outer_stride_bytes, box_rows, box_chunks);
+    if (r != CUDA_SUCCESS) set_error(encode_tiled() ? "cuTensorMapEncodeTiled failed with CUresult %d" : "cuTensorMapEncodeTiled is not available", (int)r);
+    return r == CUDA_SUCCESS;
 }
 
 // 3-D map over fp32 rows for stores: (columns, rows, outer), row and outer strides in bytes
