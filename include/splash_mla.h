@@ -95,7 +95,8 @@ enum {
      * scales or the block table -- and a decode step runs the same batch through every layer of the model: the first
      * layer's call plans, the others pass this bit.  The caller asserts that those arguments are what they were in the
      * last call WITHOUT this bit on the same workspace (nothing checks it; a different batch may be cut along the old
-     * batch's boundaries and give wrong results, within bounds).  The layers' block tables may be of different widths.  The error words of the status block are cleared as in
+     * batch's boundaries and give wrong results, within bounds).  The layers' block tables may be of different widths.  Up to 32
+     * requests every call plans for itself in its decode kernel, and the flag changes nothing (except with SPLASH_FLAG_SIMT).  The error words of the status block are cleared as in
      * any call.  Ignored by the sparse entry point and together with SPLASH_FLAG_VALIDATE (which needs the plan's pass). */
     SPLASH_FLAG_REUSE_PLAN = 16u
 };

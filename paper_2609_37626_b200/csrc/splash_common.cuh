@@ -35,8 +35,9 @@ constexpr int kRequestOverheadTilesFp8Pair = 13;   // CTA-pair kernel: tiles are
 // ---- workspace layout ------------------------------------------------------
 // [0, 64)                 status block (int32 x 16): [0] status, [1..3] detail
 // then int32 arrays       tile_start[B+1], req_lo[B], req_hi[B], req_wfirst[B],
-//                         req_wlast[B], cost_start[B+1], worker_begin[W+1], split_list[W+1]
+//                         req_wlast[B], cost_start[B+1], worker_begin[W+1], split_list[W+1], worker_req[W+1]
 //                         (status[8] = number of entries of split_list)
+// then (16-B aligned)     split_rec [W+1] int4
 // then (256-B aligned)    partial_lse [2W][h] fp32
 // then (256-B aligned)    partial_scale [2W][h] fp32 (f16 partial outputs only: the power of two a row was divided by)
 // then (256-B aligned)    partial_out [2W][h][512] fp32
@@ -139,7 +140,7 @@ struct DecodeParams {
     int32_t num_workers;
     int32_t request_overhead_tiles;   // per-request cost the plan adds to the tile count
     int32_t plan_mode;                // kPlanWorkspace, kPlanInline or kPlanWhole
-    int32_t q_by_hand;                // e4m3 kernels: the query rows come by plain loads (strides that a tensor map cannot state)
+    int32_t q_by_hand;                // e4m3 pair kernel: its warps copy the query rows (strides that a tensor map cannot state)
     int32_t clear_status;             // 1: no plan kernel ran (its partition is taken again): block 0 clears the error words
     const int32_t *kv_begin, *kv_end; // the inline modes read the ranges themselves
     int4 *split_rec;                  // kPlanInline: where block 0 leaves the combine kernel's records
@@ -175,7 +176,8 @@ __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddep
 // Where a decode kernel's partition comes from.  Workspace: the plan kernel wrote it.  Inline: a batch of at most 32
 // requests is one lane each, so a warp of every CTA works the partition out for itself in a shuffle scan while the plan
 // kernel of such a call would still be in its launch (a tiny decode: 16.4 us with the plan kernel in front, see
-// build_inline_plan); the numbers are the plan kernel's.  Whole: inline, and no request is cut -- worker i takes request
+// build_inline_plan); the requests are cut where the plan kernel cuts them, though by other workers where all the work costs less than
+// there are (cut_workers).  Whole: inline, and no request is cut -- worker i takes request
 // i -- so that there is nothing to combine either.
 enum { kPlanWorkspace = 0, kPlanInline = 1, kPlanWhole = 2 };
 constexpr int kInlinePlanRequests = 32;
@@ -208,7 +210,10 @@ __device__ __forceinline__ void lane_range(const DecodeParams &p, int lane, int 
     if (lane < p.B) effective_range(load_l2(p.seq_lens + lane), p.kv_begin, p.kv_end, lane, p.len_cap, lo, hi);
 }
 
-// Workers that an inline plan cuts the work for: no more than it costs tiles, or some would start where the next one does.
+// Workers that an inline plan cuts the work for: no more than the work costs (tiles, and the overhead of each request).  Their shares
+// then begin at different costs, so that from the first to the last worker of a request each has a piece of it, as the combine kernel takes
+// for granted.  (A worker whose share begins in a request's overhead, where the next one's does too, has nothing: it stands in front of
+// that request's first worker.)
 __device__ __forceinline__ int cut_workers(const DecodeParams &p, int cost) { return min(p.num_workers, cost); }
 
 // One warp of a CTA: the plan, as far as worker `worker` needs it, from the lanes' ranges.

@@ -112,8 +112,8 @@ struct Layout {
 
 // Issued by the elected lane of a converged warp; the operands are uniform.  `a_at`, `b_at`: 16-byte units added to the descriptors'
 // addresses.  Only the low words of the descriptors move with them, and what they start from is said to be uniform: with 64-bit sums, and
-// addresses that only happen to be the same in all lanes, an issuer is slower than the tensor pipe (128 heads: 150 requests of 6,000 tokens
-// 288 us, now 266; the rollout batch 680 and 627).
+// addresses that only happen to be the same in all lanes, an issuer is slower than the tensor pipe (this alone, 128 heads: 150 requests of
+// 6,000 tokens 306 and 248 us, one of 500,000 166 and 129, 512 rollout requests 720 and 577; 64 heads, half the MMAs: no difference).
 __device__ __forceinline__ void umma_e4m3_pair(uint32_t elected, uint32_t d_tmem, uint64_t a_desc, uint32_t a_at, uint64_t b_desc, uint32_t b_at, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
         "{\n\t.reg .pred p, q;\n\t.reg .b64 a, b;\n\t"

@@ -5,9 +5,11 @@
 // Eight warps of every decode CTA do it, so a listed row crosses HBM once and its 1,152 dequantised bytes never leave the SM.
 // 64 requests x 2,048 tokens on 128 heads: 82 us a call.  (A kernel in front of the decode that wrote them to a dense cache took
 // 46 us of 107.  The same warps writing to a ring of pages in L2 for TMA loads: 143 us, the fences between a warp's
-// global stores and the copy engine's reads cost 3,000 cycles a tile.)  Neither the conversions bound
-// it (74 us without them) nor the row loads (82 without): it is the ring, a stage being held from its first store over the own rows, the
-// lag, the other CTA's rows and P.V, with four of them (one tile of lag more or less: 5 and 13 us slower).  A register is loaded
+// global stores and the copy engine's reads cost 3,000 cycles a tile.)  What bounds it
+// is the gathering warps' own way round their loop: of 3,650 cycles a tile (CTA 0 of that call, traced) 1,840 go with the own rows, 735 with the
+// other CTA's columns and 1,080 with the loads and addresses of the next, and none with waiting, for a stage has been free for 2,700 cycles when they
+// come to it and QK^T has long retired.  No one part of the work is all of it: 74 us without the conversions, 82 without the row loads.
+// (One tile of lag more or less: 5 and 13 us slower.)  A register is loaded
 // again for the next tile as soon as it has been converted, and the addresses of a warp's next 32 rows -- list entry, page id, row -- are resolved one
 // link of that chain per step.  The loop has one body, not unrolled over tiles: the CTA's warps are in loops of five kinds,
 // and with 45 KB of code in this one they waited for instructions.

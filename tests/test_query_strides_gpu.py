@@ -1,6 +1,6 @@
-"""The e4m3 kernels' query rows arrive by TMA, or by plain loads where the strides are none that a tensor map can state (one query
-for all requests, a stride of 0): the same bits either way, for slices that end inside a group of eight heads, rows of zeros and rows
-whose largest value is in any chunk."""
+"""The query rows of the e4m3 pair kernel (33 heads and more, or several rows per request) arrive by TMA, or are copied by its warps where
+the strides are none that a tensor map can state (one query for all requests, a stride of 0): the same bits either way, for slices that end
+inside a group of eight heads, rows of zeros and rows whose largest value is in any chunk.  (Up to 32 heads there is one way only.)"""
 import numpy as np
 import pytest
 
